@@ -74,7 +74,7 @@ namespace {
 
 constexpr int kBT = 256;          // threads of the per-problem passes
 constexpr int kScal = 8;          // doubles of per-problem solver scalars
-// scal[8p + 0] ball scale * mu, 1 ||d||, 2 gamma, 3 power-iteration sum
+// scal[8p + 2] gamma, 3 power-iteration sum
 
 cudaStream_t as_stream(void *s) { return static_cast<cudaStream_t>(s); }
 
@@ -128,7 +128,10 @@ __global__ void __launch_bounds__(kBT)
 k_bs_dual_residual(const BProb *__restrict__ tab, const float2 *__restrict__ u, float2 *__restrict__ r,
                    const float2 *__restrict__ y, const double *__restrict__ mu, double *__restrict__ part) {
   const BProb P = tab[blockIdx.y];
-  const float inv_mu = float(1.0 / mu[blockIdx.y]);
+  __shared__ float inv_mu_s;
+  if (threadIdx.x == 0) inv_mu_s = float(1.0 / mu[blockIdx.y]);
+  __syncthreads();
+  const float inv_mu = inv_mu_s;
   double acc = 0;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < P.m; i += int64_t(gridDim.x) * blockDim.x) {
     const int64_t k = P.vis_off + i;
@@ -141,23 +144,32 @@ k_bs_dual_residual(const BProb *__restrict__ tab, const float2 *__restrict__ u, 
   if (threadIdx.x == 0) part[int64_t(blockIdx.y) * gridDim.x + blockIdx.x] = t;
 }
 
-// thread per problem: scal[0] = max(0, 1 - eps/||d||) mu, scal[1] = ||d||
-__global__ void k_bs_ball_scale(int np, int nbx, const double *__restrict__ part, const double *__restrict__ eps,
-                                const double *__restrict__ mu, double *__restrict__ scal) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= np) return;
-  double s = 0;
-  for (int i = 0; i < nbx; ++i) s += part[int64_t(p) * nbx + i];
-  const double nd = sqrt(s);
-  const double f = (nd > 0) ? fmax(0.0, 1.0 - eps[p] / nd) : 0.0;
-  scal[p * kScal + 0] = f * mu[p];
-  scal[p * kScal + 1] = nd;
+// f(sum of problem blockIdx.y's nbx block partials), the same float in every
+// thread: each block that needs it adds the (at most 64) partials itself, in one
+// warp, and one thread evaluates f (FP64 divisions and roots in every thread of
+// every block cost more than the launch they save).
+template <class F>
+__device__ __forceinline__ float of_problem_sum(const double *__restrict__ part, int nbx, F f) {
+  __shared__ float r;
+  if (threadIdx.x < 32) {
+    double v = 0;
+    for (int i = threadIdx.x; i < nbx; i += 32) v += part[int64_t(blockIdx.y) * nbx + i];
+    v = warp_sum_d(v);
+    if (threadIdx.x == 0) r = f(v);
+  }
+  __syncthreads();
+  return r;
 }
 
-__global__ void k_bs_dual_update(const BProb *__restrict__ tab, const float2 *__restrict__ d,
-                                 const double *__restrict__ scal, float2 *__restrict__ u) {
+// u = f d, f = max(0, 1 - eps/||d||) mu with ||d||^2 the sum of the problem's partials
+__global__ void __launch_bounds__(kBT)
+k_bs_dual_update(const BProb *__restrict__ tab, const float2 *__restrict__ d, const double *__restrict__ part, int nbx,
+                 const double *__restrict__ eps, const double *__restrict__ mu, float2 *__restrict__ u) {
   const BProb P = tab[blockIdx.y];
-  const float f = float(scal[blockIdx.y * kScal + 0]);
+  const float f = of_problem_sum(part, nbx, [&](double s) {
+    const double nd = sqrt(s);
+    return float(((nd > 0) ? fmax(0.0, 1.0 - eps[blockIdx.y] / nd) : 0.0) * mu[blockIdx.y]);
+  });
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < P.m; i += int64_t(gridDim.x) * blockDim.x)
     u[P.vis_off + i] = cscale(d[P.vis_off + i], f);
 }
@@ -184,18 +196,20 @@ k_bs_image_part(const BProb *__restrict__ tab, const float *__restrict__ x, doub
   const BProb P = tab[blockIdx.y];
   const int64_t n = int64_t(P.N) * P.N;
   double acc = 0;
+  float mx = 0.f;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
-    const double v = x[P.img_off + i];
-    acc = MODE == 0 ? fmax(acc, fabs(v)) : acc + v * v;
+    const float v = x[P.img_off + i];
+    if (MODE == 0) mx = fmaxf(mx, fabsf(v));
+    else acc += double(v) * v;
   }
   if (MODE == 0) {
-    for (int o = 16; o; o >>= 1) acc = fmax(acc, __shfl_xor_sync(0xffffffffu, acc, o));
-    __shared__ double red[kBT / 32];
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    __shared__ float red[kBT / 32];
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = mx;
     __syncthreads();
     if (threadIdx.x == 0) {
-      double t = 0;
-      for (int i = 0; i < kBT / 32; ++i) t = fmax(t, red[i]);
+      float t = 0.f;
+      for (int i = 0; i < kBT / 32; ++i) t = fmaxf(t, red[i]);
       part[int64_t(blockIdx.y) * gridDim.x + blockIdx.x] = t;
     }
   } else {
@@ -204,25 +218,29 @@ k_bs_image_part(const BProb *__restrict__ tab, const float *__restrict__ x, doub
   }
 }
 
-// thread per problem: MODE 0: scal[2] = frac * max(part); MODE 1: scal[3] = sum(part)
-template <int MODE>
-__global__ void k_bs_image_scalar(int np, int nbx, const double *__restrict__ part, double frac,
-                                  double *__restrict__ scal) {
+// thread per problem: scal[2] = frac * max(part)
+__global__ void k_bs_gamma(int np, int nbx, const double *__restrict__ part, double frac, double *__restrict__ scal) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= np) return;
   double v = 0;
-  for (int i = 0; i < nbx; ++i) v = MODE == 0 ? fmax(v, part[int64_t(p) * nbx + i]) : v + part[int64_t(p) * nbx + i];
-  if (MODE == 0) scal[p * kScal + 2] = frac * v;
-  else scal[p * kScal + 3] = v;
+  for (int i = 0; i < nbx; ++i) v = fmax(v, part[int64_t(p) * nbx + i]);
+  scal[p * kScal + 2] = frac * v;
 }
 
-// x = z / sqrt(scal[3]) (power iteration), or the unit impulse at the image centre
-// (start) when scal is null
-__global__ void k_bs_scale_image(const BProb *__restrict__ tab, const float *__restrict__ z,
-                                 const double *__restrict__ scal, float *__restrict__ x) {
+// x = z / sqrt(s), s the sum of the problem's partials, left in scal[3] (power
+// iteration), or the unit impulse at the image centre (start) when scal is null
+__global__ void __launch_bounds__(kBT)
+k_bs_scale_image(const BProb *__restrict__ tab, const float *__restrict__ z, const double *__restrict__ part, int nbx,
+                 double *__restrict__ scal, float *__restrict__ x) {
   const BProb P = tab[blockIdx.y];
   const int64_t n = int64_t(P.N) * P.N;
-  const float f = scal ? float(1.0 / sqrt(scal[blockIdx.y * kScal + 3])) : 0.f;
+  float f = 0.f;
+  if (scal) {
+    f = of_problem_sum(part, nbx, [&](double s) {
+      if (blockIdx.x == 0) scal[blockIdx.y * kScal + 3] = s;
+      return float(1.0 / sqrt(s));
+    });
+  }
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
     x[P.img_off + i] = scal ? z[P.img_off + i] * f : (i == int64_t(P.N / 2) * P.N + P.N / 2 ? 1.f : 0.f);
 }
@@ -346,11 +364,9 @@ wproj_status dr_iteration(wproj_batch *b, const float2 *y, int inner, float lamb
     WPROJ_TRY(bphi_adj(b, u, x, z, 1, s));   // x = z - Re Phi^H u
     WPROJ_TRY(bphi(b, x, r, s));             // r = Phi x
     k_bs_dual_residual<<<dim3(nbm, b->np), kBT, 0, s>>>(tab, u, r, y, b->mu.as<double>(), part);
-    k_bs_ball_scale<<<ceil_div(b->np, 128), 128, 0, s>>>(b->np, nbm, part, b->eps.as<double>(), b->mu.as<double>(),
-                                                         scal);
-    k_bs_dual_update<<<dim3(nbm, b->np), kBT, 0, s>>>(tab, r, scal, u);
+    k_bs_dual_update<<<dim3(nbm, b->np), kBT, 0, s>>>(tab, r, part, nbm, b->eps.as<double>(), b->mu.as<double>(), u);
     WPROJ_CHECK_LAUNCH("batch dual step");
-    b->launches += 3;
+    b->launches += 2;
   }
   WPROJ_TRY(bphi_adj(b, u, x, z, 1, s));     // x = P_B(z)
   float *px = x;
@@ -371,14 +387,13 @@ wproj_status power_mu(wproj_batch *b, int iters, cudaStream_t s) {
   float2 *r = b->r.as<float2>();
   double *scal = b->scal.as<double>(), *part = b->part.as<double>();
   const int nbn = nbx_for(b->max_img);
-  k_bs_scale_image<<<dim3(nbn, b->np), kBT, 0, s>>>(tab, nullptr, nullptr, x);
+  k_bs_scale_image<<<dim3(nbn, b->np), kBT, 0, s>>>(tab, nullptr, nullptr, 0, nullptr, x);
   WPROJ_CHECK_LAUNCH("batch power start");
   for (int it = 0; it < iters; ++it) {
     WPROJ_TRY(bphi(b, x, r, s));
     WPROJ_TRY(bphi_adj(b, r, z, nullptr, 0, s));
     k_bs_image_part<1><<<dim3(nbn, b->np), kBT, 0, s>>>(tab, z, part);
-    k_bs_image_scalar<1><<<ceil_div(b->np, 128), 128, 0, s>>>(b->np, nbn, part, 0.0, scal);
-    k_bs_scale_image<<<dim3(nbn, b->np), kBT, 0, s>>>(tab, z, scal, x);
+    k_bs_scale_image<<<dim3(nbn, b->np), kBT, 0, s>>>(tab, z, part, nbn, scal, x);
     WPROJ_CHECK_LAUNCH("batch power iteration");
   }
   k_bs_mu<<<ceil_div(b->np, 128), 128, 0, s>>>(b->np, scal, b->mu.as<double>());
@@ -646,8 +661,8 @@ wproj_status batch_solve_impl(wproj_batch *b, const float2 *y, const double *eps
       WPROJ_TRY(bphi_adj(b, y, b->z.as<float>(), nullptr, 0, s));
     }
     k_bs_image_part<0><<<dim3(nbn, b->np), kBT, 0, s>>>(tab, b->z.as<float>(), b->part.as<double>());
-    k_bs_image_scalar<0><<<ceil_div(b->np, 128), 128, 0, s>>>(b->np, nbn, b->part.as<double>(), prm.gamma_frac,
-                                                              b->scal.as<double>());
+    k_bs_gamma<<<ceil_div(b->np, 128), 128, 0, s>>>(b->np, nbn, b->part.as<double>(), prm.gamma_frac,
+                                                    b->scal.as<double>());
     WPROJ_CHECK_LAUNCH("batch dr init");
     WPROJ_CUDA(cudaMemsetAsync(b->u.ptr, 0, sizeof(float2) * b->m, s));
   }

@@ -235,10 +235,19 @@ k_grid(const int32_t *__restrict__ chunk_tile, const int64_t *__restrict__ chunk
   }
 }
 
-// tile_prob / tab (batches): blockIdx.x is a tile of the whole batch
-__global__ void k_grid_reduce(const int32_t *__restrict__ tile_chunk_ptr, const float2 *__restrict__ partial,
-                              int G, int TS, int nT, const int32_t *__restrict__ tile_prob,
-                              const BProb *__restrict__ tab, float2 *__restrict__ Xt2) {
+// Sum of each tile's chunk partials.  A block takes 32 cells of one tile (grid:
+// tiles x cells / 32), thread (cell, j) the chunks c0 + j, c0 + j + 8, ...; the 8
+// sums of a cell are added in j order, so the order is fixed.  Bound by latency
+// (the partials sit in L2): with a block per tile and one thread walking all
+// chunks of a cell, a 128^2 grid (16 tiles of ~150 chunks) kept 16 SMs busy for
+// 118 us; with 512 blocks of 8 chunk lanes a pair of Phi and Phi^H there fell from
+// 177 to 107 us (with the row sums of the tile stream a warp each).
+// tile_prob / tab (batches): blockIdx.x is a tile of the whole batch.
+constexpr int kRedLanes = 8;
+__global__ void __launch_bounds__(32 * kRedLanes)
+k_grid_reduce(const int32_t *__restrict__ tile_chunk_ptr, const float2 *__restrict__ partial, int G, int TS, int nT,
+              const int32_t *__restrict__ tile_prob, const BProb *__restrict__ tab, float2 *__restrict__ Xt2) {
+  __shared__ float2 red[kRedLanes][32];
   int tile = blockIdx.x;
   const int c0 = tile_chunk_ptr[tile], c1 = tile_chunk_ptr[tile + 1];
   if (tile_prob) {
@@ -250,9 +259,15 @@ __global__ void k_grid_reduce(const int32_t *__restrict__ tile_chunk_ptr, const 
   }
   const int tu = tile / nT, tv = tile % nT;
   const int cells = TS * TS;
-  for (int i = threadIdx.x; i < cells; i += blockDim.x) {
-    float2 s = make_float2(0.f, 0.f);
-    for (int c = c0; c < c1; ++c) s = cadd(s, partial[int64_t(c) * cells + i]);
+  const int i = blockIdx.y * 32 + (threadIdx.x & 31), j = threadIdx.x >> 5;   // TS * TS is a multiple of 32
+  float2 s = make_float2(0.f, 0.f);
+#pragma unroll 4
+  for (int c = c0 + j; c < c1; c += kRedLanes) s = cadd(s, partial[int64_t(c) * cells + i]);
+  red[j][threadIdx.x & 31] = s;
+  __syncthreads();
+  if (j == 0) {
+#pragma unroll
+    for (int q = 1; q < kRedLanes; ++q) s = cadd(s, red[q][threadIdx.x]);
     const int lu = i / TS, lv = i % TS;
     Xt2[int64_t(tu * TS + lu) * G + tv * TS + lv] = s;
   }
@@ -349,8 +364,8 @@ wproj_status grid(wproj_plan *p, const float2 *y, float2 *Xt2, cudaStream_t s) {
     WPROJ_CHECK_LAUNCH("grid");
   }
   ScopedTimer t(p, TC_REDUCE, s);
-  k_grid_reduce<<<g.nT * g.nT, 256, 0, s>>>(p->tile_chunk_ptr.as<int32_t>(), p->grid_partial.as<float2>(), g.G, g.tile,
-                                             g.nT, nullptr, nullptr, Xt2);
+  k_grid_reduce<<<dim3(g.nT * g.nT, g.tile * g.tile / 32), 32 * kRedLanes, 0, s>>>(
+      p->tile_chunk_ptr.as<int32_t>(), p->grid_partial.as<float2>(), g.G, g.tile, g.nT, nullptr, nullptr, Xt2);
   WPROJ_CHECK_LAUNCH("grid reduce");
   return WPROJ_OK;
 }
@@ -393,7 +408,8 @@ wproj_status batch_grid(const BatchOps &b, const float2 *y, float2 *partial, flo
       b.chunk_tile, b.chunk_lo, b.chunk_hi, b.meta, b.col, b.val, nullptr, y, 0, kTile, 0, b.chunk_prob, b.tab,
       partial);
   WPROJ_CHECK_LAUNCH("batch grid");
-  k_grid_reduce<<<(unsigned)b.n_tiles, 256, 0, s>>>(b.tile_chunk_ptr, partial, 0, kTile, 0, b.tile_prob, b.tab, Xt2);
+  k_grid_reduce<<<dim3((unsigned)b.n_tiles, kTile), 32 * kRedLanes, 0, s>>>(b.tile_chunk_ptr, partial, 0, kTile, 0,
+                                                                       b.tile_prob, b.tab, Xt2);
   WPROJ_CHECK_LAUNCH("batch grid reduce");
   return WPROJ_OK;
 }

@@ -37,21 +37,29 @@ k_dual_residual(int64_t m, const float2 *__restrict__ u, float2 *__restrict__ r,
   if (threadIdx.x == 0) part[blockIdx.x] = t;
 }
 
-// scal[0] = max(0, 1 - eps/||d||) * mu
-__global__ void k_ball_scale(const double *__restrict__ part, int n, double eps, double mu,
-                             double *__restrict__ scal) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s = 0;
-  for (int i = 0; i < n; ++i) s += part[i];
-  const double nd = sqrt(s);
-  const double f = (nd > 0) ? fmax(0.0, 1.0 - eps / nd) : 0.0;
-  scal[0] = f * mu;
-  scal[1] = nd;
+// f(sum of the n block partials), the same float in every thread of the block:
+// every block of the pass that needs it adds them again (n <= kRedBlocks, in L2)
+// instead of waiting for a launch of its own; one thread evaluates f (FP64
+// divisions and roots in every thread would cost more than that launch).
+template <class F>
+__device__ __forceinline__ float of_sum(const double *__restrict__ part, int n, F f) {
+  __shared__ float r;
+  double v = 0;
+  for (int i = threadIdx.x; i < n; i += kRedThreads) v += part[i];
+  v = block_sum_d<kRedThreads>(v);
+  if (threadIdx.x == 0) r = f(v);
+  __syncthreads();
+  return r;
 }
 
-__global__ void k_dual_update(int64_t m, const float2 *__restrict__ d, const double *__restrict__ scal,
-                              float2 *__restrict__ u) {
-  const float f = float(scal[0]);
+// u = f d, f = max(0, 1 - eps/||d||) mu with ||d||^2 = the sum of part
+__global__ void __launch_bounds__(kRedThreads)
+k_dual_update(int64_t m, const float2 *__restrict__ d, const double *__restrict__ part, int n, double eps, double mu,
+              float2 *__restrict__ u) {
+  const float f = of_sum(part, n, [&](double s) {
+    const double nd = sqrt(s);
+    return float(((nd > 0) ? fmax(0.0, 1.0 - eps / nd) : 0.0) * mu);
+  });
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < m; i += int64_t(gridDim.x) * blockDim.x)
     u[i] = cscale(d[i], f);
 }
@@ -84,12 +92,12 @@ k_absmax_part(int64_t n, const float *__restrict__ x, double *__restrict__ part)
   }
 }
 
-// scal[2] = frac * max(part)
+// scal[2] = frac * max(part); one warp
 __global__ void k_gamma(const double *__restrict__ part, int n, double frac, double *__restrict__ scal) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
   double mx = 0;
-  for (int i = 0; i < n; ++i) mx = fmax(mx, part[i]);
-  scal[2] = frac * mx;
+  for (int i = threadIdx.x; i < n; i += 32) mx = fmax(mx, part[i]);
+  for (int o = 16; o; o >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (threadIdx.x == 0) scal[2] = frac * mx;
 }
 
 template <int ABS>
@@ -115,17 +123,22 @@ k_resid_part(int64_t m, const float2 *__restrict__ a, const float2 *__restrict__
   if (threadIdx.x == 0) part[blockIdx.x] = t;
 }
 
-__global__ void k_sum_parts(const double *__restrict__ part, int n, double *__restrict__ out) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  double s = 0;
-  for (int i = 0; i < n; ++i) s += part[i];
-  *out = s;
+__global__ void __launch_bounds__(kRedThreads)
+k_sum_parts(const double *__restrict__ part, int n, double *__restrict__ out) {
+  double v = 0;
+  for (int i = threadIdx.x; i < n; i += kRedThreads) v += part[i];
+  v = block_sum_d<kRedThreads>(v);
+  if (threadIdx.x == 0) *out = v;
 }
 
-// x = z / sqrt(scal[3])
-__global__ void k_normalise(int64_t n, const float *__restrict__ z, const double *__restrict__ scal,
-                            float *__restrict__ x) {
-  const float f = float(1.0 / sqrt(scal[3]));
+// x = z / sqrt(s), s = the sum of part, which block 0 leaves in *sum
+__global__ void __launch_bounds__(kRedThreads)
+k_normalise(int64_t n, const float *__restrict__ z, const double *__restrict__ part, int nb, double *__restrict__ sum,
+            float *__restrict__ x) {
+  const float f = of_sum(part, nb, [&](double s) {
+    if (blockIdx.x == 0) *sum = s;
+    return float(1.0 / sqrt(s));
+  });
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
     x[i] = z[i] * f;
 }
@@ -168,10 +181,9 @@ wproj_status power_norm2_impl(wproj_plan *p, int iters, double *out, cudaStream_
     WPROJ_TRY(apply_phi_adj(p, r, z, nullptr, nullptr, 0, s));
     const int nb = grid_for(n);
     k_sum_part<0><<<nb, kRedThreads, 0, s>>>(n, z, part);
-    k_sum_parts<<<1, 1, 0, s>>>(part, nb, scal + 3);
-    k_normalise<<<grid_for(n), kRedThreads, 0, s>>>(n, z, scal, x);
+    k_normalise<<<nb, kRedThreads, 0, s>>>(n, z, part, nb, scal + 3, x);
     WPROJ_CHECK_LAUNCH("power iteration");
-    p->launches += 3;
+    p->launches += 2;
   }
   double h = 0;
   WPROJ_CUDA(cudaMemcpyAsync(&h, scal + 3, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -221,7 +233,7 @@ wproj_status solve_bpdn_impl(wproj_plan *p, const float2 *y, double eps, const w
     }
     ScopedTimer t(p, TC_SOLVER, s);
     k_absmax_part<<<nbn, kRedThreads, 0, s>>>(n, z, part);
-    k_gamma<<<1, 1, 0, s>>>(part, nbn, prm.gamma_frac, scal);
+    k_gamma<<<1, 32, 0, s>>>(part, nbn, prm.gamma_frac, scal);
     WPROJ_CUDA(cudaMemsetAsync(u, 0, sizeof(float2) * m, s));
     WPROJ_CHECK_LAUNCH("dr init");
     p->launches += 2;
@@ -235,10 +247,9 @@ wproj_status solve_bpdn_impl(wproj_plan *p, const float2 *y, double eps, const w
       WPROJ_TRY(apply_phi(p, x, nullptr, r, s));               // r = Phi x
       ScopedTimer t(p, TC_SOLVER, s);
       k_dual_residual<<<nbm, kRedThreads, 0, s>>>(m, u, r, y, float(1.0 / mu), part);
-      k_ball_scale<<<1, 1, 0, s>>>(part, nbm, eps, mu, scal);
-      k_dual_update<<<nbm, kRedThreads, 0, s>>>(m, r, scal, u);
+      k_dual_update<<<nbm, kRedThreads, 0, s>>>(m, r, part, nbm, eps, mu, u);
       WPROJ_CHECK_LAUNCH("dual step");
-      p->launches += 3;
+      p->launches += 2;
     }
     WPROJ_TRY(apply_phi_adj(p, u, x, nullptr, zi, 1, s));     // x = P_B(zi)
     if (psi) WPROJ_TRY(dwt2_impl(N, lev, psi, x, alpha, wk, &p->launches, s));
@@ -256,12 +267,12 @@ wproj_status solve_bpdn_impl(wproj_plan *p, const float2 *y, double eps, const w
     // residual ||y - Phi x|| and ||x||_1
     WPROJ_TRY(apply_phi(p, x, nullptr, r, s));
     k_resid_part<<<nbm, kRedThreads, 0, s>>>(m, r, y, part);
-    k_sum_parts<<<1, 1, 0, s>>>(part, nbm, scal + 4);
+    k_sum_parts<<<1, kRedThreads, 0, s>>>(part, nbm, scal + 4);
     if (psi) WPROJ_TRY(dwt2_impl(N, lev, psi, x, alpha, wk, &p->launches, s));
     k_sum_part<1><<<nbn, kRedThreads, 0, s>>>(n, alpha, part);
-    k_sum_parts<<<1, 1, 0, s>>>(part, nbn, scal + 5);
+    k_sum_parts<<<1, kRedThreads, 0, s>>>(part, nbn, scal + 5);
     WPROJ_CHECK_LAUNCH("solve info");
-    double h[4];   // gamma, ||d||, ||y - Phi x||^2, ||x||_1
+    double h[4];   // gamma, power-iteration sum, ||y - Phi x||^2, ||x||_1
     WPROJ_CUDA(cudaMemcpyAsync(h, scal + 2, sizeof(double) * 4, cudaMemcpyDeviceToHost, s));
     WPROJ_CUDA(cudaStreamSynchronize(s));
     info->iters_done = prm.iters;

@@ -194,16 +194,27 @@ int chunk_stride(int64_t n) {
   return 1;
 }
 
-// y_k = sum over row k's segments s and warps w of partial[4 s + w], in that
-// order, times the row scale
-__global__ void k_stream_reduce(int64_t m, const int64_t *__restrict__ seg_base, const float2 *__restrict__ partial,
-                                const float *__restrict__ row_scale, float2 *__restrict__ y) {
-  const int64_t k = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+// y_k = sum over row k's segments s and warps w of partial[4 s + w], times the
+// row scale.  A warp takes a row: lane l sums the partials l, l + 32, ... of its
+// contiguous range and the lanes are added in a fixed tree.  (A thread per row
+// read with a stride of the row's range and filled 5 blocks at 1229 rows: 12 us
+// against 4.)
+__global__ void __launch_bounds__(256)
+k_stream_reduce(int64_t m, const int64_t *__restrict__ seg_base, const float2 *__restrict__ partial,
+                const float *__restrict__ row_scale, float2 *__restrict__ y) {
+  const int lane = threadIdx.x & 31;
+  const int64_t k = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
   if (k >= m) return;
   float2 acc = make_float2(0.f, 0.f);
-  for (int64_t i = seg_base[k] * kWarps; i < seg_base[k + 1] * kWarps; ++i) acc = cadd(acc, partial[i]);
-  if (row_scale) acc = cscale(acc, row_scale[k]);
-  y[k] = acc;
+  const int64_t i1 = seg_base[k + 1] * kWarps;
+#pragma unroll 4
+  for (int64_t i = seg_base[k] * kWarps + lane; i < i1; i += 32) acc = cadd(acc, partial[i]);
+#pragma unroll
+  for (int o = 16; o; o >>= 1) {
+    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
+    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
+  }
+  if (lane == 0) y[k] = row_scale ? cscale(acc, row_scale[k]) : acc;
 }
 
 template <int VDT, bool DEGRID>
@@ -262,7 +273,7 @@ wproj_status degrid_stream(wproj_plan *p, const float2 *Xt, float2 *partial, cud
 }
 
 wproj_status degrid_stream_reduce(wproj_plan *p, const float2 *partial, float2 *y, cudaStream_t s) {
-  k_stream_reduce<<<ceil_div(p->m, 256), 256, 0, s>>>(
+  k_stream_reduce<<<ceil_div(p->m, 8), 256, 0, s>>>(
       p->m, p->seg_base.as<int64_t>(), partial,
       p->g.value_dtype == WPROJ_VAL_F32 ? nullptr : p->row_scale.as<float>(), y);
   WPROJ_CHECK_LAUNCH("degrid (tile stream) reduce");

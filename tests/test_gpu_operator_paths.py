@@ -1,0 +1,77 @@
+"""Phi and Phi^H through every storage and work split against the stored G itself:
+the rows the plan exports (FP64 copies of its own values) applied by SciPy between
+the oracle's FP64 transforms, so that only the operator kernels are under test.
+
+Tolerance: FP32 sums and transforms.  A transform of up to 12 radix-4 / radix-2
+stages and a sum of n terms in blocks each lose a few units of 2^-24 of the 2-norm;
+1e-5 (170 units) covers both with the stored values taken as exact."""
+import numpy as np
+import pytest
+import scipy.sparse
+import torch
+
+from oracle import wproj_oracle as O
+from paper_1307_3424_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+L = synth.fov_L()
+
+
+@pytest.fixture(scope="module")
+def wp():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1307_3424_gb300 import wproj
+    return wproj
+
+
+def exported(plan):
+    c = plan.csr()
+    col, val = c.rows(0, c.m)
+    val = val.cpu()
+    if c.value_dtype == "f32":
+        val = val.numpy().astype(np.complex128)
+    else:
+        v = val.float().numpy().astype(np.float64)
+        rs = np.repeat(c.row_scale.cpu().numpy().astype(np.float64), np.diff(c.row_ptr.cpu().numpy()))
+        val = (v[:, 0] + 1j * v[:, 1]) * rs
+    return scipy.sparse.csr_matrix((val, col.cpu().numpy().astype(np.int64), c.row_ptr.cpu().numpy()),
+                                   shape=(c.m, c.n_cols))
+
+
+def uvw_cells(rng, M, N, wmax, edge=0.0):
+    """Uniform disk, w_c ~ U[0, wmax] cells; a share `edge` of the rows at the band's
+    corner, where kernels wrap around the grid."""
+    uv = synth.uv_points(rng, M, synth.band_limit(N, L), N, "uniform")
+    k = int(edge * M)
+    uv[:k] = -synth.band_limit(N, L) * (1 - 3.0 * rng.uniform(0, 1, (k, 2)) / N)
+    w = 2.0 * rng.uniform(0, wmax, M) / (L * L)
+    return np.ascontiguousarray(np.concatenate([uv, w[:, None]], axis=1))
+
+
+def check_operators(plan, N, W, rng, tol=1e-5):
+    geo = O.Geometry(N, L, W=W)
+    G = exported(plan)
+    x = rng.standard_normal((N, N)).astype(np.float32)
+    y = (rng.standard_normal(G.shape[0]) + 1j * rng.standard_normal(G.shape[0])).astype(np.complex64)
+    xg, yg = torch.from_numpy(x).cuda(), torch.from_numpy(y).cuda()
+    yr, xr = O.phi(geo, G, x.astype(np.float64)), np.real(O.phi_adj(geo, G, y.astype(np.complex128)))
+    for _ in range(2):      # a second pass on the same buffers gives the same bits
+        py, px = plan.phi(xg).cpu().numpy(), plan.phi_adj(yg).cpu().numpy()
+        assert np.linalg.norm(py - yr) <= tol * np.linalg.norm(yr)
+        assert np.linalg.norm(px - xr) <= tol * np.linalg.norm(xr)
+        assert np.abs(py - yr).max() <= 30 * tol * np.abs(yr).max()   # no row and no cell left out
+        assert np.abs(px - xr).max() <= 30 * tol * np.abs(xr).max()
+
+
+# dense rows: 16^2 grid (one 16-cell tile), one to ~100 chunks a tile, each format
+@pytest.mark.parametrize("N,M,wmax,fmt,value", [(8, 5, 0.5, "auto", "f32"), (16, 700, 2.0, "columns", "f32"),
+                                                (32, 40, 4.0, "mask", "f32"), (64, 300, 30.0, "mask", "f32"),
+                                                (64, 300, 30.0, "mask", "bf16"), (128, 33, 60.0, "columns", "f16")])
+def test_dense_rows(wp, N, M, wmax, fmt, value):
+    rng = np.random.default_rng(N + M)
+    plan = wp.Plan(N, L, value_dtype=value, index_format=fmt)
+    plan.build_kernels(torch.from_numpy(uvw_cells(rng, M, N, wmax)).cuda(), 0.99)
+    check_operators(plan, N, 4, rng)
+    plan.close()
