@@ -47,6 +47,9 @@ __device__ __forceinline__ float abs2_rn(float2 z) {
   return __fadd_rn(__fmul_rn(z.x, z.x), __fmul_rn(z.y, z.y));
 }
 
+// GELU, the erf form
+__device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
+
 // Kaiser-Bessel gridding kernel of support W (unnormalised), t in cells
 __device__ __forceinline__ double kb_dev(double t, int W, double beta) {
   const double r = 2.0 * t / W;

@@ -17,11 +17,24 @@
 //            128B-swizzle K-major shared-memory descriptors, commits each slice
 //            to its stage's `empty` barrier and the tile to `acc_full`;
 //   warps 2-5  epilogue: wait for `acc_full`, read the accumulator with
-//            tcgen05.ld (warp w reads tensor-memory lanes 32 (w mod 4) ..), add
-//            the bias, transpose each 32 x 32 block through shared memory so that
-//            stores are row-contiguous, store, and release the accumulator.
+//            tcgen05.ld (warp w reads tensor-memory lanes 32 (w mod 4) .., a lane
+//            one row of the tile), add the bias, apply GELU where asked, store
+//            32 bytes a lane (st.global.v8: whole sectors), and release the
+//            accumulator.
 // So the loads of tile i + 1 and the MMAs of tile i + 1 overlap the epilogue of
 // tile i.  Four stages of 48 KB (BN = 256); 1 CTA per SM.
+//
+// What bounds it: at large K the tensor cores; at the network's K = 256 the
+// epilogue and the output's bytes (65536 x 3072 FP32, 805 MB).  Storing 4 bytes a
+// lane after a transpose through shared memory took ~130 instructions per 32 x
+// 32 block in the one epilogue warp of each scheduler (330 us for that output);
+// a lane's own row in 32-byte stores takes ~50.
+//
+// Split K: a product with fewer tiles than SMs (weight gradients: 2 to 24 tiles
+// of K = batch) is cut into `splits` ranges of K slices, each range a work unit
+// of its own with its own FP32 partial product; the caller adds the partials in
+// order.  At 152 units against 2 tiles of 64 slices the chain of slices a CTA
+// walks falls from 64 to 2.
 //
 // Shapes: M, N multiples of 128, K a multiple of 64 (the callers pad).  Every
 // wait is bounded (2 s); a wait that runs out sets *err and its role stops, the
@@ -127,22 +140,82 @@ template <int BN>
 struct GemmSmem {
   unsigned char a[kStages][kSliceA];     // 1024-byte aligned (swizzle atoms)
   unsigned char b[kStages][BN * kBK * 2];
-  float epi[4][32 * 33];                 // epilogue transposes, one block per warp
   uint64_t full[kStages], empty[kStages], acc_full[2], acc_empty[2], never;
   uint32_t tmem_base;
 };
 
-template <int BN, bool OUT_BF16>
+// Z (FP32, optional with the other) and H (BF16): what the epilogue writes.
+// act: H = GELU(Z).  A store is 32 bytes a lane when `vec` (outputs 32-byte, bias
+// 16-byte aligned; rows are multiples of 128 elements), else element by element.
+struct EpiArgs {
+  const float *bias;
+  float *z;
+  __nv_bfloat16 *h;
+  int act, splits, vec;
+};
+
+__device__ __forceinline__ void st_global_v8(void *p, const uint32_t (&v)[8]) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+               "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+               : "memory");
+}
+
+// one lane's 32 consecutive elements of a row (already biased): Z at z, H at h
+__device__ __forceinline__ void store_row32(const float (&v)[32], float *z, __nv_bfloat16 *h, int act, int vec) {
+  if (z) {
+    if (vec) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        uint32_t w[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) w[i] = __float_as_uint(v[8 * q + i]);
+        st_global_v8(z + 8 * q, w);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) z[i] = v[i];
+    }
+  }
+  if (h) {
+    __nv_bfloat162 b[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      b[i] = act ? __floats2bfloat162_rn(gelu(v[2 * i]), gelu(v[2 * i + 1])) : __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+    if (vec) {
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        uint32_t w[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) w[i] = *reinterpret_cast<const uint32_t *>(&b[8 * q + i]);
+        st_global_v8(h + 16 * q, w);
+      }
+    } else {
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        h[2 * i] = b[i].x;
+        h[2 * i + 1] = b[i].y;
+      }
+    }
+  }
+}
+
+template <int BN>
 __global__ void __launch_bounds__(kThreads, 1)
 k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M, int N, int K,
-          const float *__restrict__ bias, void *__restrict__ C, int *__restrict__ err) {
+          const EpiArgs ep, int *__restrict__ err) {
   constexpr int kAccCols = BN;
   constexpr int kSliceB = BN * kBK * 2;
   extern __shared__ unsigned char smem_raw[];
   GemmSmem<BN> &sm =
       *reinterpret_cast<GemmSmem<BN> *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nN = N / BN, n_tiles = (M / kBM) * nN, nk = K / kBK;
+  // work unit t: split t mod splits of tile t / splits, K slices [k0, k1)
+  const int nN = N / BN, nk_all = K / kBK, sp_n = ep.splits, n_units = (M / kBM) * nN * sp_n;
+  auto slices = [&](int t, int &k0, int &k1) {
+    const int sp = t % sp_n;
+    k0 = int(int64_t(nk_all) * sp / sp_n);
+    k1 = int(int64_t(nk_all) * (sp + 1) / sp_n);
+  };
   if (threadIdx.x == 0) {
     for (int i = 0; i < kStages; ++i) {
       mbar_init(&sm.full[i], 1);    // the producer's arrive.expect_tx
@@ -174,9 +247,11 @@ k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
       uint32_t it = 0;
-      for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x) {
-        const int m0 = (t / nN) * kBM, n0 = (t % nN) * BN;
-        for (int k = 0; k < nk; ++k, ++it) {
+      for (int t = blockIdx.x; t < n_units && ok; t += gridDim.x) {
+        const int tile = t / sp_n, m0 = (tile / nN) * kBM, n0 = (tile % nN) * BN;
+        int k0, k1;
+        slices(t, k0, k1);
+        for (int k = k0; k < k1; ++k, ++it) {
           const int st = int(it % kStages);
           const uint32_t ph = (it / kStages) & 1u;
           if (!mbar_wait_bounded(&sm.empty[st], ph ^ 1u)) { ok = false; break; }
@@ -191,12 +266,14 @@ k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     if (lane == 0 && ok) {
       const uint32_t idesc = instr_desc(kBM, BN);
       uint32_t it = 0, ti = 0;
-      for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++ti) {
+      for (int t = blockIdx.x; t < n_units && ok; t += gridDim.x, ++ti) {
+        int k0, k1;
+        slices(t, k0, k1);
         const uint32_t buf = ti & 1u, aph = (ti >> 1) & 1u;
         if (!mbar_wait_bounded(&sm.acc_empty[buf], aph ^ 1u)) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         const uint32_t acc = tmem + buf * kAccCols;
-        for (int k = 0; k < nk; ++k, ++it) {
+        for (int k = k0; k < k1; ++k, ++it) {
           const int st = int(it % kStages);
           const uint32_t ph = (it / kStages) & 1u;
           if (!mbar_wait_bounded(&sm.full[st], ph)) { ok = false; break; }
@@ -206,7 +283,7 @@ k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
           for (int j = 0; j < kBK / 16; ++j) {   // K = 16 per MMA: 32 bytes along the swizzled row
             const uint64_t ad = smem_desc_sw128(a0 + j * 32);
             const uint64_t bd = smem_desc_sw128(b0 + j * 32);
-            const uint32_t accum = (k > 0 || j > 0) ? 1u : 0u;
+            const uint32_t accum = (k > k0 || j > 0) ? 1u : 0u;
             asm volatile(
                 "{\n\t.reg .pred p;\n\t"
                 "setp.ne.b32 p, %4, 0;\n\t"
@@ -234,10 +311,10 @@ k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   } else {
     // ---- epilogue (warps 2-5): tensor-memory lanes 32 (warp mod 4) ..
     const int lg = warp & 3;
-    float *blk = sm.epi[warp - 2];
     uint32_t ti = 0;
-    for (int t = blockIdx.x; t < n_tiles && ok; t += gridDim.x, ++ti) {
-      const int m0 = (t / nN) * kBM, n0 = (t % nN) * BN;
+    for (int t = blockIdx.x; t < n_units && ok; t += gridDim.x, ++ti) {
+      const int tile = t / sp_n, m0 = (tile / nN) * kBM, n0 = (tile % nN) * BN;
+      const int64_t row = (int64_t(t % sp_n) * M + m0 + lg * 32 + lane) * N + n0;   // this lane's row of its partial
       const uint32_t buf = ti & 1u, aph = (ti >> 1) & 1u;
       if (!mbar_wait_bounded(&sm.acc_full[buf], aph)) { ok = false; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -255,20 +332,21 @@ k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
               "=r"(r[30]), "=r"(r[31])
             : "r"(taddr)
             : "memory");
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        float bv[32];   // the same 32 values in every lane
 #pragma unroll
-        for (int i = 0; i < 32; ++i) blk[lane * 33 + i] = __uint_as_float(r[i]);
-        __syncwarp();
-        const int col = n0 + c0 + lane;
-        const float bv = bias ? __ldg(bias + col) : 0.f;
-#pragma unroll 4
-        for (int i = 0; i < 32; ++i) {
-          const int64_t rr = m0 + lg * 32 + i;
-          const float v = blk[i * 33 + lane] + bv;
-          if (OUT_BF16) reinterpret_cast<__nv_bfloat16 *>(C)[rr * N + col] = __float2bfloat16_rn(v);
-          else reinterpret_cast<float *>(C)[rr * N + col] = v;
+        for (int i = 0; i < 32; i += 4) {
+          float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (ep.bias) {
+            const float *bp = ep.bias + n0 + c0 + i;
+            b4 = ep.vec ? __ldg(reinterpret_cast<const float4 *>(bp)) : make_float4(bp[0], bp[1], bp[2], bp[3]);
+          }
+          bv[i] = b4.x; bv[i + 1] = b4.y; bv[i + 2] = b4.z; bv[i + 3] = b4.w;
         }
-        __syncwarp();
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        float v[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]) + bv[i];
+        store_row32(v, ep.z ? ep.z + row + c0 : nullptr, ep.h ? ep.h + row + c0 : nullptr, ep.act, ep.vec);
       }
       // this warp is done with the accumulator
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -322,41 +400,62 @@ wproj_status tensor_map(CUtensorMap *map, const __nv_bfloat16 *p, int rows, int 
 }
 
 template <int BN>
-wproj_status launch_gemm(int M, int N, int K, const __nv_bfloat16 *A, const __nv_bfloat16 *B, const float *bias,
-                         void *C, bool out_bf16, int *err, cudaStream_t s) {
+wproj_status launch_gemm(int M, int N, int K, const __nv_bfloat16 *A, const __nv_bfloat16 *B, const EpiArgs &ep, int sms,
+                         int *err, cudaStream_t s) {
   CUtensorMap ta, tb;
   WPROJ_TRY(tensor_map(&ta, A, M, K, kBM));
   WPROJ_TRY(tensor_map(&tb, B, N, K, BN));
-  int dev = 0, sms = 0;
-  WPROJ_CUDA(cudaGetDevice(&dev));
-  WPROJ_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  const int n_tiles = (M / kBM) * (N / BN);
-  const int grid = std::max(1, std::min(n_tiles, sms));
+  const int grid = std::max(1, std::min((M / kBM) * (N / BN) * ep.splits, sms));
   const size_t smem = sizeof(GemmSmem<BN>) + 1024;
-  if (out_bf16) {
-    WPROJ_CUDA(cudaFuncSetAttribute(k_gemm_ws<BN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_gemm_ws<BN, true><<<grid, kThreads, smem, s>>>(ta, tb, M, N, K, bias, C, err);
-  } else {
-    WPROJ_CUDA(cudaFuncSetAttribute(k_gemm_ws<BN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_gemm_ws<BN, false><<<grid, kThreads, smem, s>>>(ta, tb, M, N, K, bias, C, err);
-  }
+  WPROJ_CUDA(cudaFuncSetAttribute(k_gemm_ws<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  k_gemm_ws<BN><<<grid, kThreads, smem, s>>>(ta, tb, M, N, K, ep, err);
   WPROJ_CHECK_LAUNCH("gemm");
+  return WPROJ_OK;
+}
+
+wproj_status sm_count(int *sms) {
+  int dev = 0;
+  WPROJ_CUDA(cudaGetDevice(&dev));
+  WPROJ_CUDA(cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev));
   return WPROJ_OK;
 }
 
 }  // namespace
 
+// Ranges of K that fill the SMs: one when the tiles do, at most one per K slice.
+wproj_status gemm_splits(int M, int N, int K, int *splits) {
+  int sms = 0;
+  WPROJ_TRY(sm_count(&sms));
+  const int tiles = (M / kBM) * (N % 256 == 0 ? N / 256 : N / 128);
+  *splits = std::max(1, std::min(sms / std::max(1, tiles), K / kBK));
+  return WPROJ_OK;
+}
+
 // C = A B^T (+ bias); M, N multiples of 128, K a multiple of 64; A and B 16-byte
-// aligned (TMA); err: device int.  Tiles of 128 x 256 when N is a multiple of
-// 256, else 128 x 128.
-wproj_status gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16 *A, const __nv_bfloat16 *B, const float *bias,
-                          void *C, bool out_bf16, int *err, cudaStream_t s) {
+// aligned (TMA); err: device int.  Tiles of 128 x 256 when N is a multiple of 256
+// and they fill the SMs (or the K ranges do), else 128 x 128: 4096 x 256 x 256
+// has 32 of the former and 64 of the latter.
+wproj_status gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16 *A, const __nv_bfloat16 *B, const GemmOut &o,
+                          int *err, cudaStream_t s) {
   if (M % kBM || N % 128 || K % kBK || M <= 0 || N <= 0 || K <= 0)
     return fail(WPROJ_ERR_INVALID_ARG, "gemm: M, N must be multiples of 128 and K of 64");
   if ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(B)) & 15)
     return fail(WPROJ_ERR_INVALID_ARG, "gemm: A and B must be 16-byte aligned");
-  if (N % 256 == 0) return launch_gemm<256>(M, N, K, A, B, bias, C, out_bf16, err, s);
-  return launch_gemm<128>(M, N, K, A, B, bias, C, out_bf16, err, s);
+  if (o.splits < 1 || o.splits > K / kBK || (o.splits > 1 && (o.bias || o.bf16)))
+    return fail(WPROJ_ERR_INVALID_ARG, "gemm: invalid K split");
+  int sms = 0;
+  WPROJ_TRY(sm_count(&sms));
+  EpiArgs ep;
+  ep.bias = o.bias;
+  ep.z = o.f32;
+  ep.h = o.bf16;
+  ep.act = o.gelu ? 1 : 0;
+  ep.splits = o.splits;
+  ep.vec = ((reinterpret_cast<uintptr_t>(o.f32) | reinterpret_cast<uintptr_t>(o.bf16)) & 31) == 0 &&
+           (reinterpret_cast<uintptr_t>(o.bias) & 15) == 0;
+  if (N % 256 == 0 && (M / kBM) * (N / 256) * (2 * o.splits) > sms)
+    return launch_gemm<256>(M, N, K, A, B, ep, sms, err, s);
+  return launch_gemm<128>(M, N, K, A, B, ep, sms, err, s);
 }
 
 }  // namespace wproj
@@ -384,8 +483,11 @@ extern "C" wproj_status wproj_gemm_bf16(int32_t m, int32_t n, int32_t k, const v
   int *err = nullptr;
   WPROJ_CUDA(cudaGetSymbolAddress(reinterpret_cast<void **>(&err), g_gemm_err));
   WPROJ_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
-  WPROJ_TRY(gemm_bf16_tn(m, n, k, static_cast<const __nv_bfloat16 *>(a), static_cast<const __nv_bfloat16 *>(b), bias,
-                         c, out_bf16 != 0, err, s));
+  GemmOut o;
+  o.bias = bias;
+  if (out_bf16) o.bf16 = static_cast<__nv_bfloat16 *>(c);
+  else o.f32 = static_cast<float *>(c);
+  WPROJ_TRY(gemm_bf16_tn(m, n, k, static_cast<const __nv_bfloat16 *>(a), static_cast<const __nv_bfloat16 *>(b), o, err, s));
   int h = 0;
   WPROJ_CUDA(cudaMemcpyAsync(&h, err, sizeof(int), cudaMemcpyDeviceToHost, s));
   WPROJ_CUDA(cudaStreamSynchronize(s));

@@ -36,9 +36,10 @@ struct wproj_mlp {
   wproj::DevBuf W2t, W3t, W4t;          // BF16 transposes [in x out]
   int64_t step = 0;
   int64_t cap = 0;                      // batch capacity of the activation buffers
-  wproj::DevBuf Z1, Z2, Z3, H1, H2, H3, Y, dY, dYt, Ht, dZt, dH, dZ, dZ1, part, err;
-  wproj::DevBuf csum;                   // column-sum partials and the first layer's sums
-  int64_t csum_off = 0;
+  int64_t fcap = 0;                     // rows of the inference buffers (H1 .. H3)
+  wproj::DevBuf Z1, Z2, Z3, H1, H2, H3, Y, dY, dYt, Ht, dZt, dH, dZ, part, loss, err;
+  wproj::DevBuf split;                  // partial products of the split-K GEMMs
+  wproj::DevBuf csum;                   // column-sum partials of 64-row blocks
 };
 
 namespace wproj {
@@ -47,135 +48,302 @@ namespace {
 
 using namespace mlpk;
 
-__device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.f + erff(z * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_d(float z) {
   return 0.5f * (1.f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * __expf(-0.5f * z * z);
 }
 
-// first layer on the FP32 cores: Z1 = x0 W1^T + b1, H1 = GELU(Z1)
-__global__ void k_in_fwd(int64_t B, const float *__restrict__ x0, const float *__restrict__ P, float *__restrict__ Z1,
-                         __nv_bfloat16 *__restrict__ H1) {
-  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= B * kH) return;
-  const int64_t b = i / kH;
-  const int j = int(i % kH);
-  const float *W1 = P + oW1 + j * kIn;
-  const float z = P[oB1 + j] + W1[0] * x0[b * 3] + W1[1] * x0[b * 3 + 1] + W1[2] * x0[b * 3 + 2];
-  Z1[i] = z;
-  H1[i] = __float2bfloat16_rn(gelu(z));
+// first layer on the FP32 cores: Z1 = x0 W1^T + b1 (kept when Z1 is given),
+// H1 = GELU(Z1).  Thread j of a block holds weights of units 2j, 2j + 1 and walks
+// the block's rows, so the weights are read once a block and a warp stores whole
+// 128-byte lines (a thread per element read seven words for each BF16 it wrote:
+// 49 against 12 us for 65536 rows).
+constexpr int kInRows = 32;
+__global__ void __launch_bounds__(kH / 2)
+k_in_fwd(int64_t B, const float *__restrict__ x0, const float *__restrict__ P, float *__restrict__ Z1,
+         __nv_bfloat16 *__restrict__ H1) {
+  __shared__ float xs[kInRows * kIn];
+  const int64_t b0 = int64_t(blockIdx.x) * kInRows;
+  const int nb = int(B - b0 < kInRows ? B - b0 : kInRows);
+  for (int i = threadIdx.x; i < nb * kIn; i += blockDim.x) xs[i] = x0[b0 * kIn + i];
+  const int j = 2 * threadIdx.x;
+  float w[2][kIn], bias[2];
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    bias[u] = P[oB1 + j + u];
+#pragma unroll
+    for (int c = 0; c < kIn; ++c) w[u][c] = P[oW1 + (j + u) * kIn + c];
+  }
+  __syncthreads();
+#pragma unroll 4
+  for (int r = 0; r < nb; ++r) {
+    float z[2];
+#pragma unroll
+    for (int u = 0; u < 2; ++u) z[u] = bias[u] + w[u][0] * xs[3 * r] + w[u][1] * xs[3 * r + 1] + w[u][2] * xs[3 * r + 2];
+    const int64_t i = (b0 + r) * kH + j;
+    if (Z1) *reinterpret_cast<float2 *>(Z1 + i) = make_float2(z[0], z[1]);
+    *reinterpret_cast<__nv_bfloat162 *>(H1 + i) = __floats2bfloat162_rn(gelu(z[0]), gelu(z[1]));
+  }
 }
 
-__global__ void k_gelu_fwd(int64_t n, const float *__restrict__ Z, __nv_bfloat16 *__restrict__ H) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    H[i] = __float2bfloat16_rn(gelu(Z[i]));
+// ---- 64 x 64 blocks of a row-major matrix ----------------------------------------
+// The backward passes walk 64 x 64 blocks with 256 threads: thread (tx, ty) takes
+// columns 4 tx .. 4 tx + 3 of rows ty, ty + 16, ty + 32, ty + 48.  What the GEMMs
+// need of a block (BF16 rows, the BF16 transpose, column sums) leaves in one pass.
+constexpr int kBlk = 64;
+constexpr int kTLd = kBlk + 2;   // transposed rows of 33 words: 2-way store conflicts
+
+struct BlockSmem {
+  __nv_bfloat16 t[kBlk][kTLd];
+  float red[16][kBlk];
+};
+
+// the block's transpose from sm.t to out (leading dimension R) at (c0, r0); every
+// thread stores 32 bytes
+__device__ __forceinline__ void store_transposed(const BlockSmem &sm, __nv_bfloat16 *__restrict__ out, int64_t R,
+                                                 int64_t r0, int64_t c0) {
+  const int c = threadIdx.x >> 2, q = (threadIdx.x & 3) * 16;
+  const uint32_t *src = reinterpret_cast<const uint32_t *>(&sm.t[c][q]);
+  uint4 *dst = reinterpret_cast<uint4 *>(out + (c0 + c) * R + r0 + q);
+  dst[0] = make_uint4(src[0], src[1], src[2], src[3]);
+  dst[1] = make_uint4(src[4], src[5], src[6], src[7]);
 }
 
-// loss partials and dY = d loss / d y (BF16); rows [0, B)
+__device__ __forceinline__ void put_bf16x4(__nv_bfloat16 *p, __nv_bfloat162 a, __nv_bfloat162 b) {
+  uint2 u;
+  u.x = *reinterpret_cast<uint32_t *>(&a);
+  u.y = *reinterpret_cast<uint32_t *>(&b);
+  *reinterpret_cast<uint2 *>(p) = u;
+}
+
+// A sum in two floats: every addition keeps its error (Knuth's two-sum) and every
+// square its rounding (fma), so the pair carries about 48 bits; magnitudes at
+// which that could overflow or underflow, and non-finite ones, go to FP64.  FP64
+// per element (a convert, an FMA and a divide) took 263 us for 4096 x 3072 losses.
+struct Sum2 {
+  float hi = 0.f, lo = 0.f;
+  double wide = 0;
+  __device__ __forceinline__ void two_sum(float v) {
+    const float t = __fadd_rn(hi, v), z = __fsub_rn(t, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(v, z)));
+    hi = t;
+  }
+  __device__ __forceinline__ void add(float v) {
+    if (fabsf(v) <= 1e30f) two_sum(v);
+    else wide += double(v);
+  }
+  __device__ __forceinline__ void add_square(float a) {
+    const float p = __fmul_rn(a, a);
+    if (p >= 1e-30f && p <= 1e30f) {
+      lo = __fadd_rn(lo, __fmaf_rn(a, a, -p));
+      two_sum(p);
+    } else if (a != 0.f) {
+      wide += double(a) * a;
+    }
+  }
+  __device__ __forceinline__ double value() const { return double(hi) + double(lo) + wide; }
+};
+
+// Loss partials and dY = d loss / d y as BF16 rows, its transpose and its column
+// sums over the block's 64 rows (bias gradient partials [row block][column]).
+// Bound by memory: reads y and the targets, writes dY twice.
 __global__ void __launch_bounds__(256)
 k_loss(int64_t B, const float *__restrict__ Y, const float *__restrict__ Tv, const float *__restrict__ Tm,
-       float mask_weight, __nv_bfloat16 *__restrict__ dY, double *__restrict__ part) {
-  const float sv = 2.f / float(B * kOutV), sm = mask_weight / float(B * kOutM);
-  double acc = 0;
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < B * kOut; i += int64_t(gridDim.x) * blockDim.x) {
-    const int64_t b = i / kOut;
-    const int j = int(i % kOut);
-    const float y = Y[i];
-    float g;
-    if (j < kOutV) {
-      const float d = y - Tv[b * kOutV + j];
-      acc += double(d) * d / double(B * kOutV);
-      g = sv * d;
-    } else {
-      const float t = Tm[b * kOutM + (j - kOutV)];
-      // BCE with logits: max(y, 0) - t y + log(1 + e^{-|y|})
-      acc += double(mask_weight) * (fmaxf(y, 0.f) - t * y + log1pf(__expf(-fabsf(y)))) / double(B * kOutM);
-      g = sm * (1.f / (1.f + __expf(-y)) - t);
-    }
-    dY[i] = __float2bfloat16_rn(g);
-  }
-  const double t = block_sum_d<256>(acc);
-  if (threadIdx.x == 0) part[blockIdx.x] = t;
-}
-
-__global__ void k_sum_part_d(const double *__restrict__ part, int n, double *__restrict__ out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
-    double s = 0;
-    for (int i = 0; i < n; ++i) s += part[i];
-    *out = s;
-  }
-}
-
-// out[c][r] = in[r][c], R x C BF16
-__global__ void k_transpose(int64_t R, int64_t C, const __nv_bfloat16 *__restrict__ in, __nv_bfloat16 *__restrict__ out) {
-  __shared__ __nv_bfloat16 t[32][33];
-  const int64_t r0 = int64_t(blockIdx.y) * 32, c0 = int64_t(blockIdx.x) * 32;
-  for (int i = threadIdx.y; i < 32; i += blockDim.y)
-    if (r0 + i < R && c0 + threadIdx.x < C) t[i][threadIdx.x] = in[(r0 + i) * C + c0 + threadIdx.x];
-  __syncthreads();
-  for (int i = threadIdx.y; i < 32; i += blockDim.y)
-    if (c0 + i < C && r0 + threadIdx.x < R) out[(c0 + i) * R + r0 + threadIdx.x] = t[threadIdx.x][i];
-}
-
-// Column sums in two passes with a fixed order: block (32 columns x 8 row
-// groups) over rows [1024 y, 1024 (y + 1)) -> part[y][NV][col]; then k_sum_chunks.
-// NV = 1: sum_r in[r][j]; NV = 4 (first layer): sum_r in[r][j] (x0[r][0..2], 1).
-constexpr int kChunkRows = 1024;
-template <class T, int NV>
-__global__ void __launch_bounds__(256)
-k_colsum_part(int64_t R, int C, const T *__restrict__ in, const float *__restrict__ x0, float *__restrict__ part) {
-  __shared__ float red[8][NV][32];
-  const int j = blockIdx.x * 32 + threadIdx.x, g = threadIdx.y;
-  const int64_t r0 = int64_t(blockIdx.y) * kChunkRows;
-  const int64_t r1 = r0 + kChunkRows < R ? r0 + kChunkRows : R;
-  float acc[NV];
+       float mask_weight, __nv_bfloat16 *__restrict__ dY, __nv_bfloat16 *__restrict__ dYt, float *__restrict__ csum,
+       double *__restrict__ part) {
+  __shared__ BlockSmem sm;
+  const int64_t c0 = int64_t(blockIdx.x) * kBlk, r0 = int64_t(blockIdx.y) * kBlk;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const bool is_val = c0 < kOutV;   // 64 divides kOutV: a block is all values or all mask
+  const float s = is_val ? 2.f / float(B * kOutV) : mask_weight / float(B * kOutM);
+  const float *T = is_val ? Tv + c0 : Tm + (c0 - kOutV);
+  const int ldt = is_val ? kOutV : kOutM;
+  Sum2 acc;
+  float cs[4] = {0.f, 0.f, 0.f, 0.f};
+  float4 yv[4], tv[4];
 #pragma unroll
-  for (int v = 0; v < NV; ++v) acc[v] = 0.f;
-  if (j < C) {
-    for (int64_t r = r0 + g; r < r1; r += 8) {
-      const float d = float(in[r * C + j]);
-      if constexpr (NV == 1) {
-        acc[0] += d;
+  for (int i = 0; i < 4; ++i) {
+    const int64_t r = r0 + ty + 16 * i;
+    yv[i] = *reinterpret_cast<const float4 *>(Y + r * kOut + c0 + 4 * tx);
+    const float *tp = T + r * ldt + 4 * tx;
+    tv[i] = (reinterpret_cast<uintptr_t>(tp) & 15) == 0 ? __ldg(reinterpret_cast<const float4 *>(tp))
+                                                         : make_float4(tp[0], tp[1], tp[2], tp[3]);
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const float y4[4] = {yv[i].x, yv[i].y, yv[i].z, yv[i].w}, t4[4] = {tv[i].x, tv[i].y, tv[i].z, tv[i].w};
+    __nv_bfloat16 g[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float y = y4[q], t = t4[q];
+      float gf;
+      if (is_val) {
+        const float d = y - t;
+        acc.add_square(d);
+        gf = s * d;
       } else {
-        acc[0] += d * x0[r * 3];
-        acc[1] += d * x0[r * 3 + 1];
-        acc[2] += d * x0[r * 3 + 2];
-        acc[3] += d;
+        // BCE with logits: max(y, 0) - t y + log(1 + e^{-|y|})
+        acc.add(fmaxf(y, 0.f) - t * y + log1pf(__expf(-fabsf(y))));
+        gf = s * (1.f / (1.f + __expf(-y)) - t);
       }
+      g[q] = __float2bfloat16_rn(gf);
+      cs[q] += __bfloat162float(g[q]);
+      sm.t[4 * tx + q][ty + 16 * i] = g[q];
     }
+    put_bf16x4(dY + (r0 + ty + 16 * i) * kOut + c0 + 4 * tx, __nv_bfloat162(g[0], g[1]), __nv_bfloat162(g[2], g[3]));
   }
 #pragma unroll
-  for (int v = 0; v < NV; ++v) red[g][v][threadIdx.x] = acc[v];
+  for (int q = 0; q < 4; ++q) sm.red[ty][4 * tx + q] = cs[q];
   __syncthreads();
-  if (g == 0 && j < C) {
+  store_transposed(sm, dYt, B, r0, c0);
+  if (threadIdx.x < kBlk) {
+    float t = 0.f;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-      float t = 0.f;
-      for (int q = 0; q < 8; ++q) t += red[q][v][threadIdx.x];
-      part[(int64_t(blockIdx.y) * NV + v) * C + j] = t;
+    for (int q = 0; q < 16; ++q) t += sm.red[q][threadIdx.x];
+    csum[int64_t(blockIdx.y) * kOut + c0 + threadIdx.x] = t;
+  }
+  const double t = block_sum_d<256>(acc.value());
+  if (threadIdx.x == 0)
+    part[int64_t(blockIdx.y) * gridDim.x + blockIdx.x] =
+        t * (is_val ? 1.0 / double(B * kOutV) : double(mask_weight) / double(B * kOutM));
+}
+
+__global__ void __launch_bounds__(1024) k_sum_part_d(const double *__restrict__ part, int n, double *__restrict__ out) {
+  double v = 0;
+  for (int i = threadIdx.x; i < n; i += 1024) v += part[i];
+  v = block_sum_d<1024>(v);
+  if (threadIdx.x == 0) *out = v;
+}
+
+// dZ = dH GELU'(Z): BF16 rows and transpose for the next GEMMs and the column sums
+// (IN = false); for the first layer (IN = true) only the four column sums of
+// dZ (x0, 1), which are its gradients.
+template <bool IN>
+__global__ void __launch_bounds__(256)
+k_gelu_bwd(int64_t B, const float *__restrict__ dH, const float *__restrict__ Z,
+           const float *__restrict__ x0, __nv_bfloat16 *__restrict__ dZ, __nv_bfloat16 *__restrict__ dZt,
+           float *__restrict__ csum) {
+  __shared__ BlockSmem sm;
+  constexpr int NV = IN ? 4 : 1;
+  const int64_t c0 = int64_t(blockIdx.x) * kBlk, r0 = int64_t(blockIdx.y) * kBlk;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  float cs[NV][4];
+#pragma unroll
+  for (int v = 0; v < NV; ++v)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) cs[v][q] = 0.f;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int64_t r = r0 + ty + 16 * i, at = r * kH + c0 + 4 * tx;
+    const float4 d = *reinterpret_cast<const float4 *>(dH + at);
+    const float4 z = *reinterpret_cast<const float4 *>(Z + at);
+    const float g[4] = {d.x * gelu_d(z.x), d.y * gelu_d(z.y), d.z * gelu_d(z.z), d.w * gelu_d(z.w)};
+    if constexpr (IN) {
+      const float a = x0[r * kIn], b = x0[r * kIn + 1], c = x0[r * kIn + 2];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        cs[0][q] += g[q] * a;
+        cs[1][q] += g[q] * b;
+        cs[2][q] += g[q] * c;
+        cs[3][q] += g[q];
+      }
+    } else {
+      __nv_bfloat16 h[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        h[q] = __float2bfloat16_rn(g[q]);
+        cs[0][q] += __bfloat162float(h[q]);
+        sm.t[4 * tx + q][ty + 16 * i] = h[q];
+      }
+      put_bf16x4(dZ + at, __nv_bfloat162(h[0], h[1]), __nv_bfloat162(h[2], h[3]));
     }
   }
+#pragma unroll
+  for (int v = 0; v < NV; ++v) {
+    if (v) __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sm.red[ty][4 * tx + q] = cs[v][q];
+    __syncthreads();
+    if (threadIdx.x < kBlk) {
+      float t = 0.f;
+#pragma unroll
+      for (int q = 0; q < 16; ++q) t += sm.red[q][threadIdx.x];
+      csum[(int64_t(blockIdx.y) * NV + v) * kH + c0 + threadIdx.x] = t;
+    }
+  }
+  if constexpr (!IN) store_transposed(sm, dZt, B, r0, c0);
 }
 
-// out[v][j] = sum over chunks of part[chunk][v][j], chunks in order
-__global__ void k_sum_chunks(int nchunk, int nv, int C, const float *__restrict__ part, float *__restrict__ out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nv * C) return;
+// out[i] = sum over p < n of in[p len + i], in order: 8 lanes of partials per 32 elements
+__global__ void __launch_bounds__(256)
+k_sum_rows(int n, int64_t len, const float *__restrict__ in, float *__restrict__ out) {
+  __shared__ float red[8][33];
+  const int x = threadIdx.x & 31, g = threadIdx.x >> 5;
+  const int64_t i = int64_t(blockIdx.x) * 32 + x;
   float t = 0.f;
-  for (int c = 0; c < nchunk; ++c) t += part[int64_t(c) * nv * C + i];
-  out[i] = t;
-}
-
-// dZ = dH * GELU'(Z) as BF16 (next GEMM) and, when dZf is given, FP32
-__global__ void k_gelu_bwd(int64_t n, const float *__restrict__ dH, const float *__restrict__ Z,
-                           __nv_bfloat16 *__restrict__ dZ, float *__restrict__ dZf) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
-    const float g = dH[i] * gelu_d(Z[i]);
-    if (dZ) dZ[i] = __float2bfloat16_rn(g);
-    if (dZf) dZf[i] = g;
+  if (i < len) {
+#pragma unroll 4
+    for (int p = g; p < n; p += 8) t += in[int64_t(p) * len + i];
+  }
+  red[g][x] = t;
+  __syncthreads();
+  if (g == 0 && i < len) {
+#pragma unroll
+    for (int q = 1; q < 8; ++q) t += red[q][x];
+    out[i] = t;
   }
 }
 
-// first layer gradients from out[v][j] of the 4-way column sums
+// BF16 transposes of the three layers' activations (blockIdx.z), B x kH each
+__global__ void __launch_bounds__(256)
+k_transpose_h(int64_t B, const __nv_bfloat16 *__restrict__ h1, const __nv_bfloat16 *__restrict__ h2,
+              const __nv_bfloat16 *__restrict__ h3, __nv_bfloat16 *__restrict__ out) {
+  __shared__ BlockSmem sm;
+  const __nv_bfloat16 *in = blockIdx.z == 0 ? h1 : (blockIdx.z == 1 ? h2 : h3);
+  const int64_t c0 = int64_t(blockIdx.x) * kBlk, r0 = int64_t(blockIdx.y) * kBlk;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint2 u = *reinterpret_cast<const uint2 *>(in + (r0 + ty + 16 * i) * kH + c0 + 4 * tx);
+    const __nv_bfloat162 a = *reinterpret_cast<const __nv_bfloat162 *>(&u.x), b = *reinterpret_cast<const __nv_bfloat162 *>(&u.y);
+    sm.t[4 * tx][ty + 16 * i] = a.x;
+    sm.t[4 * tx + 1][ty + 16 * i] = a.y;
+    sm.t[4 * tx + 2][ty + 16 * i] = b.x;
+    sm.t[4 * tx + 3][ty + 16 * i] = b.y;
+  }
+  __syncthreads();
+  store_transposed(sm, out + int64_t(blockIdx.z) * B * kH, B, r0, c0);
+}
+
+// BF16 copies and transposes of W2, W3 (256 x 256) and W4 (3072 x 256) from the
+// FP32 master parameters: block = one 64 x 64 block, W2's 16 first, then W3's, W4's
+constexpr int kWBlocks = 2 * (kH / kBlk) * (kH / kBlk) + (kOut / kBlk) * (kH / kBlk);
+__global__ void __launch_bounds__(256)
+k_weights(const float *__restrict__ P, __nv_bfloat16 *__restrict__ w2, __nv_bfloat16 *__restrict__ w2t,
+          __nv_bfloat16 *__restrict__ w3, __nv_bfloat16 *__restrict__ w3t, __nv_bfloat16 *__restrict__ w4,
+          __nv_bfloat16 *__restrict__ w4t) {
+  __shared__ BlockSmem sm;
+  constexpr int kSq = (kH / kBlk) * (kH / kBlk);
+  const int which = blockIdx.x < kSq ? 0 : (blockIdx.x < 2 * kSq ? 1 : 2);
+  const int b = blockIdx.x - which * kSq, R = which == 2 ? kOut : kH;
+  const float *in = P + (which == 0 ? oW2 : (which == 1 ? oW3 : oW4));
+  __nv_bfloat16 *o = which == 0 ? w2 : (which == 1 ? w3 : w4), *ot = which == 0 ? w2t : (which == 1 ? w3t : w4t);
+  const int64_t r0 = int64_t(b / (kH / kBlk)) * kBlk, c0 = int64_t(b % (kH / kBlk)) * kBlk;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int64_t at = (r0 + ty + 16 * i) * kH + c0 + 4 * tx;
+    const float4 v = *reinterpret_cast<const float4 *>(in + at);   // every matrix starts on a multiple of 4 floats
+    const __nv_bfloat16 h[4] = {__float2bfloat16_rn(v.x), __float2bfloat16_rn(v.y), __float2bfloat16_rn(v.z),
+                                __float2bfloat16_rn(v.w)};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sm.t[4 * tx + q][ty + 16 * i] = h[q];
+    put_bf16x4(o + at, __nv_bfloat162(h[0], h[1]), __nv_bfloat162(h[2], h[3]));
+  }
+  __syncthreads();
+  store_transposed(sm, ot, R, r0, c0);
+}
+
+// first layer gradients from the 4-way column sums of the row blocks
 __global__ void k_in_grad(const float *__restrict__ s4, float *__restrict__ G) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= kH) return;
@@ -198,118 +366,126 @@ __global__ void k_adam(int64_t n, float *__restrict__ P, const float *__restrict
   }
 }
 
-__global__ void k_to_bf16(int64_t n, const float *__restrict__ in, __nv_bfloat16 *__restrict__ out) {
-  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
-    out[i] = __float2bfloat16_rn(in[i]);
-}
-
 int blocks_for(int64_t n) { return (int)std::min<int64_t>(152 * 16, std::max<int64_t>(1, ceil_div(n, 256))); }
 
-// column sums of an R x C matrix (NV = 1), or the first layer's four (NV = 4)
-template <class T, int NV>
-wproj_status colsum(int64_t R, int C, const T *in, const float *x0, float *scratch, float *out, cudaStream_t s) {
-  const int nchunk = ceil_div(R, kChunkRows);
-  k_colsum_part<T, NV><<<dim3(ceil_div(C, 32), nchunk), dim3(32, 8), 0, s>>>(R, C, in, x0, scratch);
-  k_sum_chunks<<<ceil_div(NV * C, 256), 256, 0, s>>>(nchunk, NV, C, scratch, out);
-  WPROJ_CHECK_LAUNCH("column sums");
+wproj_status sum_rows(int n, int64_t len, const float *in, float *out, cudaStream_t s) {
+  k_sum_rows<<<ceil_div(len, 32), 256, 0, s>>>(n, len, in, out);
+  WPROJ_CHECK_LAUNCH("row sums");
   return WPROJ_OK;
 }
 
-wproj_status transpose(int64_t R, int64_t C, const __nv_bfloat16 *in, __nv_bfloat16 *out, cudaStream_t s) {
-  k_transpose<<<dim3(ceil_div(C, 32), ceil_div(R, 32)), dim3(32, 8), 0, s>>>(R, C, in, out);
-  WPROJ_CHECK_LAUNCH("transpose");
-  return WPROJ_OK;
-}
-
-// BF16 copies and transposes of W2..W4 from the master parameters
 wproj_status refresh_weights(wproj_mlp *n, cudaStream_t s) {
-  const float *P = n->P.as<float>();
-  k_to_bf16<<<blocks_for(kH * kH), 256, 0, s>>>(kH * kH, P + oW2, n->W2b.as<__nv_bfloat16>());
-  k_to_bf16<<<blocks_for(kH * kH), 256, 0, s>>>(kH * kH, P + oW3, n->W3b.as<__nv_bfloat16>());
-  k_to_bf16<<<blocks_for(int64_t(kOut) * kH), 256, 0, s>>>(int64_t(kOut) * kH, P + oW4, n->W4b.as<__nv_bfloat16>());
+  k_weights<<<kWBlocks, 256, 0, s>>>(n->P.as<float>(), n->W2b.as<__nv_bfloat16>(), n->W2t.as<__nv_bfloat16>(),
+                                     n->W3b.as<__nv_bfloat16>(), n->W3t.as<__nv_bfloat16>(), n->W4b.as<__nv_bfloat16>(),
+                                     n->W4t.as<__nv_bfloat16>());
   WPROJ_CHECK_LAUNCH("weights to bf16");
-  WPROJ_TRY(transpose(kH, kH, n->W2b.as<__nv_bfloat16>(), n->W2t.as<__nv_bfloat16>(), s));
-  WPROJ_TRY(transpose(kH, kH, n->W3b.as<__nv_bfloat16>(), n->W3t.as<__nv_bfloat16>(), s));
-  WPROJ_TRY(transpose(kOut, kH, n->W4b.as<__nv_bfloat16>(), n->W4t.as<__nv_bfloat16>(), s));
+  return WPROJ_OK;
+}
+
+// activations of inference, B rows
+wproj_status ensure_forward(wproj_mlp *n, int64_t B) {
+  if (n->fcap >= B) return WPROJ_OK;
+  n->fcap = 0;
+  WPROJ_TRY(n->H1.alloc(2 * B * kH));
+  WPROJ_TRY(n->H2.alloc(2 * B * kH));
+  WPROJ_TRY(n->H3.alloc(2 * B * kH));
+  n->fcap = B;
   return WPROJ_OK;
 }
 
 wproj_status ensure_batch(wproj_mlp *n, int64_t B) {
+  WPROJ_TRY(ensure_forward(n, B));
   if (n->cap >= B) return WPROJ_OK;
+  n->cap = 0;
   WPROJ_TRY(n->Z1.alloc(sizeof(float) * B * kH));
   WPROJ_TRY(n->Z2.alloc(sizeof(float) * B * kH));
   WPROJ_TRY(n->Z3.alloc(sizeof(float) * B * kH));
-  WPROJ_TRY(n->H1.alloc(2 * B * kH));
-  WPROJ_TRY(n->H2.alloc(2 * B * kH));
-  WPROJ_TRY(n->H3.alloc(2 * B * kH));
   WPROJ_TRY(n->Y.alloc(sizeof(float) * B * kOut));
   WPROJ_TRY(n->dY.alloc(2 * B * kOut));
   WPROJ_TRY(n->dYt.alloc(2 * B * kOut));
-  WPROJ_TRY(n->Ht.alloc(2 * B * kH));
+  WPROJ_TRY(n->Ht.alloc(3 * 2 * B * kH));
   WPROJ_TRY(n->dZt.alloc(2 * B * kH));
   WPROJ_TRY(n->dH.alloc(sizeof(float) * B * kH));
   WPROJ_TRY(n->dZ.alloc(2 * B * kH));
-  WPROJ_TRY(n->dZ1.alloc(sizeof(float) * B * kH));
-  // column-sum partials: up to ceil(B / 1024) chunks x max(3072, 4 x 256) columns, then 4 x 256 results
-  n->csum_off = int64_t(ceil_div(B, kChunkRows)) * kOut;
-  WPROJ_TRY(n->csum.alloc(sizeof(float) * (n->csum_off + 4 * kH)));
+  WPROJ_TRY(n->csum.alloc(sizeof(float) * (B / kBlk) * kOut));   // covers 4 x 256 columns too
+  WPROJ_TRY(n->part.alloc(sizeof(double) * (B / kBlk) * (kOut / kBlk)));
   n->cap = B;
   return WPROJ_OK;
 }
 
-wproj_status gemm(int M, int N, int K, const void *A, const void *B, const float *bias, void *C, wproj_mlp *n,
-                  cudaStream_t s) {
-  return gemm_bf16_tn(M, N, K, static_cast<const __nv_bfloat16 *>(A), static_cast<const __nv_bfloat16 *>(B), bias,
-                      C, false, n->err.as<int>(), s);
+// C = A B^T (+ bias), FP32 and, when H is given, BF16 (GELU) outputs
+wproj_status gemm(int M, int N, int K, const void *A, const void *B, const float *bias, float *Z, __nv_bfloat16 *H,
+                  wproj_mlp *n, cudaStream_t s) {
+  GemmOut o;
+  o.bias = bias;
+  o.f32 = Z;
+  o.bf16 = H;
+  o.gelu = H != nullptr;
+  return gemm_bf16_tn(M, N, K, static_cast<const __nv_bfloat16 *>(A), static_cast<const __nv_bfloat16 *>(B), o,
+                      n->err.as<int>(), s);
 }
 
-// forward of B rows (B a multiple of 128) into n->Y
-wproj_status forward(wproj_mlp *n, const float *x0, int64_t B, float *Y, cudaStream_t s) {
+// Weight gradient C = A B^T in FP32 (K = the batch, few tiles) with K split over the
+// idle SMs: partial products in n->split, added in order into C.  The gradients of
+// the activations are not split: they are rounded to BF16 for the next layer, and
+// another order of their FP32 sum moves some of those roundings.
+wproj_status gemm_wgrad(int M, int N, int K, const void *A, const void *B, float *C, wproj_mlp *n, cudaStream_t s) {
+  GemmOut o;
+  WPROJ_TRY(gemm_splits(M, N, K, &o.splits));
+  WPROJ_TRY(n->split.ensure(sizeof(float) * size_t(o.splits) * M * N));
+  o.f32 = o.splits > 1 ? n->split.as<float>() : C;
+  WPROJ_TRY(gemm_bf16_tn(M, N, K, static_cast<const __nv_bfloat16 *>(A), static_cast<const __nv_bfloat16 *>(B), o,
+                         n->err.as<int>(), s));
+  return o.splits > 1 ? sum_rows(o.splits, int64_t(M) * N, n->split.as<float>(), C, s) : WPROJ_OK;
+}
+
+// forward of B rows (B a multiple of 128) into Y; train: keep Z1 .. Z3 for backward
+wproj_status forward(wproj_mlp *n, const float *x0, int64_t B, float *Y, bool train, cudaStream_t s) {
   const float *P = n->P.as<float>();
-  k_in_fwd<<<ceil_div(B * kH, 256), 256, 0, s>>>(B, x0, P, n->Z1.as<float>(), n->H1.as<__nv_bfloat16>());
+  auto *H1 = n->H1.as<__nv_bfloat16>(), *H2 = n->H2.as<__nv_bfloat16>(), *H3 = n->H3.as<__nv_bfloat16>();
+  k_in_fwd<<<ceil_div(B, kInRows), kH / 2, 0, s>>>(B, x0, P, train ? n->Z1.as<float>() : nullptr, H1);
   WPROJ_CHECK_LAUNCH("mlp layer 1");
-  WPROJ_TRY(gemm((int)B, kH, kH, n->H1.ptr, n->W2b.ptr, P + oB2, n->Z2.ptr, n, s));
-  k_gelu_fwd<<<blocks_for(B * kH), 256, 0, s>>>(B * kH, n->Z2.as<float>(), n->H2.as<__nv_bfloat16>());
-  WPROJ_TRY(gemm((int)B, kH, kH, n->H2.ptr, n->W3b.ptr, P + oB3, n->Z3.ptr, n, s));
-  k_gelu_fwd<<<blocks_for(B * kH), 256, 0, s>>>(B * kH, n->Z3.as<float>(), n->H3.as<__nv_bfloat16>());
-  WPROJ_CHECK_LAUNCH("mlp gelu");
-  return gemm((int)B, kOut, kH, n->H3.ptr, n->W4b.ptr, P + oB4, Y, n, s);
+  WPROJ_TRY(gemm((int)B, kH, kH, H1, n->W2b.ptr, P + oB2, train ? n->Z2.as<float>() : nullptr, H2, n, s));
+  WPROJ_TRY(gemm((int)B, kH, kH, H2, n->W3b.ptr, P + oB3, train ? n->Z3.as<float>() : nullptr, H3, n, s));
+  return gemm((int)B, kOut, kH, H3, n->W4b.ptr, P + oB4, Y, nullptr, n, s);
 }
 
 // loss (device double at *loss_d) and gradients into n->Gr for B rows
 wproj_status backward(wproj_mlp *n, const float *x0, const float *Tv, const float *Tm, int64_t B, float mask_weight,
                       double *loss_d, cudaStream_t s) {
-  float *G = n->Gr.as<float>();
-  const float *Z[3] = {n->Z1.as<float>(), n->Z2.as<float>(), n->Z3.as<float>()};
-  const __nv_bfloat16 *H[3] = {n->H1.as<__nv_bfloat16>(), n->H2.as<__nv_bfloat16>(), n->H3.as<__nv_bfloat16>()};
-  const int nb = blocks_for(B * kOut);
-  k_loss<<<nb, 256, 0, s>>>(B, n->Y.as<float>(), Tv, Tm, mask_weight, n->dY.as<__nv_bfloat16>(), n->part.as<double>());
-  k_sum_part_d<<<1, 32, 0, s>>>(n->part.as<double>(), nb, loss_d);
+  float *G = n->Gr.as<float>(), *csum = n->csum.as<float>();
+  auto *Ht = n->Ht.as<__nv_bfloat16>();
+  auto *dZ = n->dZ.as<__nv_bfloat16>(), *dZt = n->dZt.as<__nv_bfloat16>();
+  const int nrb = int(B / kBlk);
+  const dim3 lg(kOut / kBlk, nrb), hg(kH / kBlk, nrb);
+  k_loss<<<lg, 256, 0, s>>>(B, n->Y.as<float>(), Tv, Tm, mask_weight, n->dY.as<__nv_bfloat16>(),
+                            n->dYt.as<__nv_bfloat16>(), csum, n->part.as<double>());
+  k_sum_part_d<<<1, 1024, 0, s>>>(n->part.as<double>(), int(lg.x * lg.y), loss_d);
+  k_transpose_h<<<dim3(kH / kBlk, nrb, 3), 256, 0, s>>>(B, n->H1.as<__nv_bfloat16>(), n->H2.as<__nv_bfloat16>(),
+                                                        n->H3.as<__nv_bfloat16>(), Ht);
   WPROJ_CHECK_LAUNCH("mlp loss");
   // layer 4
-  WPROJ_TRY(transpose(B, kOut, n->dY.as<__nv_bfloat16>(), n->dYt.as<__nv_bfloat16>(), s));
-  WPROJ_TRY(transpose(B, kH, H[2], n->Ht.as<__nv_bfloat16>(), s));
-  WPROJ_TRY(gemm(kOut, kH, (int)B, n->dYt.ptr, n->Ht.ptr, nullptr, G + oW4, n, s));
-  WPROJ_TRY((colsum<__nv_bfloat16, 1>(B, kOut, n->dY.as<__nv_bfloat16>(), nullptr, n->csum.as<float>(), G + oB4, s)));
-  WPROJ_TRY(gemm((int)B, kH, kOut, n->dY.ptr, n->W4t.ptr, nullptr, n->dH.ptr, n, s));
+  float *dH = n->dH.as<float>();
+  WPROJ_TRY(sum_rows(nrb, kOut, csum, G + oB4, s));
+  WPROJ_TRY(gemm_wgrad(kOut, kH, (int)B, n->dYt.ptr, Ht + 2 * B * kH, G + oW4, n, s));
+  WPROJ_TRY(gemm((int)B, kH, kOut, n->dY.ptr, n->W4t.ptr, nullptr, dH, nullptr, n, s));
   // layers 3 and 2
   const __nv_bfloat16 *Wt[2] = {n->W3t.as<__nv_bfloat16>(), n->W2t.as<__nv_bfloat16>()};
+  const float *Z[2] = {n->Z3.as<float>(), n->Z2.as<float>()};
   const int64_t oW[2] = {oW3, oW2}, oB[2] = {oB3, oB2};
   for (int l = 0; l < 2; ++l) {
-    const int zi = 2 - l;   // Z3 then Z2
-    k_gelu_bwd<<<blocks_for(B * kH), 256, 0, s>>>(B * kH, n->dH.as<float>(), Z[zi], n->dZ.as<__nv_bfloat16>(), nullptr);
+    k_gelu_bwd<false><<<hg, 256, 0, s>>>(B, dH, Z[l], nullptr, dZ, dZt, csum);
     WPROJ_CHECK_LAUNCH("mlp gelu backward");
-    WPROJ_TRY(transpose(B, kH, n->dZ.as<__nv_bfloat16>(), n->dZt.as<__nv_bfloat16>(), s));
-    WPROJ_TRY(transpose(B, kH, H[zi - 1], n->Ht.as<__nv_bfloat16>(), s));
-    WPROJ_TRY(gemm(kH, kH, (int)B, n->dZt.ptr, n->Ht.ptr, nullptr, G + oW[l], n, s));
-    WPROJ_TRY((colsum<__nv_bfloat16, 1>(B, kH, n->dZ.as<__nv_bfloat16>(), nullptr, n->csum.as<float>(), G + oB[l], s)));
-    WPROJ_TRY(gemm((int)B, kH, kH, n->dZ.ptr, Wt[l], nullptr, n->dH.ptr, n, s));
+    WPROJ_TRY(sum_rows(nrb, kH, csum, G + oB[l], s));
+    WPROJ_TRY(gemm_wgrad(kH, kH, (int)B, dZt, Ht + (1 - l) * B * kH, G + oW[l], n, s));
+    WPROJ_TRY(gemm((int)B, kH, kH, dZ, Wt[l], nullptr, dH, nullptr, n, s));
   }
   // layer 1
-  k_gelu_bwd<<<blocks_for(B * kH), 256, 0, s>>>(B * kH, n->dH.as<float>(), Z[0], nullptr, n->dZ1.as<float>());
-  WPROJ_TRY((colsum<float, 4>(B, kH, n->dZ1.as<float>(), x0, n->csum.as<float>(), n->csum.as<float>() + n->csum_off, s)));
-  k_in_grad<<<1, kH, 0, s>>>(n->csum.as<float>() + n->csum_off, G);
+  k_gelu_bwd<true><<<hg, 256, 0, s>>>(B, dH, n->Z1.as<float>(), x0, nullptr, nullptr, csum);
   WPROJ_CHECK_LAUNCH("mlp layer 1 backward");
+  WPROJ_TRY(sum_rows(nrb, 4 * kH, csum, dH, s));   // dH is spent: its first 4 kH floats take the sums
+  k_in_grad<<<1, kH, 0, s>>>(dH, G);
+  WPROJ_CHECK_LAUNCH("mlp layer 1 gradients");
   return WPROJ_OK;
 }
 
@@ -486,11 +662,11 @@ wproj_status build_learned_impl(wproj_plan *p, wproj_mlp *n, const double *uvw, 
   WPROJ_CUDA(cudaMemsetAsync(x0.ptr, 0, sizeof(float) * 3 * (m + 128), s));
   k_features<<<ceil_div(m, 256), 256, 0, s>>>(m, uvw, p->g.du, p->g.L, x0.as<float>());
   WPROJ_CHECK_LAUNCH("mlp features");
-  WPROJ_TRY(ensure_batch(n, chunk));
+  WPROJ_TRY(ensure_forward(n, chunk));
   for (int64_t r = 0; r < m; r += chunk) {
     const int64_t nr = std::min(chunk, m - r);
     const int64_t B = (nr + 127) / 128 * 128;   // padded rows read zero features
-    WPROJ_TRY(forward(n, x0.as<float>() + 3 * r, B, Y.as<float>(), s));
+    WPROJ_TRY(forward(n, x0.as<float>() + 3 * r, B, Y.as<float>(), false, s));
     k_judge<<<(unsigned)nr, 256, 0, s>>>(r, uvw, p->row_ptr.as<int64_t>(), p->col.as<int32_t>(), p->val.as<float2>(),
                                          Y.as<float>(), p->g.G, p->g.du, p->g.W, p->g.beta, e, relmax, err_p,
                                          pass.as<int8_t>());
@@ -528,7 +704,7 @@ wproj_status mlp_create(wproj_mlp *n) {
   WPROJ_TRY(n->W2t.alloc(2 * kH * kH));
   WPROJ_TRY(n->W3t.alloc(2 * kH * kH));
   WPROJ_TRY(n->W4t.alloc(2 * int64_t(kOut) * kH));
-  WPROJ_TRY(n->part.alloc(sizeof(double) * (152 * 16 + 8)));
+  WPROJ_TRY(n->loss.alloc(sizeof(double)));
   WPROJ_TRY(n->err.alloc(sizeof(int)));
   WPROJ_CUDA(cudaMemset(n->P.ptr, 0, sizeof(float) * kParams));
   WPROJ_CUDA(cudaMemset(n->Mo.ptr, 0, sizeof(float) * kParams));
@@ -554,10 +730,10 @@ wproj_status mlp_get_params(const wproj_mlp *n, float *p, cudaStream_t s) {
 }
 
 wproj_status mlp_forward(wproj_mlp *n, const float *x0, int64_t m, float *y, int64_t chunk, cudaStream_t s) {
-  WPROJ_TRY(ensure_batch(n, chunk));
+  WPROJ_TRY(ensure_forward(n, chunk));
   for (int64_t r = 0; r < m; r += chunk) {
     const int64_t B = std::min<int64_t>(chunk, m - r);
-    WPROJ_TRY(forward(n, x0 + 3 * r, B, y + r * kOut, s));
+    WPROJ_TRY(forward(n, x0 + 3 * r, B, y + r * kOut, false, s));
   }
   return check_err(n, s);
 }
@@ -565,9 +741,9 @@ wproj_status mlp_forward(wproj_mlp *n, const float *x0, int64_t m, float *y, int
 wproj_status mlp_gradients(wproj_mlp *n, const float *x0, const float *Tv, const float *Tm, int64_t B,
                            double mask_weight, double *loss, float *grad, cudaStream_t s) {
   WPROJ_TRY(ensure_batch(n, B));
-  WPROJ_TRY(forward(n, x0, B, n->Y.as<float>(), s));
-  WPROJ_TRY(backward(n, x0, Tv, Tm, B, float(mask_weight), n->part.as<double>() + 152 * 16, s));
-  WPROJ_CUDA(cudaMemcpyAsync(loss, n->part.as<double>() + 152 * 16, sizeof(double), cudaMemcpyDeviceToHost, s));
+  WPROJ_TRY(forward(n, x0, B, n->Y.as<float>(), true, s));
+  WPROJ_TRY(backward(n, x0, Tv, Tm, B, float(mask_weight), n->loss.as<double>(), s));
+  WPROJ_CUDA(cudaMemcpyAsync(loss, n->loss.as<double>(), sizeof(double), cudaMemcpyDeviceToHost, s));
   if (grad) WPROJ_CUDA(cudaMemcpyAsync(grad, n->Gr.ptr, sizeof(float) * kParams, cudaMemcpyDefault, s));
   return check_err(n, s);
 }
@@ -581,7 +757,7 @@ wproj_status mlp_train(wproj_mlp *n, const float *x0, const float *Tv, const flo
   const int64_t nbatch = m / B;
   for (int it = 0; it < steps; ++it) {
     const int64_t r = (it % nbatch) * B;
-    WPROJ_TRY(forward(n, x0 + 3 * r, B, n->Y.as<float>(), s));
+    WPROJ_TRY(forward(n, x0 + 3 * r, B, n->Y.as<float>(), true, s));
     WPROJ_TRY(backward(n, x0 + 3 * r, Tv + r * kOutV, Tm + r * kOutM, B, float(mask_weight), dl.as<double>() + it, s));
     n->step += 1;
     const float c1 = 1.f - powf(0.9f, float(n->step)), c2 = 1.f - powf(0.999f, float(n->step));

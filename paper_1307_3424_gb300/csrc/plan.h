@@ -208,6 +208,7 @@ wproj_status fft2d_generic(const float2 *in, float2 *out, int n, int batch, int 
 // box FFT for the kernel build: nb boxes of S x S, in place; tables per box
 struct BoxBatch;
 wproj_status box_fft(wproj_plan *p, const BoxBatch &bb, cudaStream_t s);
+wproj_status box_g_table(int S, const float *lsq, float *g, cudaStream_t s);   // BoxBatch::gtab
 
 wproj_status phi_forward_fft_into(wproj_plan *p, const float *x, float2 *inter, float2 *Xt, cudaStream_t s);
 // batches: F Z A and A Z^H F^H for the np problems plist (device) of one grid size 2^logG
@@ -249,8 +250,16 @@ wproj_status rebuild_cells(wproj_plan *p, cudaStream_t s);
 wproj_status batch_grid_cells(const BatchOps &b, const float2 *y, float2 *Xt2, cudaStream_t s);
 
 // gemm.cu: C = A B^T (+ bias) on the tcgen05 tensor cores, BF16 in, FP32 accumulate
-wproj_status gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16 *A, const __nv_bfloat16 *B, const float *bias,
-                          void *C, bool out_bf16, int *err, cudaStream_t s);
+struct GemmOut {
+  const float *bias = nullptr;
+  float *f32 = nullptr;            // FP32 product; with splits > 1, `splits` partial products of M x N
+  __nv_bfloat16 *bf16 = nullptr;   // BF16 product, or its GELU
+  bool gelu = false;
+  int splits = 1;                  // ranges of K, each with its own partial product (FP32 only, no bias)
+};
+wproj_status gemm_splits(int M, int N, int K, int *splits);   // ranges that fill the SMs
+wproj_status gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16 *A, const __nv_bfloat16 *B, const GemmOut &o,
+                          int *err, cudaStream_t s);
 
 // mlp.cu: the learned-kernel network
 int64_t mlp_num_params();
