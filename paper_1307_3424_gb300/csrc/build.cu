@@ -996,7 +996,7 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
     max_nb = std::max<int>(max_nb, (int)std::min<int64_t>(std::min<int64_t>(cls_ptr[c + 1] - cls_ptr[c], kMaxBatchBoxes),
                                                             std::max<int64_t>(1, batch_bytes(S) / per)));
   }
-  DevBuf Kbuf, Au, Av, bmode, bwf, bwd, bsel, hcnt, hq, lcoord, lsq, bsid;
+  DevBuf Kbuf, Au, Av, bmode, bwf, bwd, bsel, hcnt, hq, lcoord, lsq, gtab, bsid;
   // Pass 2 needs every box's transform again.  When the device has room for all
   // of them (and, with a margin, for G, whose size is at most 1.5x theirs), pass
   // 1 keeps them and pass 2 emits without recomputing the tables and FFTs;
@@ -1026,6 +1026,7 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
   WPROJ_TRY(hq.alloc(sizeof(unsigned long long) * kHistBins * size_t(max_nb)));
   WPROJ_TRY(lcoord.alloc(sizeof(double) * p->box_max));
   WPROJ_TRY(lsq.alloc(sizeof(float) * p->box_max));
+  if (g.chirp == WPROJ_CHIRP_EXACT) WPROJ_TRY(gtab.alloc(sizeof(float) * p->box_max * p->box_max));
 
   const double e_target = e + kSelectMargin;
   const int vdt = g.value_dtype;
@@ -1126,6 +1127,7 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
       k_coord_tables<<<ceil_div(S, 256), 256, 0, s>>>(S, g.L, g.extension == WPROJ_EXT_CLAMP,
                                                       lcoord.as<double>(), lsq.as<float>());
       WPROJ_CHECK_LAUNCH("coord tables");
+      if (g.chirp == WPROJ_CHIRP_EXACT) WPROJ_TRY(box_g_table(S, lsq.as<float>(), gtab.as<float>(), s));
       for (int64_t b0 = glo; b0 < ghi; b0 += nbmax) {
         const int nb = (int)std::min<int64_t>(nbmax, ghi - b0);
         const int32_t *ids = d_ids.as<int32_t>() + b0;
@@ -1144,7 +1146,7 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
           WPROJ_CHECK_LAUNCH("box tables");
           bb.Au = Au.as<float2>(); bb.Av = Av.as<float2>();
           bb.mode = bmode.as<int8_t>(); bb.wf = bwf.as<float>(); bb.wd = bwd.as<double>();
-          bb.lsq = lsq.as<float>(); bb.lcoord = lcoord.as<double>();
+          bb.lsq = lsq.as<float>(); bb.gtab = gtab.as<float>(); bb.lcoord = lcoord.as<double>();
           if (sid) {
             bb.screens = p->screens.as<float2>();
             bb.bsid = bsid.as<int32_t>();

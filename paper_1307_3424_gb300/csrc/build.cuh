@@ -15,6 +15,7 @@ struct BoxBatch {
   const float *wf = nullptr;      // [nb] w as float (remainder term)
   const double *wd = nullptr;     // [nb] w (FP64 phase path)
   const float *lsq = nullptr;     // [S] l_P^2 (float)
+  const float *gtab = nullptr;    // [S][S] g(l_P^2 + l_Q^2), g(x) = x^2 / (2 (1 + n)^2) (exact chirp)
   const double *lcoord = nullptr; // [S] l_P (after clamping)
   float2 *K = nullptr;            // [nb][S][S] kernel values, natural order (offset s at s mod S)
   // direction-dependent screens (S = G): screens[bsid[b]] multiplies box b's samples;

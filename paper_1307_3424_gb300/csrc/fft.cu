@@ -28,35 +28,21 @@ __global__ void k_twiddles(float2 *tw) {
   tw[i] = make_float2(float(cs), float(sn));
 }
 
-// padded index -> image index (or -1): offset p - N/2 sits at (p - N/2) mod G
-__device__ __forceinline__ int pad_to_img(int P, int N, int G) {
-  const int h = N >> 1;
-  if (P < h) return P + h;
-  if (P >= G - h) return P - G + h;
-  return -1;
-}
-__device__ __forceinline__ int img_to_pad(int p, int N, int G) {
-  const int h = N >> 1;
-  return (p >= h) ? p - h : p - h + G;
-}
+// Padded position tq + m G / 16 of a length-G axis -> image index: offset p - N/2
+// sits at (p - N/2) mod G, N = G / 2, so m < 4 holds the image's upper half, m >= 12
+// its lower half and the rest is padding: 8 of a thread's 16 elements, known at
+// compile time, are zeros that are never read or are cropped before the store.
+__device__ __forceinline__ constexpr bool in_image(int m) { return m < 4 || m >= 12; }
+__device__ __forceinline__ int pad_to_img(int m, int P, int G) { return m < 4 ? P + G / 4 : P - G + G / 4; }
 
-// Block copy of TOT elements into shared memory, element idx from ld(idx) and
-// stored by st(idx, v): all of a thread's loads are issued before its first
-// store, so a thread keeps TOT / T loads in flight instead of one.
-template <int TOT, int T, class LD, class ST>
-__device__ __forceinline__ void staged_copy(LD ld, ST st) {
-  constexpr int PER = (TOT + T - 1) / T;
-  float2 r[PER];
-#pragma unroll
-  for (int i = 0; i < PER; ++i) {
-    const int idx = int(threadIdx.x) + i * T;
-    r[i] = (TOT % T == 0 || idx < TOT) ? ld(idx) : make_float2(0.f, 0.f);
-  }
-#pragma unroll
-  for (int i = 0; i < PER; ++i) {
-    const int idx = int(threadIdx.x) + i * T;
-    if (TOT % T == 0 || idx < TOT) st(idx, r[i]);
-  }
+// thread -> (transform of the block, thread of the transform): rows / columns
+template <class Cfg> __device__ __forceinline__ void row_thread(int &c, int &tq) {
+  c = int(threadIdx.x) / Cfg::TN;
+  tq = int(threadIdx.x) % Cfg::TN;
+}
+template <class Cfg> __device__ __forceinline__ void col_thread(int &c, int &tq) {
+  c = int(threadIdx.x) % Cfg::C;
+  tq = int(threadIdx.x) / Cfg::C;
 }
 
 // ---- Phi: F Z A --------------------------------------------------------------
@@ -72,30 +58,26 @@ __device__ __forceinline__ void phi_fwd_rows_body(const float *__restrict__ x, c
   using Cfg = RowCfg<LOGN>;
   constexpr int G = 1 << LOGN;
   extern __shared__ float2 sm[];
-  const int p0 = blk * Cfg::C;
-  staged_copy<Cfg::C * G, Cfg::T>(
-      [&](int idx) {
-        const int c = idx / G, Q = idx % G;
-        const int p = p0 + c;
-        float2 v = make_float2(0.f, 0.f);
-        if (p < N) {
-          const int q = pad_to_img(Q, N, G);
-          if (q >= 0) {
-            const float s = inv_a[p] * inv_a[q];
-            if (xc) v = cscale(xc[int64_t(p) * N + q], s);
-            else v = make_float2(x[int64_t(p) * N + q] * s, 0.f);
-          }
-        }
-        return v;
-      },
-      [&](int idx, float2 v) { sm[(idx / G) * Cfg::LD + idx % G] = v; });
-  __syncthreads();
-  fft_block<LOGN, Cfg::C, Cfg::T, -1>(sm, Cfg::LD, tw);
-  for (int idx = threadIdx.x; idx < Cfg::C * G; idx += Cfg::T) {
-    const int c = idx / G, Q = idx % G;
-    const int p = p0 + c;
-    if (p < N) inter[int64_t(p) * G + Q] = sm[c * Cfg::LD + Q];
+  int c, tq;
+  row_thread<Cfg>(c, tq);
+  const int p = blk * Cfg::C + c;
+  const bool ok = p < N;
+  const float ap = ok ? inv_a[p] : 0.f;
+  float2 v[kFftE];
+#pragma unroll
+  for (int m = 0; m < kFftE; ++m) {
+    v[m] = make_float2(0.f, 0.f);
+    if (in_image(m) && ok) {
+      const int q = pad_to_img(m, tq + m * Cfg::TN, G);
+      const float s = ap * inv_a[q];
+      if (xc) v[m] = cscale(xc[int64_t(p) * N + q], s);
+      else v[m].x = x[int64_t(p) * N + q] * s;
+    }
   }
+  float2 *out = inter + int64_t(p) * G;
+  fft_run<LOGN, -1>(v, tq, sm + c * Cfg::LD, tw, [&](int, int Q, float2 o) {
+    if (ok) out[Q] = o;
+  });
 }
 
 template <int LOGN>
@@ -119,20 +101,19 @@ __device__ __forceinline__ void phi_fwd_cols_body(const float2 *__restrict__ int
   using Cfg = ColCfg<LOGN>;
   constexpr int G = 1 << LOGN;
   extern __shared__ float2 sm[];
-  const int Q0 = blk * Cfg::C;
-  staged_copy<Cfg::C * G, Cfg::T>(
-      [&](int idx) {
-        const int P = idx / Cfg::C, c = idx % Cfg::C;
-        const int p = pad_to_img(P, N, G);
-        return (p >= 0 && Q0 + c < G) ? inter[int64_t(p) * G + Q0 + c] : make_float2(0.f, 0.f);
-      },
-      [&](int idx, float2 v) { sm[(idx % Cfg::C) * Cfg::LD + idx / Cfg::C] = v; });
-  __syncthreads();
-  fft_block<LOGN, Cfg::C, Cfg::T, -1>(sm, Cfg::LD, tw);
-  for (int idx = threadIdx.x; idx < Cfg::C * G; idx += Cfg::T) {
-    const int P = idx / Cfg::C, c = idx % Cfg::C;
-    if (Q0 + c < G) Xt[int64_t(P) * G + Q0 + c] = cscale(sm[c * Cfg::LD + P], scale);
+  int c, tq;
+  col_thread<Cfg>(c, tq);
+  const int Q = blk * Cfg::C + c;
+  const bool ok = Q < G;
+  float2 v[kFftE];
+#pragma unroll
+  for (int m = 0; m < kFftE; ++m) {
+    v[m] = make_float2(0.f, 0.f);
+    if (in_image(m) && ok) v[m] = inter[int64_t(pad_to_img(m, tq + m * Cfg::TN, G)) * G + Q];
   }
+  fft_run<LOGN, -1>(v, tq, sm + c * Cfg::LD, tw, [&](int, int P, float2 o) {
+    if (ok) Xt[int64_t(P) * G + Q] = cscale(o, scale);
+  });
 }
 
 template <int LOGN>
@@ -158,19 +139,17 @@ __device__ __forceinline__ void phi_adj_cols_body(const float2 *__restrict__ Xt2
   using Cfg = ColCfg<LOGN>;
   constexpr int G = 1 << LOGN;
   extern __shared__ float2 sm[];
-  const int Q0 = blk * Cfg::C;
-  staged_copy<Cfg::C * G, Cfg::T>(
-      [&](int idx) {
-        const int P = idx / Cfg::C, c = idx % Cfg::C;
-        return (Q0 + c < G) ? Xt2[int64_t(P) * G + Q0 + c] : make_float2(0.f, 0.f);
-      },
-      [&](int idx, float2 v) { sm[(idx % Cfg::C) * Cfg::LD + idx / Cfg::C] = v; });
-  __syncthreads();
-  fft_block<LOGN, Cfg::C, Cfg::T, +1>(sm, Cfg::LD, tw);
-  for (int idx = threadIdx.x; idx < Cfg::C * N; idx += Cfg::T) {
-    const int p = idx / Cfg::C, c = idx % Cfg::C;
-    if (Q0 + c < G) inter[int64_t(p) * G + Q0 + c] = sm[c * Cfg::LD + img_to_pad(p, N, G)];
-  }
+  int c, tq;
+  col_thread<Cfg>(c, tq);
+  const int Q = blk * Cfg::C + c;
+  const bool ok = Q < G;
+  float2 v[kFftE];
+#pragma unroll
+  for (int m = 0; m < kFftE; ++m)
+    v[m] = ok ? Xt2[int64_t(tq + m * Cfg::TN) * G + Q] : make_float2(0.f, 0.f);
+  fft_run<LOGN, +1>(v, tq, sm + c * Cfg::LD, tw, [&](int m, int P, float2 o) {
+    if (in_image(m) && ok) inter[int64_t(pad_to_img(m, P, G)) * G + Q] = o;
+  });
 }
 
 template <int LOGN>
@@ -196,29 +175,28 @@ __device__ __forceinline__ void phi_adj_rows_body(const float2 *__restrict__ int
   using Cfg = RowCfg<LOGN>;
   constexpr int G = 1 << LOGN;
   extern __shared__ float2 sm[];
-  const int p0 = blk * Cfg::C;
-  staged_copy<Cfg::C * G, Cfg::T>(
-      [&](int idx) {
-        const int p = p0 + idx / G;
-        return (p < N) ? inter[int64_t(p) * G + idx % G] : make_float2(0.f, 0.f);
-      },
-      [&](int idx, float2 v) { sm[(idx / G) * Cfg::LD + idx % G] = v; });
-  __syncthreads();
-  fft_block<LOGN, Cfg::C, Cfg::T, +1>(sm, Cfg::LD, tw);
-  for (int idx = threadIdx.x; idx < Cfg::C * N; idx += Cfg::T) {
-    const int c = idx / N, q = idx % N;
-    const int p = p0 + c;
-    if (p >= N) continue;
-    const float s = inv_a[p] * inv_a[q] * scale;
-    const float2 v = sm[c * Cfg::LD + img_to_pad(q, N, G)];
-    const int64_t o = int64_t(p) * N + q;
-    if (mode == 0) {
-      if (x_re) x_re[o] = v.x * s;
-      if (x_c) x_c[o] = cscale(v, s);
-    } else {
-      x_re[o] = z[o] - v.x * s;
+  int c, tq;
+  row_thread<Cfg>(c, tq);
+  const int p = blk * Cfg::C + c;
+  const bool ok = p < N;
+  const float2 *in = inter + int64_t(p) * G;
+  float2 v[kFftE];
+#pragma unroll
+  for (int m = 0; m < kFftE; ++m) v[m] = ok ? in[tq + m * Cfg::TN] : make_float2(0.f, 0.f);
+  const float ap = ok ? inv_a[p] : 0.f;
+  fft_run<LOGN, +1>(v, tq, sm + c * Cfg::LD, tw, [&](int m, int Q, float2 f) {
+    if (in_image(m) && ok) {
+      const int q = pad_to_img(m, Q, G);
+      const float s = ap * inv_a[q] * scale;
+      const int64_t o = int64_t(p) * N + q;
+      if (mode == 0) {
+        if (x_re) x_re[o] = f.x * s;
+        if (x_c) x_c[o] = cscale(f, s);
+      } else {
+        x_re[o] = z[o] - f.x * s;
+      }
     }
-  }
+  });
 }
 
 template <int LOGN>
@@ -248,52 +226,51 @@ k_fft_rows(const float2 *__restrict__ in, float2 *__restrict__ out, int64_t n_ro
   using Cfg = RowCfg<LOGN>;
   constexpr int N = 1 << LOGN;
   extern __shared__ float2 sm[];
-  const int64_t r0 = int64_t(blockIdx.x) * Cfg::C;
-  staged_copy<Cfg::C * N, Cfg::T>(
-      [&](int idx) {
-        const int64_t r = r0 + idx / N;
-        return (r < n_rows) ? in[r * N + idx % N] : make_float2(0.f, 0.f);
-      },
-      [&](int idx, float2 v) { sm[(idx / N) * Cfg::LD + idx % N] = v; });
-  __syncthreads();
-  fft_block<LOGN, Cfg::C, Cfg::T, DIR>(sm, Cfg::LD, tw);
-  for (int idx = threadIdx.x; idx < Cfg::C * N; idx += Cfg::T) {
-    const int c = idx / N, i = idx % N;
-    if (r0 + c < n_rows) out[(r0 + c) * N + i] = sm[c * Cfg::LD + i];
-  }
+  int c, tq;
+  row_thread<Cfg>(c, tq);
+  const int64_t r = int64_t(blockIdx.x) * Cfg::C + c;
+  const bool ok = r < n_rows;
+  float2 v[kFftE];
+#pragma unroll
+  for (int m = 0; m < kFftE; ++m) v[m] = ok ? in[r * N + tq + m * Cfg::TN] : make_float2(0.f, 0.f);
+  fft_run<LOGN, DIR>(v, tq, sm + c * Cfg::LD, tw, [&](int, int i, float2 o) {
+    if (ok) out[r * N + i] = o;
+  });
 }
 
 // columns of `batch` N x N arrays, flattened as batch * N global columns
 template <int LOGN, int DIR>
-__global__ void __launch_bounds__(ColCfg<LOGN>::T)
+__global__ void __launch_bounds__(BoxColCfg<LOGN>::T)
 k_fft_cols(const float2 *__restrict__ in, float2 *__restrict__ out, int64_t n_cols, float scale,
            const float2 *__restrict__ tw) {
-  using Cfg = ColCfg<LOGN>;
+  using Cfg = BoxColCfg<LOGN>;
   constexpr int N = 1 << LOGN;
   extern __shared__ float2 sm[];
-  const int64_t g0 = int64_t(blockIdx.x) * Cfg::C;
-  staged_copy<Cfg::C * N, Cfg::T>(
-      [&](int idx) {
-        const int P = idx / Cfg::C;
-        const int64_t gc = g0 + idx % Cfg::C;
-        if (gc >= n_cols) return make_float2(0.f, 0.f);
-        const int64_t b = gc >> LOGN, Q = gc & (N - 1);
-        return in[(b * N + P) * N + Q];
-      },
-      [&](int idx, float2 v) { sm[(idx % Cfg::C) * Cfg::LD + idx / Cfg::C] = v; });
-  __syncthreads();
-  fft_block<LOGN, Cfg::C, Cfg::T, DIR>(sm, Cfg::LD, tw);
-  for (int idx = threadIdx.x; idx < Cfg::C * N; idx += Cfg::T) {
-    const int P = idx / Cfg::C, c = idx % Cfg::C;
-    const int64_t gc = g0 + c;
-    if (gc < n_cols) {
-      const int64_t b = gc >> LOGN, Q = gc & (N - 1);
-      out[(b * N + P) * N + Q] = cscale(sm[c * Cfg::LD + P], scale);
-    }
-  }
+  int c, tq;
+  col_thread<Cfg>(c, tq);
+  const int64_t gc = int64_t(blockIdx.x) * Cfg::C + c;
+  const bool ok = gc < n_cols;
+  const int64_t at = ((gc >> LOGN) << (2 * LOGN)) + (gc & (N - 1));
+  float2 v[kFftE];
+#pragma unroll
+  for (int m = 0; m < kFftE; ++m) v[m] = ok ? in[at + int64_t(tq + m * Cfg::TN) * N] : make_float2(0.f, 0.f);
+  fft_run<LOGN, DIR>(v, tq, sm + c * Cfg::LD, tw, [&](int, int P, float2 o) {
+    if (ok) out[at + int64_t(P) * N] = cscale(o, scale);
+  });
 }
 
 // ---- kernel build: S x S boxes ---------------------------------------------------
+
+// g(x) of the exact chirp's FP32 remainder at every sample of an S x S box: the
+// root and the division once per sample position instead of once per box sample.
+__global__ void k_g_table(int S, const float *__restrict__ lsq, float *__restrict__ g) {
+  const int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i >= int64_t(S) * S) return;
+  const float x = lsq[i / S] + lsq[i % S];
+  const float n = sqrtf(1.f - x);
+  const float d = 1.f + n;
+  g[i] = (x * x) / (2.f * d * d);
+}
 
 // f[P][Q] = Au[P] Av[Q] e^{2 pi i w g(x)}: the chirp (Eq. 4 / Eq. 5) times the KB
 // tap polynomial, at box offsets P' = P (P < S/2) or P - S; Au, Av carry the
@@ -305,13 +282,10 @@ __device__ __forceinline__ float2 box_value(const BoxBatch &bb, int b, int P, in
   const int mode = bb.mode[b];
   if (mode == 1) {
     // exact chirp: phase w (1 - n) = w x / 2 + w g(x), g = x^2 / (2 (1 + n)^2), the
-    // remainder |w g| <= 1/4 cycle so FP32 keeps it to ~1e-7 cycles
-    const float x = bb.lsq[P] + bb.lsq[Q];
-    const float n = sqrtf(1.f - x);
-    const float d = 1.f + n;
-    const float g = (x * x) / (2.f * d * d);
+    // remainder |w g| <= 1/4 cycle so FP32 keeps it to ~1e-7 cycles; g does not
+    // depend on the box and comes from a table of the class (k_g_table)
     float sn, cs;
-    sincospif(2.f * (bb.wf[b] * g), &sn, &cs);
+    sincospif(2.f * (bb.wf[b] * __ldg(bb.gtab + int64_t(P) * bb.S + Q)), &sn, &cs);
     f = cmul(f, make_float2(cs, sn));
   } else if (mode == 2) {
     // large w: the full phase argument in FP64, reduced mod 1
@@ -337,22 +311,26 @@ k_box_rows(BoxBatch bb, const float2 *__restrict__ tw) {
   using Cfg = RowCfg<LOGN>;
   constexpr int S = 1 << LOGN;
   extern __shared__ float2 sm[];
-  const int64_t n_rows = int64_t(bb.nb) * S;
-  const int64_t r0 = int64_t(blockIdx.x) * Cfg::C;
-  for (int idx = threadIdx.x; idx < Cfg::C * S; idx += Cfg::T) {
-    const int c = idx / S, Q = idx % S;
-    const int64_t r = r0 + c;
-    float2 v = make_float2(0.f, 0.f);
-    if (r < n_rows) v = box_value(bb, int(r >> LOGN), int(r & (S - 1)), Q);
-    sm[c * Cfg::LD + Q] = v;
+  int c, tq;
+  row_thread<Cfg>(c, tq);
+  const int64_t r = int64_t(blockIdx.x) * Cfg::C + c;
+  const bool ok = r < int64_t(bb.nb) * S;
+  const int b = int(r >> LOGN), P = int(r & (S - 1));
+  // a thread's samples go through its own slots of the exchange buffer, so that
+  // the chirp's code exists once and not 16 times
+  float2 *own = sm + c * Cfg::LD;
+#pragma unroll 2
+  for (int m = 0; m < kFftE; ++m) {
+    const int Q = tq + m * Cfg::TN;
+    own[fft_pad(Q)] = ok ? box_value(bb, b, P, Q) : make_float2(0.f, 0.f);
   }
+  float2 v[kFftE];
+#pragma unroll
+  for (int m = 0; m < kFftE; ++m) v[m] = own[fft_pad(tq + m * Cfg::TN)];
   __syncthreads();
-  fft_block<LOGN, Cfg::C, Cfg::T, +1>(sm, Cfg::LD, tw);
-  for (int idx = threadIdx.x; idx < Cfg::C * S; idx += Cfg::T) {
-    const int c = idx / S, Q = idx % S;
-    const int64_t r = r0 + c;
-    if (r < n_rows) bb.K[r * S + Q] = sm[c * Cfg::LD + Q];
-  }
+  fft_run<LOGN, +1>(v, tq, own, tw, [&](int, int Q, float2 o) {
+    if (ok) bb.K[r * S + Q] = o;
+  });
 }
 
 // ---- separable kernel boxes (linear chirp, Eq. 5) ------------------------------------
@@ -492,7 +470,7 @@ wproj_status fft2d_impl(const float2 *in, float2 *out, int batch, int inverse, c
                         cudaStream_t s) {
   constexpr int N = 1 << LOGN;
   using RC = RowCfg<LOGN>;
-  using CC = ColCfg<LOGN>;
+  using CC = BoxColCfg<LOGN>;
   const int64_t rows = int64_t(batch) * N;
   if (inverse) {
     WPROJ_TRY(set_smem(k_fft_rows<LOGN, +1>, RC::SMEM));
@@ -513,7 +491,7 @@ template <int LOGN>
 wproj_status box_fft_impl(wproj_plan *p, const BoxBatch &bb, cudaStream_t s) {
   constexpr int S = 1 << LOGN;
   using RC = RowCfg<LOGN>;
-  using CC = ColCfg<LOGN>;
+  using CC = BoxColCfg<LOGN>;
   const float2 *tw = p->twiddle.as<float2>();
   const int64_t rows = int64_t(bb.nb) * S;
   WPROJ_TRY(set_smem(k_box_rows<LOGN>, RC::SMEM));
@@ -672,6 +650,12 @@ wproj_status box_fft_separable_impl(wproj_plan *p, const BoxBatch &bb, cudaStrea
   k_box_outer<<<(int)std::min<int64_t>(152 * 32, ceil_div(n, 256)), 256, 0, s>>>(bb.nb, S, Au, Av,
                                                                                 1.0f / (float(S) * float(S)), bb.K);
   WPROJ_CHECK_LAUNCH("separable boxes");
+  return WPROJ_OK;
+}
+
+wproj_status box_g_table(int S, const float *lsq, float *g, cudaStream_t s) {
+  k_g_table<<<ceil_div(int64_t(S) * S, 256), 256, 0, s>>>(S, lsq, g);
+  WPROJ_CHECK_LAUNCH("chirp remainder table");
   return WPROJ_OK;
 }
 
