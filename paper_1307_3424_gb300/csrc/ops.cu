@@ -182,10 +182,12 @@ k_grid(const int32_t *__restrict__ chunk_tile, const int64_t *__restrict__ chunk
   extern __shared__ float2 acc[];   // [WARPS][TS*TS]
   const int c = blockIdx.x;
   int cbase = 0;
+  const int stride = TS * TS;   // cells of a partial tile
   if (chunk_prob) {
     const BProb &P = tab[chunk_prob[c]];
     logG = P.logG;
     nT = P.nT;
+    TS = min(TS, P.G);   // a 16 x 16 grid is one tile of 16 x 16
     cbase = int(P.grid_off);
   }
   const int tile = chunk_tile[c];
@@ -226,7 +228,7 @@ k_grid(const int32_t *__restrict__ chunk_tile, const int64_t *__restrict__ chunk
     if (more) cur = nxt;
   }
   __syncthreads();
-  float2 *out = partial + int64_t(c) * cells;
+  float2 *out = partial + int64_t(c) * stride;
   for (int i = threadIdx.x; i < cells; i += blockDim.x) {
     float2 s = acc[i];
 #pragma unroll
@@ -250,19 +252,21 @@ k_grid_reduce(const int32_t *__restrict__ tile_chunk_ptr, const float2 *__restri
   __shared__ float2 red[kRedLanes][32];
   int tile = blockIdx.x;
   const int c0 = tile_chunk_ptr[tile], c1 = tile_chunk_ptr[tile + 1];
+  const int stride = TS * TS;
   if (tile_prob) {
     const BProb &P = tab[tile_prob[tile]];
     G = P.G;
     nT = P.nT;
+    TS = min(TS, G);
     tile -= int(P.tile_off);
     Xt2 += P.grid_off;
   }
   const int tu = tile / nT, tv = tile % nT;
-  const int cells = TS * TS;
   const int i = blockIdx.y * 32 + (threadIdx.x & 31), j = threadIdx.x >> 5;   // TS * TS is a multiple of 32
+  if (blockIdx.y * 32 >= TS * TS) return;
   float2 s = make_float2(0.f, 0.f);
 #pragma unroll 4
-  for (int c = c0 + j; c < c1; c += kRedLanes) s = cadd(s, partial[int64_t(c) * cells + i]);
+  for (int c = c0 + j; c < c1; c += kRedLanes) s = cadd(s, partial[int64_t(c) * stride + i]);
   red[j][threadIdx.x & 31] = s;
   __syncthreads();
   if (j == 0) {

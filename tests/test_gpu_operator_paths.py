@@ -75,3 +75,25 @@ def test_dense_rows(wp, N, M, wmax, fmt, value):
     plan.build_kernels(torch.from_numpy(uvw_cells(rng, M, N, wmax)).cuda(), 0.99)
     check_operators(plan, N, 4, rng)
     plan.close()
+
+
+# problems on 16^2 grids (one tile of 16 x 16 cells) beside larger ones
+@pytest.mark.parametrize("ns", [(16, 32, 64), (64, 16, 128), (8, 64)])
+def test_batch_matches_single_plans(wp, ns):
+    rng = np.random.default_rng(sum(ns))
+    ms = [7 * n + 3 for n in ns]
+    uvw = [uvw_cells(rng, m, n, 1.0, edge=0.2) for m, n in zip(ms, ns)]
+    b = wp.Batch(ns, L)
+    b.build_kernels(torch.from_numpy(np.concatenate(uvw)).cuda(), ms, 0.99)
+    b.tune()
+    x = torch.from_numpy(rng.standard_normal(b.pixels).astype(np.float32)).cuda()
+    y = torch.view_as_complex(torch.from_numpy(rng.standard_normal((b.m, 2)).astype(np.float32)).cuda())
+    px, py = b.split_images(b.phi_adj(y)), b.split_vis(b.phi(x))
+    for i, (n, u) in enumerate(zip(ns, uvw)):
+        p = wp.Plan(n, L, box="rule")
+        p.build_kernels(torch.from_numpy(u).cuda(), 0.99)
+        ry, rx = p.phi(b.split_images(x)[i].contiguous()), p.phi_adj(b.split_vis(y)[i].contiguous())
+        assert float((py[i] - ry).norm() / ry.norm()) <= 1e-5
+        assert float((px[i] - rx).norm() / rx.norm()) <= 1e-5
+        p.close()
+    b.close()
