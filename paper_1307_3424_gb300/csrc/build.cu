@@ -12,9 +12,10 @@
 // the gridding taps.  Each row keeps the smallest set of entries, largest
 // modulus first, that holds a fraction e of the row energy (Section 3.2).
 //
-// Pipeline (boxes processed in batches sized to stay in L2):
+// Pipeline (boxes processed in batches):
 //   plan rows -> per-box tables -> 2 FFT passes -> 3-level energy-weighted
-//   radix select (exact integer prefix) -> per-tile counts  [phase 1]
+//   radix select (exact integer prefix) -> per-tile counts  [phase 1; boxes of 32^2
+//   and 64^2 cells in one kernel after the tables, a block per box]
 //   scan counts -> allocate G exactly -> tables + FFT again -> emit  [phase 2]
 //   -> tile lists for gridding, row pieces for degridding.
 #include <math.h>
@@ -24,6 +25,7 @@
 #include <vector>
 
 #include "build.cuh"
+#include "fft.cuh"
 #include "plan.h"
 
 namespace wproj {
@@ -213,8 +215,11 @@ struct SelState {
   int32_t n_tie;
 };
 
+// The FP64 units bound this kernel (Bessel functions of the taps): a tap of either
+// axis per lane, one call for all of them, and what depends only on the geometry
+// (gmax) comes from the host.
 __global__ void k_box_tables(const int32_t *__restrict__ ids, const double *__restrict__ uvw,
-                             const double2 *__restrict__ delta, GridGeom g, int S,
+                             const double2 *__restrict__ delta, GridGeom g, double gmax, int S,
                              const double *__restrict__ lcoord, float2 *__restrict__ Au,
                              float2 *__restrict__ Av, int8_t *__restrict__ mode,
                              float *__restrict__ wf, double *__restrict__ wd,
@@ -224,27 +229,21 @@ __global__ void k_box_tables(const int32_t *__restrict__ ids, const double *__re
   const int k = ids[b];
   const double w = uvw[3 * int64_t(k) + 2];
   const double2 dl = delta[k];
-  __shared__ double tapu[8], tapv[8];
+  __shared__ double tap[16];
+  const double *tapu = tap, *tapv = tap + 8;
   __shared__ int md;
   const int W = g.W;
   const int ntap = (W == 1) ? 1 : W;
-  if (threadIdx.x < ntap) {
-    const int t = (W == 1) ? 0 : int(threadIdx.x) - W / 2 + 1;
-    tapu[threadIdx.x] = (W == 1) ? 1.0 : kb_dev(dl.x - t, W, g.beta);
-    tapv[threadIdx.x] = (W == 1) ? 1.0 : kb_dev(dl.y - t, W, g.beta);
+  if (threadIdx.x < 16 && (threadIdx.x & 7) < ntap) {
+    const int t = (W == 1) ? 0 : int(threadIdx.x & 7) - W / 2 + 1;
+    tap[threadIdx.x] = (W == 1) ? 1.0 : kb_dev((threadIdx.x < 8 ? dl.x : dl.y) - t, W, g.beta);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
     double eu = 0, ev = 0;
     for (int i = 0; i < ntap; ++i) { eu += tapu[i] * tapu[i]; ev += tapv[i] * tapv[i]; }
     int m_ = 0;
-    if (g.chirp == WPROJ_CHIRP_EXACT) {
-      const double lmax = g.extension == WPROJ_EXT_CLAMP ? 0.5 * g.L : g.L;
-      const double x = 2.0 * lmax * lmax;
-      const double d = 1.0 + sqrt(1.0 - x);
-      const double gmax = x * x / (2.0 * d * d);
-      m_ = (fabs(w) * gmax <= 0.25) ? 1 : 2;
-    }
+    if (g.chirp == WPROJ_CHIRP_EXACT) m_ = (fabs(w) * gmax <= 0.25) ? 1 : 2;
     md = m_;
     mode[b] = int8_t(m_);
     wf[b] = float(w);
@@ -617,6 +616,183 @@ k_tie_alloc(const int32_t *__restrict__ ids, const int64_t *__restrict__ seg_bas
   }
 }
 
+// ---- small boxes: transform, selection and tile counts in one kernel ---------------------
+
+// Warp sum of 64-bit integers (modulo 2^64) by three redux.sync of 22, 22 and 20 bits
+__device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v) {
+  const unsigned a = __reduce_add_sync(0xffffffffu, unsigned(v) & 0x3fffffu);
+  const unsigned b = __reduce_add_sync(0xffffffffu, unsigned(v >> 22) & 0x3fffffu);
+  const unsigned c = __reduce_add_sync(0xffffffffu, unsigned(v >> 44));
+  return (unsigned long long)a + ((unsigned long long)b << 22) + ((unsigned long long)c << 44);
+}
+
+// A block takes one S x S box (S = 32 or 64), 16 samples a thread: chirp x taps, row
+// transform, column transform (the passes of k_box_rows and k_fft_cols), then the
+// row's threshold on the samples it holds.  The threshold is the largest key t whose
+// samples of key >= t hold the target energy, found by bisection over the keys with
+// exact integer sums, which is the key the radix select finds; ties and per-tile
+// counts as there.  Phase 2 only transforms (select = 0).
+// Bound by issue: ~30 rounds of 16 compare-adds and a block sum.  The separate
+// kernels passed over the box six times and over 24 KB of histogram per box and
+// level, more than the box itself: 28 ms for 262144 boxes, most of 64^2, against 12.5.
+template <int LOGN>
+__global__ void __launch_bounds__((1 << (2 * LOGN)) / kFftE)
+k_box_small(const BoxBatch bb, const float2 *__restrict__ tw, float scale, int select, double e_target, GridGeom g,
+            const int32_t *__restrict__ ids, const int2 *__restrict__ j0, const int64_t *__restrict__ seg_base,
+            const SelState *__restrict__ sel, int32_t *__restrict__ seg_cnt, int32_t *__restrict__ seg_tieb,
+            uint32_t *__restrict__ r_thr, int32_t *__restrict__ r_ntie, int8_t *__restrict__ r_all,
+            float *__restrict__ r_max) {
+  constexpr int S = 1 << LOGN, TN = S / kFftE, T = S * TN, NW = T / 32;
+  constexpr int LDR = fft_ld(S, LOGN <= 5 ? 2 : 4), LDC = fft_ld(S, 1);   // exchange and matrix rows; columns
+  __shared__ float2 buf[S * (LDR > LDC ? LDR : LDC)];
+  __shared__ unsigned long long part[2][NW];
+  __shared__ unsigned long long s_target;
+  __shared__ unsigned s_max[NW];
+  __shared__ int s_all, s_eq, tile_gt[16], tile_eq[16];
+  const int b = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
+  float2 v[kFftE];
+  {   // rows: thread tq of row P holds columns tq + m TN
+    const int P = t / TN, tq = t % TN;
+    float2 *own = buf + P * LDR;
+#pragma unroll 2
+    for (int m = 0; m < kFftE; ++m) own[fft_pad(tq + m * TN)] = box_value(bb, b, P, tq + m * TN);
+#pragma unroll
+    for (int m = 0; m < kFftE; ++m) v[m] = own[fft_pad(tq + m * TN)];
+    __syncthreads();
+    float2 o[kFftE];
+    fft_run<LOGN, +1>(v, tq, own, tw, [&](int m, int, float2 x) { o[m] = x; });
+#pragma unroll
+    for (int m = 0; m < kFftE; ++m) own[tq + m * TN] = o[m];
+  }
+  __syncthreads();
+  const int c = t % S, tq = t / S;   // columns: thread tq of column c holds rows tq + m TN
+#pragma unroll
+  for (int m = 0; m < kFftE; ++m) v[m] = buf[(tq + m * TN) * LDR + c];
+  __syncthreads();
+  unsigned key[kFftE];
+  {
+    float2 *Kb = bb.K + int64_t(b) * S * S + c;
+    fft_run<LOGN, +1>(v, tq, buf + c * LDC, tw, [&](int m, int P, float2 x) {
+      const float2 k = cscale(x, scale);
+      Kb[P * S] = k;
+      key[m] = __float_as_uint(abs2_rn(k));
+    });
+  }
+  if (!select) return;
+  const int qexp = sel[b].qexp;
+  unsigned long long q[kFftE], sum = 0;
+  unsigned mx = 0;
+#pragma unroll
+  for (int m = 0; m < kFftE; ++m) {
+    q[m] = fixed_energy(__uint_as_float(key[m]), qexp);
+    sum += q[m];
+    mx = max(mx, key[m]);
+  }
+  sum = warp_sum_u64(sum);
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if (lane == 0) {
+    part[0][w] = sum;
+    s_max[w] = mx;
+  }
+  if (t < 16) tile_gt[t] = tile_eq[t] = 0;
+  __syncthreads();
+  unsigned long long tot = 0;
+#pragma unroll
+  for (int i = 0; i < NW; ++i) {
+    tot += part[0][i];
+    mx = max(mx, s_max[i]);
+  }
+  if (t == 0) {
+    const double tgt = e_target * double(tot);
+    s_all = !(tgt < double(tot));
+    s_eq = 0;
+    const unsigned long long x = (unsigned long long)ceil(tgt);
+    s_target = x < 1 ? 1 : x;
+  }
+  __syncthreads();
+  const bool all = s_all != 0;
+  const unsigned long long target = s_target;
+  unsigned lo = 0, hi = mx + 1;          // energy of keys >= lo reaches the target, of keys >= hi does not
+  unsigned long long q_hi = 0;           // energy of keys >= hi
+  if (!all) {
+    for (int it = 1; hi - lo > 1; ++it) {
+      const unsigned mid = lo + ((hi - lo) >> 1);
+      unsigned long long f = 0;
+#pragma unroll
+      for (int m = 0; m < kFftE; ++m) f += key[m] >= mid ? q[m] : 0ull;
+      f = warp_sum_u64(f);
+      if (lane == 0) part[it & 1][w] = f;   // two buffers: one barrier a round
+      __syncthreads();
+      f = 0;
+#pragma unroll
+      for (int i = 0; i < NW; ++i) f += part[it & 1][i];
+      if (f >= target) lo = mid;
+      else { hi = mid; q_hi = f; }
+    }
+  }
+  const unsigned thr = all ? 0u : lo;
+  // per-tile counts: rows of one thread's samples lie in at most three tiles of one column
+  const int k = ids[b], logT = 31 - __clz(g.tile), Gm = g.G - 1;
+  const int2 jk = j0[k];
+  const AxisTiles tu = axis_tiles(jk.x, S, g.G, g.tile), tv = axis_tiles(jk.y, S, g.G, g.tile);
+  const int pv = axis_tile_pos(tv, ((jk.y + (c < S / 2 ? c : c - S)) & Gm) >> logT);
+  int rpos = -1, rgt = 0, req = 0, neq = 0;
+  auto flush = [&]() {
+    if (rgt) atomicAdd(&tile_gt[rpos], rgt);
+    if (req) atomicAdd(&tile_eq[rpos], req);
+    neq += req;
+  };
+#pragma unroll
+  for (int m = 0; m < kFftE; ++m) {
+    const int P = tq + m * TN, su = P < S / 2 ? P : P - S;
+    const int pos = axis_tile_pos(tu, ((jk.x + su) & Gm) >> logT) * tv.nt + pv;
+    if (pos != rpos) {
+      flush();
+      rpos = pos;
+      rgt = req = 0;
+    }
+    rgt += all || key[m] > thr;
+    req += !all && key[m] == thr;
+  }
+  flush();
+  neq = __reduce_add_sync(0xffffffffu, neq);
+  if (lane == 0 && neq) atomicAdd(&s_eq, neq);
+  __syncthreads();
+  if (t) return;
+  int n_tie = 0x7fffffff;
+  if (!all) {
+    const unsigned long long qthr = fixed_energy(__uint_as_float(thr), qexp), rem = target - q_hi;
+    long long nt = qthr > 0 ? (long long)((rem + qthr - 1) / qthr) : (long long)s_eq;
+    if (nt > (long long)s_eq) nt = s_eq;
+    n_tie = int(nt < 0 ? 0 : nt);
+  }
+  // ties go to the earliest tiles (k_tie_alloc)
+  const int64_t base = seg_base[k];
+  const int nt = tu.nt * tv.nt, ntie = all ? 0 : n_tie;
+  int excl = 0;
+  for (int i = 0; i < nt; ++i) {
+    seg_tieb[base + i] = min(excl, ntie);
+    seg_cnt[base + i] = tile_gt[i] + min(tile_eq[i], max(0, ntie - excl));
+    excl += tile_eq[i];
+  }
+  r_thr[k] = thr;
+  r_ntie[k] = n_tie;
+  r_all[k] = int8_t(all);
+  r_max[k] = sqrtf(__uint_as_float(mx));
+}
+
+template <int LOGN>
+wproj_status box_small(const BoxBatch &bb, const float2 *tw, bool select, double e_target, const GridGeom &g,
+                       const int32_t *ids, const int2 *j0, const int64_t *seg_base, const SelState *sel,
+                       int32_t *seg_cnt, int32_t *seg_tieb, uint32_t *r_thr, int32_t *r_ntie, int8_t *r_all, float *r_max,
+                       cudaStream_t s) {
+  constexpr int S = 1 << LOGN;
+  k_box_small<LOGN><<<bb.nb, S * S / kFftE, 0, s>>>(bb, tw, 1.0f / (float(S) * float(S)), select ? 1 : 0, e_target, g, ids,
+                                                    j0, seg_base, sel, seg_cnt, seg_tieb, r_thr, r_ntie, r_all, r_max);
+  WPROJ_CHECK_LAUNCH("small boxes");
+  return WPROJ_OK;
+}
+
 // ---- emission -------------------------------------------------------------------------
 
 // One warp per (box, touched tile) segment, lane = tile column: the warp walks
@@ -655,6 +831,7 @@ k_emit(const float2 *__restrict__ K, int S, const int32_t *__restrict__ ids,
     const int64_t sid = seg_base[k] + seg;
     const int tie0 = seg_tieb[sid];
     const int cnt = seg_cnt[sid];
+    if (cnt == 0 && !rec) continue;   // a small kernel's box touches more tiles than its support
     // COLUMNS: entries at seg_off in col / val; TILE_MASK: the segment's record
     const int64_t o = rec ? 0 : seg_off[sid];
     unsigned char *rp = rec ? stream + seg_rec[sid] : nullptr;
@@ -666,8 +843,11 @@ k_emit(const float2 *__restrict__ K, int S, const int32_t *__restrict__ ids,
     int tie_run = 0, sel_run = 0;
     unsigned my_w = 0;    // lane r keeps row r's selection word and prefix
     int my_pre = 0;
+    // rows of the tile inside the box
+    const unsigned rmask = __ballot_sync(0xffffffffu, lane < TS && ((tile_u * TS + lane - tu.a) & Gm) < S);
+    const int r0 = max(0, __ffs(int(rmask)) - 1), r1 = 32 - __clz(int(rmask));
 #pragma unroll 4
-    for (int r = 0; r < 32; ++r) {
+    for (int r = r0; r < r1; ++r) {
       bool gt = false, eq = false;
       int kidx = 0;
       if (r < TS && col_in) {
@@ -704,6 +884,7 @@ k_emit(const float2 *__restrict__ K, int S, const int32_t *__restrict__ ids,
       sel_run += __popc(sw);
     }
     if (lane == 0 && sel_run != cnt) atomicOr(err, ERR_EMIT);
+    if (lane >= r1) my_pre = sel_run;   // rows past the box
     if (rec) {
       reinterpret_cast<uint32_t *>(rp + kRecHeader)[lane] = my_w;
       reinterpret_cast<uint16_t *>(rp + kRecPrefix)[lane] = uint16_t(my_pre);
@@ -984,17 +1165,15 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
   WPROJ_TRY(r_all.alloc(sizeof(int8_t) * m));
   WPROJ_TRY(r_max.alloc(sizeof(float) * m));
 
+  // boxes of 32^2 and 64^2 cells take the one-kernel form (the linear chirp's boxes are
+  // outer products of two short transforms)
+  auto small_box = [&](int S) { return (S == 32 || S == 64) && (g.chirp == WPROJ_CHIRP_EXACT || sid); };
   p->box_min = 1 << 30;
   p->box_max = 0;
-  int max_nb = 1;
   for (int c = 0; c < 9; ++c) {
     if (cls_ptr[c + 1] <= cls_ptr[c]) continue;
-    const int S = 16 << c;
-    p->box_min = std::min(p->box_min, S);
-    p->box_max = std::max(p->box_max, S);
-    const int64_t per = int64_t(S) * S * sizeof(float2);
-    max_nb = std::max<int>(max_nb, (int)std::min<int64_t>(std::min<int64_t>(cls_ptr[c + 1] - cls_ptr[c], kMaxBatchBoxes),
-                                                            std::max<int64_t>(1, batch_bytes(S) / per)));
+    p->box_min = std::min(p->box_min, 16 << c);
+    p->box_max = std::max(p->box_max, 16 << c);
   }
   DevBuf Kbuf, Au, Av, bmode, bwf, bwd, bsel, hcnt, hq, lcoord, lsq, gtab, bsid;
   // Pass 2 needs every box's transform again.  When the device has room for all
@@ -1013,6 +1192,18 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
       if (!keep_all) cudaGetLastError();   // fall back to recomputing
     }
   }
+  // boxes per batch: what fits in Kbuf, or (small boxes written to Kall) in the tables
+  auto batch_boxes = [&](int c) {
+    const int S = 16 << c;
+    const int64_t n = std::min<int64_t>(cls_ptr[c + 1] - cls_ptr[c], kMaxBatchBoxes);
+    if (keep_all && small_box(S)) return (int)n;
+    return (int)std::min<int64_t>(n, std::max<int64_t>(1, int64_t(batch_bytes(S) / (size_t(S) * S * sizeof(float2)))));
+  };
+  int max_nb = 1, max_nb_hist = 1;
+  for (int c = 0; c < 9; ++c) {
+    max_nb = std::max(max_nb, batch_boxes(c));
+    if (!small_box(16 << c)) max_nb_hist = std::max(max_nb_hist, batch_boxes(c));
+  }
   if (!keep_all)
     WPROJ_TRY(Kbuf.alloc(std::max<size_t>(kBuildBatchBytes, size_t(p->box_max) * p->box_max * sizeof(float2))));
   WPROJ_TRY(Au.alloc(sizeof(float2) * size_t(max_nb) * p->box_max));
@@ -1022,12 +1213,20 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
   WPROJ_TRY(bwd.alloc(sizeof(double) * max_nb));
   WPROJ_TRY(bsel.alloc(sizeof(SelState) * max_nb));
   if (sid) WPROJ_TRY(bsid.alloc(sizeof(int32_t) * max_nb));
-  WPROJ_TRY(hcnt.alloc(sizeof(unsigned) * kHistBins * size_t(max_nb)));
-  WPROJ_TRY(hq.alloc(sizeof(unsigned long long) * kHistBins * size_t(max_nb)));
+  WPROJ_TRY(hcnt.alloc(sizeof(unsigned) * kHistBins * size_t(max_nb_hist)));
+  WPROJ_TRY(hq.alloc(sizeof(unsigned long long) * kHistBins * size_t(max_nb_hist)));
   WPROJ_TRY(lcoord.alloc(sizeof(double) * p->box_max));
   WPROJ_TRY(lsq.alloc(sizeof(float) * p->box_max));
   if (g.chirp == WPROJ_CHIRP_EXACT) WPROJ_TRY(gtab.alloc(sizeof(float) * p->box_max * p->box_max));
 
+  // largest remainder g of the exact chirp over the box (x = l^2 + m^2 <= 2 lmax^2)
+  double gmax = 0;
+  {
+    const double lmax = g.extension == WPROJ_EXT_CLAMP ? 0.5 * g.L : g.L;
+    const double x = 2.0 * lmax * lmax;
+    const double d = 1.0 + sqrt(1.0 - x);
+    gmax = x * x / (2.0 * d * d);
+  }
   const double e_target = e + kSelectMargin;
   const int vdt = g.value_dtype;
   const int vb = vdt == WPROJ_VAL_F32 ? 8 : 4;
@@ -1122,8 +1321,8 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
       if (ghi <= glo) continue;
       const int S = 16 << c;
       const int64_t per = int64_t(S) * S;
-      const int nbmax = (int)std::min<int64_t>(std::min<int64_t>(ghi - glo, kMaxBatchBoxes),
-                                               std::max<int64_t>(1, batch_bytes(S) / (per * 8)));
+      const int nbmax = batch_boxes(c);
+      const bool small = small_box(S);
       k_coord_tables<<<ceil_div(S, 256), 256, 0, s>>>(S, g.L, g.extension == WPROJ_EXT_CLAMP,
                                                       lcoord.as<double>(), lsq.as<float>());
       WPROJ_CHECK_LAUNCH("coord tables");
@@ -1139,7 +1338,7 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
         const bool transform = phase == 1 || !keep_all;
         ScopedTimer t_fft(p, TC_BFFT, s);
         if (transform) {
-          k_box_tables<<<nb, 128, 0, s>>>(ids, uvw, d_delta.as<double2>(), g, S, lcoord.as<double>(),
+          k_box_tables<<<nb, 128, 0, s>>>(ids, uvw, d_delta.as<double2>(), g, gmax, S, lcoord.as<double>(),
                                           Au.as<float2>(), Av.as<float2>(), bmode.as<int8_t>(),
                                           bwf.as<float>(), bwd.as<double>(), bsel.as<SelState>(), sid,
                                           sid ? p->screen_max2.as<float>() : nullptr, bsid.as<int32_t>());
@@ -1151,9 +1350,17 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
             bb.screens = p->screens.as<float2>();
             bb.bsid = bsid.as<int32_t>();
           }
-          WPROJ_TRY(box_fft(p, bb, s));
+          if (small) {   // phase 1: with the selection and the counts
+            const auto run = S == 32 ? box_small<5> : box_small<6>;
+            WPROJ_TRY(run(bb, p->twiddle.as<float2>(), phase == 1, e_target, g, ids, d_j0.as<int2>(),
+                          d_segbase.as<int64_t>(), bsel.as<SelState>(), p->seg_cnt.as<int32_t>(), d_tieb.as<int32_t>(),
+                          r_thr.as<uint32_t>(), r_ntie.as<int32_t>(), r_all.as<int8_t>(), r_max.as<float>(), s));
+          } else {
+            WPROJ_TRY(box_fft(p, bb, s));
+          }
         }
         t_fft.stop();
+        if (phase == 1 && small) continue;
         const dim3 hgrid(ceil_div(per, kSelChunk), nb);
         if (phase == 1) {
           ScopedTimer t_sel(p, TC_BSEL, s);

@@ -35,16 +35,6 @@ __global__ void k_twiddles(float2 *tw) {
 __device__ __forceinline__ constexpr bool in_image(int m) { return m < 4 || m >= 12; }
 __device__ __forceinline__ int pad_to_img(int m, int P, int G) { return m < 4 ? P + G / 4 : P - G + G / 4; }
 
-// thread -> (transform of the block, thread of the transform): rows / columns
-template <class Cfg> __device__ __forceinline__ void row_thread(int &c, int &tq) {
-  c = int(threadIdx.x) / Cfg::TN;
-  tq = int(threadIdx.x) % Cfg::TN;
-}
-template <class Cfg> __device__ __forceinline__ void col_thread(int &c, int &tq) {
-  c = int(threadIdx.x) % Cfg::C;
-  tq = int(threadIdx.x) / Cfg::C;
-}
-
 // ---- Phi: F Z A --------------------------------------------------------------
 
 // Each pass is a device body (block `blk` of one transform set) called by a
@@ -270,39 +260,6 @@ __global__ void k_g_table(int S, const float *__restrict__ lsq, float *__restric
   const float n = sqrtf(1.f - x);
   const float d = 1.f + n;
   g[i] = (x * x) / (2.f * d * d);
-}
-
-// f[P][Q] = Au[P] Av[Q] e^{2 pi i w g(x)}: the chirp (Eq. 4 / Eq. 5) times the KB
-// tap polynomial, at box offsets P' = P (P < S/2) or P - S; Au, Av carry the
-// separable part of the phase, w (l^2 + m^2) / 2, and the taps.
-__device__ __forceinline__ float2 box_value(const BoxBatch &bb, int b, int P, int Q) {
-  const float2 a = bb.Au[int64_t(b) * bb.S + P];
-  const float2 c = bb.Av[int64_t(b) * bb.S + Q];
-  float2 f = cmul(a, c);
-  const int mode = bb.mode[b];
-  if (mode == 1) {
-    // exact chirp: phase w (1 - n) = w x / 2 + w g(x), g = x^2 / (2 (1 + n)^2), the
-    // remainder |w g| <= 1/4 cycle so FP32 keeps it to ~1e-7 cycles; g does not
-    // depend on the box and comes from a table of the class (k_g_table)
-    float sn, cs;
-    sincospif(2.f * (bb.wf[b] * __ldg(bb.gtab + int64_t(P) * bb.S + Q)), &sn, &cs);
-    f = cmul(f, make_float2(cs, sn));
-  } else if (mode == 2) {
-    // large w: the full phase argument in FP64, reduced mod 1
-    const double l = bb.lcoord[P], m = bb.lcoord[Q];
-    const double x = l * l + m * m;
-    const double ph = bb.wd[b] * x / (1.0 + sqrt(1.0 - x));
-    const double fr = ph - floor(ph);
-    float sn, cs;
-    sincospif(2.f * float(fr), &sn, &cs);
-    f = cmul(f, make_float2(cs, sn));
-  }
-  if (bb.screens) {
-    const int S = bb.S, h = S / 2;
-    const float2 a = bb.screens[(int64_t(bb.bsid[b]) * S + ((P + h) & (S - 1))) * S + ((Q + h) & (S - 1))];
-    f = cmul(f, a);
-  }
-  return f;
 }
 
 template <int LOGN>

@@ -191,4 +191,14 @@ template <int LOGN> struct BoxColCfg {
   static constexpr size_t SMEM = size_t(C) * LD * sizeof(float2);
 };
 
+// thread -> (transform of the block, thread of the transform): rows / columns
+template <class Cfg> __device__ __forceinline__ void row_thread(int &c, int &tq) {
+  c = int(threadIdx.x) / Cfg::TN;
+  tq = int(threadIdx.x) % Cfg::TN;
+}
+template <class Cfg> __device__ __forceinline__ void col_thread(int &c, int &tq) {
+  c = int(threadIdx.x) % Cfg::C;
+  tq = int(threadIdx.x) / Cfg::C;
+}
+
 }  // namespace wproj

@@ -97,3 +97,18 @@ def test_batch_matches_single_plans(wp, ns):
         assert float((px[i] - rx).norm() / rx.norm()) <= 1e-5
         p.close()
     b.close()
+
+
+# boxes built by one block each (32^2 and 64^2 cells): kept energy, cardinality and
+# values against the oracle, with whole boxes (e = 1), single entries (small e), w = 0
+# (mirror-symmetric kernels: ties at the cut) and each tap count
+@pytest.mark.parametrize("N,e,W,wmax", [(16, 0.99, 4, 0.0), (32, 0.05, 4, 4.0), (32, 0.9, 8, 4.0), (64, 0.999, 6, 4.0),
+                                        (64, 1.0, 4, 2.0), (128, 0.99, 4, 4.0)])
+def test_small_boxes(wp, N, e, W, wmax):
+    from test_gpu_parity import check_build
+    rng = np.random.default_rng(N + W)
+    uvw = uvw_cells(rng, 40, N, wmax, edge=0.2)
+    plan = wp.Plan(N, L, kb_support=W, box="rule")
+    plan.build_kernels(torch.from_numpy(uvw).cuda(), e)
+    check_build(plan, O.Geometry(N, L, W=W), uvw, e, "rule")
+    plan.close()
