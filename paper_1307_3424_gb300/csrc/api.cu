@@ -42,9 +42,36 @@ wproj_status DevBuf::alloc(size_t n) {
   bytes = n;
   return WPROJ_OK;
 }
+wproj_status DevBuf::reuse(size_t n) {
+  if (ptr && own && n > 0 && bytes >= n && bytes - n <= n / 8) return WPROJ_OK;
+  return alloc(n);
+}
 wproj_status DevBuf::ensure(size_t n) {
   if (ptr && bytes >= n) return WPROJ_OK;
   return alloc(n);
+}
+
+static thread_local ScratchScope *t_scratch = nullptr;
+
+ScratchScope::ScratchScope(DevBuf &b, size_t bytes) : block(b), outer(t_scratch) {
+  if (block.ensure(bytes) != WPROJ_OK) block.release();   // no room: every buffer its own allocation
+  t_scratch = this;
+}
+ScratchScope::~ScratchScope() {
+  t_scratch = outer;
+  if (block.bytes > kScratchKeep) block.release();
+}
+wproj_status TmpBuf::alloc(size_t n) {
+  release();
+  const size_t need = (std::max<size_t>(n, 16) + 255) & ~size_t(255);
+  if (t_scratch && t_scratch->block.bytes - t_scratch->used >= need) {
+    ptr = t_scratch->block.as<char>() + t_scratch->used;
+    t_scratch->used += need;
+    bytes = n;
+    own = false;
+    return WPROJ_OK;
+  }
+  return DevBuf::alloc(n);
 }
 
 EventTimer::~EventTimer() {

@@ -1017,7 +1017,7 @@ __global__ void k_chunk_fill(int n_tiles, const int64_t *__restrict__ tile_ptr,
 
 wproj_status make_row_pieces(int64_t m, const int64_t *row_ptr, int64_t piece, DevBuf &piece_row, DevBuf &piece_lo,
                              DevBuf &piece_len, DevBuf &row_piece_ptr, int64_t *n_pieces, cudaStream_t s) {
-  DevBuf npc, pbase;
+  TmpBuf npc, pbase;
   WPROJ_TRY(npc.alloc(sizeof(int32_t) * std::max<int64_t>(1, m)));
   WPROJ_TRY(pbase.alloc(sizeof(int64_t) * (m + 1)));
   k_npieces<<<ceil_div(m, 256), 256, 0, s>>>(m, row_ptr, piece, npc.as<int32_t>());
@@ -1044,7 +1044,7 @@ wproj_status make_row_pieces(int64_t m, const int64_t *row_ptr, int64_t piece, D
 wproj_status make_tile_chunks(int n_tiles, const int64_t *tptr, const int64_t *cum, int64_t n_seg, int64_t nnz,
                               int64_t chunk, DevBuf &chunk_tile, DevBuf &chunk_lo, DevBuf &chunk_hi,
                               DevBuf &tile_chunk_ptr, int64_t *n_chunks, cudaStream_t s) {
-  DevBuf nch, chbase;
+  TmpBuf nch, chbase;
   WPROJ_TRY(nch.alloc(sizeof(int32_t) * n_tiles));
   WPROJ_TRY(chbase.alloc(sizeof(int64_t) * (n_tiles + 1)));
   k_tile_chunks<<<ceil_div(n_tiles, 256), 256, 0, s>>>(n_tiles, tptr, cum, n_seg, nnz, chunk, nch.as<int32_t>());
@@ -1097,13 +1097,16 @@ wproj_status set_screens_impl(wproj_plan *p, const float2 *screens, int n, cudaS
 wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, double e, cudaStream_t s,
                                 const int32_t *sid) {
   auto t_start = std::chrono::steady_clock::now();
+  // the previous G's buffers are overwritten where they fit: no kernel may still read them
+  WPROJ_CUDA(cudaDeviceSynchronize());
+  ScratchScope scope(p->scratch, (size_t(4) << 20) + size_t(384) * size_t(m));
   const GridGeom &g = p->g;
   p->built = false;
   p->dr_valid = false;
   p->m = p->nnz = p->n_seg = p->n_chunks = p->n_pieces = 0;
 
   // ---- rows
-  DevBuf d_j0, d_delta, d_Sk, d_ntile, d_sclass, d_err, d_segbase;
+  TmpBuf d_j0, d_delta, d_Sk, d_ntile, d_sclass, d_err, d_segbase;
   WPROJ_TRY(d_j0.alloc(sizeof(int2) * m));
   WPROJ_TRY(d_delta.alloc(sizeof(double2) * m));
   WPROJ_TRY(d_Sk.alloc(sizeof(int32_t) * m));
@@ -1136,11 +1139,11 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
   WPROJ_CUDA(cudaMemcpy(&last_nt, d_ntile.as<int32_t>() + (m - 1), sizeof(int32_t), cudaMemcpyDeviceToHost));
   const int64_t n_seg = last_base + last_nt;
   if (n_seg >= (int64_t(1) << 31)) return fail(WPROJ_ERR_UNSUPPORTED, "build_kernels: too many (row, tile) segments");
-  WPROJ_TRY(p->seg_off.alloc(sizeof(int64_t) * std::max<int64_t>(1, n_seg)));
-  WPROJ_TRY(p->seg_cnt.alloc(sizeof(int32_t) * std::max<int64_t>(1, n_seg)));
-  WPROJ_TRY(p->seg_row.alloc(sizeof(int32_t) * std::max<int64_t>(1, n_seg)));
-  DevBuf d_cntgt, d_cnteq, d_tieb;
-  WPROJ_TRY(p->seg_tile.alloc(sizeof(int32_t) * std::max<int64_t>(1, n_seg)));
+  WPROJ_TRY(p->seg_off.reuse(sizeof(int64_t) * std::max<int64_t>(1, n_seg)));
+  WPROJ_TRY(p->seg_cnt.reuse(sizeof(int32_t) * std::max<int64_t>(1, n_seg)));
+  WPROJ_TRY(p->seg_row.reuse(sizeof(int32_t) * std::max<int64_t>(1, n_seg)));
+  TmpBuf d_cntgt, d_cnteq, d_tieb;
+  WPROJ_TRY(p->seg_tile.reuse(sizeof(int32_t) * std::max<int64_t>(1, n_seg)));
   WPROJ_TRY(d_cntgt.alloc(sizeof(int32_t) * std::max<int64_t>(1, n_seg)));
   WPROJ_TRY(d_cnteq.alloc(sizeof(int32_t) * std::max<int64_t>(1, n_seg)));
   WPROJ_TRY(d_tieb.alloc(sizeof(int32_t) * std::max<int64_t>(1, n_seg)));
@@ -1151,7 +1154,7 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
   WPROJ_CHECK_LAUNCH("seg fill");
 
   // ---- group rows by box size (stable: rows ascending inside a group)
-  DevBuf d_ids, d_cls_ptr;
+  TmpBuf d_ids, d_cls_ptr;
   WPROJ_TRY(d_ids.alloc(sizeof(int32_t) * m));
   WPROJ_TRY(d_cls_ptr.alloc(sizeof(int64_t) * 10));
   WPROJ_TRY(stable_bin_sort(d_sclass.as<int32_t>(), m, 9, d_ids.as<int32_t>(), d_cls_ptr.as<int64_t>(), s));
@@ -1159,7 +1162,7 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
   WPROJ_CUDA(cudaMemcpy(cls_ptr, d_cls_ptr.ptr, sizeof(cls_ptr), cudaMemcpyDeviceToHost));
 
   // per-row selection results
-  DevBuf r_thr, r_ntie, r_all, r_max;
+  TmpBuf r_thr, r_ntie, r_all, r_max;
   WPROJ_TRY(r_thr.alloc(sizeof(uint32_t) * m));
   WPROJ_TRY(r_ntie.alloc(sizeof(int32_t) * m));
   WPROJ_TRY(r_all.alloc(sizeof(int8_t) * m));
@@ -1175,7 +1178,8 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
     p->box_min = std::min(p->box_min, 16 << c);
     p->box_max = std::max(p->box_max, 16 << c);
   }
-  DevBuf Kbuf, Au, Av, bmode, bwf, bwd, bsel, hcnt, hq, lcoord, lsq, gtab, bsid;
+  DevBuf Kbuf;
+  TmpBuf Au, Av, bmode, bwf, bwd, bsel, hcnt, hq, lcoord, lsq, gtab, bsid;
   // Pass 2 needs every box's transform again.  When the device has room for all
   // of them (and, with a margin, for G, whose size is at most 1.5x theirs), pass
   // 1 keeps them and pass 2 emits without recomputing the tables and FFTs;
@@ -1231,7 +1235,7 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
   const int vdt = g.value_dtype;
   const int vb = vdt == WPROJ_VAL_F32 ? 8 : 4;
   const int n_tiles = g.nT * g.nT;
-  DevBuf tile_seg, tptr;
+  TmpBuf tile_seg, tptr;
   bool want_runs = false;   // TILE_RUNS: emitted as columns, then transcoded
   int64_t n_rec = 0;        // TILE_RUNS: records (segments holding entries), tile order
 
@@ -1280,10 +1284,10 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
         p->col.release();
         p->val.release();
         p->seg_meta.release();
-        DevBuf rsz;
+        TmpBuf rsz;
         WPROJ_TRY(rsz.alloc(sizeof(int32_t) * std::max<int64_t>(1, n_seg)));
-        WPROJ_TRY(p->rec_off.alloc(sizeof(int64_t) * (n_seg + 1)));
-        WPROJ_TRY(p->seg_rec.alloc(sizeof(int64_t) * std::max<int64_t>(1, n_seg)));
+        WPROJ_TRY(p->rec_off.reuse(sizeof(int64_t) * (n_seg + 1)));
+        WPROJ_TRY(p->seg_rec.reuse(sizeof(int64_t) * std::max<int64_t>(1, n_seg)));
         int64_t total = 0;
         if (n_seg > 0) {
           k_rec_size<<<ceil_div(n_seg, 256), 256, 0, s>>>(n_seg, tile_seg.as<int32_t>(), p->seg_cnt.as<int32_t>(), vb,
@@ -1300,7 +1304,7 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
           WPROJ_CHECK_LAUNCH("record offsets");
         }
         WPROJ_CUDA(cudaMemcpy(p->rec_off.as<int64_t>() + n_seg, &total, sizeof(int64_t), cudaMemcpyHostToDevice));
-        WPROJ_TRY(p->stream.alloc(std::max<int64_t>(16, total)));
+        WPROJ_TRY(p->stream.reuse(std::max<int64_t>(16, total)));
         WPROJ_CUDA(cudaMemsetAsync(p->stream.ptr, 0, std::max<int64_t>(16, total), s));   // record padding
         p->stream_bytes = total;
       } else {
@@ -1308,10 +1312,10 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
         p->seg_rec.release();
         p->rec_off.release();
         p->stream_bytes = 0;
-        WPROJ_TRY(p->col.alloc(sizeof(int32_t) * std::max<int64_t>(1, p->nnz)));
-        WPROJ_TRY(p->val.alloc(int64_t(vb) * std::max<int64_t>(1, p->nnz)));
+        WPROJ_TRY(p->col.reuse(sizeof(int32_t) * std::max<int64_t>(1, p->nnz)));
+        WPROJ_TRY(p->val.reuse(int64_t(vb) * std::max<int64_t>(1, p->nnz)));
       }
-      WPROJ_TRY(p->row_ptr.alloc(sizeof(int64_t) * (m + 1)));
+      WPROJ_TRY(p->row_ptr.reuse(sizeof(int64_t) * (m + 1)));
       k_row_ptr<<<ceil_div(m + 1, 256), 256, 0, s>>>(m, d_segbase.as<int64_t>(), p->seg_off.as<int64_t>(),
                                                      d_ntile.as<int32_t>(), n_seg, p->nnz, p->row_ptr.as<int64_t>());
       WPROJ_CHECK_LAUNCH("row ptr");
@@ -1410,7 +1414,7 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
   }
   // row scales (max |K| per row) for the 16-bit value forms
   if (vdt != WPROJ_VAL_F32) {
-    WPROJ_TRY(p->row_scale.alloc(sizeof(float) * m));
+    WPROJ_TRY(p->row_scale.reuse(sizeof(float) * m));
     WPROJ_CUDA(cudaMemcpyAsync(p->row_scale.ptr, r_max.ptr, sizeof(float) * m, cudaMemcpyDeviceToDevice, s));
   } else {
     p->row_scale.release();
@@ -1442,18 +1446,18 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
     p->piece_lo.release();
     p->piece_len.release();
     p->row_piece_ptr.release();
-    WPROJ_TRY(p->piece_partial.alloc(sizeof(float2)));
+    WPROJ_TRY(p->piece_partial.reuse(sizeof(float2)));
   } else if (p->fmt == WPROJ_INDEX_TILE_MASK) {
     p->n_pieces = 0;
     p->piece_row.release();
     p->piece_lo.release();
     p->piece_len.release();
     p->row_piece_ptr.release();
-    WPROJ_TRY(p->piece_partial.alloc(sizeof(float2) * std::max<int64_t>(1, kStreamWarps * n_seg)));
+    WPROJ_TRY(p->piece_partial.reuse(sizeof(float2) * std::max<int64_t>(1, kStreamWarps * n_seg)));
   } else {
     WPROJ_TRY(make_row_pieces(m, p->row_ptr.as<int64_t>(), degrid_piece(p->nnz), p->piece_row, p->piece_lo,
                               p->piece_len, p->row_piece_ptr, &p->n_pieces, s));
-    WPROJ_TRY(p->piece_partial.alloc(sizeof(float2) * std::max<int64_t>(1, p->n_pieces)));
+    WPROJ_TRY(p->piece_partial.reuse(sizeof(float2) * std::max<int64_t>(1, p->n_pieces)));
   }
 
   // ---- gridding: chunks of one tile's segments (tile order), balanced by entries
@@ -1462,10 +1466,10 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
     const int64_t chunk = grid_chunk(p->nnz);
     // the gridding's items in tile order: all segments, or the records of TILE_RUNS
     const int64_t n_items = p->fmt == WPROJ_INDEX_TILE_RUNS ? n_rec : n_seg;
-    DevBuf cntsorted, cum;
+    TmpBuf cntsorted, cum;
     WPROJ_TRY(cntsorted.alloc(sizeof(int32_t) * std::max<int64_t>(1, n_items)));
     WPROJ_TRY(cum.alloc(sizeof(int64_t) * std::max<int64_t>(1, n_items)));
-    if (!rec) WPROJ_TRY(p->seg_meta.alloc(sizeof(SegMeta) * std::max<int64_t>(1, n_seg)));
+    if (!rec) WPROJ_TRY(p->seg_meta.reuse(sizeof(SegMeta) * std::max<int64_t>(1, n_seg)));
     if (n_items > 0) {
       k_gather_cnt<<<ceil_div(n_items, 256), 256, 0, s>>>(n_items, tile_seg.as<int32_t>(), p->seg_cnt.as<int32_t>(),
                                                         p->seg_off.as<int64_t>(), p->seg_row.as<int32_t>(),
@@ -1477,22 +1481,22 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
     WPROJ_TRY(make_tile_chunks(n_tiles, tptr.as<int64_t>(), cum.as<int64_t>(), n_items, p->nnz, chunk, p->chunk_tile,
                                p->chunk_lo, p->chunk_hi, p->tile_chunk_ptr, &p->n_chunks, s));
     // column format: a cell-major copy for the gridding (packed rows need m <= 2^22)
-    p->has_cells = false;
-    p->tile_ent.release();
-    p->cell_ent.release();
-    p->cell_val.release();
-    if (!rec && g.tile == 32 && m <= (int64_t(1) << 22)) {
+    p->has_cells = !rec && g.tile == 32 && m <= (int64_t(1) << 22);
+    if (p->has_cells) {
       WPROJ_TRY(build_cells(p, tptr.as<int64_t>(), cum.as<int64_t>(), n_seg, s));
-      p->has_cells = true;
+    } else {
+      p->tile_ent.release();
+      p->cell_ent.release();
+      p->cell_val.release();
     }
-    WPROJ_TRY(p->grid_partial.alloc(sizeof(float2) * size_t(p->n_chunks) * g.tile * g.tile));
+    WPROJ_TRY(p->grid_partial.reuse(sizeof(float2) * size_t(p->n_chunks) * g.tile * g.tile));
   }
-  WPROJ_TRY(p->ytmp.alloc(sizeof(float2) * m));
+  WPROJ_TRY(p->ytmp.reuse(sizeof(float2) * m));
   WPROJ_CUDA(cudaMemcpyAsync(&herr, d_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));
   WPROJ_CUDA(cudaStreamSynchronize(s));
   if (herr & ERR_EMIT) return fail(WPROJ_ERR_CUDA, "build_kernels: emission pass disagrees with the counting pass");
   // first segment of every row, closed by n_seg (per-row reduction of segment partials)
-  WPROJ_TRY(p->seg_base.alloc(sizeof(int64_t) * (m + 1)));
+  WPROJ_TRY(p->seg_base.reuse(sizeof(int64_t) * (m + 1)));
   WPROJ_CUDA(cudaMemcpy(p->seg_base.ptr, d_segbase.ptr, sizeof(int64_t) * m, cudaMemcpyDeviceToDevice));
   WPROJ_CUDA(cudaMemcpy(p->seg_base.as<int64_t>() + m, &n_seg, sizeof(int64_t), cudaMemcpyHostToDevice));
   p->m = m;

@@ -404,10 +404,10 @@ __global__ void k_tile_ent(int n_tiles, const int64_t *__restrict__ tptr, const 
 wproj_status build_cells(wproj_plan *p, const int64_t *tptr, const int64_t *cum, int64_t n_seg, cudaStream_t s) {
   const int n_tiles = p->g.nT * p->g.nT;
   const int vb = p->g.value_dtype == WPROJ_VAL_F32 ? 8 : 4;
-  WPROJ_TRY(p->tile_ent.alloc(sizeof(int64_t) * (n_tiles + 1)));
+  WPROJ_TRY(p->tile_ent.reuse(sizeof(int64_t) * (n_tiles + 1)));
   // 4 entries of padding: the gridding reads whole 16-byte words of 4 entries
-  WPROJ_TRY(p->cell_ent.alloc(sizeof(uint32_t) * (p->nnz + kCellPad)));
-  WPROJ_TRY(p->cell_val.alloc(int64_t(vb) * (p->nnz + kCellPad)));
+  WPROJ_TRY(p->cell_ent.reuse(sizeof(uint32_t) * (p->nnz + kCellPad)));
+  WPROJ_TRY(p->cell_val.reuse(int64_t(vb) * (p->nnz + kCellPad)));
   k_tile_ent<<<ceil_div(n_tiles + 1, 256), 256, 0, s>>>(n_tiles, tptr, cum, n_seg, p->nnz,
                                                        p->tile_ent.as<int64_t>());
   WPROJ_CHECK_LAUNCH("tile entries");
@@ -428,7 +428,7 @@ wproj_status build_cells(wproj_plan *p, const int64_t *tptr, const int64_t *cum,
   const int64_t cap = std::max<int64_t>(1, p->nnz / (int64_t(n_tiles) * 4096));
   p->cell_parts = (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(want, cap), 64));
   if (p->cell_parts > 1) {
-    WPROJ_TRY(p->cell_partial.alloc(sizeof(float2) * size_t(n_tiles) * p->cell_parts * 1024));
+    WPROJ_TRY(p->cell_partial.reuse(sizeof(float2) * size_t(n_tiles) * p->cell_parts * 1024));
   } else {
     p->cell_partial.release();
   }

@@ -14,18 +14,41 @@ namespace wproj {
 struct DevBuf {
   void *ptr = nullptr;
   size_t bytes = 0;
+  bool own = true;   // false: the memory belongs to a scratch block
   DevBuf() = default;
   DevBuf(const DevBuf &) = delete;
   DevBuf &operator=(const DevBuf &) = delete;
   ~DevBuf() { release(); }
   void release() {
-    if (ptr) cudaFree(ptr);
+    if (ptr && own) cudaFree(ptr);
     ptr = nullptr;
     bytes = 0;
+    own = true;
   }
   wproj_status alloc(size_t n);           // exact size, contents undefined
   wproj_status ensure(size_t n);          // grow (contents discarded)
+  wproj_status reuse(size_t n);           // keep an allocation of n to 9/8 n bytes, else as alloc
   template <class T> T *as() const { return static_cast<T *>(ptr); }
+};
+
+// Temporaries of a build: parts of one scratch block while a ScratchScope of the
+// thread is open (a build makes 60 to 100 of them, and a cudaMalloc with its cudaFree
+// costs ~60 us: 7.5 of the 50 ms of 262144 short rows), allocations of their own
+// outside it or when the block is used up.  Nothing is handed out twice within a
+// scope, so a buffer dropped while kernels still read it stays theirs.
+struct TmpBuf : DevBuf {
+  wproj_status alloc(size_t n);
+};
+
+// The block belongs to the plan (kept up to kScratchKeep bytes, freed with it); the
+// scope ends after the build has synchronised its stream.
+constexpr size_t kScratchKeep = size_t(64) << 20;
+struct ScratchScope {
+  ScratchScope(DevBuf &block, size_t bytes);
+  ~ScratchScope();
+  DevBuf &block;
+  size_t used = 0;
+  ScratchScope *outer;
 };
 
 // One (row, tile) segment of G as the gridding reads it: entries [off, off+cnt)
@@ -159,6 +182,7 @@ struct wproj_plan {
   wproj::DevBuf row_piece_ptr;   // int32[m+1]
 
   // work buffers
+  wproj::DevBuf scratch;     // temporaries of a build
   wproj::DevBuf Xt;          // float2[G*G]  F Z A x
   wproj::DevBuf Xt2;         // float2[G*G]  G^H y
   wproj::DevBuf inter;       // float2[N*G]  between FFT passes

@@ -656,7 +656,7 @@ wproj_status build_runs(wproj_plan *p, const int2 *j0, const int32_t *Sk, int32_
   const int logG = ilog2(g.G);
   const int nb_rows = grid_blocks(m, 1), nb_seg = grid_blocks(std::max<int64_t>(1, n_seg), 8);
   // ---- counting passes
-  DevBuf pc, nr, bytes, err;
+  TmpBuf pc, nr, bytes, err;
   WPROJ_TRY(pc.alloc(sizeof(int32_t) * m));
   WPROJ_TRY(nr.alloc(sizeof(int32_t) * m));
   WPROJ_TRY(bytes.alloc(sizeof(int32_t) * std::max<int64_t>(1, n_seg)));
@@ -679,14 +679,14 @@ wproj_status build_runs(wproj_plan *p, const int2 *j0, const int32_t *Sk, int32_
   if (herr) return fail(WPROJ_ERR_UNSUPPORTED, "build_kernels: a row or segment holds more than 64 runs");
   // ---- row-major copy
   {
-    WPROJ_TRY(p->rm_vptr.alloc(sizeof(int64_t) * (m + 1)));
-    WPROJ_TRY(p->rm_rptr.alloc(sizeof(int64_t) * (m + 1)));
-    WPROJ_TRY(p->rm_org.alloc(sizeof(uint32_t) * m));
+    WPROJ_TRY(p->rm_vptr.reuse(sizeof(int64_t) * (m + 1)));
+    WPROJ_TRY(p->rm_rptr.reuse(sizeof(int64_t) * (m + 1)));
+    WPROJ_TRY(p->rm_org.reuse(sizeof(uint32_t) * m));
     int64_t n_vals = 0, n_runs = 0;
     WPROJ_TRY(scan_total(pc.as<int32_t>(), p->rm_vptr.as<int64_t>(), m, &n_vals, s));
     WPROJ_TRY(scan_total(nr.as<int32_t>(), p->rm_rptr.as<int64_t>(), m, &n_runs, s));
-    WPROJ_TRY(p->rm_run.alloc(sizeof(uint32_t) * std::max<int64_t>(1, n_runs)));
-    WPROJ_TRY(p->rm_val.alloc(int64_t(vb) * std::max<int64_t>(4, n_vals)));
+    WPROJ_TRY(p->rm_run.reuse(sizeof(uint32_t) * std::max<int64_t>(1, n_runs)));
+    WPROJ_TRY(p->rm_val.reuse(int64_t(vb) * std::max<int64_t>(4, n_vals)));
     WPROJ_CUDA(cudaMemsetAsync(p->rm_val.ptr, 0, int64_t(vb) * std::max<int64_t>(4, n_vals), s));
     k_rm_build<<<nb_rows, 64, 0, s>>>(m, p->row_ptr.as<int64_t>(), p->col.as<int32_t>(),
                                       p->val.as<unsigned char>(), vb, j0, Sk, logG, nullptr, nullptr, nullptr,
@@ -702,7 +702,7 @@ wproj_status build_runs(wproj_plan *p, const int2 *j0, const int32_t *Sk, int32_
     const int n_tiles = g.nT * g.nT;
     int64_t nr_ = 0;
     {
-      DevBuf flag, pos, tmp;
+      TmpBuf flag, pos, tmp;
       WPROJ_TRY(flag.alloc(sizeof(int32_t) * std::max<int64_t>(1, n_seg)));
       WPROJ_TRY(pos.alloc(sizeof(int64_t) * (n_seg + 1)));
       WPROJ_TRY(tmp.alloc(sizeof(int32_t) * std::max<int64_t>(1, n_seg)));
@@ -722,10 +722,10 @@ wproj_status build_runs(wproj_plan *p, const int2 *j0, const int32_t *Sk, int32_
       WPROJ_CUDA(cudaStreamSynchronize(s));
     }
     *n_rec = nr_;
-    DevBuf bytes_t;
+    TmpBuf bytes_t;
     WPROJ_TRY(bytes_t.alloc(sizeof(int32_t) * std::max<int64_t>(1, nr_)));
-    WPROJ_TRY(p->rec_off.alloc(sizeof(int64_t) * (nr_ + 1)));
-    WPROJ_TRY(p->seg_rec.alloc(sizeof(int64_t) * std::max<int64_t>(1, n_seg)));
+    WPROJ_TRY(p->rec_off.reuse(sizeof(int64_t) * (nr_ + 1)));
+    WPROJ_TRY(p->seg_rec.reuse(sizeof(int64_t) * std::max<int64_t>(1, n_seg)));
     WPROJ_CUDA(cudaMemsetAsync(p->seg_rec.ptr, 0xff, sizeof(int64_t) * std::max<int64_t>(1, n_seg), s));   // -1
     int64_t total = 0;
     if (nr_ > 0) {
@@ -738,7 +738,7 @@ wproj_status build_runs(wproj_plan *p, const int2 *j0, const int32_t *Sk, int32_
     } else {
       WPROJ_CUDA(cudaMemsetAsync(p->rec_off.ptr, 0, sizeof(int64_t), s));
     }
-    WPROJ_TRY(p->stream.alloc(std::max<int64_t>(16, total)));
+    WPROJ_TRY(p->stream.reuse(std::max<int64_t>(16, total)));
     WPROJ_CUDA(cudaMemsetAsync(p->stream.ptr, 0, std::max<int64_t>(16, total), s));
     p->stream_bytes = total;
     if (n_seg > 0) {

@@ -103,7 +103,7 @@ template <class Tin, class Tout>
 wproj_status exclusive_scan(const Tin *in, Tout *out, int64_t n, cudaStream_t s) {
   if (n <= 0) return WPROJ_OK;
   const int64_t nb = (n + kScanTile - 1) / kScanTile;
-  DevBuf sums;
+  TmpBuf sums;
   WPROJ_TRY(sums.alloc(sizeof(Tout) * (nb + 1)));
   k_block_sums<Tin, Tout><<<(unsigned)nb, kScanThreads, 0, s>>>(in, n, sums.as<Tout>());
   WPROJ_CHECK_LAUNCH("scan block sums");
@@ -185,7 +185,7 @@ wproj_status stable_bin_sort(const int32_t *key, int64_t n, int n_bins, int32_t 
   int64_t chunk = (n + n_blocks - 1) / n_blocks;
   chunk = std::max<int64_t>(32, (chunk + 31) / 32 * 32);
   n_blocks = (int)std::max<int64_t>(1, (n + chunk - 1) / chunk);
-  DevBuf hist, offs;
+  TmpBuf hist, offs;
   const int64_t nh = int64_t(n_bins) * n_blocks;
   WPROJ_TRY(hist.alloc(sizeof(int32_t) * nh));
   WPROJ_TRY(offs.alloc(sizeof(int64_t) * nh));
