@@ -626,15 +626,21 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
   return (unsigned long long)a + ((unsigned long long)b << 22) + ((unsigned long long)c << 44);
 }
 
+// Rounds of bisection before the samples left between the bounds go to one warp:
+// 31-bit keys, so that 2^17 keys (1/64 octave of energy) are left
+constexpr int kSelRounds = 15;
+
 // A block takes one S x S box (S = 32 or 64), 16 samples a thread: chirp x taps, row
 // transform, column transform (the passes of k_box_rows and k_fft_cols), then the
 // row's threshold on the samples it holds.  The threshold is the largest key t whose
 // samples of key >= t hold the target energy, found by bisection over the keys with
-// exact integer sums, which is the key the radix select finds; ties and per-tile
-// counts as there.  Phase 2 only transforms (select = 0).
-// Bound by issue: ~30 rounds of 16 compare-adds and a block sum.  The separate
+// exact integer sums, which is the key the radix select finds: 14 rounds over all
+// samples, the last bits by one warp over the few samples left (all rounds over all
+// samples when more than 32 are).  Ties and per-tile counts as there.  Phase 2 only
+// transforms (select = 0).
+// Bound by issue: rounds of 16 compare-adds and a block sum.  The separate
 // kernels passed over the box six times and over 24 KB of histogram per box and
-// level, more than the box itself: 28 ms for 262144 boxes, most of 64^2, against 12.5.
+// level, more than the box itself: 28 ms for 262144 boxes, most of 64^2, against 9.6 (12.3 with all rounds over all samples).
 template <int LOGN>
 __global__ void __launch_bounds__((1 << (2 * LOGN)) / kFftE)
 k_box_small(const BoxBatch bb, const float2 *__restrict__ tw, float scale, int select, double e_target, GridGeom g,
@@ -649,6 +655,8 @@ k_box_small(const BoxBatch bb, const float2 *__restrict__ tw, float scale, int s
   __shared__ unsigned long long s_target;
   __shared__ unsigned s_max[NW];
   __shared__ int s_all, s_eq, tile_gt[16], tile_eq[16];
+  __shared__ unsigned s_n, s_lo, s_key[32];
+  __shared__ unsigned long long s_above, s_q[32];
   const int b = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
   float2 v[kFftE];
   {   // rows: thread tq of row P holds columns tq + m TN
@@ -706,6 +714,9 @@ k_box_small(const BoxBatch bb, const float2 *__restrict__ tw, float scale, int s
     const double tgt = e_target * double(tot);
     s_all = !(tgt < double(tot));
     s_eq = 0;
+    s_n = 0;
+    s_lo = 0;
+    s_above = 0;
     const unsigned long long x = (unsigned long long)ceil(tgt);
     s_target = x < 1 ? 1 : x;
   }
@@ -716,6 +727,46 @@ k_box_small(const BoxBatch bb, const float2 *__restrict__ tw, float scale, int s
   unsigned long long q_hi = 0;           // energy of keys >= hi
   if (!all) {
     for (int it = 1; hi - lo > 1; ++it) {
+      if (it == kSelRounds) {   // few samples are left between lo and hi: hand them to one warp
+        unsigned n = 0;
+#pragma unroll
+        for (int m = 0; m < kFftE; ++m) n += key[m] >= lo && key[m] < hi;
+        if (n) {
+          unsigned at = atomicAdd(&s_n, n);
+#pragma unroll
+          for (int m = 0; m < kFftE; ++m)
+            if (key[m] >= lo && key[m] < hi) {
+              if (at < 32) {
+                s_key[at] = key[m];
+                s_q[at] = q[m];
+              }
+              ++at;
+            }
+        }
+        __syncthreads();
+        if (s_n <= 32) {
+          if (w == 0) {   // each lane: the energy of keys >= its own; the largest key that reaches the target
+            const unsigned kk = lane < int(s_n) ? s_key[lane] : 0u;
+            const unsigned long long qq = lane < int(s_n) ? s_q[lane] : 0ull;
+            unsigned long long f = q_hi, above = q_hi;
+            for (int i = 0; i < int(s_n); ++i) {
+              const unsigned ki = __shfl_sync(0xffffffffu, kk, i);
+              const unsigned long long qi = __shfl_sync(0xffffffffu, qq, i);
+              if (ki >= kk) f += qi;
+              if (ki > kk) above += qi;
+            }
+            const unsigned best = __reduce_max_sync(0xffffffffu, lane < int(s_n) && f >= target ? kk : 0u);
+            if (lane < int(s_n) && kk == best) {   // equal keys write the same words
+              s_lo = kk;
+              s_above = above;
+            }
+          }
+          __syncthreads();
+          lo = s_lo;
+          q_hi = s_above;
+          break;
+        }
+      }
       const unsigned mid = lo + ((hi - lo) >> 1);
       unsigned long long f = 0;
 #pragma unroll
