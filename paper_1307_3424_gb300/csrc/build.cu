@@ -208,7 +208,6 @@ struct SelState {
   int32_t qexp;         // fixed-point scale 2^qexp: the largest power of two <= 2^62 / E_closed
   uint32_t prefix;
   uint32_t maxkey;
-  int32_t n_above;
   int32_t done;
   int32_t all;
   uint32_t thr_key;
@@ -313,18 +312,24 @@ __device__ __forceinline__ unsigned long long fixed_energy(float a2, int qexp) {
 }
 __host__ __device__ constexpr int lvl_bits(int L) { return L == 2 ? 9 : 11; }
 
+// All keys of a bin share their exponent, so the energies of a bin are their
+// significands shifted alike: the histogram adds significands (24 bits, shifted right
+// where the scale asks for it, as fixed_energy does) in two 32-bit words, low 16 bits
+// and the rest, and shifts the bin's sum once.  64-bit shared-memory atomics, and a
+// second histogram of counts that only the last level's single bin needed (its
+// energy over its key's), made the first level 121 us per 64 boxes of 512^2; 37 us so.
+__device__ __forceinline__ int energy_shift(unsigned e8, int qexp) { return int(e8 ? e8 : 1u) - 150 + qexp; }
+
 template <int LEVEL>
 __global__ void __launch_bounds__(256)
-k_sel_hist(const float2 *__restrict__ K, int S, SelState *__restrict__ sel,
-           unsigned *__restrict__ hcnt, unsigned long long *__restrict__ hq) {
-  __shared__ unsigned scnt[kHistBins];
-  __shared__ unsigned long long sq[kHistBins];
+k_sel_hist(const float2 *__restrict__ K, int S, SelState *__restrict__ sel, unsigned long long *__restrict__ hq) {
+  __shared__ unsigned slo[kHistBins], shi[kHistBins];
   __shared__ unsigned smax;
   const int b = blockIdx.y;
   const SelState st = sel[b];
   if (st.done) return;
   constexpr int nb = 1 << lvl_bits(LEVEL);
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) { scnt[i] = 0; sq[i] = 0; }
+  for (int i = threadIdx.x; i < nb; i += blockDim.x) { slo[i] = 0; shi[i] = 0; }
   if (threadIdx.x == 0) smax = 0;
   __syncthreads();
   const int64_t n = int64_t(S) * S;
@@ -332,6 +337,12 @@ k_sel_hist(const float2 *__restrict__ K, int S, SelState *__restrict__ sel,
   const int64_t hi = min(n, lo + kSelChunk);
   const float2 *Kb = K + int64_t(b) * n;
   unsigned lmax = 0;
+  auto add = [&](unsigned bin, unsigned sum) {
+    if (sum) {
+      atomicAdd(&slo[bin], sum & 0xffffu);
+      atomicAdd(&shi[bin], sum >> 16);
+    }
+  };
   // A thread takes kRun consecutive samples (16-byte loads; S^2 and the
   // chunk bounds are multiples of kRun) and adds a run of samples in one bin with
   // one pair of atomics: neighbouring samples of a kernel have similar
@@ -344,45 +355,38 @@ k_sel_hist(const float2 *__restrict__ K, int S, SelState *__restrict__ sel,
     float4 pk[kRun / 2];
 #pragma unroll
     for (int h = 0; h < kRun / 2; ++h) pk[h] = __ldg(reinterpret_cast<const float4 *>(Kb + i0) + h);
-    unsigned rbin = 0xffffffffu, rcnt = 0;
-    unsigned long long rq = 0;
+    unsigned rbin = 0, rsum = 0;
 #pragma unroll
     for (int j = 0; j < kRun; ++j) {
       const float4 &v = pk[j >> 1];
-      const float a2 = abs2_rn((j & 1) ? make_float2(v.z, v.w) : make_float2(v.x, v.y));
-      const unsigned key = __float_as_uint(a2);
+      const unsigned key = __float_as_uint(abs2_rn((j & 1) ? make_float2(v.z, v.w) : make_float2(v.x, v.y)));
       if (LEVEL == 0) lmax = max(lmax, key);
       if (LEVEL > 0 && (key >> lvl_shift(LEVEL - 1)) != st.prefix) continue;
       const unsigned bin = (key >> lvl_shift(LEVEL)) & (nb - 1);
-      const unsigned long long q = fixed_energy(a2, st.qexp);
+      const unsigned e8 = key >> 23;
+      const int sh = energy_shift(e8, st.qexp);
+      unsigned m = (key & 0x7fffffu) | (e8 ? 0x800000u : 0u);
+      if (sh < 0) m = sh > -32 ? m >> -sh : 0u;
       if (bin != rbin) {
-        if (rcnt) {
-          atomicAdd(&scnt[rbin], rcnt);
-          atomicAdd(&sq[rbin], rq);
-        }
+        add(rbin, rsum);
         rbin = bin;
-        rcnt = 0;
-        rq = 0;
+        rsum = 0;
       }
-      rcnt += 1;
-      rq += q;
+      rsum += m;
     }
-    if (rcnt) {
-      atomicAdd(&scnt[rbin], rcnt);
-      atomicAdd(&sq[rbin], rq);
-    }
+    add(rbin, rsum);
   }
   if (LEVEL == 0) {
-    for (int o = 16; o; o >>= 1) lmax = max(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
+    lmax = __reduce_max_sync(0xffffffffu, lmax);
     if ((threadIdx.x & 31) == 0) atomicMax(&smax, lmax);
   }
   __syncthreads();
-  unsigned *gc = hcnt + int64_t(b) * kHistBins;
   unsigned long long *gq = hq + int64_t(b) * kHistBins;
   for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-    if (scnt[i]) {
-      atomicAdd(&gc[i], scnt[i]);
-      atomicAdd(&gq[i], sq[i]);
+    const unsigned long long m = ((unsigned long long)shi[i] << 16) + slo[i];
+    if (m) {
+      const unsigned e8 = LEVEL == 0 ? unsigned(i) >> 3 : (LEVEL == 1 ? st.prefix >> 3 : st.prefix >> 14);
+      atomicAdd(&gq[i], m << max(0, min(39, energy_shift(e8, st.qexp))));
     }
   }
   if (LEVEL == 0 && threadIdx.x == 0) atomicMax(&sel[b].maxkey, smax);
@@ -422,8 +426,7 @@ __device__ __forceinline__ unsigned long long block_incl_scan256(unsigned long l
 
 template <int LEVEL>
 __global__ void __launch_bounds__(256)
-k_sel_find(SelState *__restrict__ sel, const unsigned *__restrict__ hcnt,
-           const unsigned long long *__restrict__ hq, double e_target) {
+k_sel_find(SelState *__restrict__ sel, const unsigned long long *__restrict__ hq, double e_target) {
   __shared__ unsigned long long red[9];
   __shared__ unsigned long long wt[8];
   __shared__ long long redc[9];
@@ -432,16 +435,13 @@ k_sel_find(SelState *__restrict__ sel, const unsigned *__restrict__ hcnt,
   if (st.done) return;
   constexpr int nb = 1 << lvl_bits(LEVEL);
   constexpr int PER = nb / 256;
-  const unsigned *gc = hcnt + int64_t(b) * kHistBins;
   const unsigned long long *gq = hq + int64_t(b) * kHistBins;
   // thread t holds the reversed bins j = t*PER .. t*PER+PER-1 (bin = nb-1-j)
   unsigned long long q[PER];
-  unsigned c[PER];
   unsigned long long tq = 0;
   for (int i = 0; i < PER; ++i) {
     const int bin = nb - 1 - (threadIdx.x * PER + i);
     q[i] = gq[bin];
-    c[i] = gc[bin];
     tq += q[i];
   }
   if (LEVEL == 0) {
@@ -463,29 +463,29 @@ k_sel_find(SelState *__restrict__ sel, const unsigned *__restrict__ hcnt,
   long long below = 0;
   unsigned long long run = st.q_above + excl_thread;
   unsigned long long q_before = 0;    // q of bins above the crossing bin (this thread's share)
-  long long c_before = 0;
   for (int i = 0; i < PER; ++i) {
     run += q[i];
-    if (run < st.target) { ++below; q_before += q[i]; c_before += c[i]; }
+    if (run < st.target) { ++below; q_before += q[i]; }
   }
   const long long jstar = block_sum256<long long>(below, redc);
   const unsigned long long qb = block_sum256<unsigned long long>(q_before, red);
-  const long long cb = block_sum256<long long>(c_before, redc);
-  __shared__ unsigned cstar;
-  if (threadIdx.x == (int)(jstar / PER) && jstar < nb) cstar = c[jstar % PER];
+  __shared__ unsigned long long qstar;   // energy of the crossing bin
+  if (threadIdx.x == (int)(jstar / PER) && jstar < nb) qstar = gq[nb - 1 - int(jstar)];
   __syncthreads();
   if (threadIdx.x == 0) {
     const int binstar = nb - 1 - int(jstar);
     st.q_above += qb;
-    st.n_above += int32_t(cb);
     st.prefix = (LEVEL == 0) ? unsigned(binstar) : ((st.prefix << lvl_bits(LEVEL)) | unsigned(binstar));
     if (LEVEL == 2) {
       st.thr_key = st.prefix;
       const unsigned long long qthr =
           fixed_energy(__uint_as_float(st.thr_key), st.qexp);
       const unsigned long long rem = st.target - st.q_above;
-      long long nt = (qthr > 0) ? (long long)((rem + qthr - 1) / qthr) : (long long)cstar;
-      if (nt > (long long)cstar) nt = cstar;
+      // the crossing bin holds one key: its energy over the key's is the number of ties
+      // (a bin that crosses has energy)
+      const long long cstar = qthr > 0 ? (long long)(qstar / qthr) : 0x7fffffff;
+      long long nt = (qthr > 0) ? (long long)((rem + qthr - 1) / qthr) : cstar;
+      if (nt > cstar) nt = cstar;
       if (nt < 0) nt = 0;
       st.n_tie = int32_t(nt);
       st.done = 1;
@@ -1230,7 +1230,7 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
     p->box_max = std::max(p->box_max, 16 << c);
   }
   DevBuf Kbuf;
-  TmpBuf Au, Av, bmode, bwf, bwd, bsel, hcnt, hq, lcoord, lsq, gtab, bsid;
+  TmpBuf Au, Av, bmode, bwf, bwd, bsel, hq, lcoord, lsq, gtab, bsid;
   // Pass 2 needs every box's transform again.  When the device has room for all
   // of them (and, with a margin, for G, whose size is at most 1.5x theirs), pass
   // 1 keeps them and pass 2 emits without recomputing the tables and FFTs;
@@ -1268,7 +1268,6 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
   WPROJ_TRY(bwd.alloc(sizeof(double) * max_nb));
   WPROJ_TRY(bsel.alloc(sizeof(SelState) * max_nb));
   if (sid) WPROJ_TRY(bsid.alloc(sizeof(int32_t) * max_nb));
-  WPROJ_TRY(hcnt.alloc(sizeof(unsigned) * kHistBins * size_t(max_nb_hist)));
   WPROJ_TRY(hq.alloc(sizeof(unsigned long long) * kHistBins * size_t(max_nb_hist)));
   WPROJ_TRY(lcoord.alloc(sizeof(double) * p->box_max));
   WPROJ_TRY(lsq.alloc(sizeof(float) * p->box_max));
@@ -1419,18 +1418,15 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
         const dim3 hgrid(ceil_div(per, kSelChunk), nb);
         if (phase == 1) {
           ScopedTimer t_sel(p, TC_BSEL, s);
-          WPROJ_CUDA(cudaMemsetAsync(hcnt.ptr, 0, sizeof(unsigned) * kHistBins * nb, s));
           WPROJ_CUDA(cudaMemsetAsync(hq.ptr, 0, sizeof(unsigned long long) * kHistBins * nb, s));
-          k_sel_hist<0><<<hgrid, 256, 0, s>>>(bb.K, S, bsel.as<SelState>(), hcnt.as<unsigned>(), hq.as<unsigned long long>());
-          k_sel_find<0><<<nb, 256, 0, s>>>(bsel.as<SelState>(), hcnt.as<unsigned>(), hq.as<unsigned long long>(), e_target);
-          WPROJ_CUDA(cudaMemsetAsync(hcnt.ptr, 0, sizeof(unsigned) * kHistBins * nb, s));
+          k_sel_hist<0><<<hgrid, 256, 0, s>>>(bb.K, S, bsel.as<SelState>(), hq.as<unsigned long long>());
+          k_sel_find<0><<<nb, 256, 0, s>>>(bsel.as<SelState>(), hq.as<unsigned long long>(), e_target);
           WPROJ_CUDA(cudaMemsetAsync(hq.ptr, 0, sizeof(unsigned long long) * kHistBins * nb, s));
-          k_sel_hist<1><<<hgrid, 256, 0, s>>>(bb.K, S, bsel.as<SelState>(), hcnt.as<unsigned>(), hq.as<unsigned long long>());
-          k_sel_find<1><<<nb, 256, 0, s>>>(bsel.as<SelState>(), hcnt.as<unsigned>(), hq.as<unsigned long long>(), e_target);
-          WPROJ_CUDA(cudaMemsetAsync(hcnt.ptr, 0, sizeof(unsigned) * kHistBins * nb, s));
+          k_sel_hist<1><<<hgrid, 256, 0, s>>>(bb.K, S, bsel.as<SelState>(), hq.as<unsigned long long>());
+          k_sel_find<1><<<nb, 256, 0, s>>>(bsel.as<SelState>(), hq.as<unsigned long long>(), e_target);
           WPROJ_CUDA(cudaMemsetAsync(hq.ptr, 0, sizeof(unsigned long long) * kHistBins * nb, s));
-          k_sel_hist<2><<<hgrid, 256, 0, s>>>(bb.K, S, bsel.as<SelState>(), hcnt.as<unsigned>(), hq.as<unsigned long long>());
-          k_sel_find<2><<<nb, 256, 0, s>>>(bsel.as<SelState>(), hcnt.as<unsigned>(), hq.as<unsigned long long>(), e_target);
+          k_sel_hist<2><<<hgrid, 256, 0, s>>>(bb.K, S, bsel.as<SelState>(), hq.as<unsigned long long>());
+          k_sel_find<2><<<nb, 256, 0, s>>>(bsel.as<SelState>(), hq.as<unsigned long long>(), e_target);
           WPROJ_CHECK_LAUNCH("select");
           const int nt_box = box_tiles(S, g);
           const int smem_tiles = std::min(nt_box, 4096);
