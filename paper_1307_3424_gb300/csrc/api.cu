@@ -413,9 +413,10 @@ wproj_status wproj_get_stats(wproj_plan *p, wproj_stats *out) {
   out->t_build_select_ms = p->timer.ms[TC_BSEL];
   out->t_build_emit_ms = p->timer.ms[TC_BEMIT];
   out->n_build_fft = p->timer.count[TC_BFFT];
-  out->runs_bytes = p->fmt == WPROJ_INDEX_TILE_RUNS
-                        ? p->rm_vals * (p->g.value_dtype == WPROJ_VAL_F32 ? 8 : 4) + p->rm_runs * 4 + p->m * 20
-                        : 0;
+  const int vbytes = p->g.value_dtype == WPROJ_VAL_F32 ? 8 : 4;
+  out->runs_bytes = p->fmt != WPROJ_INDEX_TILE_RUNS ? 0
+                    : p->slices.use                 ? p->slices.d_steps * 32 * (vbytes + 2) + p->slices.d_slices * 24
+                                                    : p->rm_vals * vbytes + p->rm_runs * 4 + p->m * 20;
   return WPROJ_OK;
 }
 

@@ -41,6 +41,10 @@ struct wproj_batch {
   wproj::DevBuf row_ptr, col, val, meta, tptr, cum, tile_prob;
   bool has_cells = false;   // cell-major copy for the gridding (every problem has one)
   wproj::DevBuf tile_ent, cell_ent, cell_val;
+  // interleaved slices of every problem (when every problem's boxes allow them)
+  bool has_slices = false;
+  wproj::SliceCopy slices;
+  wproj::DevBuf d_chunk_prob, g_chunk_prob;
   // schedule
   int64_t piece = 0, chunk = 0, n_pieces = 0, n_chunks = 0;
   int lpp = 32;   // degridding lanes per row piece (32, 16, 8 or 4: the row-split schedule)
@@ -89,6 +93,14 @@ __global__ void k_add_i32(int64_t n, const int32_t *__restrict__ src, int32_t ad
 __global__ void k_add_i64(int64_t n, const int64_t *__restrict__ src, int64_t add, int64_t *__restrict__ dst) {
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
     dst[i] = src[i] + add;
+}
+// rows of a problem (-1: none) as rows of the batch
+__global__ void k_add_row(int64_t n, const int32_t *__restrict__ src, int32_t add, int32_t *__restrict__ dst) {
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x)
+    dst[i] = src[i] < 0 ? -1 : src[i] + add;
+}
+__global__ void k_fill_i32(int64_t n, int32_t v, int32_t *__restrict__ dst) {
+  for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) dst[i] = v;
 }
 __global__ void k_cat_meta(int64_t n, const SegMeta *__restrict__ src, int64_t ent_add, int row_add,
                            SegMeta *__restrict__ dst) {
@@ -282,6 +294,25 @@ BatchOps ops_of(const wproj_batch *b) {
   return o;
 }
 
+SliceOps slices_of(const wproj_batch *b) {
+  SliceOps o = b->slices.ops();
+  o.d_chunk_prob = b->d_chunk_prob.as<int32_t>();
+  o.g_chunk_prob = b->g_chunk_prob.as<int32_t>();
+  o.tile_prob = b->tile_prob.as<int32_t>();
+  o.tab = b->tab.as<BProb>();
+  return o;
+}
+
+wproj_status bdegrid(wproj_batch *b, const float2 *Xt, float2 *y, cudaStream_t s) {
+  if (b->has_slices) return batch_degrid_slices(slices_of(b), b->slices.d_smem, Xt, y, s);
+  return batch_degrid(ops_of(b), Xt, b->piece_partial.as<float2>(), y, s);
+}
+wproj_status bgrid(wproj_batch *b, const float2 *y, float2 *Xt2, cudaStream_t s) {
+  if (b->has_slices)
+    return batch_grid_slices(slices_of(b), b->slices.g_smem, y, b->slices.partial.as<float2>(), Xt2, s);
+  return batch_grid(ops_of(b), y, b->grid_partial.as<float2>(), Xt2, s);
+}
+
 wproj_status bphi(wproj_batch *b, const float *x, float2 *y, cudaStream_t s) {
   for (auto &c : b->cls) {
     if (c.np == 0) continue;
@@ -289,14 +320,14 @@ wproj_status bphi(wproj_batch *b, const float *x, float2 *y, cudaStream_t s) {
                             b->interb.as<float2>(), b->Xt.as<float2>(), b->twiddle.as<float2>(), s));
     b->launches += 2;
   }
-  b->launches += 2;
-  return batch_degrid(ops_of(b), b->Xt.as<float2>(), b->piece_partial.as<float2>(), y, s);
+  b->launches += b->has_slices ? 1 : 2;
+  return bdegrid(b, b->Xt.as<float2>(), y, s);
 }
 
 // mode 0: x_re = Re Phi^H y; mode 1: x_re = z - Re Phi^H y
 wproj_status bphi_adj(wproj_batch *b, const float2 *y, float *x_re, const float *z, int mode, cudaStream_t s) {
-  WPROJ_TRY(batch_grid(ops_of(b), y, b->grid_partial.as<float2>(), b->Xt2.as<float2>(), s));
-  b->launches += 2;
+  WPROJ_TRY(bgrid(b, y, b->Xt2.as<float2>(), s));
+  b->launches += b->has_slices && !b->slices.n_multi ? 1 : 2;
   for (auto &c : b->cls) {
     if (c.np == 0) continue;
     WPROJ_TRY(batch_phi_adj(c.logG, c.np, c.plist.as<int32_t>(), b->tab.as<BProb>(), b->Xt2.as<float2>(),
@@ -309,7 +340,7 @@ wproj_status bphi_adj(wproj_batch *b, const float2 *y, float *x_re, const float 
 wproj_status set_pieces(wproj_batch *b, int64_t piece, cudaStream_t s) {
   WPROJ_TRY(make_row_pieces(b->m, b->row_ptr.as<int64_t>(), piece, b->piece_row, b->piece_lo, b->piece_len,
                             b->row_piece_ptr, &b->n_pieces, s));
-  WPROJ_TRY(b->piece_partial.alloc(sizeof(float2) * std::max<int64_t>(1, b->n_pieces)));
+  WPROJ_TRY(b->piece_partial.alloc(sizeof(float2) * (b->has_slices ? 1 : std::max<int64_t>(1, b->n_pieces))));
   b->piece = piece;
   if (b->dr_exec) {   // the captured iteration holds the old buffers
     cudaGraphExecDestroy(b->dr_exec);
@@ -326,7 +357,8 @@ wproj_status set_chunks(wproj_batch *b, int64_t chunk, cudaStream_t s) {
                                                           b->tab.as<BProb>(), b->chunk_tile.as<int32_t>(),
                                                           b->chunk_prob.as<int32_t>());
   WPROJ_CHECK_LAUNCH("chunk problems");
-  WPROJ_TRY(b->grid_partial.alloc(sizeof(float2) * size_t(std::max<int64_t>(1, b->n_chunks)) * kTile * kTile));
+  WPROJ_TRY(b->grid_partial.alloc(b->has_slices ? sizeof(float2)
+                                                : sizeof(float2) * size_t(std::max<int64_t>(1, b->n_chunks)) * kTile * kTile));
   b->chunk = chunk;
   if (b->dr_exec) {   // the captured iteration holds the old buffers
     cudaGraphExecDestroy(b->dr_exec);
@@ -401,6 +433,95 @@ wproj_status power_mu(wproj_batch *b, int iters, cudaStream_t s) {
   return WPROJ_OK;
 }
 
+// The problems' slices end to end: offsets shifted by what lies before the problem;
+// the closing element of one problem's offsets is the first of the next one's.
+wproj_status concat_slices(wproj_batch *b, const std::vector<wproj_plan *> &plans, cudaStream_t s) {
+  SliceCopy &c = b->slices;
+  c.release();
+  b->d_chunk_prob.release();
+  b->g_chunk_prob.release();
+  if (!b->has_slices) return WPROJ_OK;
+  for (auto *pl : plans) {
+    const SliceCopy &q = pl->slices;
+    c.d_chunks += q.d_chunks;
+    c.d_slices += q.d_slices;
+    c.d_steps += q.d_steps;
+    c.g_chunks += q.g_chunks;
+    c.g_steps += q.g_steps;
+    c.g_nrows += q.g_nrows;
+    c.n_multi += q.n_multi;
+    c.d_smem = std::max(c.d_smem, q.d_smem);
+    c.g_smem = std::max(c.g_smem, q.g_smem);
+  }
+  const int64_t de = std::max<int64_t>(1, c.d_steps) * 32, ge = std::max<int64_t>(1, c.g_steps) * 32;
+  WPROJ_TRY(c.d_slice_base.alloc(sizeof(int64_t) * (c.d_chunks + 1)));
+  WPROJ_TRY(c.slice_ptr.alloc(sizeof(int64_t) * (c.d_slices + 1)));
+  WPROJ_TRY(c.srow.alloc(sizeof(int32_t) * 4 * std::max<int64_t>(1, c.d_slices)));
+  WPROJ_TRY(c.rect.alloc(sizeof(int4) * c.d_chunks));
+  WPROJ_TRY(b->d_chunk_prob.alloc(sizeof(int32_t) * c.d_chunks));
+  WPROJ_TRY(c.d_idx.alloc(sizeof(uint16_t) * de));
+  WPROJ_TRY(c.d_val.alloc(sizeof(float2) * de));
+  WPROJ_TRY(c.g_chunk_tile.alloc(sizeof(int32_t) * c.g_chunks));
+  WPROJ_TRY(c.tile_chunk_ptr.alloc(sizeof(int32_t) * (b->tiles + 1)));
+  WPROJ_TRY(c.g_base.alloc(sizeof(int64_t) * (c.g_chunks + 1)));
+  WPROJ_TRY(c.g_slp.alloc(sizeof(uint32_t) * 33 * c.g_chunks));
+  WPROJ_TRY(c.g_perm.alloc(sizeof(uint16_t) * 1024 * c.g_chunks));
+  WPROJ_TRY(c.g_row_base.alloc(sizeof(int64_t) * (c.g_chunks + 1)));
+  WPROJ_TRY(c.g_rows.alloc(sizeof(int32_t) * std::max<int64_t>(1, c.g_nrows)));
+  WPROJ_TRY(c.g_idx.alloc(sizeof(uint16_t) * ge));
+  WPROJ_TRY(c.g_val.alloc(sizeof(float2) * ge));
+  if (c.n_multi > 0) {
+    WPROJ_TRY(c.multi.alloc(sizeof(int32_t) * c.n_multi));
+    WPROJ_TRY(c.partial.alloc(sizeof(float2) * 1024 * c.g_chunks));
+  }
+  WPROJ_TRY(b->g_chunk_prob.alloc(sizeof(int32_t) * c.g_chunks));
+  auto nb = [](int64_t n) { return std::max(1, std::min(ceil_div(n, 256), 152 * 8)); };
+  auto copy = [&](void *d, const void *src, size_t n) {
+    return n ? cudaMemcpyAsync(d, src, n, cudaMemcpyDeviceToDevice, s) : cudaSuccess;
+  };
+  int64_t dc = 0, ds = 0, dst = 0, gc = 0, gst = 0, gr = 0, mu = 0;   // before the problem
+  for (int p = 0; p < b->np; ++p) {
+    const SliceCopy &q = plans[p]->slices;
+    const BProb &P = b->prob[p];
+    const int nt = P.nT * P.nT;
+    k_add_i64<<<nb(q.d_chunks + 1), 256, 0, s>>>(q.d_chunks + 1, q.d_slice_base.as<int64_t>(), ds,
+                                                 c.d_slice_base.as<int64_t>() + dc);
+    k_add_i64<<<nb(q.d_slices + 1), 256, 0, s>>>(q.d_slices + 1, q.slice_ptr.as<int64_t>(), dst,
+                                                 c.slice_ptr.as<int64_t>() + ds);
+    k_fill_i32<<<nb(q.d_chunks), 256, 0, s>>>(q.d_chunks, p, b->d_chunk_prob.as<int32_t>() + dc);
+    k_add_row<<<nb(4 * q.d_slices), 256, 0, s>>>(4 * q.d_slices, q.srow.as<int32_t>(), int32_t(P.vis_off),
+                                                 c.srow.as<int32_t>() + 4 * ds);
+    k_add_i32<<<nb(nt + 1), 256, 0, s>>>(nt + 1, q.tile_chunk_ptr.as<int32_t>(), int32_t(gc),
+                                         c.tile_chunk_ptr.as<int32_t>() + P.tile_off);
+    k_add_i64<<<nb(q.g_chunks + 1), 256, 0, s>>>(q.g_chunks + 1, q.g_base.as<int64_t>(), gst, c.g_base.as<int64_t>() + gc);
+    k_add_i64<<<nb(q.g_chunks + 1), 256, 0, s>>>(q.g_chunks + 1, q.g_row_base.as<int64_t>(), gr,
+                                                 c.g_row_base.as<int64_t>() + gc);
+    k_add_row<<<nb(q.g_nrows), 256, 0, s>>>(q.g_nrows, q.g_rows.as<int32_t>(), int32_t(P.vis_off),
+                                            c.g_rows.as<int32_t>() + gr);
+    k_fill_i32<<<nb(q.g_chunks), 256, 0, s>>>(q.g_chunks, p, b->g_chunk_prob.as<int32_t>() + gc);
+    if (q.n_multi)
+      k_add_i32<<<nb(q.n_multi), 256, 0, s>>>(q.n_multi, q.multi.as<int32_t>(), int32_t(P.tile_off),
+                                              c.multi.as<int32_t>() + mu);
+    WPROJ_CHECK_LAUNCH("batch slice concatenation");
+    WPROJ_CUDA(copy(c.rect.as<int4>() + dc, q.rect.ptr, sizeof(int4) * q.d_chunks));
+    WPROJ_CUDA(copy(c.d_idx.as<uint16_t>() + dst * 32, q.d_idx.ptr, sizeof(uint16_t) * 32 * q.d_steps));
+    WPROJ_CUDA(copy(c.d_val.as<float2>() + dst * 32, q.d_val.ptr, sizeof(float2) * 32 * q.d_steps));
+    WPROJ_CUDA(copy(c.g_chunk_tile.as<int32_t>() + gc, q.g_chunk_tile.ptr, sizeof(int32_t) * q.g_chunks));
+    WPROJ_CUDA(copy(c.g_slp.as<uint32_t>() + gc * 33, q.g_slp.ptr, sizeof(uint32_t) * 33 * q.g_chunks));
+    WPROJ_CUDA(copy(c.g_perm.as<uint16_t>() + gc * 1024, q.g_perm.ptr, sizeof(uint16_t) * 1024 * q.g_chunks));
+    WPROJ_CUDA(copy(c.g_idx.as<uint16_t>() + gst * 32, q.g_idx.ptr, sizeof(uint16_t) * 32 * q.g_steps));
+    WPROJ_CUDA(copy(c.g_val.as<float2>() + gst * 32, q.g_val.ptr, sizeof(float2) * 32 * q.g_steps));
+    dc += q.d_chunks;
+    ds += q.d_slices;
+    dst += q.d_steps;
+    gc += q.g_chunks;
+    gst += q.g_steps;
+    gr += q.g_nrows;
+    mu += q.n_multi;
+  }
+  return WPROJ_OK;
+}
+
 template <class F>
 wproj_status time_ms(F &&f, int reps, cudaStream_t s, double *ms) {
   cudaEvent_t a, c;
@@ -439,13 +560,30 @@ wproj_status batch_build_impl(wproj_batch *b, const double *uvw, const int64_t *
       for (auto *p : v) if (p) wproj_plan_destroy(p);
     }
   } guard{plans};
+  // slices everywhere, or the other forms everywhere: a problem that cannot take them
+  // (a box over 64 cells, a grid under 32) makes those built with them build again
   int64_t vis = 0;
-  for (int p = 0; p < np; ++p) {
-    wproj_grid_desc d = b->desc[p];
-    d.index_format = WPROJ_INDEX_COLUMNS;
-    WPROJ_TRY(wproj_plan_create(&plans[p], &d));
-    WPROJ_TRY(build_kernels_impl(plans[p], uvw + 3 * vis, m[p], e, s));
-    vis += m[p];
+  bool want = true;
+  for (int p = 0; p < np; ++p) want = want && b->desc[p].box <= 64 && 2 * b->desc[p].n >= kTile;
+  for (bool done = false; !done;) {
+    done = true;
+    vis = 0;
+    for (int p = 0; p < np; ++p) {
+      wproj_grid_desc d = b->desc[p];
+      d.index_format = WPROJ_INDEX_COLUMNS;
+      if (!plans[p]) WPROJ_TRY(wproj_plan_create(&plans[p], &d));
+      wproj_plan *pl = plans[p];
+      if (want || !pl->built || pl->slices.use) {
+        pl->in_batch = want;
+        pl->no_slices = !want;
+        WPROJ_TRY(build_kernels_impl(pl, uvw + 3 * vis, m[p], e, s));
+      }
+      vis += m[p];
+      if (want && !pl->slices.use) {
+        want = false;
+        done = false;
+      }
+    }
   }
   // ---- offsets
   b->prob.assign(np, BProb{});
@@ -494,8 +632,10 @@ wproj_status batch_build_impl(wproj_batch *b, const double *uvw, const int64_t *
   WPROJ_CUDA(cudaMemcpyAsync(b->tab.ptr, b->prob.data(), sizeof(BProb) * np, cudaMemcpyHostToDevice, s));
   // ---- concatenate G and the per-problem tables
   WPROJ_TRY(b->row_ptr.alloc(sizeof(int64_t) * (vis + 1)));
-  WPROJ_TRY(b->col.alloc(sizeof(int32_t) * std::max<int64_t>(1, nnz)));
-  WPROJ_TRY(b->val.alloc(sizeof(float2) * std::max<int64_t>(1, nnz)));
+  // the column form serves the operators only where slices do not
+  b->has_slices = want;
+  WPROJ_TRY(b->col.alloc(sizeof(int32_t) * (want ? 1 : std::max<int64_t>(1, nnz))));
+  WPROJ_TRY(b->val.alloc(sizeof(float2) * (want ? 1 : std::max<int64_t>(1, nnz))));
   WPROJ_TRY(b->meta.alloc(sizeof(SegMeta) * std::max<int64_t>(1, nseg)));
   WPROJ_TRY(b->tptr.alloc(sizeof(int64_t) * (tiles + 1)));
   WPROJ_TRY(b->tile_prob.alloc(sizeof(int32_t) * tiles));
@@ -512,12 +652,13 @@ wproj_status batch_build_impl(wproj_batch *b, const double *uvw, const int64_t *
     b->cell_ent.release();
     b->cell_val.release();
   }
+  WPROJ_TRY(concat_slices(b, plans, s));
   int64_t ent = 0, sg = 0;
   for (int p = 0; p < np; ++p) {
     wproj_plan *pl = plans[p];
     const BProb &P = b->prob[p];
     const int nt = P.nT * P.nT;
-    if (pl->nnz > 0) {
+    if (pl->nnz > 0 && !b->has_slices) {
       k_add_i32<<<std::min(ceil_div(pl->nnz, 256), 152 * 8), 256, 0, s>>>(pl->nnz, pl->col.as<int32_t>(),
                                                                           int32_t(P.grid_off), b->col.as<int32_t>() + ent);
       WPROJ_CUDA(cudaMemcpyAsync(b->val.as<float2>() + ent, pl->val.ptr, sizeof(float2) * pl->nnz,
@@ -603,14 +744,26 @@ wproj_status batch_tune_impl(wproj_batch *b, wproj_batch_schedule *out, cudaStre
   int bl = b->lpp;
   WPROJ_CUDA(cudaMemsetAsync(b->Xt.ptr, 0, sizeof(float2) * b->grid, s));
   WPROJ_CUDA(cudaMemsetAsync(b->u.ptr, 0, sizeof(float2) * b->m, s));
+  if (b->has_slices) {   // no schedule to pick: the set one stays, both operators are timed
+    double d_ms = 0, g_ms = 0;
+    WPROJ_TRY(time_ms([&] { return bdegrid(b, b->Xt.as<float2>(), b->r.as<float2>(), s); }, 5, s, &d_ms));
+    WPROJ_TRY(time_ms([&] { return bgrid(b, b->u.as<float2>(), b->Xt2.as<float2>(), s); }, 5, s, &g_ms));
+    if (out) {
+      out->piece = b->piece;
+      out->lanes_per_piece = b->lpp;
+      out->chunk = b->chunk;
+      out->degrid_ms = d_ms;
+      out->grid_ms = g_ms;
+    }
+    return WPROJ_OK;
+  }
   // row split: pieces of at most `piece` entries, each taken by 32, 16, 8 or 4 lanes
   for (int64_t pc : pieces) {
     WPROJ_TRY(set_pieces(b, pc, s));
     for (int l : lanes) {
       b->lpp = l;
       double ms = 0;
-      WPROJ_TRY(time_ms([&] { return batch_degrid(ops_of(b), b->Xt.as<float2>(), b->piece_partial.as<float2>(),
-                                                  b->r.as<float2>(), s); }, 5, s, &ms));
+      WPROJ_TRY(time_ms([&] { return bdegrid(b, b->Xt.as<float2>(), b->r.as<float2>(), s); }, 5, s, &ms));
       if (ms < best) { best = ms; bp = pc; bl = l; }
     }
   }
@@ -622,8 +775,7 @@ wproj_status batch_tune_impl(wproj_batch *b, wproj_batch_schedule *out, cudaStre
   for (int64_t ch : chunks) {
     WPROJ_TRY(set_chunks(b, ch, s));
     double ms = 0;
-    WPROJ_TRY(time_ms([&] { return batch_grid(ops_of(b), b->u.as<float2>(), b->grid_partial.as<float2>(),
-                                              b->Xt2.as<float2>(), s); }, 5, s, &ms));
+    WPROJ_TRY(time_ms([&] { return bgrid(b, b->u.as<float2>(), b->Xt2.as<float2>(), s); }, 5, s, &ms));
     if (ms < best) { best = ms; bc = ch; }
   }
   WPROJ_TRY(set_chunks(b, bc, s));

@@ -1100,13 +1100,9 @@ wproj_status make_tile_chunks(int n_tiles, const int64_t *tptr, const int64_t *c
   WPROJ_TRY(chbase.alloc(sizeof(int64_t) * (n_tiles + 1)));
   k_tile_chunks<<<ceil_div(n_tiles, 256), 256, 0, s>>>(n_tiles, tptr, cum, n_seg, nnz, chunk, nch.as<int32_t>());
   WPROJ_CHECK_LAUNCH("tile chunks");
-  WPROJ_TRY(exclusive_scan_i32_to_i64(nch.as<int32_t>(), chbase.as<int64_t>(), n_tiles, s));
-  int64_t lb = 0;
-  int32_t ln = 0;
-  WPROJ_CUDA(cudaMemcpyAsync(&lb, chbase.as<int64_t>() + (n_tiles - 1), sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-  WPROJ_CUDA(cudaMemcpyAsync(&ln, nch.as<int32_t>() + (n_tiles - 1), sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+  WPROJ_TRY(exclusive_scan_total(nch.as<int32_t>(), chbase.as<int64_t>(), n_tiles, s));
+  WPROJ_CUDA(cudaMemcpyAsync(n_chunks, chbase.as<int64_t>() + n_tiles, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
   WPROJ_CUDA(cudaStreamSynchronize(s));
-  *n_chunks = lb + ln;
   WPROJ_TRY(chunk_tile.alloc(sizeof(int32_t) * *n_chunks));
   WPROJ_TRY(chunk_lo.alloc(sizeof(int64_t) * *n_chunks));
   WPROJ_TRY(chunk_hi.alloc(sizeof(int64_t) * *n_chunks));
@@ -1466,18 +1462,39 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
   } else {
     p->row_scale.release();
   }
+  // boxes of at most 64 x 64 cells in the column form: interleaved slices
+  p->slices.use = false;
+  TmpBuf row_runs;   // with slices: an upper bound of each row's runs
+  if (p->fmt == WPROJ_INDEX_COLUMNS && p->box_max <= 64 && g.tile == 32 && !p->no_slices && n_seg > 0) {
+    p->m = m;
+    WPROJ_TRY(row_runs.alloc(sizeof(int32_t) * m));
+    TmpBuf cnt, cum;
+    WPROJ_TRY(cnt.alloc(sizeof(int32_t) * n_seg));
+    WPROJ_TRY(cum.alloc(sizeof(int64_t) * n_seg));
+    WPROJ_TRY(p->seg_meta.reuse(sizeof(SegMeta) * n_seg));
+    k_gather_cnt<<<ceil_div(n_seg, 256), 256, 0, s>>>(n_seg, tile_seg.as<int32_t>(), p->seg_cnt.as<int32_t>(),
+                                                    p->seg_off.as<int64_t>(), p->seg_row.as<int32_t>(),
+                                                    cnt.as<int32_t>(), p->seg_meta.as<SegMeta>());
+    WPROJ_CHECK_LAUNCH("segments in tile order");
+    WPROJ_TRY(exclusive_scan_i32_to_i64(cnt.as<int32_t>(), cum.as<int64_t>(), n_seg, s));
+    WPROJ_TRY(build_slices(p, d_j0.as<int2>(), d_Sk.as<int32_t>(), tptr.as<int64_t>(), cum.as<int64_t>(), n_seg,
+                           row_runs.as<int32_t>(), s));
+  }
+  if (!p->slices.use) p->slices.release();
   if (want_runs) {
     p->m = m;
     p->n_seg = n_seg;
-    const wproj_status st = build_runs(p, d_j0.as<int2>(), d_Sk.as<int32_t>(), tile_seg.as<int32_t>(),
+    const wproj_status st = build_runs(p, d_j0.as<int2>(), d_Sk.as<int32_t>(),
+                                       p->slices.use ? row_runs.as<int32_t>() : nullptr, tile_seg.as<int32_t>(),
                                        tptr.as<int64_t>(), &n_rec, s);
     if (st == WPROJ_OK) {
       p->fmt = WPROJ_INDEX_TILE_RUNS;
+      p->seg_meta.release();
     } else if (!(st == WPROJ_ERR_UNSUPPORTED && g.index_format == WPROJ_INDEX_AUTO)) {
       return st;
     }   // AUTO: rows with more than 64 runs keep the column form
   }
-  if (p->fmt != WPROJ_INDEX_TILE_RUNS) {
+  if (p->fmt != WPROJ_INDEX_TILE_RUNS || p->slices.use) {
     p->rm_vptr.release();
     p->rm_rptr.release();
     p->rm_org.release();
@@ -1504,7 +1521,7 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
   } else {
     WPROJ_TRY(make_row_pieces(m, p->row_ptr.as<int64_t>(), degrid_piece(p->nnz), p->piece_row, p->piece_lo,
                               p->piece_len, p->row_piece_ptr, &p->n_pieces, s));
-    WPROJ_TRY(p->piece_partial.reuse(sizeof(float2) * std::max<int64_t>(1, p->n_pieces)));
+    WPROJ_TRY(p->piece_partial.reuse(sizeof(float2) * (p->slices.use ? 1 : std::max<int64_t>(1, p->n_pieces))));
   }
 
   // ---- gridding: chunks of one tile's segments (tile order), balanced by entries
@@ -1528,7 +1545,7 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
     WPROJ_TRY(make_tile_chunks(n_tiles, tptr.as<int64_t>(), cum.as<int64_t>(), n_items, p->nnz, chunk, p->chunk_tile,
                                p->chunk_lo, p->chunk_hi, p->tile_chunk_ptr, &p->n_chunks, s));
     // column format: a cell-major copy for the gridding (packed rows need m <= 2^22)
-    p->has_cells = !rec && g.tile == 32 && m <= (int64_t(1) << 22);
+    p->has_cells = !rec && !p->slices.use && g.tile == 32 && m <= (int64_t(1) << 22);
     if (p->has_cells) {
       WPROJ_TRY(build_cells(p, tptr.as<int64_t>(), cum.as<int64_t>(), n_seg, s));
     } else {
@@ -1536,7 +1553,8 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
       p->cell_ent.release();
       p->cell_val.release();
     }
-    WPROJ_TRY(p->grid_partial.reuse(sizeof(float2) * size_t(p->n_chunks) * g.tile * g.tile));
+    WPROJ_TRY(p->grid_partial.reuse(p->slices.use ? sizeof(float2)
+                                                  : sizeof(float2) * size_t(p->n_chunks) * g.tile * g.tile));
   }
   WPROJ_TRY(p->ytmp.reuse(sizeof(float2) * m));
   WPROJ_CUDA(cudaMemcpyAsync(&herr, d_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));

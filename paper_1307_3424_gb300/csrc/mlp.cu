@@ -674,6 +674,7 @@ wproj_status build_learned_impl(wproj_plan *p, wproj_mlp *n, const double *uvw, 
   }
   WPROJ_TRY(check_err(n, s));
   WPROJ_TRY(rebuild_cells(p, s));
+  WPROJ_TRY(rebuild_slices(p, s));
   k_count_pass<<<1, 256, 0, s>>>(m, pass.as<int8_t>(), err_p, cnt.as<unsigned long long>(), cnt.as<double>() + 1);
   WPROJ_CHECK_LAUNCH("mlp pass count");
   unsigned long long np_ = 0;

@@ -301,7 +301,7 @@ wproj_status launch_degrid_cols(wproj_plan *p, const float2 *Xt, float2 *partial
 }  // namespace
 
 wproj_status degrid(wproj_plan *p, const float2 *Xt, float2 *y, cudaStream_t s) {
-  p->launches += p->fmt == WPROJ_INDEX_TILE_RUNS ? 1 : 2;
+  p->launches += p->slices.use || p->fmt == WPROJ_INDEX_TILE_RUNS ? 1 : 2;
   return degrid_into(p, Xt, p->piece_partial.as<float2>(), y, s);
 }
 
@@ -309,6 +309,10 @@ wproj_status degrid(wproj_plan *p, const float2 *Xt, float2 *y, cudaStream_t s) 
 // (degrid_partials(p) float2); the kernels and their launch shape are those of
 // degrid().
 wproj_status degrid_into(wproj_plan *p, const float2 *Xt, float2 *partial, float2 *y, cudaStream_t s) {
+  if (p->slices.use) {   // short rows: no partial sums
+    ScopedTimer t(p, TC_DEGRID, s);
+    return degrid_slices(p, Xt, y, s);
+  }
   if (p->fmt == WPROJ_INDEX_TILE_RUNS) {   // warp per row, no partial sums
     ScopedTimer t(p, TC_DEGRID, s);
     return degrid_runs(p, Xt, y, s);
@@ -347,7 +351,10 @@ wproj_status grid(wproj_plan *p, const float2 *y, float2 *Xt2, cudaStream_t s) {
         p->seg_meta.as<SegMeta>(), p->col.as<int32_t>(), p->val.ptr, rs, y, logG, g.tile, g.nT, nullptr,    \
         nullptr, p->grid_partial.as<float2>());                                                             \
   } while (0)
-    if (p->fmt == WPROJ_INDEX_TILE_RUNS) {
+    if (p->slices.use) {
+      p->launches -= p->slices.n_multi ? 0 : 1;
+      return grid_slices(p, y, Xt2, s);
+    } else if (p->fmt == WPROJ_INDEX_TILE_RUNS) {
       int nl = 0;
       WPROJ_TRY(grid_runs(p, y, Xt2, &nl, s));
       p->launches += nl - 2;

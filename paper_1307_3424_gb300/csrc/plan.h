@@ -25,7 +25,7 @@ struct DevBuf {
     bytes = 0;
     own = true;
   }
-  wproj_status alloc(size_t n);           // exact size, contents undefined
+  virtual wproj_status alloc(size_t n);   // exact size, contents undefined
   wproj_status ensure(size_t n);          // grow (contents discarded)
   wproj_status reuse(size_t n);           // keep an allocation of n to 9/8 n bytes, else as alloc
   template <class T> T *as() const { return static_cast<T *>(ptr); }
@@ -37,7 +37,7 @@ struct DevBuf {
 // outside it or when the block is used up.  Nothing is handed out twice within a
 // scope, so a buffer dropped while kernels still read it stays theirs.
 struct TmpBuf : DevBuf {
-  wproj_status alloc(size_t n);
+  wproj_status alloc(size_t n) override;
 };
 
 // The block belongs to the plan (kept up to kScratchKeep bytes, freed with it); the
@@ -94,6 +94,51 @@ struct BatchOps {
   const void *cell_val = nullptr;
 };
 
+// The short-row operators' view of G (slices.cu).  A step is 32 values with their
+// 2-byte indices.  The arrays of a batch are its problems' end to end.
+struct SliceOps {
+  int logG = 0;                          // plans; a batch's chunk names its problem
+  const float *row_scale = nullptr;      // by row; null for f32
+  // degridding: chunks of one tile's rows
+  int64_t d_chunks = 0;
+  const int64_t *d_slice_base = nullptr; // first slice of each chunk, closed
+  const int64_t *slice_ptr = nullptr;    // first step of each slice, closed
+  const int32_t *srow = nullptr;         // four rows a slice (-1: none)
+  const int4 *rect = nullptr;            // patch of each chunk: u0, v0, rows, columns
+  const uint16_t *d_idx = nullptr;       // 1 + place in the patch; 0: pad
+  const void *d_val = nullptr;
+  // gridding: chunks of one tile's segments
+  int64_t g_chunks = 0;
+  const int32_t *g_chunk_tile = nullptr; // tile within its problem
+  const int32_t *tile_chunk_ptr = nullptr;
+  const int32_t *multi = nullptr;        // tiles of several chunks
+  int64_t n_multi = 0;
+  const int64_t *g_base = nullptr;       // first step of each chunk
+  const uint32_t *g_slp = nullptr;       // 33 per chunk: first step of its 32 slices, closed
+  const uint16_t *g_perm = nullptr;      // 1024 per chunk: the cells in slice order
+  const int64_t *g_row_base = nullptr;   // first row of each chunk's list, closed
+  const int32_t *g_rows = nullptr;
+  const uint16_t *g_idx = nullptr;       // 1 + place in the chunk's rows; 0: pad
+  const void *g_val = nullptr;
+  const int32_t *d_chunk_prob = nullptr, *g_chunk_prob = nullptr, *tile_prob = nullptr;   // batches
+  const BProb *tab = nullptr;
+};
+
+// Patch cells a plan's chunks may have per stored entry before the other forms
+// are the faster ones.
+constexpr int64_t kPatchCellsPerEntry = 4;
+
+struct SliceCopy {
+  bool use = false;    // built, and the operators take it
+  DevBuf d_slice_base, slice_ptr, srow, rect, d_idx, d_val;
+  DevBuf g_chunk_tile, g_chunk_lo, g_chunk_hi, tile_chunk_ptr, g_base, g_slp, g_perm, g_row_base, g_rows, g_idx, g_val, multi;
+  DevBuf partial;      // float2[g_chunks * 1024] when a tile has several chunks
+  int64_t d_chunks = 0, d_slices = 0, d_steps = 0, g_chunks = 0, g_steps = 0, g_nrows = 0, n_multi = 0;
+  size_t d_smem = 0, g_smem = 0;
+  SliceOps ops() const;
+  void release();
+};
+
 // Timing accumulator for one class of kernels.
 // (TC_B*: the kernel build: box tables + box FFTs, selection + counts, emission)
 enum TimerClass { TC_FFT = 0, TC_DEGRID, TC_GRID, TC_REDUCE, TC_SOLVER, TC_BFFT, TC_BSEL, TC_BEMIT, TC_COUNT };
@@ -143,7 +188,11 @@ struct wproj_plan {
   wproj::DevBuf seg_rec;     // int64[n_seg] byte offset of each segment's record (TILE_MASK)
   wproj::DevBuf rec_off;     // int64[n_seg+1] byte offset of the records in stream order (TILE_MASK)
   wproj::DevBuf seg_tile;    // int32[n_seg] tile index of each segment
-  // TILE_RUNS: the row-major copy of the degridding (runs padded to even lengths);
+  // boxes of at most 64 x 64 cells: interleaved slices for both operators
+  wproj::SliceCopy slices;
+  bool in_batch = false;     // built for a batch, whose operators run on the whole
+  bool no_slices = false;    // a batch some of whose problems cannot take slices
+  // TILE_RUNS without slices: the row-major copy of the degridding (runs padded to even lengths);
   // the tile-major records of the gridding live in `stream` / `rec_off` / `seg_rec`
   int64_t rm_runs = 0, rm_vals = 0;
   wproj::DevBuf rm_vptr;     // int64[m+1] first stored value of each row
@@ -306,11 +355,21 @@ wproj_status apply_phi(wproj_plan *p, const float *x, const float2 *xc, float2 *
 wproj_status apply_phi_adj(wproj_plan *p, const float2 *y, float *x_re, float2 *x_cplx,
                            const float *z, int mode, cudaStream_t s);
 
+// slices.cu: short rows (boxes of at most 64 x 64 cells)
+wproj_status build_slices(wproj_plan *p, const int2 *j0, const int32_t *Sk, const int64_t *tptr, const int64_t *cum,
+                          int64_t n_seg, int32_t *row_runs, cudaStream_t s);
+wproj_status rebuild_slices(wproj_plan *p, cudaStream_t s);
+wproj_status degrid_slices(wproj_plan *p, const float2 *Xt, float2 *y, cudaStream_t s);
+wproj_status grid_slices(wproj_plan *p, const float2 *y, float2 *Xt2, cudaStream_t s);
+wproj_status batch_degrid_slices(const SliceOps &o, size_t smem, const float2 *Xt, float2 *y, cudaStream_t s);
+wproj_status batch_grid_slices(const SliceOps &o, size_t smem, const float2 *y, float2 *partial, float2 *Xt2,
+                               cudaStream_t s);
+
 // runs.cu (TILE_RUNS format): both copies from the column form in col / val, which
 // is then released; tile_seg / tptr = segments in tile order, compacted in place
 // to the n_rec segments that hold entries
-wproj_status build_runs(wproj_plan *p, const int2 *j0, const int32_t *Sk, int32_t *tile_seg, int64_t *tptr,
-                        int64_t *n_rec, cudaStream_t s);
+wproj_status build_runs(wproj_plan *p, const int2 *j0, const int32_t *Sk, const int32_t *row_runs, int32_t *tile_seg,
+                        int64_t *tptr, int64_t *n_rec, cudaStream_t s);
 wproj_status degrid_runs(wproj_plan *p, const float2 *Xt, float2 *y, cudaStream_t s);
 wproj_status grid_runs(wproj_plan *p, const float2 *y, float2 *Xt2, int *launches, cudaStream_t s);
 wproj_status runs_export(const wproj_plan *p, int64_t k0, int64_t k1, int32_t *col_out, void *val_out,
@@ -327,9 +386,10 @@ wproj_status make_tile_chunks(int n_tiles, const int64_t *tptr, const int64_t *c
 
 // scan.cu
 wproj_status exclusive_scan_i32_to_i64(const int32_t *in, int64_t *out, int64_t n, cudaStream_t s);
+wproj_status exclusive_scan_total(const int32_t *in, int64_t *out, int64_t n, cudaStream_t s);
 wproj_status exclusive_scan_i64(const int64_t *in, int64_t *out, int64_t n, cudaStream_t s);
 // stable counting sort of ids [0, n) by key[i] in [0, n_bins): out_ids, bin_ptr[n_bins+1]
 wproj_status stable_bin_sort(const int32_t *key, int64_t n, int n_bins, int32_t *out_ids,
-                             int64_t *bin_ptr, cudaStream_t s);
+                             int64_t *bin_ptr, cudaStream_t s, bool wait = true);
 
 }  // namespace wproj

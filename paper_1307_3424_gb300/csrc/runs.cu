@@ -441,8 +441,8 @@ __device__ __forceinline__ void row_runs32(unsigned w, int &nr, int &pc, unsigne
 __global__ void __launch_bounds__(64)
 k_rm_build(int64_t m, const int64_t *__restrict__ row_ptr, const int32_t *__restrict__ col,
            const unsigned char *__restrict__ val, int vb, const int2 *__restrict__ j0, const int32_t *__restrict__ Sk,
-           int logG, int32_t *__restrict__ out_pc, int32_t *__restrict__ out_nr, int *__restrict__ err,
-           const int64_t *__restrict__ vptr,
+           int logG, const int32_t *__restrict__ row_runs, int32_t *__restrict__ out_pc, int32_t *__restrict__ out_nr,
+           int *__restrict__ err, const int64_t *__restrict__ vptr,
            const int64_t *__restrict__ rptr, uint32_t *__restrict__ org, uint32_t *__restrict__ runs,
            unsigned char *__restrict__ rm_val) {
   __shared__ unsigned long long bm[64], lpad_s[64], rpad_s[64];
@@ -451,6 +451,7 @@ k_rm_build(int64_t m, const int64_t *__restrict__ row_ptr, const int32_t *__rest
   const int t = threadIdx.x, lane = t & 31;
   const int G = 1 << logG, Gm = G - 1;
   for (int64_t k = blockIdx.x; k < m; k += gridDim.x) {
+    if (row_runs && row_runs[k] <= kMaxRuns) continue;   // only the limit is asked for, and the row is within it
     const int S = Sk[k];
     const int au = (j0[k].x - S / 2) & Gm, av = (j0[k].y - S / 2) & Gm;
     bm[t] = 0;
@@ -642,14 +643,16 @@ int grid_blocks(int64_t units, int per_block) {
 
 }  // namespace
 
-// Both copies from the column form held in p->col / p->val (CSR order), then the
-// column form is released.  tile_seg / tptr: segments in tile order and the
+// Both copies (the records alone when the plan has slices) from the column form held
+// in p->col / p->val (CSR order), then the column form is released.  tile_seg / tptr: segments in tile order and the
 // first of each tile; on success they are compacted in place to the segments
 // that hold entries (the records; *n_rec of them).  A row or segment of more
 // than kMaxRuns runs returns WPROJ_ERR_UNSUPPORTED before anything is
 // allocated, and the column form stays as it was.
-wproj_status build_runs(wproj_plan *p, const int2 *j0, const int32_t *Sk, int32_t *tile_seg, int64_t *tptr,
-                        int64_t *n_rec, cudaStream_t s) {
+// row_runs (plans with slices): an upper bound of each row's runs; rows within the
+// limit by it are not counted again.
+wproj_status build_runs(wproj_plan *p, const int2 *j0, const int32_t *Sk, const int32_t *row_runs, int32_t *tile_seg,
+                        int64_t *tptr, int64_t *n_rec, cudaStream_t s) {
   const GridGeom &g = p->g;
   const int64_t m = p->m, n_seg = p->n_seg;
   const int vb = g.value_dtype == WPROJ_VAL_F32 ? 8 : 4;
@@ -663,7 +666,7 @@ wproj_status build_runs(wproj_plan *p, const int2 *j0, const int32_t *Sk, int32_
   WPROJ_TRY(err.alloc(sizeof(int)));
   WPROJ_CUDA(cudaMemsetAsync(err.ptr, 0, sizeof(int), s));
   k_rm_build<<<nb_rows, 64, 0, s>>>(m, p->row_ptr.as<int64_t>(), p->col.as<int32_t>(), p->val.as<unsigned char>(),
-                                    vb, j0, Sk, logG, pc.as<int32_t>(), nr.as<int32_t>(), err.as<int>(), nullptr,
+                                    vb, j0, Sk, logG, row_runs, pc.as<int32_t>(), nr.as<int32_t>(), err.as<int>(), nullptr,
                                     nullptr, nullptr, nullptr, nullptr);
   WPROJ_CHECK_LAUNCH("runs: row counts");
   if (n_seg > 0) {
@@ -677,8 +680,8 @@ wproj_status build_runs(wproj_plan *p, const int2 *j0, const int32_t *Sk, int32_
   WPROJ_CUDA(cudaMemcpyAsync(&herr, err.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));
   WPROJ_CUDA(cudaStreamSynchronize(s));
   if (herr) return fail(WPROJ_ERR_UNSUPPORTED, "build_kernels: a row or segment holds more than 64 runs");
-  // ---- row-major copy
-  {
+  // ---- row-major copy (the slices serve the operators where they exist)
+  if (!p->slices.use) {
     WPROJ_TRY(p->rm_vptr.reuse(sizeof(int64_t) * (m + 1)));
     WPROJ_TRY(p->rm_rptr.reuse(sizeof(int64_t) * (m + 1)));
     WPROJ_TRY(p->rm_org.reuse(sizeof(uint32_t) * m));
@@ -689,7 +692,7 @@ wproj_status build_runs(wproj_plan *p, const int2 *j0, const int32_t *Sk, int32_
     WPROJ_TRY(p->rm_val.reuse(int64_t(vb) * std::max<int64_t>(4, n_vals)));
     WPROJ_CUDA(cudaMemsetAsync(p->rm_val.ptr, 0, int64_t(vb) * std::max<int64_t>(4, n_vals), s));
     k_rm_build<<<nb_rows, 64, 0, s>>>(m, p->row_ptr.as<int64_t>(), p->col.as<int32_t>(),
-                                      p->val.as<unsigned char>(), vb, j0, Sk, logG, nullptr, nullptr, nullptr,
+                                      p->val.as<unsigned char>(), vb, j0, Sk, logG, nullptr, nullptr, nullptr, nullptr,
                                       p->rm_vptr.as<int64_t>(), p->rm_rptr.as<int64_t>(), p->rm_org.as<uint32_t>(),
                                       p->rm_run.as<uint32_t>(), p->rm_val.as<unsigned char>());
     WPROJ_CHECK_LAUNCH("runs: row-major copy");

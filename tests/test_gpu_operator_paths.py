@@ -77,7 +77,32 @@ def test_dense_rows(wp, N, M, wmax, fmt, value):
     plan.close()
 
 
-# problems on 16^2 grids (one tile of 16 x 16 cells) beside larger ones
+# short rows (boxes of at most 64 x 64 cells) on interleaved slices: grids whose
+# patches wrap round the whole axis (32^2, 64^2) and larger ones; one row, a tile of
+# rows split over several chunks, rows at the grid's edge; runs of 2 to 64 cells
+# (w up to 4 cells; e = 1 keeps whole boxes), each value type and storage
+@pytest.mark.parametrize("N,M,wmax,W,e,fmt,value", [
+    (16, 40, 1.0, 4, 0.99, "auto", "f32"), (32, 1, 0.0, 4, 0.99, "auto", "f32"), (32, 900, 4.0, 4, 0.99, "auto", "f32"),
+    (32, 300, 4.0, 8, 1.0, "columns", "f32"), (64, 1500, 4.0, 6, 0.999, "auto", "f32"),
+    (64, 1500, 0.3, 4, 0.9, "auto", "bf16"), (128, 6001, 4.0, 4, 0.99, "auto", "f16"),
+    (128, 3000, 2.0, 8, 0.99, "runs", "bf16"), (256, 20000, 1.0, 4, 0.99, "columns", "f32"),
+    (256, 2000, 4.0, 4, 1.0, "auto", "f32"), (512, 9, 3.0, 4, 0.99, "auto", "f32"), (512, 9, 3.0, 4, 0.99, "auto", "bf16"),
+])
+def test_short_rows(wp, N, M, wmax, W, e, fmt, value):
+    rng = np.random.default_rng(N + M + W)
+    uvw = uvw_cells(rng, M, N, wmax, edge=0.2)
+    if M > 1000:
+        uvw[: M // 2, :2] = uvw[0, :2]      # half of the rows in one tile: several chunks
+        uvw[: M // 2, :2] += rng.uniform(0, 0.5, (M // 2, 2)) / L
+        uvw = uvw[np.abs(uvw[:, :2]).max(axis=1) < synth.band_limit(N, L) * (1 - 1e-9)]
+    plan = wp.Plan(N, L, kb_support=W, box="rule", value_dtype=value, index_format=fmt)
+    plan.build_kernels(torch.from_numpy(np.ascontiguousarray(uvw)).cuda(), e)
+    check_operators(plan, N, W, rng)
+    plan.close()
+
+
+# a batch takes slices only when every problem can (a 16^2 grid, one tile of 16 x 16
+# cells, cannot)
 @pytest.mark.parametrize("ns", [(16, 32, 64), (64, 16, 128), (8, 64)])
 def test_batch_matches_single_plans(wp, ns):
     rng = np.random.default_rng(sum(ns))
