@@ -313,9 +313,28 @@ wproj_status bgrid(wproj_batch *b, const float2 *y, float2 *Xt2, cudaStream_t s)
   return batch_grid(ops_of(b), y, b->grid_partial.as<float2>(), Xt2, s);
 }
 
-wproj_status bphi(wproj_batch *b, const float *x, float2 *y, cudaStream_t s) {
-  for (auto &c : b->cls) {
+// the size classes up to 1024^2, largest first (its blocks are the longest)
+FftClasses small_classes(const wproj_batch *b) {
+  FftClasses cl;
+  for (int lg = kBatchMaxLog; lg >= 4; --lg) {
+    const auto &c = b->cls[lg];
     if (c.np == 0) continue;
+    cl.logG[cl.n] = c.logG;
+    cl.np[cl.n] = c.np;
+    cl.plist[cl.n++] = c.plist.as<int32_t>();
+  }
+  return cl;
+}
+
+wproj_status bphi(wproj_batch *b, const float *x, float2 *y, cudaStream_t s) {
+  const FftClasses cl = small_classes(b);
+  if (cl.n) {
+    WPROJ_TRY(batch_phi_fwd_all(cl, b->tab.as<BProb>(), x, b->inv_a.as<float>(), b->interb.as<float2>(),
+                                b->Xt.as<float2>(), b->twiddle.as<float2>(), s));
+    b->launches += 2;
+  }
+  for (auto &c : b->cls) {
+    if (c.np == 0 || c.logG <= kBatchMaxLog) continue;
     WPROJ_TRY(batch_phi_fwd(c.logG, c.np, c.plist.as<int32_t>(), b->tab.as<BProb>(), x, b->inv_a.as<float>(),
                             b->interb.as<float2>(), b->Xt.as<float2>(), b->twiddle.as<float2>(), s));
     b->launches += 2;
@@ -328,8 +347,14 @@ wproj_status bphi(wproj_batch *b, const float *x, float2 *y, cudaStream_t s) {
 wproj_status bphi_adj(wproj_batch *b, const float2 *y, float *x_re, const float *z, int mode, cudaStream_t s) {
   WPROJ_TRY(bgrid(b, y, b->Xt2.as<float2>(), s));
   b->launches += b->has_slices && !b->slices.n_multi ? 1 : 2;
+  const FftClasses cl = small_classes(b);
+  if (cl.n) {
+    WPROJ_TRY(batch_phi_adj_all(cl, b->tab.as<BProb>(), b->Xt2.as<float2>(), b->inv_a.as<float>(),
+                                b->interb.as<float2>(), x_re, z, mode, b->twiddle.as<float2>(), s));
+    b->launches += 2;
+  }
   for (auto &c : b->cls) {
-    if (c.np == 0) continue;
+    if (c.np == 0 || c.logG <= kBatchMaxLog) continue;
     WPROJ_TRY(batch_phi_adj(c.logG, c.np, c.plist.as<int32_t>(), b->tab.as<BProb>(), b->Xt2.as<float2>(),
                             b->inv_a.as<float>(), b->interb.as<float2>(), x_re, z, mode, b->twiddle.as<float2>(), s));
     b->launches += 2;

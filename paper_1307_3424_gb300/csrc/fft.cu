@@ -9,6 +9,8 @@
 //    Douglas-Rachford dual step).
 //  * The kernel build: batched S x S inverse transforms of the chirp times the
 //    KB tap polynomial, with the chirp generated in the first pass's load.
+#include <algorithm>
+
 #include "build.cuh"
 #include "fft.cuh"
 #include "plan.h"
@@ -40,12 +42,11 @@ __device__ __forceinline__ int pad_to_img(int m, int P, int G) { return m < 4 ? 
 // Each pass is a device body (block `blk` of one transform set) called by a
 // kernel for one plan and by a kernel for a batch of same-size problems
 // (blockIdx.y = problem of the size class, offsets from its BProb entry).
-template <int LOGN>
+template <int LOGN, class Cfg>
 __device__ __forceinline__ void phi_fwd_rows_body(const float *__restrict__ x, const float2 *__restrict__ xc,
                                                   const float *__restrict__ inv_a, int N,
                                                   float2 *__restrict__ inter, const float2 *__restrict__ tw,
                                                   int blk) {
-  using Cfg = RowCfg<LOGN>;
   constexpr int G = 1 << LOGN;
   extern __shared__ float2 sm[];
   int c, tq;
@@ -74,7 +75,7 @@ template <int LOGN>
 __global__ void __launch_bounds__(RowCfg<LOGN>::T)
 k_phi_fwd_rows(const float *__restrict__ x, const float2 *__restrict__ xc, const float *__restrict__ inv_a, int N,
                float2 *__restrict__ inter, const float2 *__restrict__ tw) {
-  phi_fwd_rows_body<LOGN>(x, xc, inv_a, N, inter, tw, blockIdx.x);
+  phi_fwd_rows_body<LOGN, RowCfg<LOGN>>(x, xc, inv_a, N, inter, tw, blockIdx.x);
 }
 
 template <int LOGN>
@@ -82,13 +83,12 @@ __global__ void __launch_bounds__(RowCfg<LOGN>::T)
 k_bphi_fwd_rows(const BProb *__restrict__ tab, const int32_t *__restrict__ plist, const float *__restrict__ x,
                 const float *__restrict__ inv_a, float2 *__restrict__ inter, const float2 *__restrict__ tw) {
   const BProb P = tab[plist[blockIdx.y]];
-  phi_fwd_rows_body<LOGN>(x + P.img_off, nullptr, inv_a + P.inva_off, P.N, inter + P.inter_off, tw, blockIdx.x);
+  phi_fwd_rows_body<LOGN, RowCfg<LOGN>>(x + P.img_off, nullptr, inv_a + P.inva_off, P.N, inter + P.inter_off, tw, blockIdx.x);
 }
 
-template <int LOGN>
+template <int LOGN, class Cfg>
 __device__ __forceinline__ void phi_fwd_cols_body(const float2 *__restrict__ inter, int N, float2 *__restrict__ Xt,
                                                   float scale, const float2 *__restrict__ tw, int blk) {
-  using Cfg = ColCfg<LOGN>;
   constexpr int G = 1 << LOGN;
   extern __shared__ float2 sm[];
   int c, tq;
@@ -110,7 +110,7 @@ template <int LOGN>
 __global__ void __launch_bounds__(ColCfg<LOGN>::T)
 k_phi_fwd_cols(const float2 *__restrict__ inter, int N, float2 *__restrict__ Xt, float scale,
                const float2 *__restrict__ tw) {
-  phi_fwd_cols_body<LOGN>(inter, N, Xt, scale, tw, blockIdx.x);
+  phi_fwd_cols_body<LOGN, ColCfg<LOGN>>(inter, N, Xt, scale, tw, blockIdx.x);
 }
 
 template <int LOGN>
@@ -118,15 +118,14 @@ __global__ void __launch_bounds__(ColCfg<LOGN>::T)
 k_bphi_fwd_cols(const BProb *__restrict__ tab, const int32_t *__restrict__ plist, const float2 *__restrict__ inter,
                 float2 *__restrict__ Xt, const float2 *__restrict__ tw) {
   const BProb P = tab[plist[blockIdx.y]];
-  phi_fwd_cols_body<LOGN>(inter + P.inter_off, P.N, Xt + P.grid_off, 1.0f / P.G, tw, blockIdx.x);
+  phi_fwd_cols_body<LOGN, ColCfg<LOGN>>(inter + P.inter_off, P.N, Xt + P.grid_off, 1.0f / P.G, tw, blockIdx.x);
 }
 
 // ---- Phi^H: A Z^H F^H -----------------------------------------------------------
 
-template <int LOGN>
+template <int LOGN, class Cfg>
 __device__ __forceinline__ void phi_adj_cols_body(const float2 *__restrict__ Xt2, int N, float2 *__restrict__ inter,
                                                   const float2 *__restrict__ tw, int blk) {
-  using Cfg = ColCfg<LOGN>;
   constexpr int G = 1 << LOGN;
   extern __shared__ float2 sm[];
   int c, tq;
@@ -145,7 +144,7 @@ __device__ __forceinline__ void phi_adj_cols_body(const float2 *__restrict__ Xt2
 template <int LOGN>
 __global__ void __launch_bounds__(ColCfg<LOGN>::T)
 k_phi_adj_cols(const float2 *__restrict__ Xt2, int N, float2 *__restrict__ inter, const float2 *__restrict__ tw) {
-  phi_adj_cols_body<LOGN>(Xt2, N, inter, tw, blockIdx.x);
+  phi_adj_cols_body<LOGN, ColCfg<LOGN>>(Xt2, N, inter, tw, blockIdx.x);
 }
 
 template <int LOGN>
@@ -153,16 +152,15 @@ __global__ void __launch_bounds__(ColCfg<LOGN>::T)
 k_bphi_adj_cols(const BProb *__restrict__ tab, const int32_t *__restrict__ plist, const float2 *__restrict__ Xt2,
                 float2 *__restrict__ inter, const float2 *__restrict__ tw) {
   const BProb P = tab[plist[blockIdx.y]];
-  phi_adj_cols_body<LOGN>(Xt2 + P.grid_off, P.N, inter + P.inter_off, tw, blockIdx.x);
+  phi_adj_cols_body<LOGN, ColCfg<LOGN>>(Xt2 + P.grid_off, P.N, inter + P.inter_off, tw, blockIdx.x);
 }
 
 // mode 0: x_re = Re(v) s (and x_c = v s when given); mode 1: x_re = z - Re(v) s
-template <int LOGN>
+template <int LOGN, class Cfg>
 __device__ __forceinline__ void phi_adj_rows_body(const float2 *__restrict__ inter, const float *__restrict__ inv_a,
                                                   int N, float scale, float *__restrict__ x_re,
                                                   float2 *__restrict__ x_c, const float *__restrict__ z, int mode,
                                                   const float2 *__restrict__ tw, int blk) {
-  using Cfg = RowCfg<LOGN>;
   constexpr int G = 1 << LOGN;
   extern __shared__ float2 sm[];
   int c, tq;
@@ -194,7 +192,7 @@ __global__ void __launch_bounds__(RowCfg<LOGN>::T)
 k_phi_adj_rows(const float2 *__restrict__ inter, const float *__restrict__ inv_a, int N, float scale,
                float *__restrict__ x_re, float2 *__restrict__ x_c, const float *__restrict__ z, int mode,
                const float2 *__restrict__ tw) {
-  phi_adj_rows_body<LOGN>(inter, inv_a, N, scale, x_re, x_c, z, mode, tw, blockIdx.x);
+  phi_adj_rows_body<LOGN, RowCfg<LOGN>>(inter, inv_a, N, scale, x_re, x_c, z, mode, tw, blockIdx.x);
 }
 
 template <int LOGN>
@@ -203,8 +201,77 @@ k_bphi_adj_rows(const BProb *__restrict__ tab, const int32_t *__restrict__ plist
                 const float *__restrict__ inv_a, float *__restrict__ x_re, const float *__restrict__ z, int mode,
                 const float2 *__restrict__ tw) {
   const BProb P = tab[plist[blockIdx.y]];
-  phi_adj_rows_body<LOGN>(inter + P.inter_off, inv_a + P.inva_off, P.N, 1.0f / P.G, x_re + P.img_off, nullptr,
+  phi_adj_rows_body<LOGN, RowCfg<LOGN>>(inter + P.inter_off, inv_a + P.inva_off, P.N, 1.0f / P.G, x_re + P.img_off, nullptr,
                           z ? z + P.img_off : nullptr, mode, tw, blockIdx.x);
+}
+
+// ---- batches: one launch per pass for all grid sizes up to 1024^2 -------------------
+// A launch per size ran the sizes one after another, each with a tail of its own and
+// too few blocks to fill the chip (64 problems: 16 launches, 180 us of transforms).
+
+// the size class, problem and block of the problem that blockIdx.x stands for
+__device__ __forceinline__ int class_block(const FftClasses &cl, int &prob, int &blk) {
+  int c = 0;
+  while (c + 1 < cl.n && int(blockIdx.x) >= cl.first[c + 1]) ++c;
+  const int q = int(blockIdx.x) - cl.first[c];
+  prob = __ldg(cl.plist[c] + q / cl.per[c]);
+  blk = q % cl.per[c];
+  return cl.logG[c];
+}
+
+#define WPROJ_BATCH_LOGN(logn, CALL) \
+  switch (logn) {                    \
+    case 4: CALL(4); break;          \
+    case 5: CALL(5); break;          \
+    case 6: CALL(6); break;          \
+    case 7: CALL(7); break;          \
+    case 8: CALL(8); break;          \
+    case 9: CALL(9); break;          \
+    default: CALL(10);               \
+  }
+
+__global__ void __launch_bounds__(256, 3)
+k_bphi_fwd_rows_all(const FftClasses cl, const BProb *__restrict__ tab, const float *__restrict__ x,
+                    const float *__restrict__ inv_a, float2 *__restrict__ inter, const float2 *__restrict__ tw) {
+  int prob, blk;
+  const int lg = class_block(cl, prob, blk);
+  const BProb P = tab[prob];
+#define CALL(L) phi_fwd_rows_body<L, BatchRowCfg<L>>(x + P.img_off, nullptr, inv_a + P.inva_off, P.N, inter + P.inter_off, tw, blk)
+  WPROJ_BATCH_LOGN(lg, CALL)
+#undef CALL
+}
+__global__ void __launch_bounds__(256, 3)
+k_bphi_fwd_cols_all(const FftClasses cl, const BProb *__restrict__ tab, const float2 *__restrict__ inter,
+                    float2 *__restrict__ Xt, const float2 *__restrict__ tw) {
+  int prob, blk;
+  const int lg = class_block(cl, prob, blk);
+  const BProb P = tab[prob];
+#define CALL(L) phi_fwd_cols_body<L, BatchColCfg<L>>(inter + P.inter_off, P.N, Xt + P.grid_off, 1.0f / P.G, tw, blk)
+  WPROJ_BATCH_LOGN(lg, CALL)
+#undef CALL
+}
+__global__ void __launch_bounds__(256, 3)
+k_bphi_adj_cols_all(const FftClasses cl, const BProb *__restrict__ tab, const float2 *__restrict__ Xt2,
+                    float2 *__restrict__ inter, const float2 *__restrict__ tw) {
+  int prob, blk;
+  const int lg = class_block(cl, prob, blk);
+  const BProb P = tab[prob];
+#define CALL(L) phi_adj_cols_body<L, BatchColCfg<L>>(Xt2 + P.grid_off, P.N, inter + P.inter_off, tw, blk)
+  WPROJ_BATCH_LOGN(lg, CALL)
+#undef CALL
+}
+__global__ void __launch_bounds__(256, 3)
+k_bphi_adj_rows_all(const FftClasses cl, const BProb *__restrict__ tab, const float2 *__restrict__ inter,
+                    const float *__restrict__ inv_a, float *__restrict__ x_re, const float *__restrict__ z, int mode,
+                    const float2 *__restrict__ tw) {
+  int prob, blk;
+  const int lg = class_block(cl, prob, blk);
+  const BProb P = tab[prob];
+#define CALL(L)                                                                                                  \
+  phi_adj_rows_body<L, BatchRowCfg<L>>(inter + P.inter_off, inv_a + P.inva_off, P.N, 1.0f / P.G, x_re + P.img_off, \
+                                       nullptr, z ? z + P.img_off : nullptr, mode, tw, blk)
+  WPROJ_BATCH_LOGN(lg, CALL)
+#undef CALL
 }
 
 // ---- generic batched 2-D FFT (rows then columns) --------------------------------
@@ -627,19 +694,62 @@ wproj_status box_fft(wproj_plan *p, const BoxBatch &bb, cudaStream_t s) {
 #undef CALL
 }
 
+// blocks of a problem and shared memory of a pass of the joint launches
+template <template <int> class Cfg>
+void batch_shape(int logG, int lines, int *per, size_t *smem) {
+#define CALL(L)                                                      \
+  static_assert(Cfg<L>::SMEM <= 48 * 1024, "no attribute is set");   \
+  *per = ceil_div(lines, Cfg<L>::C), *smem = std::max(*smem, Cfg<L>::SMEM)
+  WPROJ_BATCH_LOGN(logG, CALL)
+#undef CALL
+}
+template <template <int> class Cfg>
+int batch_blocks(FftClasses &cl, bool rows, size_t *smem) {
+  int n = 0;
+  for (int c = 0; c < cl.n; ++c) {
+    const int G = 1 << cl.logG[c];
+    batch_shape<Cfg>(cl.logG[c], rows ? G / 2 : G, &cl.per[c], smem);
+    cl.first[c] = n;
+    n += cl.per[c] * cl.np[c];
+  }
+  return n;
+}
+
+wproj_status batch_phi_fwd_all(FftClasses cl, const BProb *tab, const float *x, const float *inv_a, float2 *inter,
+                               float2 *Xt, const float2 *tw, cudaStream_t s) {
+  size_t smem = 0;
+  int n = batch_blocks<BatchRowCfg>(cl, true, &smem);
+  k_bphi_fwd_rows_all<<<n, 256, smem, s>>>(cl, tab, x, inv_a, inter, tw);
+  smem = 0;
+  n = batch_blocks<BatchColCfg>(cl, false, &smem);
+  k_bphi_fwd_cols_all<<<n, 256, smem, s>>>(cl, tab, inter, Xt, tw);
+  WPROJ_CHECK_LAUNCH("batch phi fwd");
+  return WPROJ_OK;
+}
+wproj_status batch_phi_adj_all(FftClasses cl, const BProb *tab, const float2 *Xt2, const float *inv_a, float2 *inter,
+                               float *x_re, const float *z, int mode, const float2 *tw, cudaStream_t s) {
+  size_t smem = 0;
+  int n = batch_blocks<BatchColCfg>(cl, false, &smem);
+  k_bphi_adj_cols_all<<<n, 256, smem, s>>>(cl, tab, Xt2, inter, tw);
+  smem = 0;
+  n = batch_blocks<BatchRowCfg>(cl, true, &smem);
+  k_bphi_adj_rows_all<<<n, 256, smem, s>>>(cl, tab, inter, inv_a, x_re, z, mode, tw);
+  WPROJ_CHECK_LAUNCH("batch phi adj");
+  return WPROJ_OK;
+}
+
+// the sizes above 1024^2, a launch per pass and size
 wproj_status batch_phi_fwd(int logG, int np, const int32_t *plist, const BProb *tab, const float *x,
                            const float *inv_a, float2 *inter, float2 *Xt, const float2 *tw, cudaStream_t s) {
-#define CALL(L) bphi_fwd_impl<L>(np, plist, tab, x, inv_a, inter, Xt, tw, s)
-  WPROJ_LOGN_SWITCH(logG, CALL)
-#undef CALL
+  return logG == 11 ? bphi_fwd_impl<11>(np, plist, tab, x, inv_a, inter, Xt, tw, s)
+                    : bphi_fwd_impl<12>(np, plist, tab, x, inv_a, inter, Xt, tw, s);
 }
 
 wproj_status batch_phi_adj(int logG, int np, const int32_t *plist, const BProb *tab, const float2 *Xt2,
                            const float *inv_a, float2 *inter, float *x_re, const float *z, int mode,
                            const float2 *tw, cudaStream_t s) {
-#define CALL(L) bphi_adj_impl<L>(np, plist, tab, Xt2, inv_a, inter, x_re, z, mode, tw, s)
-  WPROJ_LOGN_SWITCH(logG, CALL)
-#undef CALL
+  return logG == 11 ? bphi_adj_impl<11>(np, plist, tab, Xt2, inv_a, inter, x_re, z, mode, tw, s)
+                    : bphi_adj_impl<12>(np, plist, tab, Xt2, inv_a, inter, x_re, z, mode, tw, s);
 }
 
 }  // namespace wproj

@@ -161,7 +161,7 @@ __device__ __forceinline__ void fft_run(float2 (&v)[kFftE], int tq, float2 *s, c
 // large grids (32-byte row segments, whole sectors) and 8 below.  Blocks of the
 // small grids are kept small so that a grid of 128^2 still fills 16 blocks.
 constexpr int fft_ld(int n, int mod16) {   // exchange buffer length congruent to mod16 mod 16
-  int ld = n + n / 16;
+  int ld = n + n / 16 - 1;   // fft_pad(n - 1) + 1
   while (ld % 16 != mod16) ++ld;
   return ld;
 }
@@ -178,6 +178,25 @@ template <int LOGN> struct ColCfg {
   static constexpr int TN = N / kFftE;
   static constexpr int C = LOGN <= 5 ? 32 : (LOGN <= 8 ? 8 : 4);
   static constexpr int T = C * TN;
+  static constexpr int LD = fft_ld(N, C >= 16 ? 1 : 16 / C);
+  static constexpr size_t SMEM = size_t(C) * LD * sizeof(float2);
+};
+// Batches: every grid size up to 1024^2 in blocks of 256 threads, so that one launch
+// serves all of a batch's sizes.
+constexpr int kBatchMaxLog = 10;
+template <int LOGN> struct BatchRowCfg {
+  static constexpr int N = 1 << LOGN;
+  static constexpr int TN = N / kFftE;
+  static constexpr int T = 256;
+  static constexpr int C = T / TN;
+  static constexpr int LD = fft_ld(N, LOGN <= 5 ? 1 : 4);
+  static constexpr size_t SMEM = size_t(C) * LD * sizeof(float2);
+};
+template <int LOGN> struct BatchColCfg {
+  static constexpr int N = 1 << LOGN;
+  static constexpr int TN = N / kFftE;
+  static constexpr int T = 256;
+  static constexpr int C = T / TN;
   static constexpr int LD = fft_ld(N, C >= 16 ? 1 : 16 / C);
   static constexpr size_t SMEM = size_t(C) * LD * sizeof(float2);
 };

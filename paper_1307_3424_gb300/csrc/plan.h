@@ -285,6 +285,16 @@ wproj_status box_g_table(int S, const float *lsq, float *g, cudaStream_t s);   /
 
 wproj_status phi_forward_fft_into(wproj_plan *p, const float *x, float2 *inter, float2 *Xt, cudaStream_t s);
 // batches: F Z A and A Z^H F^H for the np problems plist (device) of one grid size 2^logG
+// the sizes up to 1024^2 in one launch per pass (first and per are the launch's), larger ones by size
+struct FftClasses {
+  int n = 0;
+  int logG[8], np[8], first[8], per[8];
+  const int32_t *plist[8];
+};
+wproj_status batch_phi_fwd_all(FftClasses cl, const BProb *tab, const float *x, const float *inv_a, float2 *inter,
+                               float2 *Xt, const float2 *tw, cudaStream_t s);
+wproj_status batch_phi_adj_all(FftClasses cl, const BProb *tab, const float2 *Xt2, const float *inv_a, float2 *inter,
+                               float *x_re, const float *z, int mode, const float2 *tw, cudaStream_t s);
 wproj_status batch_phi_fwd(int logG, int np, const int32_t *plist, const BProb *tab, const float *x,
                            const float *inv_a, float2 *inter, float2 *Xt, const float2 *tw, cudaStream_t s);
 wproj_status batch_phi_adj(int logG, int np, const int32_t *plist, const BProb *tab, const float2 *Xt2,
