@@ -851,7 +851,9 @@ wproj_status box_small(const BoxBatch &bb, const float2 *tw, bool select, double
 // word of the tile-mask format) and running popcounts give each entry's place
 // in the row-major compacted order and each tie's rank (ties are taken in the
 // same row-major order).  No block barriers: the 8 warps of a block take 8
-// segments.
+// segments.  A warp loads four rows before the first ballot (a row at a time
+// exposed the latency of its load).
+constexpr int kEmitRows = 4;
 __global__ void __launch_bounds__(256)
 k_emit(const float2 *__restrict__ K, int S, const int32_t *__restrict__ ids,
        const int2 *__restrict__ j0, const int64_t *__restrict__ seg_base,
@@ -897,42 +899,45 @@ k_emit(const float2 *__restrict__ K, int S, const int32_t *__restrict__ ids,
     // rows of the tile inside the box
     const unsigned rmask = __ballot_sync(0xffffffffu, lane < TS && ((tile_u * TS + lane - tu.a) & Gm) < S);
     const int r0 = max(0, __ffs(int(rmask)) - 1), r1 = 32 - __clz(int(rmask));
-#pragma unroll 4
-    for (int r = r0; r < r1; ++r) {
-      bool gt = false, eq = false;
-      int kidx = 0;
-      if (r < TS && col_in) {
-        const int du = (tile_u * TS + r - tu.a) & Gm;
-        if (du < S) {
-          kidx = ((du + S / 2) & (S - 1)) * S + iv;
-          const unsigned key = __float_as_uint(abs2_rn(Kb[kidx]));
-          gt = all || key > thr;
-          eq = !all && key == thr;
+    for (int rb = r0; rb < r1; rb += kEmitRows) {
+      float2 kv[kEmitRows];
+      bool in[kEmitRows];
+#pragma unroll
+      for (int u = 0; u < kEmitRows; ++u) {   // all loads of a group before its first ballot
+        const int du = (tile_u * TS + rb + u - tu.a) & Gm;
+        in[u] = rb + u < r1 && col_in && du < S;
+        kv[u] = in[u] ? __ldg(Kb + ((du + S / 2) & (S - 1)) * S + iv) : make_float2(0.f, 0.f);
+      }
+#pragma unroll
+      for (int u = 0; u < kEmitRows; ++u) {
+        const int r = rb + u;
+        if (r >= r1) break;
+        const unsigned key = __float_as_uint(abs2_rn(kv[u]));
+        const bool gt = in[u] && (all || key > thr), eq = in[u] && !all && key == thr;
+        const unsigned tw = __ballot_sync(0xffffffffu, eq);
+        const int rank = tie0 + tie_run + __popc(tw & lt);
+        const bool sel = gt || (eq && rank < ntie);
+        const unsigned sw = __ballot_sync(0xffffffffu, sel);
+        const int pos = sel_run + __popc(sw & lt);
+        if (sel && pos < cnt) {    // pos < cnt always holds when the two passes agree
+          const int64_t at = o + pos;
+          if (!rec) col[at] = (tile_u * TS + r) * g.G + cv;
+          const float2 v = kv[u];
+          if (vdt == WPROJ_VAL_F32) {
+            reinterpret_cast<float2 *>(vdst)[at] = v;
+          } else if (vdt == WPROJ_VAL_BF16) {
+            reinterpret_cast<__nv_bfloat162 *>(vdst)[at] = __floats2bfloat162_rn(v.x * inv_scale, v.y * inv_scale);
+          } else {
+            reinterpret_cast<__half2 *>(vdst)[at] = __floats2half2_rn(v.x * inv_scale, v.y * inv_scale);
+          }
         }
-      }
-      const unsigned tw = __ballot_sync(0xffffffffu, eq);
-      const int rank = tie0 + tie_run + __popc(tw & lt);
-      const bool sel = gt || (eq && rank < ntie);
-      const unsigned sw = __ballot_sync(0xffffffffu, sel);
-      const int pos = sel_run + __popc(sw & lt);
-      if (sel && pos < cnt) {    // pos < cnt always holds when the two passes agree
-        const int64_t at = o + pos;
-        if (!rec) col[at] = (tile_u * TS + r) * g.G + cv;
-        const float2 v = Kb[kidx];
-        if (vdt == WPROJ_VAL_F32) {
-          reinterpret_cast<float2 *>(vdst)[at] = v;
-        } else if (vdt == WPROJ_VAL_BF16) {
-          reinterpret_cast<__nv_bfloat162 *>(vdst)[at] = __floats2bfloat162_rn(v.x * inv_scale, v.y * inv_scale);
-        } else {
-          reinterpret_cast<__half2 *>(vdst)[at] = __floats2half2_rn(v.x * inv_scale, v.y * inv_scale);
+        if (lane == r) {
+          my_w = sw;
+          my_pre = sel_run;
         }
+        tie_run += __popc(tw);
+        sel_run += __popc(sw);
       }
-      if (lane == r) {
-        my_w = sw;
-        my_pre = sel_run;
-      }
-      tie_run += __popc(tw);
-      sel_run += __popc(sw);
     }
     if (lane == 0 && sel_run != cnt) atomicOr(err, ERR_EMIT);
     if (lane >= r1) my_pre = sel_run;   // rows past the box
