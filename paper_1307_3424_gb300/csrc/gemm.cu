@@ -6,7 +6,7 @@
 // Persistent and warp-specialised: one CTA per SM walks the 128 x BN tiles of
 // C (BN = 256 when N allows, else 128; tile t = CTA, CTA + grid, ...; tiles of
 // one row block of A are adjacent, so concurrent CTAs share A rows and B in
-// L2).  Six warps:
+// L2).  Ten warps:
 //   warp 0   TMA producer: for every 64-wide K slice of a tile, waits for a free
 //            stage, arms its `full` mbarrier with the slice's bytes and issues
 //            two cp.async.bulk.tensor loads (A: 128 rows, B: BN rows, x 64 bf16,
@@ -16,19 +16,22 @@
 //            issues four tcgen05.mma (kind::f16, K = 16) per slice from
 //            128B-swizzle K-major shared-memory descriptors, commits each slice
 //            to its stage's `empty` barrier and the tile to `acc_full`;
-//   warps 2-5  epilogue: wait for `acc_full`, read the accumulator with
+//   warps 2-9  epilogue: wait for `acc_full`, read the accumulator with
 //            tcgen05.ld (warp w reads tensor-memory lanes 32 (w mod 4) .., a lane
-//            one row of the tile), add the bias, apply GELU where asked, store
-//            32 bytes a lane (st.global.v8: whole sectors), and release the
-//            accumulator.
+//            one row of the tile; warps 2-5 the left half of the columns, 6-9 the
+//            right), add the bias, apply GELU where asked, put blocks of 32 x 32
+//            into swizzled shared memory and hand them to TMA (two blocks of a
+//            warp in flight), and release the accumulator.
 // So the loads of tile i + 1 and the MMAs of tile i + 1 overlap the epilogue of
-// tile i.  Four stages of 48 KB (BN = 256); 1 CTA per SM.
+// tile i.  BN = 256: three stages of 48 KB and 64 KB of staging; 1 CTA per SM.
 //
 // What bounds it: at large K the tensor cores; at the network's K = 256 the
-// epilogue and the output's bytes (65536 x 3072 FP32, 805 MB).  Storing 4 bytes a
-// lane after a transpose through shared memory took ~130 instructions per 32 x
-// 32 block in the one epilogue warp of each scheduler (330 us for that output);
-// a lane's own row in 32-byte stores takes ~50.
+// epilogue and the output's bytes (65536 x 3072 FP32, 805 MB): 143 us, 83 %
+// of the copy bandwidth.  A lane storing its own row 32 bytes at a time (whole
+// sectors, but a warp's store touches 32 lines) from four epilogue warps took 268 us;
+// sixteen warps with one staging block each 155 us, though they hide more of the
+// GELU's latency (65536 x 256 x 256 with GELU: 41 us with four, 35 with eight, 31
+// with sixteen).
 //
 // Split K: a product with fewer tiles than SMs (weight gradients: 2 to 24 tiles
 // of K = batch) is cut into `splits` ranges of K slices, each range a work unit
@@ -52,8 +55,10 @@ namespace {
 
 constexpr int kBM = 128, kBK = 64;      // tile rows; K slice (64 bf16 = one 128-byte swizzle row)
 constexpr int kSliceA = kBM * kBK * 2;   // bytes of one A slice: 16 KB
-constexpr int kStages = 4;
-constexpr int kThreads = 192;            // 6 warps
+constexpr int kEpiWarps = 8;
+constexpr int kOutBufs = 2;              // staging blocks a warp
+constexpr int kThreads = 64 + 32 * kEpiWarps;
+constexpr int kStage = 32 * 32 * 4;      // a warp's staging block: 32 rows of 128 bytes
 constexpr unsigned long long kGemmWaitNs = 2000000000ull;
 
 // Test hook (wproj_gemm_test_hook): when g_gemm_unset_wait is nonzero every
@@ -115,6 +120,15 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
       : "memory");
 }
 
+// 2-D tiled TMA store of a staged box at (x = column, y = row); one bulk group each
+__device__ __forceinline__ void tma_store_2d(const CUtensorMap *map, const void *src, int x, int y) {
+  asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(
+                   reinterpret_cast<uint64_t>(map)),
+               "r"(x), "r"(y), "r"(su32(src))
+               : "memory");
+  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+}
+
 // Shared-memory matrix descriptor (tcgen05) of a K-major operand in the
 // 128-byte-swizzled layout TMA writes: start address >> 4, leading byte offset
 // (unused for swizzled K-major; 1), stride byte offset 1024 (8 rows of 128 B),
@@ -138,73 +152,36 @@ __host__ __device__ constexpr uint32_t instr_desc(int M, int N) {
 // columns, two of them 2 BN (512 at most: the whole tensor memory).
 template <int BN>
 struct GemmSmem {
+  static constexpr int kStages = BN == 256 ? 3 : 4;
   unsigned char a[kStages][kSliceA];     // 1024-byte aligned (swizzle atoms)
   unsigned char b[kStages][BN * kBK * 2];
+  unsigned char out[kEpiWarps][kOutBufs][kStage];
   uint64_t full[kStages], empty[kStages], acc_full[2], acc_empty[2], never;
   uint32_t tmem_base;
 };
 
 // Z (FP32, optional with the other) and H (BF16): what the epilogue writes.
-// act: H = GELU(Z).  A store is 32 bytes a lane when `vec` (outputs 32-byte, bias
-// 16-byte aligned; rows are multiples of 128 elements), else element by element.
+// act: H = GELU(Z).  By TMA when `tma` (outputs and bias 16-byte aligned), else
+// element by element.
 struct EpiArgs {
   const float *bias;
   float *z;
   __nv_bfloat16 *h;
-  int act, splits, vec;
+  int act, splits, tma;
 };
 
-__device__ __forceinline__ void st_global_v8(void *p, const uint32_t (&v)[8]) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
-               "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
-               : "memory");
-}
-
-// one lane's 32 consecutive elements of a row (already biased): Z at z, H at h
-__device__ __forceinline__ void store_row32(const float (&v)[32], float *z, __nv_bfloat16 *h, int act, int vec) {
-  if (z) {
-    if (vec) {
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        uint32_t w[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) w[i] = __float_as_uint(v[8 * q + i]);
-        st_global_v8(z + 8 * q, w);
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < 32; ++i) z[i] = v[i];
-    }
-  }
-  if (h) {
-    __nv_bfloat162 b[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i)
-      b[i] = act ? __floats2bfloat162_rn(gelu(v[2 * i]), gelu(v[2 * i + 1])) : __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-    if (vec) {
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        uint32_t w[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) w[i] = *reinterpret_cast<const uint32_t *>(&b[8 * q + i]);
-        st_global_v8(h + 16 * q, w);
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        h[2 * i] = b[i].x;
-        h[2 * i + 1] = b[i].y;
-      }
-    }
-  }
+__device__ __forceinline__ void st_shared_v4(uint32_t at, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
 template <int BN>
 __global__ void __launch_bounds__(kThreads, 1)
-k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, int M, int N, int K,
+k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
+          const __grid_constant__ CUtensorMap tmZ, const __grid_constant__ CUtensorMap tmH, int M, int N, int K,
           const EpiArgs ep, int *__restrict__ err) {
+  constexpr int kStages = GemmSmem<BN>::kStages;
   constexpr int kAccCols = BN;
-  constexpr int kSliceB = BN * kBK * 2;
+  constexpr int kSliceB = BN * kBK * 2, kCols = BN / (kEpiWarps / 4);   // columns of an epilogue warp
   extern __shared__ unsigned char smem_raw[];
   GemmSmem<BN> &sm =
       *reinterpret_cast<GemmSmem<BN> *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -223,7 +200,7 @@ k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(&sm.acc_full[i], 1);    // one tcgen05.commit
-      mbar_init(&sm.acc_empty[i], 4);   // one arrive per epilogue warp
+      mbar_init(&sm.acc_empty[i], kEpiWarps);   // one arrive per epilogue warp
     }
     mbar_init(&sm.never, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -309,17 +286,28 @@ k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
       }
     }
   } else {
-    // ---- epilogue (warps 2-5): tensor-memory lanes 32 (warp mod 4) ..
-    const int lg = warp & 3;
-    uint32_t ti = 0;
+    // ---- epilogue (warps 2-9): tensor-memory lanes 32 (warp mod 4) .., half the columns
+    const int lg = warp & 3, ch = (warp - 2) / 4 * kCols;
+    uint32_t ti = 0, blk = 0;   // blk: blocks this warp staged
+    // the staging block to fill next, once TMA has read what was there
+    auto stage = [&]() {
+      if (lane == 0) asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kOutBufs - 1) : "memory");
+      __syncwarp();
+      return sm.out[warp - 2][blk++ % kOutBufs];
+    };
+    auto send = [&](const CUtensorMap *map, const unsigned char *p, int x, int y) {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) tma_store_2d(map, p, x, y);
+    };
     for (int t = blockIdx.x; t < n_units && ok; t += gridDim.x, ++ti) {
       const int tile = t / sp_n, m0 = (tile / nN) * kBM, n0 = (tile % nN) * BN;
-      const int64_t row = (int64_t(t % sp_n) * M + m0 + lg * 32 + lane) * N + n0;   // this lane's row of its partial
+      const int row0 = (t % sp_n) * M + m0 + lg * 32;   // first row of its partial that this warp holds
       const uint32_t buf = ti & 1u, aph = (ti >> 1) & 1u;
       if (!mbar_wait_bounded(&sm.acc_full[buf], aph)) { ok = false; break; }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
-      for (int c0 = 0; c0 < BN; c0 += 32) {
+      for (int c0 = ch; c0 < ch + kCols; c0 += 32) {
         uint32_t r[32];
         const uint32_t taddr = tmem + (uint32_t(lg * 32) << 16) + buf * kAccCols + uint32_t(c0);
         asm volatile(
@@ -338,7 +326,7 @@ k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
           float4 b4 = make_float4(0.f, 0.f, 0.f, 0.f);
           if (ep.bias) {
             const float *bp = ep.bias + n0 + c0 + i;
-            b4 = ep.vec ? __ldg(reinterpret_cast<const float4 *>(bp)) : make_float4(bp[0], bp[1], bp[2], bp[3]);
+            b4 = ep.tma ? __ldg(reinterpret_cast<const float4 *>(bp)) : make_float4(bp[0], bp[1], bp[2], bp[3]);
           }
           bv[i] = b4.x; bv[i + 1] = b4.y; bv[i + 2] = b4.z; bv[i + 3] = b4.w;
         }
@@ -346,13 +334,52 @@ k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
         float v[32];
 #pragma unroll
         for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]) + bv[i];
-        store_row32(v, ep.z ? ep.z + row + c0 : nullptr, ep.h ? ep.h + row + c0 : nullptr, ep.act, ep.vec);
+        if (ep.z) {
+          if (ep.tma) {   // 128-byte rows, 16-byte chunks swizzled by the row (mod 8)
+            unsigned char *p = stage();
+            const uint32_t at = su32(p) + lane * 128;
+#pragma unroll
+            for (int q = 0; q < 8; ++q)
+              st_shared_v4(at + uint32_t((q ^ (lane & 7)) * 16), __float_as_uint(v[4 * q]), __float_as_uint(v[4 * q + 1]),
+                           __float_as_uint(v[4 * q + 2]), __float_as_uint(v[4 * q + 3]));
+            send(&tmZ, p, n0 + c0, row0);
+          } else {
+            float *z = ep.z + int64_t(row0 + lane) * N + n0 + c0;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) z[i] = v[i];
+          }
+        }
+        if (ep.h) {
+          __nv_bfloat162 hb[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i)
+            hb[i] = ep.act ? __floats2bfloat162_rn(gelu(v[2 * i]), gelu(v[2 * i + 1]))
+                           : __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+          if (ep.tma) {   // 64-byte rows, chunks swizzled by half the row (mod 4)
+            unsigned char *p = stage();
+            const uint32_t at = su32(p) + lane * 64;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const uint32_t *w = reinterpret_cast<const uint32_t *>(&hb[4 * q]);
+              st_shared_v4(at + uint32_t((q ^ ((lane >> 1) & 3)) * 16), w[0], w[1], w[2], w[3]);
+            }
+            send(&tmH, p, n0 + c0, row0);
+          } else {
+            __nv_bfloat16 *h = ep.h + int64_t(row0 + lane) * N + n0 + c0;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              h[2 * i] = hb[i].x;
+              h[2 * i + 1] = hb[i].y;
+            }
+          }
+        }
       }
       // this warp is done with the accumulator
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.acc_empty[buf]);
     }
+    if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // the last stores
   }
   if (!ok && lane == 0) atomicOr(err, 1);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -384,16 +411,18 @@ wproj_status encode_fn(EncodeTiledFn *out) {
   return WPROJ_OK;
 }
 
-// tensor map of a rows x K bf16 row-major matrix, box box_rows x 64 (128 B), 128-byte swizzle
-wproj_status tensor_map(CUtensorMap *map, const __nv_bfloat16 *p, int rows, int K, int box_rows) {
+// tensor map of a rows x cols row-major matrix of `elem` bytes (2: bf16, 4: f32), box of
+// box_rows rows; swizzled by the box's row bytes (128 or 64)
+wproj_status tensor_map(CUtensorMap *map, const void *p, int elem, int64_t rows, int cols, int box_rows, int box_cols) {
   EncodeTiledFn enc = nullptr;
   WPROJ_TRY(encode_fn(&enc));
-  const cuuint64_t dims[2] = {cuuint64_t(K), cuuint64_t(rows)};
-  const cuuint64_t strides[1] = {cuuint64_t(K) * 2};
-  const cuuint32_t box[2] = {cuuint32_t(kBK), cuuint32_t(box_rows)};
+  const cuuint64_t dims[2] = {cuuint64_t(cols), cuuint64_t(rows)};
+  const cuuint64_t strides[1] = {cuuint64_t(cols) * elem};
+  const cuuint32_t box[2] = {cuuint32_t(box_cols), cuuint32_t(box_rows)};
   const cuuint32_t estr[2] = {1, 1};
-  const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<__nv_bfloat16 *>(p), dims, strides, box,
-                         estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+  const CUresult r = enc(map, elem == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
+                         const_cast<void *>(p), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                         box_cols * elem == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) return fail(WPROJ_ERR_CUDA, "gemm: cuTensorMapEncodeTiled failed (" + std::to_string(int(r)) + ")");
   return WPROJ_OK;
@@ -402,13 +431,15 @@ wproj_status tensor_map(CUtensorMap *map, const __nv_bfloat16 *p, int rows, int 
 template <int BN>
 wproj_status launch_gemm(int M, int N, int K, const __nv_bfloat16 *A, const __nv_bfloat16 *B, const EpiArgs &ep, int sms,
                          int *err, cudaStream_t s) {
-  CUtensorMap ta, tb;
-  WPROJ_TRY(tensor_map(&ta, A, M, K, kBM));
-  WPROJ_TRY(tensor_map(&tb, B, N, K, BN));
+  CUtensorMap ta, tb, tz{}, th{};
+  WPROJ_TRY(tensor_map(&ta, A, 2, M, K, kBM, kBK));
+  WPROJ_TRY(tensor_map(&tb, B, 2, N, K, BN, kBK));
+  if (ep.tma && ep.z) WPROJ_TRY(tensor_map(&tz, ep.z, 4, int64_t(M) * ep.splits, N, 32, 32));
+  if (ep.tma && ep.h) WPROJ_TRY(tensor_map(&th, ep.h, 2, M, N, 32, 32));
   const int grid = std::max(1, std::min((M / kBM) * (N / BN) * ep.splits, sms));
   const size_t smem = sizeof(GemmSmem<BN>) + 1024;
   WPROJ_CUDA(cudaFuncSetAttribute(k_gemm_ws<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_gemm_ws<BN><<<grid, kThreads, smem, s>>>(ta, tb, M, N, K, ep, err);
+  k_gemm_ws<BN><<<grid, kThreads, smem, s>>>(ta, tb, tz, th, M, N, K, ep, err);
   WPROJ_CHECK_LAUNCH("gemm");
   return WPROJ_OK;
 }
@@ -451,8 +482,8 @@ wproj_status gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16 *A, const __n
   ep.h = o.bf16;
   ep.act = o.gelu ? 1 : 0;
   ep.splits = o.splits;
-  ep.vec = ((reinterpret_cast<uintptr_t>(o.f32) | reinterpret_cast<uintptr_t>(o.bf16)) & 31) == 0 &&
-           (reinterpret_cast<uintptr_t>(o.bias) & 15) == 0;
+  ep.tma = ((reinterpret_cast<uintptr_t>(o.f32) | reinterpret_cast<uintptr_t>(o.bf16) |
+             reinterpret_cast<uintptr_t>(o.bias)) & 15) == 0;
   if (N % 256 == 0 && (M / kBM) * (N / 256) * (2 * o.splits) > sms)
     return launch_gemm<256>(M, N, K, A, B, ep, sms, err, s);
   return launch_gemm<128>(M, N, K, A, B, ep, sms, err, s);
