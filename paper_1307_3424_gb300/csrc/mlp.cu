@@ -293,6 +293,26 @@ k_sum_rows(int n, int64_t len, const float *__restrict__ in, float *__restrict__
   }
 }
 
+// The same for n <= 8 in 16-byte loads, a thread four elements (len a multiple of 4):
+// six partials of 3072 x 256 took 22 us a word at a time.
+__global__ void __launch_bounds__(256)
+k_sum_few(int n, int64_t len4, const float4 *__restrict__ in, float4 *__restrict__ out) {
+  const int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x;
+  if (i >= len4) return;
+  float4 v[8];
+#pragma unroll
+  for (int p = 0; p < 8; ++p) v[p] = p < n ? __ldcs(in + p * len4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 t = v[0];
+#pragma unroll
+  for (int p = 1; p < 8; ++p) {
+    t.x += v[p].x;
+    t.y += v[p].y;
+    t.z += v[p].z;
+    t.w += v[p].w;
+  }
+  out[i] = t;
+}
+
 // BF16 transposes of the three layers' activations (blockIdx.z), B x kH each
 __global__ void __launch_bounds__(256)
 k_transpose_h(int64_t B, const __nv_bfloat16 *__restrict__ h1, const __nv_bfloat16 *__restrict__ h2,
@@ -369,7 +389,11 @@ __global__ void k_adam(int64_t n, float *__restrict__ P, const float *__restrict
 int blocks_for(int64_t n) { return (int)std::min<int64_t>(152 * 16, std::max<int64_t>(1, ceil_div(n, 256))); }
 
 wproj_status sum_rows(int n, int64_t len, const float *in, float *out, cudaStream_t s) {
-  k_sum_rows<<<ceil_div(len, 32), 256, 0, s>>>(n, len, in, out);
+  if (n <= 8 && len % 4 == 0 && ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0)
+    k_sum_few<<<ceil_div(len / 4, 256), 256, 0, s>>>(n, len / 4, reinterpret_cast<const float4 *>(in),
+                                                     reinterpret_cast<float4 *>(out));
+  else
+    k_sum_rows<<<ceil_div(len, 32), 256, 0, s>>>(n, len, in, out);
   WPROJ_CHECK_LAUNCH("row sums");
   return WPROJ_OK;
 }
