@@ -139,6 +139,11 @@ __global__ void k_chunk_prob(int64_t n, const int32_t *__restrict__ tile_prob, c
 __global__ void __launch_bounds__(kBT)
 k_bs_dual_residual(const BProb *__restrict__ tab, const float2 *__restrict__ u, float2 *__restrict__ r,
                    const float2 *__restrict__ y, const double *__restrict__ mu, double *__restrict__ part) {
+  chain_next();
+  chain_wait();
+  u = after_wait(u);
+  r = after_wait(r);
+  mu = after_wait(mu);
   const BProb P = tab[blockIdx.y];
   __shared__ float inv_mu_s;
   if (threadIdx.x == 0) inv_mu_s = float(1.0 / mu[blockIdx.y]);
@@ -177,6 +182,12 @@ __device__ __forceinline__ float of_problem_sum(const double *__restrict__ part,
 __global__ void __launch_bounds__(kBT)
 k_bs_dual_update(const BProb *__restrict__ tab, const float2 *__restrict__ d, const double *__restrict__ part, int nbx,
                  const double *__restrict__ eps, const double *__restrict__ mu, float2 *__restrict__ u) {
+  chain_next();
+  chain_wait();
+  d = after_wait(d);
+  part = after_wait(part);
+  eps = after_wait(eps);
+  mu = after_wait(mu);
   const BProb P = tab[blockIdx.y];
   const float f = of_problem_sum(part, nbx, [&](double s) {
     const double nd = sqrt(s);
@@ -189,6 +200,11 @@ k_bs_dual_update(const BProb *__restrict__ tab, const float2 *__restrict__ d, co
 // z = z + lambda (soft(2x - z, gamma) - x)
 __global__ void k_bs_dr_update(const BProb *__restrict__ tab, const float *__restrict__ x, float *__restrict__ z,
                                float lambda, const double *__restrict__ scal) {
+  chain_next();
+  chain_wait();
+  x = after_wait(x);
+  z = after_wait(z);
+  scal = after_wait(scal);
   const BProb P = tab[blockIdx.y];
   const float gamma = float(scal[blockIdx.y * kScal + 2]);
   const int64_t n = int64_t(P.N) * P.N;
@@ -205,6 +221,9 @@ __global__ void k_bs_dr_update(const BProb *__restrict__ tab, const float *__res
 template <int MODE>
 __global__ void __launch_bounds__(kBT)
 k_bs_image_part(const BProb *__restrict__ tab, const float *__restrict__ x, double *__restrict__ part) {
+  chain_next();
+  chain_wait();
+  x = after_wait(x);
   const BProb P = tab[blockIdx.y];
   const int64_t n = int64_t(P.N) * P.N;
   double acc = 0;
@@ -244,6 +263,10 @@ __global__ void k_bs_gamma(int np, int nbx, const double *__restrict__ part, dou
 __global__ void __launch_bounds__(kBT)
 k_bs_scale_image(const BProb *__restrict__ tab, const float *__restrict__ z, const double *__restrict__ part, int nbx,
                  double *__restrict__ scal, float *__restrict__ x) {
+  chain_next();
+  chain_wait();
+  z = after_wait(z);
+  part = after_wait(part);
   const BProb P = tab[blockIdx.y];
   const int64_t n = int64_t(P.N) * P.N;
   float f = 0.f;
@@ -420,8 +443,10 @@ wproj_status dr_iteration(wproj_batch *b, const float2 *y, int inner, float lamb
   for (int j = 0; j < inner; ++j) {
     WPROJ_TRY(bphi_adj(b, u, x, z, 1, s));   // x = z - Re Phi^H u
     WPROJ_TRY(bphi(b, x, r, s));             // r = Phi x
-    k_bs_dual_residual<<<dim3(nbm, b->np), kBT, 0, s>>>(tab, u, r, y, b->mu.as<double>(), part);
-    k_bs_dual_update<<<dim3(nbm, b->np), kBT, 0, s>>>(tab, r, part, nbm, b->eps.as<double>(), b->mu.as<double>(), u);
+    const dim3 gm(nbm, b->np);
+    WPROJ_CUDA(launch_chained(k_bs_dual_residual, gm, kBT, 0, s, tab, u, r, y, b->mu.as<double>(), part));
+    WPROJ_CUDA(launch_chained(k_bs_dual_update, gm, kBT, 0, s, tab, r, part, nbm, b->eps.as<double>(),
+                              b->mu.as<double>(), u));
     WPROJ_CHECK_LAUNCH("batch dual step");
     b->launches += 2;
   }
@@ -431,7 +456,7 @@ wproj_status dr_iteration(wproj_batch *b, const float2 *y, int inner, float lamb
     px = b->alpha.as<float>();
     WPROJ_TRY(batch_dwt2(tab, b->np, b->max_n, levels, psi, x, px, b->wwork.as<float>(), &b->launches, s));
   }
-  k_bs_dr_update<<<dim3(nbn, b->np), kBT, 0, s>>>(tab, px, zc, lambda, scal);
+  WPROJ_CUDA(launch_chained(k_bs_dr_update, dim3(nbn, b->np), kBT, 0, s, tab, px, zc, lambda, scal));
   WPROJ_CHECK_LAUNCH("batch dr update");
   b->launches += 1;
   return WPROJ_OK;
@@ -449,8 +474,8 @@ wproj_status power_mu(wproj_batch *b, int iters, cudaStream_t s) {
   for (int it = 0; it < iters; ++it) {
     WPROJ_TRY(bphi(b, x, r, s));
     WPROJ_TRY(bphi_adj(b, r, z, nullptr, 0, s));
-    k_bs_image_part<1><<<dim3(nbn, b->np), kBT, 0, s>>>(tab, z, part);
-    k_bs_scale_image<<<dim3(nbn, b->np), kBT, 0, s>>>(tab, z, part, nbn, scal, x);
+    WPROJ_CUDA(launch_chained(k_bs_image_part<1>, dim3(nbn, b->np), kBT, 0, s, tab, z, part));
+    WPROJ_CUDA(launch_chained(k_bs_scale_image, dim3(nbn, b->np), kBT, 0, s, tab, z, part, nbn, scal, x));
     WPROJ_CHECK_LAUNCH("batch power iteration");
   }
   k_bs_mu<<<ceil_div(b->np, 128), 128, 0, s>>>(b->np, scal, b->mu.as<double>());

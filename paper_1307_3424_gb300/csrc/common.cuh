@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 
 #include "wproj.h"
 
@@ -80,6 +81,25 @@ __device__ __forceinline__ double block_sum_d(double v) {
   return t;
 }
 
+// ---- chained launches ----------------------------------------------------------
+// The kernels of an operator or a solver step are launched (launch_chained) so that
+// the next one's blocks start once this one's have all started, set up what does not
+// depend on it and wait for it there.  The first kernel of a chain waits before it
+// calls chain_next, so whatever ran before the chain (a build, a copy) is complete
+// when a later kernel reads the plan ahead of its wait.  Every chained kernel waits,
+// in all threads and before it returns or writes; data of earlier kernels is read
+// through pointers from after_wait only, so that no load can move above the wait or
+// take the non-coherent path.  Measured without and with: a pair on a 128^2 grid (8
+// launches) 89 and 74 us, a reconstruction of it 62.5 and 50.7 ms, a batch of 64
+// problems 521 and 500 us, the 14 ms pair of dense rows the same.
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class T> __device__ __forceinline__ T *after_wait(T *p) {
+  asm volatile("" : "+l"(p)::"memory");
+  __builtin_assume(__isGlobal(p));
+  return p;
+}
+
 // ---- error state ------------------------------------------------------------
 void set_error(const std::string &msg);
 wproj_status fail(wproj_status st, const std::string &msg);
@@ -102,6 +122,21 @@ wproj_status cuda_fail(cudaError_t err, const char *what);
     wproj_status st__ = (expr);                             \
     if (st__ != WPROJ_OK) return st__;                      \
   } while (0)
+
+template <class... P, class... A>
+cudaError_t launch_chained(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A &&...a) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, k, std::forward<A>(a)...);
+}
 
 inline int ceil_div(int64_t a, int64_t b) { return (int)((a + b - 1) / b); }
 inline int ilog2(int64_t n) { int l = 0; while ((int64_t(1) << l) < n) ++l; return l; }

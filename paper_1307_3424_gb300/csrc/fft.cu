@@ -75,7 +75,9 @@ template <int LOGN>
 __global__ void __launch_bounds__(RowCfg<LOGN>::T)
 k_phi_fwd_rows(const float *__restrict__ x, const float2 *__restrict__ xc, const float *__restrict__ inv_a, int N,
                float2 *__restrict__ inter, const float2 *__restrict__ tw) {
-  phi_fwd_rows_body<LOGN, RowCfg<LOGN>>(x, xc, inv_a, N, inter, tw, blockIdx.x);
+  chain_wait();
+  chain_next();
+  phi_fwd_rows_body<LOGN, RowCfg<LOGN>>(after_wait(x), after_wait(xc), inv_a, N, inter, tw, blockIdx.x);
 }
 
 template <int LOGN>
@@ -110,7 +112,9 @@ template <int LOGN>
 __global__ void __launch_bounds__(ColCfg<LOGN>::T)
 k_phi_fwd_cols(const float2 *__restrict__ inter, int N, float2 *__restrict__ Xt, float scale,
                const float2 *__restrict__ tw) {
-  phi_fwd_cols_body<LOGN, ColCfg<LOGN>>(inter, N, Xt, scale, tw, blockIdx.x);
+  chain_next();
+  chain_wait();
+  phi_fwd_cols_body<LOGN, ColCfg<LOGN>>(after_wait(inter), N, Xt, scale, tw, blockIdx.x);
 }
 
 template <int LOGN>
@@ -144,7 +148,9 @@ __device__ __forceinline__ void phi_adj_cols_body(const float2 *__restrict__ Xt2
 template <int LOGN>
 __global__ void __launch_bounds__(ColCfg<LOGN>::T)
 k_phi_adj_cols(const float2 *__restrict__ Xt2, int N, float2 *__restrict__ inter, const float2 *__restrict__ tw) {
-  phi_adj_cols_body<LOGN, ColCfg<LOGN>>(Xt2, N, inter, tw, blockIdx.x);
+  chain_next();
+  chain_wait();
+  phi_adj_cols_body<LOGN, ColCfg<LOGN>>(after_wait(Xt2), N, inter, tw, blockIdx.x);
 }
 
 template <int LOGN>
@@ -192,7 +198,9 @@ __global__ void __launch_bounds__(RowCfg<LOGN>::T)
 k_phi_adj_rows(const float2 *__restrict__ inter, const float *__restrict__ inv_a, int N, float scale,
                float *__restrict__ x_re, float2 *__restrict__ x_c, const float *__restrict__ z, int mode,
                const float2 *__restrict__ tw) {
-  phi_adj_rows_body<LOGN, RowCfg<LOGN>>(inter, inv_a, N, scale, x_re, x_c, z, mode, tw, blockIdx.x);
+  chain_next();
+  chain_wait();
+  phi_adj_rows_body<LOGN, RowCfg<LOGN>>(after_wait(inter), inv_a, N, scale, x_re, x_c, after_wait(z), mode, tw, blockIdx.x);
 }
 
 template <int LOGN>
@@ -234,6 +242,9 @@ __global__ void __launch_bounds__(256, 3)
 k_bphi_fwd_rows_all(const FftClasses cl, const BProb *__restrict__ tab, const float *__restrict__ x,
                     const float *__restrict__ inv_a, float2 *__restrict__ inter, const float2 *__restrict__ tw) {
   int prob, blk;
+  chain_wait();
+  chain_next();
+  x = after_wait(x);
   const int lg = class_block(cl, prob, blk);
   const BProb P = tab[prob];
 #define CALL(L) phi_fwd_rows_body<L, BatchRowCfg<L>>(x + P.img_off, nullptr, inv_a + P.inva_off, P.N, inter + P.inter_off, tw, blk)
@@ -244,8 +255,11 @@ __global__ void __launch_bounds__(256, 3)
 k_bphi_fwd_cols_all(const FftClasses cl, const BProb *__restrict__ tab, const float2 *__restrict__ inter,
                     float2 *__restrict__ Xt, const float2 *__restrict__ tw) {
   int prob, blk;
+  chain_next();
   const int lg = class_block(cl, prob, blk);
   const BProb P = tab[prob];
+  chain_wait();
+  inter = after_wait(inter);
 #define CALL(L) phi_fwd_cols_body<L, BatchColCfg<L>>(inter + P.inter_off, P.N, Xt + P.grid_off, 1.0f / P.G, tw, blk)
   WPROJ_BATCH_LOGN(lg, CALL)
 #undef CALL
@@ -254,8 +268,11 @@ __global__ void __launch_bounds__(256, 3)
 k_bphi_adj_cols_all(const FftClasses cl, const BProb *__restrict__ tab, const float2 *__restrict__ Xt2,
                     float2 *__restrict__ inter, const float2 *__restrict__ tw) {
   int prob, blk;
+  chain_next();
   const int lg = class_block(cl, prob, blk);
   const BProb P = tab[prob];
+  chain_wait();
+  Xt2 = after_wait(Xt2);
 #define CALL(L) phi_adj_cols_body<L, BatchColCfg<L>>(Xt2 + P.grid_off, P.N, inter + P.inter_off, tw, blk)
   WPROJ_BATCH_LOGN(lg, CALL)
 #undef CALL
@@ -265,8 +282,12 @@ k_bphi_adj_rows_all(const FftClasses cl, const BProb *__restrict__ tab, const fl
                     const float *__restrict__ inv_a, float *__restrict__ x_re, const float *__restrict__ z, int mode,
                     const float2 *__restrict__ tw) {
   int prob, blk;
+  chain_next();
   const int lg = class_block(cl, prob, blk);
   const BProb P = tab[prob];
+  chain_wait();
+  inter = after_wait(inter);
+  z = after_wait(z);
 #define CALL(L)                                                                                                  \
   phi_adj_rows_body<L, BatchRowCfg<L>>(inter + P.inter_off, inv_a + P.inva_off, P.N, 1.0f / P.G, x_re + P.img_off, \
                                        nullptr, z ? z + P.img_off : nullptr, mode, tw, blk)
@@ -435,13 +456,14 @@ wproj_status phi_fwd_impl(wproj_plan *p, const float *x, const float2 *xc, float
   {
     using Cfg = RowCfg<LOGN>;
     WPROJ_TRY(set_smem(k_phi_fwd_rows<LOGN>, Cfg::SMEM));
-    k_phi_fwd_rows<LOGN><<<ceil_div(N, Cfg::C), Cfg::T, Cfg::SMEM, s>>>(x, xc, p->inv_a.as<float>(), N, inter, tw);
+    WPROJ_CUDA(launch_chained(k_phi_fwd_rows<LOGN>, ceil_div(N, Cfg::C), Cfg::T, Cfg::SMEM, s, x, xc,
+                              p->inv_a.as<float>(), N, inter, tw));
     WPROJ_CHECK_LAUNCH("phi fwd rows");
   }
   {
     using Cfg = ColCfg<LOGN>;
     WPROJ_TRY(set_smem(k_phi_fwd_cols<LOGN>, Cfg::SMEM));
-    k_phi_fwd_cols<LOGN><<<ceil_div(G, Cfg::C), Cfg::T, Cfg::SMEM, s>>>(inter, N, Xt, 1.0f / G, tw);
+    WPROJ_CUDA(launch_chained(k_phi_fwd_cols<LOGN>, ceil_div(G, Cfg::C), Cfg::T, Cfg::SMEM, s, inter, N, Xt, 1.0f / G, tw));
     WPROJ_CHECK_LAUNCH("phi fwd cols");
   }
   return WPROJ_OK;
@@ -455,13 +477,14 @@ wproj_status phi_fwd_into_impl(wproj_plan *p, const float *x, float2 *inter, flo
   {
     using Cfg = RowCfg<LOGN>;
     WPROJ_TRY(set_smem(k_phi_fwd_rows<LOGN>, Cfg::SMEM));
-    k_phi_fwd_rows<LOGN><<<ceil_div(N, Cfg::C), Cfg::T, Cfg::SMEM, s>>>(x, nullptr, p->inv_a.as<float>(), N, inter, tw);
+    WPROJ_CUDA(launch_chained(k_phi_fwd_rows<LOGN>, ceil_div(N, Cfg::C), Cfg::T, Cfg::SMEM, s, x, nullptr,
+                              p->inv_a.as<float>(), N, inter, tw));
     WPROJ_CHECK_LAUNCH("phi fwd rows");
   }
   {
     using Cfg = ColCfg<LOGN>;
     WPROJ_TRY(set_smem(k_phi_fwd_cols<LOGN>, Cfg::SMEM));
-    k_phi_fwd_cols<LOGN><<<ceil_div(G, Cfg::C), Cfg::T, Cfg::SMEM, s>>>(inter, N, Xt, 1.0f / G, tw);
+    WPROJ_CUDA(launch_chained(k_phi_fwd_cols<LOGN>, ceil_div(G, Cfg::C), Cfg::T, Cfg::SMEM, s, inter, N, Xt, 1.0f / G, tw));
     WPROJ_CHECK_LAUNCH("phi fwd cols");
   }
   return WPROJ_OK;
@@ -476,14 +499,14 @@ wproj_status phi_adj_impl(wproj_plan *p, const float2 *Xt2, float *x_re, float2 
   {
     using Cfg = ColCfg<LOGN>;
     WPROJ_TRY(set_smem(k_phi_adj_cols<LOGN>, Cfg::SMEM));
-    k_phi_adj_cols<LOGN><<<ceil_div(G, Cfg::C), Cfg::T, Cfg::SMEM, s>>>(Xt2, N, inter, tw);
+    WPROJ_CUDA(launch_chained(k_phi_adj_cols<LOGN>, ceil_div(G, Cfg::C), Cfg::T, Cfg::SMEM, s, Xt2, N, inter, tw));
     WPROJ_CHECK_LAUNCH("phi adj cols");
   }
   {
     using Cfg = RowCfg<LOGN>;
     WPROJ_TRY(set_smem(k_phi_adj_rows<LOGN>, Cfg::SMEM));
-    k_phi_adj_rows<LOGN><<<ceil_div(N, Cfg::C), Cfg::T, Cfg::SMEM, s>>>(
-        inter, p->inv_a.as<float>(), N, 1.0f / G, x_re, x_c, z, mode, tw);
+    WPROJ_CUDA(launch_chained(k_phi_adj_rows<LOGN>, ceil_div(N, Cfg::C), Cfg::T, Cfg::SMEM, s, inter,
+                              p->inv_a.as<float>(), N, 1.0f / G, x_re, x_c, z, mode, tw));
     WPROJ_CHECK_LAUNCH("phi adj rows");
   }
   return WPROJ_OK;
@@ -719,10 +742,10 @@ wproj_status batch_phi_fwd_all(FftClasses cl, const BProb *tab, const float *x, 
                                float2 *Xt, const float2 *tw, cudaStream_t s) {
   size_t smem = 0;
   int n = batch_blocks<BatchRowCfg>(cl, true, &smem);
-  k_bphi_fwd_rows_all<<<n, 256, smem, s>>>(cl, tab, x, inv_a, inter, tw);
+  WPROJ_CUDA(launch_chained(k_bphi_fwd_rows_all, n, 256, smem, s, cl, tab, x, inv_a, inter, tw));
   smem = 0;
   n = batch_blocks<BatchColCfg>(cl, false, &smem);
-  k_bphi_fwd_cols_all<<<n, 256, smem, s>>>(cl, tab, inter, Xt, tw);
+  WPROJ_CUDA(launch_chained(k_bphi_fwd_cols_all, n, 256, smem, s, cl, tab, inter, Xt, tw));
   WPROJ_CHECK_LAUNCH("batch phi fwd");
   return WPROJ_OK;
 }
@@ -730,10 +753,10 @@ wproj_status batch_phi_adj_all(FftClasses cl, const BProb *tab, const float2 *Xt
                                float *x_re, const float *z, int mode, const float2 *tw, cudaStream_t s) {
   size_t smem = 0;
   int n = batch_blocks<BatchColCfg>(cl, false, &smem);
-  k_bphi_adj_cols_all<<<n, 256, smem, s>>>(cl, tab, Xt2, inter, tw);
+  WPROJ_CUDA(launch_chained(k_bphi_adj_cols_all, n, 256, smem, s, cl, tab, Xt2, inter, tw));
   smem = 0;
   n = batch_blocks<BatchRowCfg>(cl, true, &smem);
-  k_bphi_adj_rows_all<<<n, 256, smem, s>>>(cl, tab, inter, inv_a, x_re, z, mode, tw);
+  WPROJ_CUDA(launch_chained(k_bphi_adj_rows_all, n, 256, smem, s, cl, tab, inter, inv_a, x_re, z, mode, tw));
   WPROJ_CHECK_LAUNCH("batch phi adj");
   return WPROJ_OK;
 }

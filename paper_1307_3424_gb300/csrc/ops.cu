@@ -250,6 +250,7 @@ __global__ void __launch_bounds__(32 * kRedLanes)
 k_grid_reduce(const int32_t *__restrict__ tile_chunk_ptr, const float2 *__restrict__ partial, int G, int TS, int nT,
               const int32_t *__restrict__ tile_prob, const BProb *__restrict__ tab, float2 *__restrict__ Xt2) {
   __shared__ float2 red[kRedLanes][32];
+  chain_next();
   int tile = blockIdx.x;
   const int c0 = tile_chunk_ptr[tile], c1 = tile_chunk_ptr[tile + 1];
   const int stride = TS * TS;
@@ -263,6 +264,8 @@ k_grid_reduce(const int32_t *__restrict__ tile_chunk_ptr, const float2 *__restri
   }
   const int tu = tile / nT, tv = tile % nT;
   const int i = blockIdx.y * 32 + (threadIdx.x & 31), j = threadIdx.x >> 5;   // TS * TS is a multiple of 32
+  chain_wait();
+  partial = after_wait(partial);
   if (blockIdx.y * 32 >= TS * TS) return;
   float2 s = make_float2(0.f, 0.f);
 #pragma unroll 4
@@ -375,8 +378,9 @@ wproj_status grid(wproj_plan *p, const float2 *y, float2 *Xt2, cudaStream_t s) {
     WPROJ_CHECK_LAUNCH("grid");
   }
   ScopedTimer t(p, TC_REDUCE, s);
-  k_grid_reduce<<<dim3(g.nT * g.nT, g.tile * g.tile / 32), 32 * kRedLanes, 0, s>>>(
-      p->tile_chunk_ptr.as<int32_t>(), p->grid_partial.as<float2>(), g.G, g.tile, g.nT, nullptr, nullptr, Xt2);
+  WPROJ_CUDA(launch_chained(k_grid_reduce, dim3(g.nT * g.nT, g.tile * g.tile / 32), 32 * kRedLanes, 0, s,
+                            p->tile_chunk_ptr.as<int32_t>(), p->grid_partial.as<float2>(), g.G, g.tile, g.nT, nullptr,
+                            nullptr, Xt2));
   WPROJ_CHECK_LAUNCH("grid reduce");
   return WPROJ_OK;
 }

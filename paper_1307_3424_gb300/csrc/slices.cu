@@ -91,7 +91,10 @@ k_slice_degrid(const SliceOps o, const float2 *__restrict__ X, float2 *__restric
   using Raw = typename RawVal<VDT>::type;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = blockIdx.x;
   const int64_t s0 = o.d_slice_base[c], s1 = o.d_slice_base[c + 1];
-  if (s0 >= s1) return;
+  if (s0 >= s1) {
+    chain_wait();
+    return;
+  }
   const int4 r = o.rect[c];
   int logG = o.logG;
   if (o.tab) {
@@ -107,10 +110,6 @@ k_slice_degrid(const SliceOps o, const float2 *__restrict__ X, float2 *__restric
     prefetch_l2(val + a, n * int(sizeof(Raw)));
     prefetch_l2(o.d_idx + a, n * 2);
   }
-  for (int a = w; a < r.z; a += kWarps) {
-    const float2 *row = X + (int64_t((r.x + a) & Gm) << logG);
-    for (int b = lane; b < r.w; b += 32) cp_async8(&sh[1 + a * ws + b], row + ((r.y + b) & Gm));
-  }
   // lane t holds the bounds of the warp's slice t (of each 32)
   long long pl = 0;
   int nl = 0;
@@ -122,6 +121,12 @@ k_slice_degrid(const SliceOps o, const float2 *__restrict__ X, float2 *__restric
     }
   };
   bounds(s0 + w + int64_t(lane) * kWarps);
+  chain_wait();
+  X = after_wait(X);
+  for (int a = w; a < r.z; a += kWarps) {
+    const float2 *row = X + (int64_t((r.x + a) & Gm) << logG);
+    for (int b = lane; b < r.w; b += 32) cp_async8(&sh[1 + a * ws + b], row + ((r.y + b) & Gm));
+  }
   Raw v[U], vn[U];
   uint16_t id[U], idn[U];
   auto load = [&](long long p, int n, int j, Raw(&a)[U], uint16_t(&b)[U]) {
@@ -143,6 +148,7 @@ k_slice_degrid(const SliceOps o, const float2 *__restrict__ X, float2 *__restric
   load(p0, n0, 0, v, id);
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
+  chain_next();
   int t = 0;
   for (int64_t s = s0 + w; s < s1; s += kWarps) {
     // the next slice
@@ -199,6 +205,8 @@ k_slice_grid(const SliceOps o, const float2 *__restrict__ y, float2 *__restrict_
   __shared__ float2 cell[1024];
   using Raw = typename RawVal<VDT>::type;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, c = blockIdx.x;
+  chain_wait();   // the first kernel of Phi^H
+  y = after_wait(y);
   // The slices are sorted by length: the warps take them to and fro, four each, step
   // by step together, so that tiles of a few entries a cell still have loads in
   // flight.  The first steps are asked for before the y are gathered.
@@ -239,7 +247,7 @@ k_slice_grid(const SliceOps o, const float2 *__restrict__ y, float2 *__restrict_
   if (threadIdx.x == 0) sh[0] = make_float2(0.f, 0.f);
   for (int i = threadIdx.x; i < nrow; i += kThreads) {
     const int k = __ldg(o.g_rows + rb + i);
-    float2 t = __ldg(y + k);
+    float2 t = y[k];
     if (o.row_scale) t = cscale(t, __ldg(o.row_scale + k));
     sh[1 + i] = t;
   }
@@ -272,6 +280,7 @@ k_slice_grid(const SliceOps o, const float2 *__restrict__ y, float2 *__restrict_
     const int sl = q * kWarps + ((q & 1) ? kWarps - 1 - w : w);
     cell[__ldg(o.g_perm + int64_t(c) * 1024 + sl * 32 + lane)] = acc[q];
   }
+  chain_next();
   __syncthreads();
   int tile = o.g_chunk_tile[c], logG = o.logG, t0 = 0;
   if (o.tab) {
@@ -293,6 +302,7 @@ k_slice_grid(const SliceOps o, const float2 *__restrict__ y, float2 *__restrict_
 __global__ void __launch_bounds__(256)
 k_slice_reduce(const SliceOps o, const float2 *__restrict__ partial, float2 *__restrict__ Xt2) {
   __shared__ float2 red[8][32];
+  chain_next();
   int tile = o.multi[blockIdx.x], logG = o.logG;
   const int c0 = o.tile_chunk_ptr[tile], c1 = o.tile_chunk_ptr[tile + 1];
   if (o.tab) {
@@ -302,6 +312,8 @@ k_slice_reduce(const SliceOps o, const float2 *__restrict__ partial, float2 *__r
     Xt2 += P.grid_off;
   }
   const int e = blockIdx.y * 32 + (threadIdx.x & 31), j = threadIdx.x >> 5;
+  chain_wait();
+  partial = after_wait(partial);
   float2 s = make_float2(0.f, 0.f);
 #pragma unroll 4
   for (int c = c0 + j; c < c1; c += 8) s = cadd(s, partial[int64_t(c) * 1024 + e]);
@@ -616,17 +628,17 @@ template <int VDT>
 wproj_status launch_degrid(const SliceOps &o, size_t smem, const float2 *X, float2 *y, cudaStream_t s) {
   constexpr int U = VDT == WPROJ_VAL_F32 ? 6 : 8;   // steps per group (two groups in registers)
   WPROJ_CUDA(cudaFuncSetAttribute(k_slice_degrid<VDT, U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_slice_degrid<VDT, U><<<(unsigned)o.d_chunks, kThreads, smem, s>>>(o, X, y);
+  WPROJ_CUDA(launch_chained(k_slice_degrid<VDT, U>, (unsigned)o.d_chunks, kThreads, smem, s, o, X, y));
   WPROJ_CHECK_LAUNCH("degrid (slices)");
   return WPROJ_OK;
 }
 template <int VDT>
 wproj_status launch_grid(const SliceOps &o, size_t smem, const float2 *y, float2 *partial, float2 *Xt2, cudaStream_t s) {
   WPROJ_CUDA(cudaFuncSetAttribute(k_slice_grid<VDT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_slice_grid<VDT><<<(unsigned)o.g_chunks, kThreads, smem, s>>>(o, y, partial, Xt2);
+  WPROJ_CUDA(launch_chained(k_slice_grid<VDT>, (unsigned)o.g_chunks, kThreads, smem, s, o, y, partial, Xt2));
   WPROJ_CHECK_LAUNCH("grid (slices)");
   if (o.n_multi > 0) {
-    k_slice_reduce<<<dim3((unsigned)o.n_multi, 32), 256, 0, s>>>(o, partial, Xt2);
+    WPROJ_CUDA(launch_chained(k_slice_reduce, dim3((unsigned)o.n_multi, 32), 256, 0, s, o, partial, Xt2));
     WPROJ_CHECK_LAUNCH("grid (slices) partial tiles");
   }
   return WPROJ_OK;

@@ -26,6 +26,10 @@ constexpr int kRedBlocks = 304;   // 2 x 152 SMs
 __global__ void __launch_bounds__(kRedThreads)
 k_dual_residual(int64_t m, const float2 *__restrict__ u, float2 *__restrict__ r,
                 const float2 *__restrict__ y, float inv_mu, double *__restrict__ part) {
+  chain_next();
+  chain_wait();
+  u = after_wait(u);
+  r = after_wait(r);
   double acc = 0;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < m; i += int64_t(gridDim.x) * blockDim.x) {
     const float2 uu = u[i], rr = r[i], yy = y[i];
@@ -56,6 +60,10 @@ __device__ __forceinline__ float of_sum(const double *__restrict__ part, int n, 
 __global__ void __launch_bounds__(kRedThreads)
 k_dual_update(int64_t m, const float2 *__restrict__ d, const double *__restrict__ part, int n, double eps, double mu,
               float2 *__restrict__ u) {
+  chain_next();
+  chain_wait();
+  d = after_wait(d);
+  part = after_wait(part);
   const float f = of_sum(part, n, [&](double s) {
     const double nd = sqrt(s);
     return float(((nd > 0) ? fmax(0.0, 1.0 - eps / nd) : 0.0) * mu);
@@ -67,6 +75,11 @@ k_dual_update(int64_t m, const float2 *__restrict__ d, const double *__restrict_
 // z = z + lambda (soft(2x - z, gamma) - x), gamma = scal[2]
 __global__ void k_dr_update(int64_t n, const float *__restrict__ x, float *__restrict__ z, float lambda,
                             const double *__restrict__ scal) {
+  chain_next();
+  chain_wait();
+  x = after_wait(x);
+  z = after_wait(z);
+  scal = after_wait(scal);
   const float gamma = float(scal[2]);
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
     const float xi = x[i], zi = z[i];
@@ -103,6 +116,9 @@ __global__ void k_gamma(const double *__restrict__ part, int n, double frac, dou
 template <int ABS>
 __global__ void __launch_bounds__(kRedThreads)
 k_sum_part(int64_t n, const float *__restrict__ x, double *__restrict__ part) {
+  chain_next();
+  chain_wait();
+  x = after_wait(x);
   double acc = 0;
   for (int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += int64_t(gridDim.x) * blockDim.x) {
     const double v = x[i];
@@ -135,6 +151,10 @@ k_sum_parts(const double *__restrict__ part, int n, double *__restrict__ out) {
 __global__ void __launch_bounds__(kRedThreads)
 k_normalise(int64_t n, const float *__restrict__ z, const double *__restrict__ part, int nb, double *__restrict__ sum,
             float *__restrict__ x) {
+  chain_next();
+  chain_wait();
+  z = after_wait(z);
+  part = after_wait(part);
   const float f = of_sum(part, nb, [&](double s) {
     if (blockIdx.x == 0) *sum = s;
     return float(1.0 / sqrt(s));
@@ -180,8 +200,8 @@ wproj_status power_norm2_impl(wproj_plan *p, int iters, double *out, cudaStream_
     WPROJ_TRY(apply_phi(p, x, nullptr, r, s));
     WPROJ_TRY(apply_phi_adj(p, r, z, nullptr, nullptr, 0, s));
     const int nb = grid_for(n);
-    k_sum_part<0><<<nb, kRedThreads, 0, s>>>(n, z, part);
-    k_normalise<<<nb, kRedThreads, 0, s>>>(n, z, part, nb, scal + 3, x);
+    WPROJ_CUDA(launch_chained(k_sum_part<0>, nb, kRedThreads, 0, s, n, z, part));
+    WPROJ_CUDA(launch_chained(k_normalise, nb, kRedThreads, 0, s, n, z, part, nb, scal + 3, x));
     WPROJ_CHECK_LAUNCH("power iteration");
     p->launches += 2;
   }
@@ -246,15 +266,15 @@ wproj_status solve_bpdn_impl(wproj_plan *p, const float2 *y, double eps, const w
       WPROJ_TRY(apply_phi_adj(p, u, x, nullptr, zi, 1, s));   // x = zi - Re Phi^H u
       WPROJ_TRY(apply_phi(p, x, nullptr, r, s));               // r = Phi x
       ScopedTimer t(p, TC_SOLVER, s);
-      k_dual_residual<<<nbm, kRedThreads, 0, s>>>(m, u, r, y, float(1.0 / mu), part);
-      k_dual_update<<<nbm, kRedThreads, 0, s>>>(m, r, part, nbm, eps, mu, u);
+      WPROJ_CUDA(launch_chained(k_dual_residual, nbm, kRedThreads, 0, s, m, u, r, y, float(1.0 / mu), part));
+      WPROJ_CUDA(launch_chained(k_dual_update, nbm, kRedThreads, 0, s, m, r, part, nbm, eps, mu, u));
       WPROJ_CHECK_LAUNCH("dual step");
       p->launches += 2;
     }
     WPROJ_TRY(apply_phi_adj(p, u, x, nullptr, zi, 1, s));     // x = P_B(zi)
     if (psi) WPROJ_TRY(dwt2_impl(N, lev, psi, x, alpha, wk, &p->launches, s));
     ScopedTimer t(p, TC_SOLVER, s);
-    k_dr_update<<<nbn, kRedThreads, 0, s>>>(n, alpha, z, float(prm.lambda), scal);
+    WPROJ_CUDA(launch_chained(k_dr_update, nbn, kRedThreads, 0, s, n, alpha, z, float(prm.lambda), scal));
     WPROJ_CHECK_LAUNCH("dr update");
     p->launches += 1;
   }

@@ -137,3 +137,60 @@ def test_small_boxes(wp, N, e, W, wmax):
     plan.build_kernels(torch.from_numpy(uvw).cuda(), e)
     check_build(plan, O.Geometry(N, L, W=W), uvw, e, "rule")
     plan.close()
+
+# passes launched one behind the other (blocks of a kernel start before the one ahead
+# has ended) against the same passes each waited for, bit for bit: inputs overwritten
+# right before and after a pass, eager and as a captured graph with copies between;
+# dense rows with and without partial tiles, short rows, a batch
+@pytest.mark.parametrize("N,M,box,value", [(64, 500, "G", "f32"), (32, 20, "G", "bf16"), (256, 3000, "rule", "f32"),
+                                           (128, 900, "rule", "f16"), (0, 0, "batch", "f32")])
+def test_back_to_back_passes(wp, N, M, box, value):
+    rng = np.random.default_rng(N + M)
+    if box == "batch":
+        ns = (64, 128, 32)
+        op = wp.Batch(ns, L)
+        op.build_kernels(torch.from_numpy(np.concatenate([uvw_cells(rng, 9 * n, n, 1.0) for n in ns])).cuda(),
+                         [9 * n for n in ns], 0.99)
+        x = torch.empty(op.pixels, dtype=torch.float32, device="cuda")
+    else:
+        op = wp.Plan(N, L, box=box, value_dtype=value)
+        op.build_kernels(torch.from_numpy(uvw_cells(rng, M, N, 20.0 if box == "G" else 2.0)).cuda(), 0.99)
+        x = torch.empty((N, N), dtype=torch.float32, device="cuda")
+    xs = torch.from_numpy(rng.standard_normal((4,) + tuple(x.shape)).astype(np.float32)).cuda()
+    y = torch.empty(op.m, dtype=torch.complex64, device="cuda")
+    z = torch.empty_like(x)
+    out = torch.empty((8,) + tuple(x.shape), dtype=torch.float32, device="cuda")
+    yo = torch.empty((8, op.m), dtype=torch.complex64, device="cuda")
+
+    def passes(wait):
+        for i in range(8):
+            x.copy_(xs[i % 4])
+            for step in range(3):      # Phi and Phi^H of each other's results
+                op.phi(x, y)
+                wait()
+                op.phi_adj(y, z)
+                wait()
+                x.copy_(z) if step == 1 else x.add_(z, alpha=0.5)
+                wait()
+            yo[i].copy_(y)
+            y.zero_()
+            out[i].copy_(z)
+
+    passes(torch.cuda.synchronize)
+    torch.cuda.synchronize()
+    want, wanty = out.clone(), yo.clone()
+    out.zero_()
+    yo.zero_()
+    passes(lambda: None)
+    torch.cuda.synchronize()
+    assert torch.equal(out, want) and torch.equal(yo, wanty)
+    out.zero_()
+    yo.zero_()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        passes(lambda: None)
+    for _ in range(2):
+        g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, want) and torch.equal(yo, wanty)
+    op.close()
