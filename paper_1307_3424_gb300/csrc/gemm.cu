@@ -215,6 +215,7 @@ k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = sm.tmem_base;
+  chain_wait();
   bool ok = true;
   if (g_gemm_unset_wait) ok = mbar_wait_bounded(&sm.never, 0, g_gemm_wait_ns);
 
@@ -381,6 +382,7 @@ k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
     }
     if (lane == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");   // the last stores
   }
+  chain_next();
   if (!ok && lane == 0) atomicOr(err, 1);
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -439,8 +441,7 @@ wproj_status launch_gemm(int M, int N, int K, const __nv_bfloat16 *A, const __nv
   const int grid = std::max(1, std::min((M / kBM) * (N / BN) * ep.splits, sms));
   const size_t smem = sizeof(GemmSmem<BN>) + 1024;
   WPROJ_CUDA(cudaFuncSetAttribute(k_gemm_ws<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  k_gemm_ws<BN><<<grid, kThreads, smem, s>>>(ta, tb, tz, th, M, N, K, ep, err);
-  WPROJ_CHECK_LAUNCH("gemm");
+  WPROJ_CUDA(launch_chained(k_gemm_ws<BN>, grid, kThreads, smem, s, ta, tb, tz, th, M, N, K, ep, err));
   return WPROJ_OK;
 }
 

@@ -62,6 +62,10 @@ __global__ void __launch_bounds__(kH / 2)
 k_in_fwd(int64_t B, const float *__restrict__ x0, const float *__restrict__ P, float *__restrict__ Z1,
          __nv_bfloat16 *__restrict__ H1) {
   __shared__ float xs[kInRows * kIn];
+  chain_wait();   // the first kernel of a pass
+  chain_next();
+  x0 = after_wait(x0);
+  P = after_wait(P);
   const int64_t b0 = int64_t(blockIdx.x) * kInRows;
   const int nb = int(B - b0 < kInRows ? B - b0 : kInRows);
   for (int i = threadIdx.x; i < nb * kIn; i += blockDim.x) xs[i] = x0[b0 * kIn + i];
@@ -151,6 +155,9 @@ k_loss(int64_t B, const float *__restrict__ Y, const float *__restrict__ Tv, con
        float mask_weight, __nv_bfloat16 *__restrict__ dY, __nv_bfloat16 *__restrict__ dYt, float *__restrict__ csum,
        double *__restrict__ part) {
   __shared__ BlockSmem sm;
+  chain_next();
+  chain_wait();
+  Y = after_wait(Y);
   const int64_t c0 = int64_t(blockIdx.x) * kBlk, r0 = int64_t(blockIdx.y) * kBlk;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const bool is_val = c0 < kOutV;   // 64 divides kOutV: a block is all values or all mask
@@ -208,6 +215,9 @@ k_loss(int64_t B, const float *__restrict__ Y, const float *__restrict__ Tv, con
 }
 
 __global__ void __launch_bounds__(1024) k_sum_part_d(const double *__restrict__ part, int n, double *__restrict__ out) {
+  chain_next();
+  chain_wait();
+  part = after_wait(part);
   double v = 0;
   for (int i = threadIdx.x; i < n; i += 1024) v += part[i];
   v = block_sum_d<1024>(v);
@@ -224,6 +234,10 @@ k_gelu_bwd(int64_t B, const float *__restrict__ dH, const float *__restrict__ Z,
            float *__restrict__ csum) {
   __shared__ BlockSmem sm;
   constexpr int NV = IN ? 4 : 1;
+  chain_next();
+  chain_wait();
+  dH = after_wait(dH);
+  Z = after_wait(Z);
   const int64_t c0 = int64_t(blockIdx.x) * kBlk, r0 = int64_t(blockIdx.y) * kBlk;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   float cs[NV][4];
@@ -277,6 +291,9 @@ k_gelu_bwd(int64_t B, const float *__restrict__ dH, const float *__restrict__ Z,
 __global__ void __launch_bounds__(256)
 k_sum_rows(int n, int64_t len, const float *__restrict__ in, float *__restrict__ out) {
   __shared__ float red[8][33];
+  chain_next();
+  chain_wait();
+  in = after_wait(in);
   const int x = threadIdx.x & 31, g = threadIdx.x >> 5;
   const int64_t i = int64_t(blockIdx.x) * 32 + x;
   float t = 0.f;
@@ -298,10 +315,13 @@ k_sum_rows(int n, int64_t len, const float *__restrict__ in, float *__restrict__
 __global__ void __launch_bounds__(256)
 k_sum_few(int n, int64_t len4, const float4 *__restrict__ in, float4 *__restrict__ out) {
   const int64_t i = int64_t(blockIdx.x) * 256 + threadIdx.x;
+  chain_next();
+  chain_wait();
+  in = after_wait(in);
   if (i >= len4) return;
   float4 v[8];
 #pragma unroll
-  for (int p = 0; p < 8; ++p) v[p] = p < n ? __ldcs(in + p * len4 + i) : make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int p = 0; p < 8; ++p) v[p] = p < n ? in[p * len4 + i] : make_float4(0.f, 0.f, 0.f, 0.f);
   float4 t = v[0];
 #pragma unroll
   for (int p = 1; p < 8; ++p) {
@@ -318,7 +338,9 @@ __global__ void __launch_bounds__(256)
 k_transpose_h(int64_t B, const __nv_bfloat16 *__restrict__ h1, const __nv_bfloat16 *__restrict__ h2,
               const __nv_bfloat16 *__restrict__ h3, __nv_bfloat16 *__restrict__ out) {
   __shared__ BlockSmem sm;
-  const __nv_bfloat16 *in = blockIdx.z == 0 ? h1 : (blockIdx.z == 1 ? h2 : h3);
+  chain_next();
+  chain_wait();
+  const __nv_bfloat16 *in = after_wait(blockIdx.z == 0 ? h1 : (blockIdx.z == 1 ? h2 : h3));
   const int64_t c0 = int64_t(blockIdx.x) * kBlk, r0 = int64_t(blockIdx.y) * kBlk;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
@@ -366,6 +388,9 @@ k_weights(const float *__restrict__ P, __nv_bfloat16 *__restrict__ w2, __nv_bflo
 // first layer gradients from the 4-way column sums of the row blocks
 __global__ void k_in_grad(const float *__restrict__ s4, float *__restrict__ G) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  chain_next();
+  chain_wait();
+  s4 = after_wait(s4);
   if (j >= kH) return;
   G[oW1 + j * kIn] = s4[j];
   G[oW1 + j * kIn + 1] = s4[kH + j];
@@ -390,11 +415,10 @@ int blocks_for(int64_t n) { return (int)std::min<int64_t>(152 * 16, std::max<int
 
 wproj_status sum_rows(int n, int64_t len, const float *in, float *out, cudaStream_t s) {
   if (n <= 8 && len % 4 == 0 && ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0)
-    k_sum_few<<<ceil_div(len / 4, 256), 256, 0, s>>>(n, len / 4, reinterpret_cast<const float4 *>(in),
-                                                     reinterpret_cast<float4 *>(out));
+    WPROJ_CUDA(launch_chained(k_sum_few, ceil_div(len / 4, 256), 256, 0, s, n, len / 4,
+                              reinterpret_cast<const float4 *>(in), reinterpret_cast<float4 *>(out)));
   else
-    k_sum_rows<<<ceil_div(len, 32), 256, 0, s>>>(n, len, in, out);
-  WPROJ_CHECK_LAUNCH("row sums");
+    WPROJ_CUDA(launch_chained(k_sum_rows, ceil_div(len, 32), 256, 0, s, n, len, in, out));
   return WPROJ_OK;
 }
 
@@ -467,8 +491,8 @@ wproj_status gemm_wgrad(int M, int N, int K, const void *A, const void *B, float
 wproj_status forward(wproj_mlp *n, const float *x0, int64_t B, float *Y, bool train, cudaStream_t s) {
   const float *P = n->P.as<float>();
   auto *H1 = n->H1.as<__nv_bfloat16>(), *H2 = n->H2.as<__nv_bfloat16>(), *H3 = n->H3.as<__nv_bfloat16>();
-  k_in_fwd<<<ceil_div(B, kInRows), kH / 2, 0, s>>>(B, x0, P, train ? n->Z1.as<float>() : nullptr, H1);
-  WPROJ_CHECK_LAUNCH("mlp layer 1");
+  WPROJ_CUDA(launch_chained(k_in_fwd, ceil_div(B, kInRows), kH / 2, 0, s, B, x0, P,
+                            train ? n->Z1.as<float>() : nullptr, H1));
   WPROJ_TRY(gemm((int)B, kH, kH, H1, n->W2b.ptr, P + oB2, train ? n->Z2.as<float>() : nullptr, H2, n, s));
   WPROJ_TRY(gemm((int)B, kH, kH, H2, n->W3b.ptr, P + oB3, train ? n->Z3.as<float>() : nullptr, H3, n, s));
   return gemm((int)B, kOut, kH, H3, n->W4b.ptr, P + oB4, Y, nullptr, n, s);
@@ -482,12 +506,11 @@ wproj_status backward(wproj_mlp *n, const float *x0, const float *Tv, const floa
   auto *dZ = n->dZ.as<__nv_bfloat16>(), *dZt = n->dZt.as<__nv_bfloat16>();
   const int nrb = int(B / kBlk);
   const dim3 lg(kOut / kBlk, nrb), hg(kH / kBlk, nrb);
-  k_loss<<<lg, 256, 0, s>>>(B, n->Y.as<float>(), Tv, Tm, mask_weight, n->dY.as<__nv_bfloat16>(),
-                            n->dYt.as<__nv_bfloat16>(), csum, n->part.as<double>());
-  k_sum_part_d<<<1, 1024, 0, s>>>(n->part.as<double>(), int(lg.x * lg.y), loss_d);
-  k_transpose_h<<<dim3(kH / kBlk, nrb, 3), 256, 0, s>>>(B, n->H1.as<__nv_bfloat16>(), n->H2.as<__nv_bfloat16>(),
-                                                        n->H3.as<__nv_bfloat16>(), Ht);
-  WPROJ_CHECK_LAUNCH("mlp loss");
+  WPROJ_CUDA(launch_chained(k_loss, lg, 256, 0, s, B, n->Y.as<float>(), Tv, Tm, mask_weight, n->dY.as<__nv_bfloat16>(),
+                            n->dYt.as<__nv_bfloat16>(), csum, n->part.as<double>()));
+  WPROJ_CUDA(launch_chained(k_sum_part_d, 1, 1024, 0, s, n->part.as<double>(), int(lg.x * lg.y), loss_d));
+  WPROJ_CUDA(launch_chained(k_transpose_h, dim3(kH / kBlk, nrb, 3), 256, 0, s, B, n->H1.as<__nv_bfloat16>(),
+                            n->H2.as<__nv_bfloat16>(), n->H3.as<__nv_bfloat16>(), Ht));
   // layer 4
   float *dH = n->dH.as<float>();
   WPROJ_TRY(sum_rows(nrb, kOut, csum, G + oB4, s));
@@ -498,18 +521,15 @@ wproj_status backward(wproj_mlp *n, const float *x0, const float *Tv, const floa
   const float *Z[2] = {n->Z3.as<float>(), n->Z2.as<float>()};
   const int64_t oW[2] = {oW3, oW2}, oB[2] = {oB3, oB2};
   for (int l = 0; l < 2; ++l) {
-    k_gelu_bwd<false><<<hg, 256, 0, s>>>(B, dH, Z[l], nullptr, dZ, dZt, csum);
-    WPROJ_CHECK_LAUNCH("mlp gelu backward");
+    WPROJ_CUDA(launch_chained(k_gelu_bwd<false>, hg, 256, 0, s, B, dH, Z[l], nullptr, dZ, dZt, csum));
     WPROJ_TRY(sum_rows(nrb, kH, csum, G + oB[l], s));
     WPROJ_TRY(gemm_wgrad(kH, kH, (int)B, dZt, Ht + (1 - l) * B * kH, G + oW[l], n, s));
     WPROJ_TRY(gemm((int)B, kH, kH, dZ, Wt[l], nullptr, dH, nullptr, n, s));
   }
   // layer 1
-  k_gelu_bwd<true><<<hg, 256, 0, s>>>(B, dH, n->Z1.as<float>(), x0, nullptr, nullptr, csum);
-  WPROJ_CHECK_LAUNCH("mlp layer 1 backward");
+  WPROJ_CUDA(launch_chained(k_gelu_bwd<true>, hg, 256, 0, s, B, dH, n->Z1.as<float>(), x0, nullptr, nullptr, csum));
   WPROJ_TRY(sum_rows(nrb, 4 * kH, csum, dH, s));   // dH is spent: its first 4 kH floats take the sums
-  k_in_grad<<<1, kH, 0, s>>>(dH, G);
-  WPROJ_CHECK_LAUNCH("mlp layer 1 gradients");
+  WPROJ_CUDA(launch_chained(k_in_grad, 1, kH, 0, s, dH, G));
   return WPROJ_OK;
 }
 

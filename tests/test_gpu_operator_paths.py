@@ -194,3 +194,26 @@ def test_back_to_back_passes(wp, N, M, box, value):
     torch.cuda.synchronize()
     assert torch.equal(out, want) and torch.equal(yo, wanty)
     op.close()
+
+
+# the GEMM's staged TMA stores (128 and 256 columns a tile, more tiles than SMs) and its
+# element by element ones (an output or a bias off the 16-byte boundary): the same bits
+@pytest.mark.parametrize("m,n,k,bf16", [(128, 128, 64, False), (512, 384, 256, True), (20480, 256, 64, True),
+                                        (4096, 1280, 128, False)])
+def test_gemm_unaligned_output(wp, m, n, k, bf16):
+    g = torch.Generator().manual_seed(m + n)
+    a, b = (torch.randn(r, k, generator=g).to(torch.bfloat16).cuda() for r in (m, n))
+    bias = torch.randn(n, generator=g).cuda()
+    ref = wp.gemm_bf16(a, b, bias, out_bf16=bf16)
+    room = torch.full((m * n + 16,), 7.0, dtype=ref.dtype, device="cuda")
+    bias1 = torch.cat([bias[:1], bias])
+    for off, bs in ((1, bias), (0, bias1[1:])):
+        room.fill_(7.0)
+        c = room[off:off + m * n]
+        st = wp.lib().wproj_gemm_bf16(m, n, k, a.data_ptr(), b.data_ptr(), bs.data_ptr(), c.data_ptr(), int(bf16),
+                                      torch.cuda.current_stream().cuda_stream)
+        assert st == 0
+        assert torch.equal(c.view(m, n), ref)
+        assert bool((room[:off] == 7).all()) and bool((room[off + m * n:] == 7).all())
+    err = (ref.double().cpu() - (a.double().cpu() @ b.double().cpu().T + bias.double().cpu())).norm() / ref.double().norm().cpu()
+    assert float(err) <= (4e-3 if bf16 else 1e-5)
