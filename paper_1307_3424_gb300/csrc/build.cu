@@ -35,11 +35,14 @@ namespace {
 __host__ __device__ __forceinline__ int64_t i64max(int64_t a, int64_t b) { return a > b ? a : b; }
 __host__ __device__ __forceinline__ int64_t i64min(int64_t a, int64_t b) { return a < b ? a : b; }
 
-constexpr size_t kBuildBatchBytes = size_t(128) << 20;   // kernel boxes in flight
-// (32 MB batches of 512^2 boxes, which stay in L2 between the passes, measured
-// slower: 866 against 638 ms for 32768 boxes; the selection's histogram
-// launches lose more parallelism than the L2 residency gains)
-size_t batch_bytes(int) { return kBuildBatchBytes; }
+// Kernel boxes in flight.  A batch of boxes is fourteen launches of 5 to 100 us: where
+// the boxes are kept for the second pass anyway (no buffer of their own), batches of
+// up to 1 GB (and 1024 boxes: 16 KB of histogram each) leave few of them; 2048 boxes of
+// 512^2: 18.0 ms in batches of 128 MB, 16.3 of 256, 15.5 of 512, 15.1 of 1 GB, 14.8 of
+// 2 GB.  (Batches that stay in L2 between the passes are slower still: 25.0 ms at
+// 32 MB; the launches lose more parallelism than the L2 hits gain.)
+constexpr size_t kBuildBatchBytes = size_t(128) << 20;
+constexpr size_t kKeptBatchBytes = size_t(1024) << 20;
 constexpr int kMaxBatchBoxes = 16384;     // grid.y limit for per-box launches
 constexpr int kHistBins = 2048;
 constexpr int kSelChunk = 8192;          // entries per histogram block
@@ -1253,7 +1256,9 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
     const int S = 16 << c;
     const int64_t n = std::min<int64_t>(cls_ptr[c + 1] - cls_ptr[c], kMaxBatchBoxes);
     if (keep_all && small_box(S)) return (int)n;
-    return (int)std::min<int64_t>(n, std::max<int64_t>(1, int64_t(batch_bytes(S) / (size_t(S) * S * sizeof(float2)))));
+    const int64_t bytes = keep_all ? std::max(kBuildBatchBytes, std::min(kKeptBatchBytes, size_t(1024) * S * S * sizeof(float2)))
+                                   : kBuildBatchBytes;
+    return (int)std::min<int64_t>(n, std::max<int64_t>(1, bytes / (int64_t(S) * S * int64_t(sizeof(float2)))));
   };
   int max_nb = 1, max_nb_hist = 1;
   for (int c = 0; c < 9; ++c) {
