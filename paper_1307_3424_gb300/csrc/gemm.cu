@@ -23,7 +23,8 @@
 //            into swizzled shared memory and hand them to TMA (two blocks of a
 //            warp in flight), and release the accumulator.
 // So the loads of tile i + 1 and the MMAs of tile i + 1 overlap the epilogue of
-// tile i.  BN = 256: three stages of 48 KB and 64 KB of staging; 1 CTA per SM.
+// tile i.  BN = 256: three stages of 48 KB and 64 KB of staging, or four and 32 KB
+// (more than 8 slices a work unit); 1 CTA per SM.
 //
 // What bounds it: at large K the tensor cores; at the network's K = 256 the
 // epilogue and the output's bytes (65536 x 3072 FP32, 805 MB): 143 us, 83 %
@@ -56,7 +57,6 @@ namespace {
 constexpr int kBM = 128, kBK = 64;      // tile rows; K slice (64 bf16 = one 128-byte swizzle row)
 constexpr int kSliceA = kBM * kBK * 2;   // bytes of one A slice: 16 KB
 constexpr int kEpiWarps = 8;
-constexpr int kOutBufs = 2;              // staging blocks a warp
 constexpr int kThreads = 64 + 32 * kEpiWarps;
 constexpr int kStage = 32 * 32 * 4;      // a warp's staging block: 32 rows of 128 bytes
 constexpr unsigned long long kGemmWaitNs = 2000000000ull;
@@ -150,9 +150,12 @@ __host__ __device__ constexpr uint32_t instr_desc(int M, int N) {
 
 // BN: tile columns (128 or 256); a tile's accumulator takes BN tensor-memory
 // columns, two of them 2 BN (512 at most: the whole tensor memory).
-template <int BN>
+// ST stages, OB staging blocks a warp: three stages and two blocks for short K (the
+// epilogue bounds it), four and one for long K (8192^3: 1431 TFLOP/s, 1282 with three
+// stages), four and two at 128 columns.
+template <int BN, int ST, int OB>
 struct GemmSmem {
-  static constexpr int kStages = BN == 256 ? 3 : 4;
+  static constexpr int kStages = ST, kOutBufs = OB;
   unsigned char a[kStages][kSliceA];     // 1024-byte aligned (swizzle atoms)
   unsigned char b[kStages][BN * kBK * 2];
   unsigned char out[kEpiWarps][kOutBufs][kStage];
@@ -174,17 +177,18 @@ __device__ __forceinline__ void st_shared_v4(uint32_t at, uint32_t a, uint32_t b
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(at), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 
-template <int BN>
+template <int BN, int ST, int OB>
 __global__ void __launch_bounds__(kThreads, 1)
 k_gemm_ws(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
           const __grid_constant__ CUtensorMap tmZ, const __grid_constant__ CUtensorMap tmH, int M, int N, int K,
           const EpiArgs ep, int *__restrict__ err) {
-  constexpr int kStages = GemmSmem<BN>::kStages;
+  constexpr int kStages = ST, kOutBufs = OB;
   constexpr int kAccCols = BN;
   constexpr int kSliceB = BN * kBK * 2, kCols = BN / (kEpiWarps / 4);   // columns of an epilogue warp
   extern __shared__ unsigned char smem_raw[];
-  GemmSmem<BN> &sm =
-      *reinterpret_cast<GemmSmem<BN> *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  using Smem = GemmSmem<BN, ST, OB>;
+  Smem &sm =
+      *reinterpret_cast<Smem *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // work unit t: split t mod splits of tile t / splits, K slices [k0, k1)
   const int nN = N / BN, nk_all = K / kBK, sp_n = ep.splits, n_units = (M / kBM) * nN * sp_n;
@@ -430,7 +434,7 @@ wproj_status tensor_map(CUtensorMap *map, const void *p, int elem, int64_t rows,
   return WPROJ_OK;
 }
 
-template <int BN>
+template <int BN, int ST, int OB>
 wproj_status launch_gemm(int M, int N, int K, const __nv_bfloat16 *A, const __nv_bfloat16 *B, const EpiArgs &ep, int sms,
                          int *err, cudaStream_t s) {
   CUtensorMap ta, tb, tz{}, th{};
@@ -439,9 +443,9 @@ wproj_status launch_gemm(int M, int N, int K, const __nv_bfloat16 *A, const __nv
   if (ep.tma && ep.z) WPROJ_TRY(tensor_map(&tz, ep.z, 4, int64_t(M) * ep.splits, N, 32, 32));
   if (ep.tma && ep.h) WPROJ_TRY(tensor_map(&th, ep.h, 2, M, N, 32, 32));
   const int grid = std::max(1, std::min((M / kBM) * (N / BN) * ep.splits, sms));
-  const size_t smem = sizeof(GemmSmem<BN>) + 1024;
-  WPROJ_CUDA(cudaFuncSetAttribute(k_gemm_ws<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  WPROJ_CUDA(launch_chained(k_gemm_ws<BN>, grid, kThreads, smem, s, ta, tb, tz, th, M, N, K, ep, err));
+  const size_t smem = sizeof(GemmSmem<BN, ST, OB>) + 1024;
+  WPROJ_CUDA(cudaFuncSetAttribute(k_gemm_ws<BN, ST, OB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  WPROJ_CUDA(launch_chained(k_gemm_ws<BN, ST, OB>, grid, kThreads, smem, s, ta, tb, tz, th, M, N, K, ep, err));
   return WPROJ_OK;
 }
 
@@ -486,8 +490,9 @@ wproj_status gemm_bf16_tn(int M, int N, int K, const __nv_bfloat16 *A, const __n
   ep.tma = ((reinterpret_cast<uintptr_t>(o.f32) | reinterpret_cast<uintptr_t>(o.bf16) |
              reinterpret_cast<uintptr_t>(o.bias)) & 15) == 0;
   if (N % 256 == 0 && (M / kBM) * (N / 256) * (2 * o.splits) > sms)
-    return launch_gemm<256>(M, N, K, A, B, ep, sms, err, s);
-  return launch_gemm<128>(M, N, K, A, B, ep, sms, err, s);
+    return K / kBK > 8 * o.splits ? launch_gemm<256, 4, 1>(M, N, K, A, B, ep, sms, err, s)
+                                  : launch_gemm<256, 3, 2>(M, N, K, A, B, ep, sms, err, s);
+  return launch_gemm<128, 4, 2>(M, N, K, A, B, ep, sms, err, s);
 }
 
 }  // namespace wproj
