@@ -99,6 +99,18 @@ k_stream(const int32_t *__restrict__ chunk_tile, const int64_t *__restrict__ chu
     }
   };
   if (pf_thread) prefetch_to(b0 + kPfAhead);
+  // degridding: this thread's cells of the chunk's tile of X, asked for before the
+  // first header (after it: 14.09 against 13.94 ms for the pair on 38 GB)
+  float2 xr[kRows];
+  if constexpr (DEGRID) {
+    const int tile = chunk_tile[c];
+    const int tu = tile / nT, tv = tile % nT;
+    chain_wait();
+    Xt = after_wait(Xt);
+#pragma unroll
+    for (int rr = 0; rr < kRows; ++rr)
+      xr[rr] = Xt[((int64_t(tu * 32 + kRows * w + rr)) << logG) + tv * 32 + lane];
+  }
   float2 acc[kRows];
 #pragma unroll
   for (int rr = 0; rr < kRows; ++rr) acc[rr] = make_float2(0.f, 0.f);
@@ -121,16 +133,6 @@ k_stream(const int32_t *__restrict__ chunk_tile, const int64_t *__restrict__ chu
       yk = y[hdr.x];
       if (row_scale) yk = cscale(yk, __ldg(row_scale + hdr.x));
     }
-  }
-  float2 xr[kRows];   // degridding: this thread's cells of the chunk's tile of X
-  if constexpr (DEGRID) {
-    const int tile = chunk_tile[c];
-    const int tu = tile / nT, tv = tile % nT;
-    chain_wait();
-    Xt = after_wait(Xt);
-#pragma unroll
-    for (int rr = 0; rr < kRows; ++rr)
-      xr[rr] = Xt[((int64_t(tu * 32 + kRows * w + rr)) << logG) + tv * 32 + lane];
   }
   for (int64_t j = j0; j < j1; ++j) {
     const int64_t offn = off + kRecValues + ((hdr.y * VB + 15) & ~15);
