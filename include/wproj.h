@@ -120,7 +120,11 @@ typedef struct {
  * else TILE_MASK when segments average >= 256 entries (dense rows), else
  * COLUMNS.  Requesting TILE_RUNS for larger boxes makes
  * wproj_build_kernels return WPROJ_ERR_UNSUPPORTED.  wproj_csr_rows exports any
- * rows in CSR order from every format. */
+ * rows in CSR order from every format.
+ * Where every box is at most 64 x 64 cells, COLUMNS and TILE_RUNS plans also hold
+ * interleaved slices of the values with 2-byte local indices, which the operators
+ * read instead (the row-major runs are then not stored); plans too sparse for them
+ * (patches of more than 4 cells an entry, pads of more than the entries) do without. */
 typedef enum {
   WPROJ_INDEX_AUTO = 0,
   WPROJ_INDEX_COLUMNS = 1,
@@ -194,8 +198,9 @@ typedef struct {
   double t_fft_ms, t_degrid_ms, t_grid_ms, t_reduce_ms, t_solver_ms;
   int64_t n_fft, n_degrid, n_grid, n_reduce, n_solver;
   int64_t launches;          /* kernels launched by Phi, Phi^H and the solver since the last reset */
-  int64_t runs_bytes;        /* TILE_RUNS: bytes of the row-major copy the degridding reads (values,
-                                runs, per-row offsets and origins); 0 for the other formats */
+  int64_t runs_bytes;        /* TILE_RUNS: bytes the degridding reads (the row-major copy's values,
+                                runs, per-row offsets and origins, or the slices that replace it);
+                                0 for the other formats */
   /* device time (ms) of the builds since the last reset when timing is on: box
      tables and FFTs (both passes), selection and per-tile counts, emission */
   double t_build_fft_ms, t_build_select_ms, t_build_emit_ms;
@@ -450,7 +455,9 @@ typedef struct wproj_batch wproj_batch;
 /* Work split of the batch operators: degridding row pieces of <= piece entries,
  * each taken by lanes_per_piece lanes of a warp (32, 16, 8 or 4: 32 / lanes pieces
  * per warp),
- * gridding chunks of about chunk entries of one grid tile. */
+ * gridding chunks of about chunk entries of one grid tile.  Batches whose boxes are
+ * all at most 64 x 64 cells, on grids of at least 32 x 32, read interleaved slices
+ * with a split of their own; the schedule is then kept but changes nothing. */
 typedef struct {
   int64_t piece;
   int64_t chunk;

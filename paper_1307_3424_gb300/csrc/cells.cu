@@ -1,5 +1,6 @@
 // Gridding X'[q] = sum_k conj(G[k, q]) y_k for G with column indices, from a
-// cell-major copy of G (Eq. 8's adjoint, Section 3.1).
+// cell-major copy of G (Eq. 8's adjoint, Section 3.1).  Short rows (boxes of at most
+// 64 x 64 cells) go through interleaved slices instead where a plan holds them.
 //
 // The copy holds, for every 32 x 32 grid tile (ascending), the tile's entries
 // sorted by cell and, within a cell, by row: one packed word per entry

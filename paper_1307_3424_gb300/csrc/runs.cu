@@ -1,5 +1,7 @@
 // Degridding and gridding for G in the run-length format (TILE_RUNS), for plans
 // whose kernel boxes are at most 64 x 64 cells (the box rule's small kernels).
+// Plans that hold interleaved slices (most of them) apply those instead; the records
+// then serve the CSR export, and the row-major copy is not built.
 //
 // A small w-kernel holds its kept entries in one contiguous run of cells per
 // grid row of its box (on the precision-form workload: 283 entries per row in
