@@ -436,9 +436,12 @@ def run_ours(args):
     grid_ms = kst["t_grid_ms"] / max(1, kst["n_grid"])
     alg_deg = nnz * b_val + M * 8 + G * G * 8
     alg_grid = nnz * b_val + M * 8 + G * G * 8
-    # G as each operator reads it: values + column indices, the tile-stream
-    # records, or (run lengths) the row-major copy and the tile-major records
-    if fmt == "columns":
+    # G as each operator reads it: the slices of short rows (values + 2-byte indices,
+    # pads not counted), values + column indices, or the tile-stream records
+    slices = fmt != "mask" and st["box_max"] <= 64
+    if slices:
+        stored_deg = stored_grid = nnz * (b_val + 2)
+    elif fmt == "columns":
         stored_deg = stored_grid = nnz * (b_val + 4)
     elif fmt == "runs":
         stored_deg, stored_grid = st["runs_bytes"], stream_bytes
@@ -447,6 +450,8 @@ def run_ours(args):
     # kernel labels as in profiles/
     deg_name, grid_name = {"mask": ("k_stream_degrid", "k_stream_grid"), "runs": ("k_runs_degrid", "k_runs_grid"),
                            "columns": ("k_degrid", "k_grid_cells")}[fmt]
+    if slices:
+        deg_name, grid_name = "k_slice_degrid", "k_slice_grid"
     if args.workload == "precision":   # the traffic figures in profiles/ are per workload
         deg_name += f"_precision_{args.value_dtype}"
         grid_name += f"_precision_{args.value_dtype}"
@@ -602,7 +607,7 @@ def run_batched(args):
     alg = info["nnz"] * 8 + info["m"] * 8 + grid_cells * 8
     dom = "grid" if sched["grid_ms"] >= sched["degrid_ms"] else "degrid"
     ms_dom = max(sched["grid_ms"], sched["degrid_ms"])
-    kname = "k_grid_cells_batch" if dom == "grid" else "k_degrid_batch"   # labels as in profiles/
+    kname = "k_slice_grid_batch" if dom == "grid" else "k_slice_degrid_batch"   # labels as in profiles/
     tr = read_profile_traffic(kname, "traffic_bytes_per_entry")   # from a smaller capture
     traffic = tr * info["nnz"] if tr is not None else None
     value = PAIRS_PER_STEP * args.steps / (t_ms * 1e-3)
