@@ -1152,8 +1152,11 @@ wproj_status set_screens_impl(wproj_plan *p, const float2 *screens, int n, cudaS
 wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, double e, cudaStream_t s,
                                 const int32_t *sid) {
   auto t_start = std::chrono::steady_clock::now();
-  // the previous G's buffers are overwritten where they fit: no kernel may still read them
-  WPROJ_CUDA(cudaDeviceSynchronize());
+  // The previous G's buffers are overwritten where they fit, so no kernel may still read
+  // them.  Freeing one of them waits for the work in flight on every stream, as freeing
+  // all of them would.  (cudaDeviceSynchronize waits as well, but fails, and breaks the
+  // capture, while any stream of the device is being captured.)
+  p->seg_base.release();
   ScratchScope scope(p->scratch, (size_t(4) << 20) + size_t(384) * size_t(m));
   const GridGeom &g = p->g;
   p->built = false;

@@ -1,0 +1,74 @@
+"""Plans built and used beside other work: another stream's capture, operators still
+running on another stream, other plans on other host threads, little free memory."""
+import numpy as np
+import pytest
+import torch
+
+from paper_1307_3424_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+L = synth.fov_L()
+
+
+@pytest.fixture(scope="module")
+def wp():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1307_3424_gb300 import wproj
+    return wproj
+
+
+def uvw_cells(seed, M, N, wmax):
+    """Uniform disk, w_c ~ U[0, wmax] cells, on the device."""
+    rng = np.random.default_rng(seed)
+    uv = synth.uv_points(rng, M, synth.band_limit(N, L), N, "uniform")
+    w = 2.0 * rng.uniform(0, wmax, M) / (L * L)
+    return torch.from_numpy(np.ascontiguousarray(np.concatenate([uv, w[:, None]], axis=1))).cuda()
+
+
+# a build, of a new plan or of one that holds a G, while another stream is captured in
+# relaxed mode: neither disturbs the other
+@pytest.mark.parametrize("again", [False, True])
+def test_build_beside_a_capture(wp, again):
+    N, M = 64, 300
+    uvw = uvw_cells(0, M, N, 1.0)
+    p, q = wp.Plan(N, L, box="rule"), wp.Plan(N, L, box="rule")
+    q.build_kernels(uvw, 0.99)
+    if again:
+        p.build_kernels(uvw, 0.99)
+    x = torch.randn(N, N, generator=torch.Generator().manual_seed(1)).cuda()
+    y = torch.empty(M, dtype=torch.complex64, device="cuda")
+    want = q.phi(x).clone()
+    side, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g, capture_error_mode="relaxed"):
+        q.phi(x, y)
+        p.build_kernels(uvw, 0.99, stream=side)
+    g.replay()
+    assert torch.equal(y, want)
+    assert torch.equal(p.phi(x), want)
+    p.close()
+    q.close()
+
+
+# a plan built again while an operator of its last G still waits on another stream: the
+# operator reads the G it was launched with
+@pytest.mark.parametrize("box,value", [("rule", "f32"), ("rule", "bf16"), ("G", "f32")])
+def test_build_waits_for_operators_in_flight(wp, box, value):
+    N, M = 64, 600
+    p = wp.Plan(N, L, box=box, value_dtype=value)
+    p.build_kernels(uvw_cells(0, M, N, 1.0), 0.99)
+    x = torch.randn(N, N, generator=torch.Generator().manual_seed(2)).cuda()
+    want = p.phi(x).clone()
+    y = torch.empty_like(want)
+    other = uvw_cells(1, M, N, 1.0)
+    side = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(400_000_000)      # about 0.2 s
+        p.phi(x, y, stream=side)
+    p.build_kernels(other, 0.99)
+    torch.cuda.synchronize()
+    assert torch.equal(y, want)
+    p.close()
