@@ -348,7 +348,9 @@ wproj_status grid(wproj_plan *p, const float2 *y, float2 *Xt2, cudaStream_t s) {
     ScopedTimer t(p, TC_GRID, s);
 #define LAUNCH_GRID(VDT)                                                                                    \
   do {                                                                                                      \
-    WPROJ_CUDA(cudaFuncSetAttribute(k_grid<VDT, kGridWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
+    /* the limit is the kernel's, not the plan's: the most any plan takes (plans of several threads) */     \
+    WPROJ_CUDA(cudaFuncSetAttribute(k_grid<VDT, kGridWarps>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
+                                    int(sizeof(float2) * kGridWarps * kTile * kTile)));                     \
     k_grid<VDT, kGridWarps><<<(unsigned)p->n_chunks, kGridWarps * 32, smem, s>>>(                           \
         p->chunk_tile.as<int32_t>(), p->chunk_lo.as<int64_t>(), p->chunk_hi.as<int64_t>(),                  \
         p->seg_meta.as<SegMeta>(), p->col.as<int32_t>(), p->val.ptr, rs, y, logG, g.tile, g.nT, nullptr,    \

@@ -50,10 +50,17 @@ constexpr int kLpr = 8;              // degridding: lanes per row
 constexpr int kRps = 32 / kLpr;      // rows per slice
 constexpr int kMaxRowsChunk = 12288; // rows of a gridding chunk (96 KB of y)
 constexpr int kMaxLen = 4096;        // entries of a row (64 x 64)
+constexpr int kMaxPatch = 96;        // sides of a patch: a tile's 32 cells and the windows of 64 around them
 
 // odd row stride of the patch in shared memory
 __host__ __device__ __forceinline__ int patch_stride(int wv) { return wv | 1; }
 __host__ __device__ __forceinline__ int patch_words(int hu, int wv) { return 1 + hu * patch_stride(wv); }
+
+// The operators' limits of dynamic shared memory: a limit belongs to the kernel, which
+// plans of other threads launch too, so it is the most that any plan takes (75 and 98 KB)
+// and not the plan's own size.
+const int kMaxDegridSmem = int(sizeof(float2)) * patch_words(kMaxPatch, kMaxPatch);
+constexpr int kMaxGridSmem = int(sizeof(float2)) * (1 + kMaxRowsChunk);
 
 template <int VDT> struct RawVal { using type = unsigned; };
 template <> struct RawVal<WPROJ_VAL_F32> { using type = float2; };
@@ -627,14 +634,14 @@ int clamp_blocks(int64_t n, int per) { return (int)std::max<int64_t>(1, std::min
 template <int VDT>
 wproj_status launch_degrid(const SliceOps &o, size_t smem, const float2 *X, float2 *y, cudaStream_t s) {
   constexpr int U = VDT == WPROJ_VAL_F32 ? 6 : 8;   // steps per group (two groups in registers)
-  WPROJ_CUDA(cudaFuncSetAttribute(k_slice_degrid<VDT, U>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  WPROJ_CUDA(cudaFuncSetAttribute(k_slice_degrid<VDT, U>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDegridSmem));
   WPROJ_CUDA(launch_chained(k_slice_degrid<VDT, U>, (unsigned)o.d_chunks, kThreads, smem, s, o, X, y));
   WPROJ_CHECK_LAUNCH("degrid (slices)");
   return WPROJ_OK;
 }
 template <int VDT>
 wproj_status launch_grid(const SliceOps &o, size_t smem, const float2 *y, float2 *partial, float2 *Xt2, cudaStream_t s) {
-  WPROJ_CUDA(cudaFuncSetAttribute(k_slice_grid<VDT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  WPROJ_CUDA(cudaFuncSetAttribute(k_slice_grid<VDT>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxGridSmem));
   WPROJ_CUDA(launch_chained(k_slice_grid<VDT>, (unsigned)o.g_chunks, kThreads, smem, s, o, y, partial, Xt2));
   WPROJ_CHECK_LAUNCH("grid (slices)");
   if (o.n_multi > 0) {

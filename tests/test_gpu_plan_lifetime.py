@@ -1,5 +1,7 @@
 """Plans built and used beside other work: another stream's capture, operators still
 running on another stream, other plans on other host threads, little free memory."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -72,3 +74,34 @@ def test_build_waits_for_operators_in_flight(wp, box, value):
     torch.cuda.synchronize()
     assert torch.equal(y, want)
     p.close()
+
+
+# two plans on two host threads, with small and with large (over 48 KB) needs of shared
+# memory: no launch of either is refused, and both give what they give alone.  A power
+# iteration is one call of some hundred operator passes, so the threads' launches mix.
+@pytest.mark.parametrize("value", ["f32", "bf16"])
+def test_plans_on_host_threads(wp, value):
+    plans = []
+    for N, M, wmax, W, e in ((128, 6000, 4.0, 8, 1.0), (32, 900, 1.0, 4, 0.99)):
+        p = wp.Plan(N, L, kb_support=W, box="rule", value_dtype=value)
+        p.build_kernels(uvw_cells(N, M, N, wmax), e)
+        plans.append((p, p.power_norm2(500)))
+    got, refused = [[], []], []
+
+    def work(i):
+        s = torch.cuda.Stream()
+        for _ in range(8):
+            try:
+                got[i].append(plans[i][0].power_norm2(500, stream=s))
+            except wp.WprojError as err:
+                refused.append(str(err))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in (0, 1)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not refused, (len(refused), refused[0])
+    for (p, alone), g in zip(plans, got):
+        assert g == [alone] * 8
+        p.close()
