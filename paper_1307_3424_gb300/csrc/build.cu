@@ -1149,8 +1149,8 @@ wproj_status set_screens_impl(wproj_plan *p, const float2 *screens, int n, cudaS
   return WPROJ_OK;
 }
 
-wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, double e, cudaStream_t s,
-                                const int32_t *sid) {
+static wproj_status build_g(wproj_plan *p, const double *uvw, int64_t m, double e, cudaStream_t s,
+                            const int32_t *sid) {
   auto t_start = std::chrono::steady_clock::now();
   // The previous G's buffers are overwritten where they fit, so no kernel may still read
   // them.  Freeing one of them waits for the work in flight on every stream, as freeing
@@ -1582,6 +1582,14 @@ wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, dou
   p->built = true;
   p->build_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_start).count();
   return WPROJ_OK;
+}
+
+wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, double e, cudaStream_t s,
+                                const int32_t *sid) {
+  const wproj_status st = build_g(p, uvw, m, e, s, sid);
+  // the next build, on any stream, writes the buffers this one's kernels may still use
+  if (st != WPROJ_OK) cudaStreamSynchronize(s);
+  return st;
 }
 
 }  // namespace wproj
