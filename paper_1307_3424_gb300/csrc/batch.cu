@@ -592,9 +592,8 @@ wproj_status time_ms(F &&f, int reps, cudaStream_t s, double *ms) {
   return st;
 }
 
-}  // namespace
-
-wproj_status batch_build_impl(wproj_batch *b, const double *uvw, const int64_t *m, double e, cudaStream_t s) {
+// lean: the forms that need least memory (build.cu)
+wproj_status batch_build_once(wproj_batch *b, const double *uvw, const int64_t *m, double e, cudaStream_t s, bool lean) {
   b->built = false;
   b->dr_valid = false;
   if (b->dr_exec) {
@@ -613,7 +612,7 @@ wproj_status batch_build_impl(wproj_batch *b, const double *uvw, const int64_t *
   // slices everywhere, or the other forms everywhere: a problem that cannot take them
   // (a box over 64 cells, a grid under 32) makes those built with them build again
   int64_t vis = 0;
-  bool want = true;
+  bool want = !lean;
   for (int p = 0; p < np; ++p) want = want && b->desc[p].box <= 64 && 2 * b->desc[p].n >= kTile;
   for (bool done = false; !done;) {
     done = true;
@@ -626,6 +625,7 @@ wproj_status batch_build_impl(wproj_batch *b, const double *uvw, const int64_t *
       if (want || !pl->built || pl->slices.use) {
         pl->in_batch = want;
         pl->no_slices = !want;
+        pl->lean = lean;
         WPROJ_TRY(build_kernels_impl(pl, uvw + 3 * vis, m[p], e, s));
       }
       vis += m[p];
@@ -783,6 +783,22 @@ wproj_status batch_build_impl(wproj_batch *b, const double *uvw, const int64_t *
   WPROJ_CUDA(cudaStreamSynchronize(s));
   b->built = true;
   return WPROJ_OK;
+}
+
+}  // namespace
+
+wproj_status batch_build_impl(wproj_batch *b, const double *uvw, const int64_t *m, double e, cudaStream_t s) {
+  wproj_status st = batch_build_once(b, uvw, m, e, s, false);
+  if (st == WPROJ_ERR_OOM) {   // no room for the slices, of the problems and end to end
+    cudaStreamSynchronize(s);
+    b->slices.release();
+    for (DevBuf *d : {&b->d_chunk_prob, &b->g_chunk_prob, &b->row_ptr, &b->col, &b->val, &b->meta, &b->tptr, &b->cum,
+                      &b->tile_prob, &b->tile_ent, &b->cell_ent, &b->cell_val, &b->piece_partial, &b->grid_partial})
+      d->release();
+    st = batch_build_once(b, uvw, m, e, s, true);
+  }
+  if (st != WPROJ_OK) cudaStreamSynchronize(s);
+  return st;
 }
 
 wproj_status batch_tune_impl(wproj_batch *b, wproj_batch_schedule *out, cudaStream_t s) {

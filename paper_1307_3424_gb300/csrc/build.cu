@@ -1149,15 +1149,16 @@ wproj_status set_screens_impl(wproj_plan *p, const float2 *screens, int n, cudaS
   return WPROJ_OK;
 }
 
+// lean: without what is there for speed only, the scratch block and the slices
 static wproj_status build_g(wproj_plan *p, const double *uvw, int64_t m, double e, cudaStream_t s,
-                            const int32_t *sid) {
+                            const int32_t *sid, bool lean) {
   auto t_start = std::chrono::steady_clock::now();
   // The previous G's buffers are overwritten where they fit, so no kernel may still read
   // them.  Freeing one of them waits for the work in flight on every stream, as freeing
   // all of them would.  (cudaDeviceSynchronize waits as well, but fails, and breaks the
   // capture, while any stream of the device is being captured.)
   p->seg_base.release();
-  ScratchScope scope(p->scratch, (size_t(4) << 20) + size_t(384) * size_t(m));
+  ScratchScope scope(p->scratch, lean ? 0 : (size_t(4) << 20) + size_t(384) * size_t(m));
   const GridGeom &g = p->g;
   p->built = false;
   p->dr_valid = false;
@@ -1239,9 +1240,10 @@ static wproj_status build_g(wproj_plan *p, const double *uvw, int64_t m, double 
   DevBuf Kbuf;
   TmpBuf Au, Av, bmode, bwf, bwd, bsel, hq, lcoord, lsq, gtab, bsid;
   // Pass 2 needs every box's transform again.  When the device has room for all
-  // of them (and, with a margin, for G, whose size is at most 1.5x theirs), pass
-  // 1 keeps them and pass 2 emits without recomputing the tables and FFTs;
-  // otherwise pass 2 recomputes them batch by batch.
+  // of them (and, with a margin, for G in the form that pass 2 writes, at most 1.5x
+  // their size), pass 1 keeps them and pass 2 emits without recomputing the tables and
+  // FFTs; otherwise pass 2 recomputes them batch by batch.  They are given back before
+  // the copies of G (slices, run lengths, cells) are made.
   int64_t k_total = 0;
   for (int c = 0; c < 9; ++c) k_total += (cls_ptr[c + 1] - cls_ptr[c]) * int64_t(16 << c) * (16 << c) * int64_t(sizeof(float2));
   DevBuf Kall;
@@ -1468,6 +1470,9 @@ static wproj_status build_g(wproj_plan *p, const double *uvw, int64_t m, double 
       }
     }
   }
+  WPROJ_CUDA(cudaStreamSynchronize(s));
+  Kall.release();
+  Kbuf.release();
   // row scales (max |K| per row) for the 16-bit value forms
   if (vdt != WPROJ_VAL_F32) {
     WPROJ_TRY(p->row_scale.reuse(sizeof(float) * m));
@@ -1478,7 +1483,7 @@ static wproj_status build_g(wproj_plan *p, const double *uvw, int64_t m, double 
   // boxes of at most 64 x 64 cells in the column form: interleaved slices
   p->slices.use = false;
   TmpBuf row_runs;   // with slices: an upper bound of each row's runs
-  if (p->fmt == WPROJ_INDEX_COLUMNS && p->box_max <= 64 && g.tile == 32 && !p->no_slices && n_seg > 0) {
+  if (p->fmt == WPROJ_INDEX_COLUMNS && p->box_max <= 64 && g.tile == 32 && !lean && !p->no_slices && n_seg > 0) {
     p->m = m;
     WPROJ_TRY(row_runs.alloc(sizeof(int32_t) * m));
     TmpBuf cnt, cum;
@@ -1584,9 +1589,30 @@ static wproj_status build_g(wproj_plan *p, const double *uvw, int64_t m, double 
   return WPROJ_OK;
 }
 
+// everything of G, its copies and the scratch block
+static void release_g(wproj_plan *p) {
+  p->slices.release();
+  for (DevBuf *b :
+       {&p->scratch, &p->row_ptr, &p->col, &p->val, &p->row_scale, &p->stream, &p->seg_rec, &p->rec_off, &p->seg_tile,
+        &p->rm_vptr, &p->rm_rptr, &p->rm_org, &p->rm_run, &p->rm_val, &p->seg_base, &p->seg_off, &p->seg_cnt, &p->seg_row,
+        &p->seg_meta, &p->tile_ent, &p->cell_ent, &p->cell_val, &p->cell_partial, &p->chunk_tile, &p->chunk_lo,
+        &p->chunk_hi, &p->tile_chunk_ptr, &p->piece_row, &p->piece_lo, &p->piece_len, &p->row_piece_ptr,
+        &p->grid_partial, &p->piece_partial, &p->ytmp})
+    b->release();
+}
+
 wproj_status build_kernels_impl(wproj_plan *p, const double *uvw, int64_t m, double e, cudaStream_t s,
                                 const int32_t *sid) {
-  const wproj_status st = build_g(p, uvw, m, e, s, sid);
+  wproj_status st = build_g(p, uvw, m, e, s, sid, p->lean);
+  // Slices take 20 (f32) or 12 bytes an entry more than the column form they are made
+  // from, the forms that they stand in for at least 12 and 8, and the last G's buffers
+  // are held during the build: where there is no room, all of it is given back and G
+  // built in the forms that need least.
+  if (st == WPROJ_ERR_OOM && !p->lean) {
+    cudaStreamSynchronize(s);
+    release_g(p);
+    st = build_g(p, uvw, m, e, s, sid, true);
+  }
   // the next build, on any stream, writes the buffers this one's kernels may still use
   if (st != WPROJ_OK) cudaStreamSynchronize(s);
   return st;

@@ -192,6 +192,7 @@ struct wproj_plan {
   wproj::SliceCopy slices;
   bool in_batch = false;     // built for a batch, whose operators run on the whole
   bool no_slices = false;    // a batch some of whose problems cannot take slices
+  bool lean = false;         // a batch built again for want of memory: least memory
   // TILE_RUNS without slices: the row-major copy of the degridding (runs padded to even lengths);
   // the tile-major records of the gridding live in `stream` / `rec_off` / `seg_rec`
   int64_t rm_runs = 0, rm_vals = 0;

@@ -105,3 +105,54 @@ def test_plans_on_host_threads(wp, value):
     for (p, alone), g in zip(plans, got):
         assert g == [alone] * 8
         p.close()
+
+
+def leave_free(gib):
+    """A tensor that takes all of the device's memory but `gib` GiB."""
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    free = torch.cuda.mem_get_info()[0]
+    return torch.empty(free - int(gib * 2 ** 30), dtype=torch.uint8, device="cuda")
+
+
+# short rows built with room for G and the older copies but not for the slices (f32 run
+# lengths, 4.35e7 entries: they fit 1.92 GiB, with slices 2.12; a batch of 2.7e7 entries:
+# 3.7 and 4.2 GiB): the same G and operators, in a form that fits
+def test_build_without_room_for_slices(wp):
+    N, M = 512, 300000
+    uvw = uvw_cells(0, M, N, 4.0)
+    x = torch.randn(N, N, generator=torch.Generator().manual_seed(3)).cuda()
+    yv = torch.randn(M, dtype=torch.complex64, generator=torch.Generator().manual_seed(4)).cuda()
+    results = []
+    for gib in (None, 2.0):
+        p = wp.Plan(N, L, box="rule")
+        fill = leave_free(gib) if gib else None
+        p.build_kernels(uvw, 0.9)
+        del fill
+        torch.cuda.empty_cache()
+        c = p.csr()
+        results.append((p.phi(x), p.phi_adj(yv), c.col.clone(), c.val.clone()))
+        p.close()
+    (y0, z0, c0, v0), (y1, z1, c1, v1) = results
+    assert torch.equal(c0, c1) and torch.equal(v0, v1)
+    assert float((y1 - y0).norm() / y0.norm()) <= 1e-5
+    assert float((z1 - z0).norm() / z0.norm()) <= 1e-5
+
+
+def test_batch_without_room_for_slices(wp):
+    N, ms = 256, [60000] * 8
+    uvw = torch.cat([uvw_cells(i, m, N, 4.0) for i, m in enumerate(ms)])
+    x = torch.randn(8 * N * N, generator=torch.Generator().manual_seed(5)).cuda()
+    yv = torch.randn(sum(ms), dtype=torch.complex64, generator=torch.Generator().manual_seed(6)).cuda()
+    results = []
+    for gib in (None, 3.95):
+        b = wp.Batch([N] * 8, L)
+        fill = leave_free(gib) if gib else None
+        b.build_kernels(uvw, ms, 0.9)
+        del fill
+        torch.cuda.empty_cache()
+        results.append((b.phi(x), b.phi_adj(yv)))
+        b.close()
+    (y0, z0), (y1, z1) = results
+    assert float((y1 - y0).norm() / y0.norm()) <= 1e-5
+    assert float((z1 - z0).norm() / z0.norm()) <= 1e-5
