@@ -761,18 +761,19 @@ wproj_status batch_build_once(wproj_batch *b, const double *uvw, const int64_t *
     p = nullptr;
   }
   // ---- size classes, work buffers, a default schedule
+  std::vector<int32_t> by_size[kMaxLogN + 1];   // live until their copies have run
   for (int lg = 0; lg <= kMaxLogN; ++lg) {
     wproj_batch::Cls &c = b->cls[lg];
     c.np = 0;
     c.plist.release();
-    std::vector<int32_t> ids;
+    std::vector<int32_t> &ids = by_size[lg];
     for (int p = 0; p < np; ++p)
       if (b->prob[p].logG == lg) ids.push_back(p);
     if (ids.empty()) continue;
     c.logG = lg;
     c.np = (int)ids.size();
     WPROJ_TRY(c.plist.alloc(sizeof(int32_t) * ids.size()));
-    WPROJ_CUDA(cudaMemcpy(c.plist.ptr, ids.data(), sizeof(int32_t) * ids.size(), cudaMemcpyHostToDevice));
+    WPROJ_CUDA(cudaMemcpyAsync(c.plist.ptr, ids.data(), sizeof(int32_t) * ids.size(), cudaMemcpyHostToDevice, s));
   }
   WPROJ_TRY(b->Xt.alloc(sizeof(float2) * grid));
   WPROJ_TRY(b->Xt2.alloc(sizeof(float2) * grid));

@@ -1299,6 +1299,7 @@ static wproj_status build_g(wproj_plan *p, const double *uvw, int64_t m, double 
   TmpBuf tile_seg, tptr;
   bool want_runs = false;   // TILE_RUNS: emitted as columns, then transcoded
   int64_t n_rec = 0;        // TILE_RUNS: records (segments holding entries), tile order
+  int64_t total = 0;        // TILE_MASK: bytes of the records (lives until its copy has run)
 
   for (int phase = 1; phase <= 2; ++phase) {
     int64_t koff = 0;   // boxes transformed so far (position in Kall)
@@ -1349,7 +1350,6 @@ static wproj_status build_g(wproj_plan *p, const double *uvw, int64_t m, double 
         WPROJ_TRY(rsz.alloc(sizeof(int32_t) * std::max<int64_t>(1, n_seg)));
         WPROJ_TRY(p->rec_off.reuse(sizeof(int64_t) * (n_seg + 1)));
         WPROJ_TRY(p->seg_rec.reuse(sizeof(int64_t) * std::max<int64_t>(1, n_seg)));
-        int64_t total = 0;
         if (n_seg > 0) {
           k_rec_size<<<ceil_div(n_seg, 256), 256, 0, s>>>(n_seg, tile_seg.as<int32_t>(), p->seg_cnt.as<int32_t>(), vb,
                                                           rsz.as<int32_t>());
@@ -1364,7 +1364,7 @@ static wproj_status build_g(wproj_plan *p, const double *uvw, int64_t m, double 
                                                              p->seg_rec.as<int64_t>());
           WPROJ_CHECK_LAUNCH("record offsets");
         }
-        WPROJ_CUDA(cudaMemcpy(p->rec_off.as<int64_t>() + n_seg, &total, sizeof(int64_t), cudaMemcpyHostToDevice));
+        WPROJ_CUDA(cudaMemcpyAsync(p->rec_off.as<int64_t>() + n_seg, &total, sizeof(int64_t), cudaMemcpyHostToDevice, s));
         WPROJ_TRY(p->stream.reuse(std::max<int64_t>(16, total)));
         WPROJ_CUDA(cudaMemsetAsync(p->stream.ptr, 0, std::max<int64_t>(16, total), s));   // record padding
         p->stream_bytes = total;
@@ -1575,13 +1575,15 @@ static wproj_status build_g(wproj_plan *p, const double *uvw, int64_t m, double 
                                                   : sizeof(float2) * size_t(p->n_chunks) * g.tile * g.tile));
   }
   WPROJ_TRY(p->ytmp.reuse(sizeof(float2) * m));
+  // first segment of every row, closed by n_seg (per-row reduction of segment partials);
+  // on the build's stream like every copy here: the legacy stream's would still be under
+  // way when a later build writes the scratch block or an operator on s reads the result
+  WPROJ_TRY(p->seg_base.reuse(sizeof(int64_t) * (m + 1)));
+  WPROJ_CUDA(cudaMemcpyAsync(p->seg_base.ptr, d_segbase.ptr, sizeof(int64_t) * m, cudaMemcpyDeviceToDevice, s));
+  WPROJ_CUDA(cudaMemcpyAsync(p->seg_base.as<int64_t>() + m, &n_seg, sizeof(int64_t), cudaMemcpyHostToDevice, s));
   WPROJ_CUDA(cudaMemcpyAsync(&herr, d_err.ptr, sizeof(int), cudaMemcpyDeviceToHost, s));
   WPROJ_CUDA(cudaStreamSynchronize(s));
   if (herr & ERR_EMIT) return fail(WPROJ_ERR_CUDA, "build_kernels: emission pass disagrees with the counting pass");
-  // first segment of every row, closed by n_seg (per-row reduction of segment partials)
-  WPROJ_TRY(p->seg_base.reuse(sizeof(int64_t) * (m + 1)));
-  WPROJ_CUDA(cudaMemcpy(p->seg_base.ptr, d_segbase.ptr, sizeof(int64_t) * m, cudaMemcpyDeviceToDevice));
-  WPROJ_CUDA(cudaMemcpy(p->seg_base.as<int64_t>() + m, &n_seg, sizeof(int64_t), cudaMemcpyHostToDevice));
   p->m = m;
   p->n_seg = n_seg;
   p->built = true;

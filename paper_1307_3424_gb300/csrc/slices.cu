@@ -823,14 +823,15 @@ wproj_status build_slices(wproj_plan *p, const int2 *j0, const int32_t *Sk, cons
   WPROJ_TRY(c.g_idx.reuse(sizeof(uint16_t) * ge));
   WPROJ_TRY(c.g_val.reuse(vb * ge));
   WPROJ_TRY(c.g_rows.reuse(sizeof(int32_t) * std::max<int64_t>(1, c.g_nrows)));
+  std::vector<int32_t> multi;   // lives until its copy has run
   if (c.g_chunks > n_tiles) {
-    std::vector<int32_t> tcp(n_tiles + 1), multi;
+    std::vector<int32_t> tcp(n_tiles + 1);
     WPROJ_CUDA(cudaMemcpy(tcp.data(), c.tile_chunk_ptr.ptr, sizeof(int32_t) * tcp.size(), cudaMemcpyDeviceToHost));
     for (int t = 0; t < n_tiles; ++t)
       if (tcp[t + 1] - tcp[t] > 1) multi.push_back(t);
     c.n_multi = int64_t(multi.size());
     WPROJ_TRY(c.multi.reuse(sizeof(int32_t) * multi.size()));
-    WPROJ_CUDA(cudaMemcpy(c.multi.ptr, multi.data(), sizeof(int32_t) * multi.size(), cudaMemcpyHostToDevice));
+    WPROJ_CUDA(cudaMemcpyAsync(c.multi.ptr, multi.data(), sizeof(int32_t) * multi.size(), cudaMemcpyHostToDevice, s));
     if (!p->in_batch) WPROJ_TRY(c.partial.reuse(sizeof(float2) * 1024 * c.g_chunks));
   }
   WPROJ_CUDA(cudaMemsetAsync(c.d_idx.ptr, 0, sizeof(uint16_t) * de, s));

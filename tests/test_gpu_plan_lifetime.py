@@ -156,3 +156,33 @@ def test_batch_without_room_for_slices(wp):
     (y0, z0), (y1, z1) = results
     assert float((y1 - y0).norm() / y0.norm()) <= 1e-5
     assert float((z1 - z0).norm() / z0.norm()) <= 1e-5
+
+
+# operators launched right after a build, on the build's own stream (which the legacy
+# stream does not order): every table that the build wrote is complete.  Segment lists
+# of the tile stream, tiles of several chunks on slices, a batch's size classes
+@pytest.mark.parametrize("box,fmt,N,M", [("G", "mask", 64, 3000), ("rule", "auto", 64, 8000), ("batch", "", 64, 2000)])
+def test_operators_right_after_a_build(wp, box, fmt, N, M):
+    side = torch.cuda.Stream()
+    uvws = [uvw_cells(i, M, N, 2.0) for i in range(6)]
+    if box == "batch":
+        op = wp.Batch([N, 32], L)
+        build = lambda u: op.build_kernels(u, [M - 300, 300], 0.9, stream=side)
+        x = torch.randn(op.pixels, generator=torch.Generator().manual_seed(7)).cuda()
+    else:
+        op = wp.Plan(N, L, box=box, index_format=fmt)
+        build = lambda u: op.build_kernels(u, 0.9, stream=side)
+        x = torch.randn(N, N, generator=torch.Generator().manual_seed(7)).cuda()
+    if box == "batch":      # the second problem's band is half as wide
+        for u in uvws:
+            u[M - 300:, :2] *= 0.5
+    yv = torch.randn(M, dtype=torch.complex64, generator=torch.Generator().manual_seed(8)).cuda()
+    y, z = torch.empty_like(yv), torch.empty_like(x)
+    torch.cuda.synchronize()
+    for u in uvws:
+        build(u)
+        op.phi(x, y, stream=side)
+        op.phi_adj(yv, z, stream=side)
+        torch.cuda.synchronize()
+        assert torch.equal(op.phi(x), y) and torch.equal(op.phi_adj(yv), z)
+    op.close()
