@@ -11,8 +11,8 @@
 //
 // Layers 2-4 and all their gradients are BF16 GEMMs on the tcgen05 tensor cores
 // (gemm.cu) with FP32 accumulation; the 3-wide first layer runs on the FP32
-// cores.  Master parameters, Adam moments and all reductions are FP32 (bias
-// gradients and losses are summed in a fixed order).  Activations and the
+// cores.  Master parameters, Adam moments and the gradients' reductions are FP32,
+// the loss is summed to FP64 precision, all in a fixed order.  Activations and the
 // gradients fed to GEMMs are rounded to BF16.  GELU is the erf form.
 #include <math.h>
 
@@ -119,32 +119,37 @@ __device__ __forceinline__ void put_bf16x4(__nv_bfloat16 *p, __nv_bfloat162 a, _
   *reinterpret_cast<uint2 *>(p) = u;
 }
 
-// A sum in two floats: every addition keeps its error (Knuth's two-sum) and every
-// square its rounding (fma), so the pair carries about 48 bits; magnitudes at
-// which that could overflow or underflow, and non-finite ones, go to FP64.  FP64
-// per element (a convert, an FMA and a divide) took 263 us for 4096 x 3072 losses.
-struct Sum2 {
-  float hi = 0.f, lo = 0.f;
+// A sum in three floats: every addition keeps its error (Knuth's two-sum), once more in
+// the next word, and every square its rounding (fma), so a thread's 16 terms lose nothing
+// that FP64 would keep (two words carry 48 bits: up to 117 units of 2^-53 off on 16 equal
+// magnitudes, three 0); magnitudes at which that could overflow or underflow, and
+// non-finite ones, go to FP64.  FP64 per element (a convert, an FMA and a divide) took
+// 263 us for 4096 x 3072 losses.
+struct Sum3 {
+  float hi = 0.f, lo = 0.f, lo2 = 0.f;
   double wide = 0;
-  __device__ __forceinline__ void two_sum(float v) {
-    const float t = __fadd_rn(hi, v), z = __fsub_rn(t, hi);
-    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(v, z)));
-    hi = t;
+  // s + v -> s, the rounding error returned
+  static __device__ __forceinline__ float two_sum(float &s, float v) {
+    const float t = __fadd_rn(s, v), z = __fsub_rn(t, s);
+    const float err = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v, z));
+    s = t;
+    return err;
   }
+  __device__ __forceinline__ void low(float v) { lo2 = __fadd_rn(lo2, two_sum(lo, v)); }
   __device__ __forceinline__ void add(float v) {
-    if (fabsf(v) <= 1e30f) two_sum(v);
+    if (fabsf(v) <= 1e30f) low(two_sum(hi, v));
     else wide += double(v);
   }
   __device__ __forceinline__ void add_square(float a) {
     const float p = __fmul_rn(a, a);
     if (p >= 1e-30f && p <= 1e30f) {
-      lo = __fadd_rn(lo, __fmaf_rn(a, a, -p));
-      two_sum(p);
+      low(__fmaf_rn(a, a, -p));
+      low(two_sum(hi, p));
     } else if (a != 0.f) {
       wide += double(a) * a;
     }
   }
-  __device__ __forceinline__ double value() const { return double(hi) + double(lo) + wide; }
+  __device__ __forceinline__ double value() const { return (double(hi) + (double(lo) + double(lo2))) + wide; }
 };
 
 // Loss partials and dY = d loss / d y as BF16 rows, its transpose and its column
@@ -164,7 +169,7 @@ k_loss(int64_t B, const float *__restrict__ Y, const float *__restrict__ Tv, con
   const float s = is_val ? 2.f / float(B * kOutV) : mask_weight / float(B * kOutM);
   const float *T = is_val ? Tv + c0 : Tm + (c0 - kOutV);
   const int ldt = is_val ? kOutV : kOutM;
-  Sum2 acc;
+  Sum3 acc;
   float cs[4] = {0.f, 0.f, 0.f, 0.f};
   float4 yv[4], tv[4];
 #pragma unroll
@@ -211,7 +216,7 @@ k_loss(int64_t B, const float *__restrict__ Y, const float *__restrict__ Tv, con
   const double t = block_sum_d<256>(acc.value());
   if (threadIdx.x == 0)
     part[int64_t(blockIdx.y) * gridDim.x + blockIdx.x] =
-        t * (is_val ? 1.0 / double(B * kOutV) : double(mask_weight) / double(B * kOutM));
+        is_val ? t / double(B * kOutV) : double(mask_weight) * t / double(B * kOutM);
 }
 
 __global__ void __launch_bounds__(1024) k_sum_part_d(const double *__restrict__ part, int n, double *__restrict__ out) {
