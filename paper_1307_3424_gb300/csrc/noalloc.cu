@@ -76,6 +76,6 @@ extern "C" wproj_status wproj_phi_noalloc(wproj_plan *p, const float *x, void *y
     p->launches += p->g.upsampling ? 4 : 2;
     WPROJ_TRY(phi_forward_fft_into(p, x, inter, Xt, s));
   }
-  p->launches += 2;
+  p->launches += degrid_launches(p);
   return degrid_into(p, Xt, partial, static_cast<float2 *>(y), s);
 }

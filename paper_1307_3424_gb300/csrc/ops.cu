@@ -303,8 +303,10 @@ wproj_status launch_degrid_cols(wproj_plan *p, const float2 *Xt, float2 *partial
 
 }  // namespace
 
+int degrid_launches(const wproj_plan *p) { return p->slices.use || p->fmt == WPROJ_INDEX_TILE_RUNS ? 1 : 2; }
+
 wproj_status degrid(wproj_plan *p, const float2 *Xt, float2 *y, cudaStream_t s) {
-  p->launches += p->slices.use || p->fmt == WPROJ_INDEX_TILE_RUNS ? 1 : 2;
+  p->launches += degrid_launches(p);
   return degrid_into(p, Xt, p->piece_partial.as<float2>(), y, s);
 }
 

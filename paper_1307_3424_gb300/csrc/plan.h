@@ -321,6 +321,7 @@ wproj_status batch_idwt2(const BProb *tab, int np, int maxN, int levels, int p, 
 
 // ops.cu
 wproj_status degrid(wproj_plan *p, const float2 *Xt, float2 *y, cudaStream_t s);
+int degrid_launches(const wproj_plan *p);   // kernels of one degridding
 wproj_status degrid_into(wproj_plan *p, const float2 *Xt, float2 *partial, float2 *y, cudaStream_t s);
 wproj_status csr_rows(const wproj_plan *p, int64_t k0, int64_t k1, int32_t *col_out, void *val_out,
                       cudaStream_t s);

@@ -186,3 +186,22 @@ def test_operators_right_after_a_build(wp, box, fmt, N, M):
         torch.cuda.synchronize()
         assert torch.equal(op.phi(x), y) and torch.equal(op.phi_adj(yv), z)
     op.close()
+
+
+# the launch count of wproj_phi_noalloc is wproj_phi's: one degridding kernel on slices and
+# run lengths, two on the column form and the tile stream
+@pytest.mark.parametrize("M,wmax,box,fmt,value", [(900, 1.0, "rule", "auto", "f32"), (900, 1.0, "rule", "columns", "bf16"),
+                                                  (9, 3.0, "rule", "auto", "f32"), (9, 3.0, "rule", "columns", "f32"),
+                                                  (90, 1.0, "G", "mask", "f32")])
+def test_launch_counts(wp, M, wmax, box, fmt, value):
+    N = 64
+    p = wp.Plan(N, L, box=box, index_format=fmt, value_dtype=value)
+    p.build_kernels(uvw_cells(0, M, N, wmax), 0.99)
+    x, y = torch.zeros(N, N, device="cuda"), torch.empty(M, dtype=torch.complex64, device="cuda")
+    counts = []
+    for call in (wp.lib().wproj_phi, wp.lib().wproj_phi_noalloc):
+        before = p.stats()["launches"]
+        assert call(p.handle, x.data_ptr(), y.data_ptr(), torch.cuda.current_stream().cuda_stream) == wp.OK
+        counts.append(p.stats()["launches"] - before)
+    assert counts[0] == counts[1]
+    p.close()
