@@ -314,6 +314,19 @@ def run_reference(args):
 # ---------------------------------------------------------------------------------
 
 
+def operator_form(fmt, slices, nnz, b_val, runs_bytes, stream_bytes):
+    """(degridding kernel, gridding kernel, bytes of G that each reads): labels as in
+    profiles/; slices where the library says that the operators read them, else values +
+    4-byte indices (columns), run lengths or tile-stream records."""
+    if slices["used"]:
+        return "k_slice_degrid", "k_slice_grid", slices["degrid_bytes"], slices["grid_bytes"]
+    if fmt == "columns":
+        return "k_degrid", "k_grid_cells", nnz * (b_val + 4), nnz * (b_val + 4)
+    if fmt == "runs":
+        return "k_runs_degrid", "k_runs_grid", runs_bytes, stream_bytes
+    return "k_stream_degrid", "k_stream_grid", stream_bytes, stream_bytes
+
+
 def read_profile_traffic(kernel: str, key: str = "traffic_bytes_per_launch"):
     """DRAM traffic of a kernel from a committed ncu summary in profiles/ (line
     '<key>: <n>' under '## <kernel>': per launch, or per entry of G)."""
@@ -355,6 +368,7 @@ def run_ours(args):
     st = plan.stats()
     csrv = plan.csr()
     fmt, n_seg, stream_bytes = csrv.index_format, csrv.n_seg, csrv.stream_bytes
+    sl = plan.slices()
     del csrv
     nnz, M, G = st["nnz"], st["m"], plan.G
 
@@ -436,22 +450,7 @@ def run_ours(args):
     grid_ms = kst["t_grid_ms"] / max(1, kst["n_grid"])
     alg_deg = nnz * b_val + M * 8 + G * G * 8
     alg_grid = nnz * b_val + M * 8 + G * G * 8
-    # G as each operator reads it: the slices of short rows (values + 2-byte indices,
-    # pads not counted), values + column indices, or the tile-stream records
-    slices = fmt != "mask" and st["box_max"] <= 64
-    if slices:
-        stored_deg = stored_grid = nnz * (b_val + 2)
-    elif fmt == "columns":
-        stored_deg = stored_grid = nnz * (b_val + 4)
-    elif fmt == "runs":
-        stored_deg, stored_grid = st["runs_bytes"], stream_bytes
-    else:
-        stored_deg = stored_grid = stream_bytes
-    # kernel labels as in profiles/
-    deg_name, grid_name = {"mask": ("k_stream_degrid", "k_stream_grid"), "runs": ("k_runs_degrid", "k_runs_grid"),
-                           "columns": ("k_degrid", "k_grid_cells")}[fmt]
-    if slices:
-        deg_name, grid_name = "k_slice_degrid", "k_slice_grid"
+    deg_name, grid_name, stored_deg, stored_grid = operator_form(fmt, sl, nnz, b_val, st["runs_bytes"], stream_bytes)
     if args.workload == "precision":   # the traffic figures in profiles/ are per workload
         deg_name += f"_precision_{args.value_dtype}"
         grid_name += f"_precision_{args.value_dtype}"
@@ -484,7 +483,7 @@ def run_ours(args):
             "warmup": args.warmup, "ms_per_step": t_ms / args.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": workload_config(wl, e, {"nnz": nnz, "segments": n_seg, "G_bytes": stored_deg + (
-                                              stored_grid if fmt == "runs" else 0), "index_format": fmt,
+                                              stored_grid if sl["used"] or fmt == "runs" else 0), "index_format": fmt,
                                               "value_dtype": args.value_dtype,
                                               "l2": "inputs larger than L2 (G exceeds L2 many times)",
                                               "parallelism": f"replicas x{ws}"}),
@@ -607,7 +606,8 @@ def run_batched(args):
     alg = info["nnz"] * 8 + info["m"] * 8 + grid_cells * 8
     dom = "grid" if sched["grid_ms"] >= sched["degrid_ms"] else "degrid"
     ms_dom = max(sched["grid_ms"], sched["degrid_ms"])
-    kname = "k_slice_grid_batch" if dom == "grid" else "k_slice_degrid_batch"   # labels as in profiles/
+    names = operator_form("columns", b.slices(), info["nnz"], 8, 0, 0)
+    kname = names[dom == "grid"] + "_batch"
     tr = read_profile_traffic(kname, "traffic_bytes_per_entry")   # from a smaller capture
     traffic = tr * info["nnz"] if tr is not None else None
     value = PAIRS_PER_STEP * args.steps / (t_ms * 1e-3)

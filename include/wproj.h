@@ -355,6 +355,12 @@ wproj_status wproj_set_timing(wproj_plan *p, int32_t enable);
 wproj_status wproj_get_stats(wproj_plan *p, wproj_stats *out);   /* synchronises */
 wproj_status wproj_reset_stats(wproj_plan *p);
 
+/* Whether the operators of the built G read interleaved slices (see
+ * wproj_index_format; a plan too sparse for them, or built with too little memory left,
+ * does without), and the bytes of G that a degridding and a gridding then read: values,
+ * indices, pads and the slices' tables (0 without slices).  Any pointer may be NULL. */
+wproj_status wproj_get_slices(const wproj_plan *p, int32_t *used, int64_t *degrid_bytes, int64_t *grid_bytes);
+
 /* Default DR parameters. */
 void wproj_dr_defaults(wproj_dr_params *prm);
 
@@ -511,6 +517,8 @@ wproj_status wproj_batch_phi_adj(wproj_batch *b, const void *y, float *x_re, voi
 wproj_status wproj_batch_solve_bpdn(wproj_batch *b, const void *y, const double *eps, const wproj_dr_params *prm,
                                     float *x_out, void *stream);
 wproj_status wproj_batch_get_info(const wproj_batch *b, wproj_batch_info *out);
+/* As wproj_get_slices, for all problems together. */
+wproj_status wproj_batch_get_slices(const wproj_batch *b, int32_t *used, int64_t *degrid_bytes, int64_t *grid_bytes);
 
 #ifdef __cplusplus
 }

@@ -379,6 +379,16 @@ wproj_status wproj_set_timing(wproj_plan *p, int32_t enable) {
   return WPROJ_OK;
 }
 
+wproj_status wproj_get_slices(const wproj_plan *p, int32_t *used, int64_t *degrid_bytes, int64_t *grid_bytes) {
+  WPROJ_TRY(check_built(p));
+  const int vbytes = p->g.value_dtype == WPROJ_VAL_F32 ? 8 : 4;
+  const bool u = p->slices.use;
+  if (used) *used = u;
+  if (degrid_bytes) *degrid_bytes = u ? p->slices.degrid_bytes(vbytes) : 0;
+  if (grid_bytes) *grid_bytes = u ? p->slices.grid_bytes(vbytes) : 0;
+  return WPROJ_OK;
+}
+
 wproj_status wproj_reset_stats(wproj_plan *p) {
   if (!p) return fail(WPROJ_ERR_INVALID_ARG, "null plan");
   fold_timer(p);
@@ -415,7 +425,7 @@ wproj_status wproj_get_stats(wproj_plan *p, wproj_stats *out) {
   out->n_build_fft = p->timer.count[TC_BFFT];
   const int vbytes = p->g.value_dtype == WPROJ_VAL_F32 ? 8 : 4;
   out->runs_bytes = p->fmt != WPROJ_INDEX_TILE_RUNS ? 0
-                    : p->slices.use                 ? p->slices.d_steps * 32 * (vbytes + 2) + p->slices.d_slices * 24
+                    : p->slices.use                 ? p->slices.degrid_bytes(vbytes)
                                                     : p->rm_vals * vbytes + p->rm_runs * 4 + p->m * 20;
   return WPROJ_OK;
 }

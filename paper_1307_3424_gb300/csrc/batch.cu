@@ -1023,6 +1023,14 @@ wproj_status wproj_batch_solve_bpdn(wproj_batch *b, const void *y, const double 
   return batch_solve_impl(b, static_cast<const float2 *>(y), eps, q, x_out, as_stream(stream));
 }
 
+wproj_status wproj_batch_get_slices(const wproj_batch *b, int32_t *used, int64_t *degrid_bytes, int64_t *grid_bytes) {
+  if (!b || !b->built) return fail(WPROJ_ERR_NOT_BUILT, "batch_get_slices: build the batch first");
+  if (used) *used = b->has_slices;
+  if (degrid_bytes) *degrid_bytes = b->has_slices ? b->slices.degrid_bytes(sizeof(float2)) : 0;
+  if (grid_bytes) *grid_bytes = b->has_slices ? b->slices.grid_bytes(sizeof(float2)) : 0;
+  return WPROJ_OK;
+}
+
 wproj_status wproj_batch_get_info(const wproj_batch *b, wproj_batch_info *out) {
   if (!b || !out) return fail(WPROJ_ERR_INVALID_ARG, "batch_get_info: null argument");
   out->n_problems = b->np;

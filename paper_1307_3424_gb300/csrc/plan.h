@@ -136,6 +136,8 @@ struct SliceCopy {
   int64_t d_chunks = 0, d_slices = 0, d_steps = 0, g_chunks = 0, g_steps = 0, g_nrows = 0, n_multi = 0;
   size_t d_smem = 0, g_smem = 0;
   SliceOps ops() const;
+  int64_t degrid_bytes(int value_bytes) const;   // of G, read by one pass
+  int64_t grid_bytes(int value_bytes) const;
   void release();
 };
 

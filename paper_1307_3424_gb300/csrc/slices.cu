@@ -701,6 +701,15 @@ SliceOps SliceCopy::ops() const {
   return o;
 }
 
+// values and indices; bounds and rows of a slice; base and patch of a chunk
+int64_t SliceCopy::degrid_bytes(int value_bytes) const {
+  return d_steps * 32 * (value_bytes + 2) + d_slices * (8 + 4 * kRps) + d_chunks * (8 + 16);
+}
+// values and indices; row lists; the cells' order, the slices' and the chunk's bounds
+int64_t SliceCopy::grid_bytes(int value_bytes) const {
+  return g_steps * 32 * (value_bytes + 2) + g_nrows * 4 + g_chunks * (2 * 1024 + 33 * 4 + 8 + 8 + 4);
+}
+
 void SliceCopy::release() {
   use = false;
   for (DevBuf *b : {&d_slice_base, &slice_ptr, &srow, &rect, &d_idx, &d_val, &g_chunk_tile, &g_chunk_lo, &g_chunk_hi,

@@ -34,6 +34,7 @@ EXPORTED = [
     "wproj_mlp_destroy", "wproj_mlp_set_params", "wproj_mlp_get_params", "wproj_mlp_targets",
     "wproj_mlp_forward", "wproj_mlp_gradients", "wproj_mlp_train", "wproj_build_kernels_learned",
     "wproj_daubechies_taps", "wproj_dwt2", "wproj_idwt2", "wproj_set_screens", "wproj_build_kernels_dde",
+    "wproj_get_slices", "wproj_batch_get_slices",
 ]
 
 
@@ -134,6 +135,8 @@ def lib() -> ctypes.CDLL:
         "wproj_set_timing": [vp, i32],
         "wproj_get_stats": [vp, P(Stats)],
         "wproj_reset_stats": [vp],
+        "wproj_get_slices": [vp, P(i32), P(i64), P(i64)],
+        "wproj_batch_get_slices": [vp, P(i32), P(i64), P(i64)],
         "wproj_dr_state_get": [vp, vp, vp, P(dbl), P(dbl), vp],
         "wproj_dr_state_set": [vp, vp, vp, dbl, dbl, vp],
         "wproj_batch_create": [P(vp), i32, P(GridDesc)],
@@ -202,6 +205,12 @@ class _CAI:
     def __init__(self, ptr: int, shape: tuple, typestr: str):
         self.__cuda_array_interface__ = {"data": (ptr, False), "shape": shape,
                                          "typestr": typestr, "version": 2, "strides": None}
+
+
+def _slices(fn, h) -> dict:
+    used, d, g = ctypes.c_int32(), ctypes.c_int64(), ctypes.c_int64()
+    _check(fn(h, ctypes.byref(used), ctypes.byref(d), ctypes.byref(g)))
+    return {"used": bool(used.value), "degrid_bytes": d.value, "grid_bytes": g.value}
 
 
 def dr_defaults() -> DRParams:
@@ -440,6 +449,11 @@ class Plan:
         _check(lib().wproj_get_stats(self._h, ctypes.byref(s)))
         return s.as_dict()
 
+    def slices(self) -> dict:
+        """used: whether the operators read interleaved slices; degrid_bytes, grid_bytes:
+        of G, read by one pass then (0 without slices)."""
+        return _slices(lib().wproj_get_slices, self._h)
+
     def reset_stats(self):
         _check(lib().wproj_reset_stats(self._h))
 
@@ -549,6 +563,10 @@ class Batch:
         out = BatchInfo()
         _check(lib().wproj_batch_get_info(self._h, ctypes.byref(out)))
         return {f: getattr(out, f) for f, _ in out._fields_}
+
+    def slices(self) -> dict:
+        """As Plan.slices, for all problems together."""
+        return _slices(lib().wproj_batch_get_slices, self._h)
 
     def phi(self, x: torch.Tensor, y: torch.Tensor | None = None, stream=None) -> torch.Tensor:
         if x.dtype != torch.float32 or x.numel() != self.pixels:

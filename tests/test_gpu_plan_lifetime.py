@@ -205,3 +205,31 @@ def test_launch_counts(wp, M, wmax, box, fmt, value):
         counts.append(p.stats()["launches"] - before)
     assert counts[0] == counts[1]
     p.close()
+
+
+# which form serves a plan or batch: slices for short rows, except where their patches would
+# hold more than four cells an entry, and nowhere else; the bytes are at least those of the
+# entries' values and 2-byte indices
+@pytest.mark.parametrize("N,M,wmax,box,fmt,value,used", [
+    (64, 900, 1.0, "rule", "auto", "f32", True), (64, 900, 1.0, "rule", "runs", "bf16", True),
+    (64, 900, 1.0, "rule", "columns", "f16", True), (512, 9, 3.0, "rule", "auto", "f32", False),
+    (512, 9, 3.0, "rule", "columns", "bf16", False), (64, 90, 1.0, "G", "mask", "f32", False),
+    (64, 90, 1.0, "G", "columns", "f32", False), (8, 40, 1.0, "rule", "auto", "f32", False)])
+def test_slices_reported(wp, N, M, wmax, box, fmt, value, used):
+    p = wp.Plan(N, L, box=box, index_format=fmt, value_dtype=value)
+    p.build_kernels(uvw_cells(0, M, N, wmax), 0.99)
+    s = p.slices()
+    least = p.csr().nnz * ((8 if value == "f32" else 4) + 2)
+    assert s["used"] == used
+    assert (min(s["degrid_bytes"], s["grid_bytes"]) >= least) if used else (s["degrid_bytes"] == s["grid_bytes"] == 0)
+    p.close()
+
+
+@pytest.mark.parametrize("ns,used", [((64, 32), True), ((64, 8), False)])
+def test_batch_slices_reported(wp, ns, used):
+    b = wp.Batch(ns, L)
+    b.build_kernels(torch.cat([uvw_cells(n, 5 * n, n, 1.0) for n in ns]), [5 * n for n in ns], 0.99)
+    s = b.slices()
+    assert s["used"] == used
+    assert (min(s["degrid_bytes"], s["grid_bytes"]) >= 10 * b.info()["nnz"]) if used else s["grid_bytes"] == 0
+    b.close()
