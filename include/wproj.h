@@ -123,8 +123,12 @@ typedef struct {
  * rows in CSR order from every format.
  * Where every box is at most 64 x 64 cells, COLUMNS and TILE_RUNS plans also hold
  * interleaved slices of the values with 2-byte local indices, which the operators
- * read instead (the row-major runs are then not stored); plans too sparse for them
- * (patches of more than 4 cells an entry, pads of more than the entries) do without. */
+ * read instead (the row-major runs and the cell-major copy are then not stored); plans
+ * too sparse for them (patches of more than 4 cells an entry, pads of more than the
+ * entries) do without, and so do plans and batches that the device has no room for with
+ * them.  Two copies of 10 bytes an entry (f32; 16-bit 6) and pads: with the column form
+ * about 32 (20) bytes an entry in all, with run lengths about 29, where the forms without
+ * slices take 24 (16) and 17. */
 typedef enum {
   WPROJ_INDEX_AUTO = 0,
   WPROJ_INDEX_COLUMNS = 1,

@@ -150,9 +150,12 @@ __host__ __device__ constexpr uint32_t instr_desc(int M, int N) {
 
 // BN: tile columns (128 or 256); a tile's accumulator takes BN tensor-memory
 // columns, two of them 2 BN (512 at most: the whole tensor memory).
-// ST stages, OB staging blocks a warp: three stages and two blocks for short K (the
-// epilogue bounds it), four and one for long K (8192^3: 1431 TFLOP/s, 1282 with three
-// stages), four and two at 128 columns.
+// ST stages, OB staging blocks a warp: three stages and two blocks for at most 8 slices
+// of K, where the epilogue bounds it and the second block helps a GELU's (20480 x 256:
+// 43 against 45 us), four and one for longer K (8192^3: 768 us against 853 with three
+// stages, 65536 x 3072 x 1024: 357 against 382), four and two at 128 columns.  65536 x
+// 3072, three stages and four: K = 256 (the network's) 181 and 175 us, 384 232 and 208,
+// 512 261 and 246; 4096 x 4096 x 512: 56 and 59.
 template <int BN, int ST, int OB>
 struct GemmSmem {
   static constexpr int kStages = ST, kOutBufs = OB;

@@ -27,7 +27,9 @@ struct DevBuf {
   }
   virtual wproj_status alloc(size_t n);   // exact size, contents undefined
   wproj_status ensure(size_t n);          // grow (contents discarded)
-  wproj_status reuse(size_t n);           // keep an allocation of n to 9/8 n bytes, else as alloc
+  // keep an allocation of n to 9/8 n bytes, else as alloc: other draws of a problem's (u, v)
+  // differ by a few per cent in the size of G, and no more than an eighth stays unused
+  wproj_status reuse(size_t n);
   template <class T> T *as() const { return static_cast<T *>(ptr); }
 };
 
@@ -124,8 +126,11 @@ struct SliceOps {
   const BProb *tab = nullptr;
 };
 
-// Patch cells a plan's chunks may have per stored entry before the other forms
-// are the faster ones.
+// Patch cells a plan's chunks may have per stored entry before the other forms are as
+// fast.  Phi + Phi^H on a 4096^2 grid, rows of ~275 entries, slices and the other forms:
+// below the line 493 and 503 us (f32, 100000 rows), 470 and 494 (bf16); beyond it, with
+// 30000 rows, 422 and 414, 410 and 382.  Fewer rows still (10000: 362 and 379, 356 and
+// 345) leave the transforms most of the time.  Batches have no such line: see slices.cu.
 constexpr int64_t kPatchCellsPerEntry = 4;
 
 struct SliceCopy {

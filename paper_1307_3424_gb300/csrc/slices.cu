@@ -31,6 +31,22 @@
 // instead of two (1.08 / 0.86 ms); a warp's four cell slices one after another
 // (gridding 0.97 / 0.75 ms, 204 against 167 us on the batch).
 //
+// Which plans take them: single plans up to kPatchCellsPerEntry patch cells an entry and
+// pads up to the entries.  Rows of 1 to 4 entries take 8 places in the degridding's copy,
+// several times the column form's bytes: Phi + Phi^H of 2e6 such rows on a 2048^2 grid
+// 252 us on slices and 185 in the column form in bf16 (243 and 984 with run lengths in
+// f32, the line's dear side).  Batches have neither line and need less memory on slices
+// (64 sparse problems of N = 256: 424 to 514 MB, 508 to 580 without).  64 problems with
+// and without slices: N = 64, 40 to 400 rows each, 28 to 38 us and 33 to 46; N = 256,
+// 6000 rows of 78 entries, 409 and 443; N = 256, 60 to 600 rows or rows of 1 to 6
+// entries, 260 to 336 and 249 to 305: sparse problems on large grids are the dear side.
+//
+// Chunk sizes: 6 to 24 (degridding) and 8 to 16 (gridding) blocks an SM are within 7 %, 32
+// for the gridding up to 80 % slower; at least 4096 entries: 2048 is 20 to 32 % slower on
+// 64^2 and 7 to 12 % on 256^2 images; a batch's 16384: 8192 makes its gridding 30 %
+// slower; at most 262144: 65536 makes the gridding of 5.8e8 entries 13 to 18 % slower,
+// 1048576 is the same.
+//
 // Building them (262144 rows, 7e7 entries): two stable sorts of the rows, a sort of each
 // tile's cells (keys in registers, 15 of the 55 exchanges through shared memory: 0.2 ms)
 // and two passes that place the values, ~2 ms of a build of 27.9 ms.
@@ -782,7 +798,7 @@ wproj_status build_slices(wproj_plan *p, const int2 *j0, const int32_t *Sk, cons
   WPROJ_CUDA(read(&words, stat.ptr, sizeof(int)));
   WPROJ_CUDA(cudaStreamSynchronize(s));
   // Worth it while the patches' cells (read from L2 once a pass) and the pads are not
-  // many times the entries, and a chunk's y fits shared memory.
+  // many times the entries (single plans only, see above), and a chunk's y fits shared memory.
   const int64_t nnz = std::max<int64_t>(1, p->nnz);
   if (!p->in_batch && n_cells > kPatchCellsPerEntry * nnz) {
     c.release();
