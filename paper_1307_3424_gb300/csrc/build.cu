@@ -1243,7 +1243,9 @@ static wproj_status build_g(wproj_plan *p, const double *uvw, int64_t m, double 
   // of them (and, with a margin, for G in the form that pass 2 writes, at most 1.5x
   // their size), pass 1 keeps them and pass 2 emits without recomputing the tables and
   // FFTs; otherwise pass 2 recomputes them batch by batch.  They are given back before
-  // the copies of G (slices, run lengths, cells) are made.
+  // the copies of G (slices, run lengths, cells) are made: room for those, and the first
+  // operators after the build are faster (a pair on 5.8e8 bf16 entries 1.62 ms, 2.87 when
+  // the boxes are freed last).
   int64_t k_total = 0;
   for (int c = 0; c < 9; ++c) k_total += (cls_ptr[c + 1] - cls_ptr[c]) * int64_t(16 << c) * (16 << c) * int64_t(sizeof(float2));
   DevBuf Kall;
